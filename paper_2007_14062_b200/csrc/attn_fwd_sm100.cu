@@ -693,7 +693,9 @@ __device__ __forceinline__ void mma_role(const KernelParams& p, SmemCtl* ctl, co
         if (fail) break;
         if (last) {
             tc_commit(&sc->q_empty[qs]);        // every Q K^T of the tile has been issued
-            pend_last = tile_steps;             // the tile's last P V is the pending one (the tile's last segment may be empty)
+            // the tile's last P V is the pending one (the tile's last segment may be empty); a tile without any step (a part
+            // of a split tile whose keys are all padding) leaves the mark of the tile before it alone
+            pend_last = pend_last || tile_steps;
         }
         mbar_arrive(&sc->sched_empty[ss]);
         ++sched_n;

@@ -181,6 +181,19 @@ def test_closed_forms_on_gpu(impl, dtype):
         assert np.abs(out[0, h][valid] - mean[valid]).max() <= TOL_OUT[dtype]
 
 
+def test_split_tiles_whose_parts_are_entirely_padding():
+    """A long layout with short sequences: most parts of the split global tiles have no key left, and a stream of work meets
+    them right behind parts that have some."""
+    wl = _small("bf16", 16, 4, 130)
+    q, k, v = synth.make_qkv(wl)
+    kpm = torch.zeros((wl.B, wl.N), dtype=torch.uint8)
+    for bi in range(wl.B):
+        kpm[bi, :300 + 170 * bi] = 1
+    out, lse = _run(wl, q, k, v, kpm)
+    rows = np.concatenate([np.arange(0, 192), np.arange(230, 330), np.arange(wl.N - 64, wl.N)])
+    _compare(wl, q, k, v, kpm, out, lse, slices=[(0, 0), (7, 2), (15, 3)], rows=rows)
+
+
 def test_two_runs_are_bit_identical():
     wl = _small("bf16", 2, 4, 16, lengths="ragged:128:1024")
     q, k, v = synth.make_qkv(wl)
