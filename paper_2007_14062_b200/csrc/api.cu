@@ -4,6 +4,8 @@
 
 #include <mutex>
 #include <new>
+#include <utility>
+#include <vector>
 
 #include "kernels.h"
 #include "../../include/bigbird.h"
@@ -41,23 +43,79 @@ int get_scratch(int device, DeviceScratch** out) {
     return BIGBIRD_OK;
 }
 
-template <typename T>
-cudaError_t upload(T** dst, const void* src, size_t count) {
-    *dst = nullptr;
-    cudaError_t e = cudaMalloc((void**)dst, (count ? count : 1) * sizeof(T));
-    if (e != cudaSuccess || count == 0) return e;
-    return cudaMemcpy(*dst, src, count * sizeof(T), cudaMemcpyHostToDevice);
+// Memory pool of a device: workspaces of calls come from it in stream order, so calls on different streams or threads never
+// share one.  It keeps up to 64 MB between calls; it is made with the first use and destroyed with the last layout that has a
+// copy on the device (what a call still in flight holds goes when that call is done).
+struct DevicePool {
+    cudaMemPool_t pool = nullptr;
+    int layouts = 0;
+};
+DevicePool g_pools[kMaxDevices];
+
+int hold_pool(int device) {
+    if (device < 0 || device >= kMaxDevices) return BIGBIRD_EUNSUPPORTED;
+    std::lock_guard<std::mutex> lock(g_mu);
+    ++g_pools[device].layouts;
+    return BIGBIRD_OK;
+}
+void release_pool(int device) {
+    std::lock_guard<std::mutex> lock(g_mu);
+    DevicePool& d = g_pools[device];
+    if (--d.layouts == 0 && d.pool) {
+        cudaMemPoolDestroy(d.pool);
+        d.pool = nullptr;
+    }
+}
+int get_pool(int device, cudaMemPool_t* out) {
+    std::lock_guard<std::mutex> lock(g_mu);
+    DevicePool& d = g_pools[device];
+    if (!d.pool) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.handleTypes = cudaMemHandleTypeNone;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        cudaError_t e = cudaMemPoolCreate(&d.pool, &props);
+        if (e != cudaSuccess) { d.pool = nullptr; return cuda_fail(e); }
+        uint64_t keep = 64ull << 20;
+        e = cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e != cudaSuccess) return cuda_fail(e);
+    }
+    *out = d.pool;
+    return BIGBIRD_OK;
 }
 
 void free_device_layout(DeviceLayout& d) {
-    cudaFree(d.row_ptr);
-    cudaFree(d.col_idx);
-    cudaFree(d.col_ptr);
-    cudaFree(d.row_idx);
-    cudaFree(d.items);
-    cudaFree(d.steps);
-    cudaFree(d.split_tile_q);
+    cudaFree(d.block);
+    if (d.device >= 0) release_pool(d.device);
     d = DeviceLayout{};
+}
+
+// Device copy of the layout: one allocation, one copy.
+cudaError_t upload_layout(const bigbird_layout* L, DeviceLayout& d) {
+    std::vector<unsigned char> host;
+    std::vector<std::pair<void**, size_t>> at;               // where each array's device address goes, and its offset
+    auto put = [&](auto** dst, const auto& v) {
+        host.resize((host.size() + 255) / 256 * 256);
+        at.emplace_back((void**)dst, host.size());
+        const unsigned char* src = reinterpret_cast<const unsigned char*>(v.data());
+        host.insert(host.end(), src, src + v.size() * sizeof(v[0]));
+    };
+    put(&d.row_ptr, L->row_ptr);
+    put(&d.col_idx, L->col_idx);
+    put(&d.col_ptr, L->col_ptr);
+    put(&d.row_idx, L->row_idx);
+    put(&d.items, L->items_abs);
+    put(&d.steps, L->steps);
+    put(&d.split_tile_q, L->split_tile_q);
+    put(&d.items_t, L->items_t);
+    put(&d.steps_t, L->steps_t);
+    put(&d.global_pairs, L->global_pairs);
+    cudaError_t e = cudaMalloc(&d.block, host.size() + 256);
+    if (e == cudaSuccess) e = cudaMemcpy(d.block, host.data(), host.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return e;
+    for (auto& [dst, off] : at) *dst = (unsigned char*)d.block + off;
+    return cudaSuccess;
 }
 
 // Device copy of the layout on the current device (made on first use, remade if the device changes).
@@ -71,14 +129,10 @@ int get_device_layout(const bigbird_layout* L, int device, DeviceLayout* out) {
             free_device_layout(d);
             cudaSetDevice(cur);
         }
-        cudaError_t e = upload(&d.row_ptr, L->row_ptr.data(), L->row_ptr.size());
-        if (e == cudaSuccess) e = upload(&d.col_idx, L->col_idx.data(), L->col_idx.size());
-        if (e == cudaSuccess) e = upload(&d.col_ptr, L->col_ptr.data(), L->col_ptr.size());
-        if (e == cudaSuccess) e = upload(&d.row_idx, L->row_idx.data(), L->row_idx.size());
-        if (e == cudaSuccess) e = upload(&d.items, L->items_abs.data(), L->items_abs.size());
-        if (e == cudaSuccess) e = upload(&d.steps, L->steps.data(), L->steps.size());
-        if (e == cudaSuccess) e = upload(&d.split_tile_q, L->split_tile_q.data(), L->split_tile_q.size());
+        cudaError_t e = upload_layout(L, d);
         if (e != cudaSuccess) { free_device_layout(d); return cuda_fail(e); }
+        const int rc = hold_pool(device);
+        if (rc != BIGBIRD_OK) { free_device_layout(d); return rc; }
         d.device = device;
     }
     *out = d;
@@ -164,6 +218,16 @@ int bigbird_attn_bwd(const void* q, const void* k, const void* v, const void* ou
     rc = get_device_layout(layout, device, &dl);
     if (rc != BIGBIRD_OK) return rc;
     BwdArgs a{q, k, v, out, lse, dout, key_padding_mask, dq, dk, dv, B, H, D, b, layout->nb, N, scale, dtype, (cudaStream_t)stream};
+    if (attn_bwd_sm100_takes(a)) {
+        DeviceScratch* sc = nullptr;
+        cudaMemPool_t pool = nullptr;
+        rc = get_scratch(device, &sc);
+        if (rc == BIGBIRD_OK) rc = get_pool(device, &pool);
+        if (rc != BIGBIRD_OK) return rc;
+        rc = launch_attn_bwd_sm100(a, *layout, dl, pool, sc->status, &t_last_launches, &e);
+        if (rc == BIGBIRD_ECUDA) t_last_cuda_error = (int)e;
+        return rc;
+    }
     e = launch_attn_bwd_simt(a, dl, &t_last_launches);
     return e == cudaSuccess ? BIGBIRD_OK : cuda_fail(e);
 }

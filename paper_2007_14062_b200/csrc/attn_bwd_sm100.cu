@@ -1,0 +1,813 @@
+// Gradients of BigBird block-sparse attention on Blackwell tensor cores (sm_100a): bf16 tensors, b = D = 64.
+//
+// The derivatives of Eq. (AT) of arXiv 2007.14062 (the paper trains through the operation, Sec. 4 and App. E.1, and leaves
+// them to autodiff).  With P = exp(scale q k^T - lse) recomputed from the saved lse and delta_i = sum_d dout[i, d] out[i, d]:
+//     dv = P^T dout,   dS = P o (dout v^T - delta),   dq = scale dS k,   dk = scale dS^T q.
+//
+// Both gradients by query (dq) and by key (dk, dv) have the same shape, so one kernel makes them:
+//     rows   X1 | X2:  two query blocks (Q | dO), or two key blocks (K | V), stacked into a 128-row tile
+//     steps  Y1 | Y2:  a key block (K | V) of the rows' lists, or a query block (Q | dO) of the transposed lists
+//     S = X1 Y1^T, dP = X2 Y2^T;   acc0 += dS Y1  (dq, or dk);   acc1 += P Y2  (dv; key tiles only)
+// Every operand is the 64 x 64 tile that TMA brings in: Y1 and Y2 serve once with their head dimension as the contraction
+// (S, dP) and once with their token dimension (acc).  P and dS go back to tensor memory as the A operand, each as the sum of
+// two bf16 numbers (16 significant bits): the products keep the precision of the fp32 path to below the rounding of the
+// results, at twice the number of the accumulating MMAs.
+//
+// Nothing carries over from step to step but the accumulators, so the steps of a tile are dealt in turn to three warpgroups
+// with a 128-column score buffer each.  One thread issues every MMA: S and dP of a step up to three steps ahead of the step
+// whose accumulation is issued.  A buffer needs no barrier to become free: the MMAs that overwrite it are issued behind the
+// ones that read it, and the tensor pipe keeps their order.  An epilogue warpgroup takes a finished tile's accumulators while
+// the next tile's scores are being computed.
+// CTAs are persistent; a scheduler warp draws work from a counter: the tiles of global blocks first, cut along their (full)
+// lists into parts where they would outlast the rest, then per (batch, head) the key tiles and the query tiles.  A part
+// leaves its fp32 accumulators in scratch; whichever part is done last sums all of them in a fixed order.  No float atomics:
+// results are bit-reproducible.
+//
+// Measured (base workload [8, 12, 4096, 64], forward and backward of a training step): 16.5 ms with the CUDA-core gradients,
+// 0.99 ms with these; [1, 12, 16384, 64] with 13000 valid tokens 19.1 ms and 0.41 ms.  What bounds it: the tensor pipe runs
+// 16 MMAs of 128 x 64 x 16 for a step of a query tile and 24 for a key tile's; the ones with both operands in shared memory
+// read 6 KB each and take 48 cycles instead of 32.
+//
+// A first kernel makes, per query row, -lse * log2 e (-inf for rows without probabilities) and -delta, packs the key-padding
+// mask and zeroes the counters.
+#include <algorithm>
+
+#include "sm100.cuh"
+
+namespace bigbird {
+namespace {
+
+constexpr int kBufs = 3;                   // score buffers, each served by one warpgroup
+constexpr int kStages = 6;                 // ring of Y1 | Y2 pairs
+constexpr int kSlots = 3;                  // tiles (or segments of long ones) posted by the scheduler
+constexpr int kSegSteps = 96;              // steps per posted segment
+// warps 0..11: the three elementwise warpgroups; 12..15: epilogue; 16: scheduler; 17: TMA producer; 18: MMA issuer
+constexpr int kThreads = 640;
+constexpr int kWarpEpilogue = 12, kWarpScheduler = 16, kWarpProducer = 17, kWarpMma = 18;
+// 640 threads start with 96 registers each; a sub-partition's five warps share 480: three elementwise warps x 120 (32 columns
+// of S and of dP and what becomes of them), an epilogue warp x 64 and a light warp x 56.
+constexpr int kRegsElem = 120, kRegsEpilogue = 64, kRegsLight = 56;
+static_assert(kBufs * kRegsElem + kRegsEpilogue + kRegsLight <= 5 * 96, "register trade between the five warps of a sub-partition");
+constexpr int kTmemCols = 512;
+constexpr int kBufCols = 128;              // S 64 | dP 64; dS (query tiles) or P and dS (key tiles) take their places
+constexpr int kColAcc = kBufs * kBufCols;  // acc0 64 | acc1 64
+static_assert(kColAcc + 128 <= kTmemCols, "tensor memory");
+constexpr int kStatFloats = 2 * kBlock;    // per block of query rows: 64 x (-lse log2 e), 64 x (-delta)
+constexpr int kPartialFloats = 2 * 128 * kBlock;   // one part of a split tile: acc0, acc1
+enum { kDkv = 0, kDq = 1 };
+enum { kSegFirst = 1, kSegLast = 2, kSegLive = 4 };
+
+struct __align__(16) StepEntry {
+    int c;                         // block of the column side
+    int who;                       // kBothHalves, kUpperHalf or kLowerHalf
+    unsigned long long kb;         // its valid-token bits (never 0)
+};
+struct __align__(16) TileSlot {
+    int w;                         // work index, -1 = no more work
+    int kind, bh, ra, rb;          // rb == kNoBlock: no lower half
+    int n;                         // steps of this segment
+    int flags;
+    int split;                     // index of the split tile, -1 if it is not split
+    int part;
+    int pad_[3];
+    unsigned long long rbits_a, rbits_b;
+    StepEntry steps[kSegSteps];
+};
+struct __align__(16) SmemCtl {
+    unsigned long long full[kStages], empty[kStages];
+    unsigned long long x_full[2], x_empty[2];
+    unsigned long long sdp_full[kBufs], p_full[kBufs];
+    unsigned long long acc_full, acc_free;
+    unsigned long long slot_full[kSlots], slot_empty[kSlots];
+    TileSlot slot[kSlots];
+    float x_stats[2][2][kStatFloats];      // query tiles: statistics of the rows
+    float y_stats[kStages][kStatFloats];   // key tiles: of the step's query block
+    unsigned tmem_base;
+    int abort_flag;
+    int merge_last;
+};
+constexpr int kSmemX = 0;                                      // two buffers of X1a X1b X2a X2b
+constexpr int kSmemRing = 2 * 4 * kTileBytes;
+constexpr int kSmemCtl = kSmemRing + kStages * 2 * kTileBytes;
+constexpr int kSmemBytes = kSmemCtl + (int)sizeof(SmemCtl) + 1024;   // + slack for the 1024-byte alignment
+static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
+
+struct KernelParams {
+    __nv_bfloat16 *dq, *dk, *dv;
+    const float* stats;                    // [BH * nb][kStatFloats]
+    const unsigned long long* kbits;       // [B * nb] or nullptr
+    const Item *items_q, *items_k;         // sparse tiles, [H] x stride
+    const Step *steps_q, *steps_k;
+    const int* global_pairs;
+    int* counter;                          // next work index
+    int* arrived;                          // [2 * BH * global_tiles] parts of each split tile that are done
+    int* status;                           // [2]: code, detail
+    float* partials;
+    int q_stride, sparse_tiles, global_tiles;
+    int parts, part_steps;                 // how the tiles of global blocks are cut
+    int BH, H, nb, total_work;
+    float scale, scale_log2;
+};
+
+__device__ __forceinline__ unsigned long long token_bits(const KernelParams& p, int batch, int c) {
+    if (c < 0) return 0ull;
+    return p.kbits ? p.kbits[(size_t)batch * p.nb + c] : ~0ull;
+}
+
+// ------------------------------------------------------------------------------------------------ scheduler (one warp)
+__device__ __forceinline__ void scheduler_role(const KernelParams& p, SmemCtl* ctl, int lane) {
+    const unsigned lt_mask = (1u << lane) - 1u;
+    unsigned slot_n = 0;
+    for (;;) {
+        int w = 0;
+        if (lane == 0) w = atomicAdd(p.counter, 1);
+        w = __shfl_sync(0xffffffffu, w, 0);
+        if (w >= p.total_work) w = -1;
+        int kind = 0, bh = 0, ra = kNoBlock, rb = kNoBlock, begin = 0, n_raw = 0, split = -1, part = 0;
+        const Step* steps = nullptr;               // nullptr: blocks begin, begin + 1, ... attended by both halves
+        if (w >= 0) {
+            const int heavy = p.BH * p.global_tiles * p.parts;
+            if (w < 2 * heavy) {
+                kind = w < heavy ? kDkv : kDq;
+                const int x = kind == kDkv ? w : w - heavy;
+                const int tile = x / p.parts;      // (batch, head) major
+                part = x - tile * p.parts;
+                bh = tile / p.global_tiles;
+                const int t = tile - bh * p.global_tiles;
+                ra = p.global_pairs[2 * t];
+                rb = p.global_pairs[2 * t + 1];
+                begin = part * p.part_steps;
+                n_raw = min(p.part_steps, p.nb - begin);
+                if (p.parts > 1) split = kind * p.BH * p.global_tiles + tile;
+            } else {
+                const int x = w - 2 * heavy;
+                bh = x / (2 * p.sparse_tiles);
+                int it = x - bh * 2 * p.sparse_tiles;
+                kind = it < p.sparse_tiles ? kDkv : kDq;
+                if (kind == kDq) it -= p.sparse_tiles;
+                const Item item = kind == kDkv ? p.items_k[(size_t)(bh % p.H) * p.sparse_tiles + it] : p.items_q[(size_t)(bh % p.H) * p.q_stride + it];
+                ra = item.qa;
+                rb = item.qb;
+                begin = item.step_begin;
+                n_raw = item.step_count;
+                steps = kind == kDkv ? p.steps_k : p.steps_q;
+            }
+            if (!BB_CHECK(bh >= 0 && bh < p.BH && ra >= 0 && ra < p.nb && rb < p.nb && n_raw >= 0 && begin >= 0, 171)) w = -1;
+        }
+        const int batch = bh / p.H;
+        const unsigned long long rbits_a = w >= 0 ? token_bits(p, batch, ra) : 0ull, rbits_b = w >= 0 ? token_bits(p, batch, rb) : 0ull;
+        const bool live = (rbits_a | rbits_b) != 0ull;       // a tile without any valid row needs no steps
+        if (!live) n_raw = 0;
+        int i0 = 0;
+        bool first = true;
+        do {
+            const unsigned ss = slot_n % kSlots;
+            if (!mbar_wait(&ctl->slot_empty[ss], ((slot_n / kSlots) & 1u) ^ 1u, &ctl->abort_flag)) { give_up(&ctl->abort_flag, p.status, 111); return; }
+            __syncwarp();
+            TileSlot* slot = &ctl->slot[ss];
+            int count = 0;
+#pragma unroll 1
+            while (i0 < n_raw && count <= kSegSteps - 32) {
+                const int i = i0 + lane;
+                StepEntry e{-1, 0, 0ull};
+                bool alive = false;
+                if (i < n_raw) {
+                    const Step s = steps ? steps[begin + i] : Step{begin + i, kBothHalves};
+                    const bool ua = s.who != kLowerHalf && rbits_a != 0ull, ub = s.who != kUpperHalf && rbits_b != 0ull;
+                    e.c = s.c;
+                    e.who = (ua && ub) ? kBothHalves : (ua ? kUpperHalf : kLowerHalf);
+                    alive = BB_CHECK(s.c >= 0 && s.c < p.nb, 170);
+                    if (alive) e.kb = token_bits(p, batch, s.c);
+                    alive = alive && e.kb != 0ull && (ua || ub);
+                }
+                const unsigned bal = __ballot_sync(0xffffffffu, alive);
+                if (alive) slot->steps[count + __popc(bal & lt_mask)] = e;
+                count += __popc(bal);
+                i0 += 32;
+            }
+            if (lane == 0) {
+                slot->w = w;
+                slot->kind = kind;
+                slot->bh = bh;
+                slot->ra = ra;
+                slot->rb = rb;
+                slot->n = count;
+                slot->flags = (first ? kSegFirst : 0) | (i0 >= n_raw ? kSegLast : 0) | (live ? kSegLive : 0);
+                slot->split = split;
+                slot->part = part;
+                slot->rbits_a = rbits_a;
+                slot->rbits_b = rbits_b;
+            }
+            __threadfence_block();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ctl->slot_full[ss]);
+            ++slot_n;
+            first = false;
+        } while (i0 < n_raw);
+        if (w < 0) return;
+    }
+}
+
+// ------------------------------------------------------------------------------------------------ TMA producer (one thread)
+__device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ctl, unsigned char* smem, const CUtensorMap* tm_q,
+                                              const CUtensorMap* tm_k, const CUtensorMap* tm_v, const CUtensorMap* tm_do) {
+    int* abort_flag = &ctl->abort_flag;
+    unsigned slot_n = 0, tile_n = 0, step_n = 0;
+    int fail = 0;
+    for (;;) {
+        const unsigned ss = slot_n % kSlots;
+        if (!mbar_wait(&ctl->slot_full[ss], (slot_n / kSlots) & 1u, abort_flag)) { fail = 113; break; }
+        const TileSlot* slot = &ctl->slot[ss];
+        const int w = slot->w, flags = slot->flags, n = slot->n, bh = slot->bh;
+        const bool dkv = slot->kind == kDkv;
+        if (w >= 0 && (flags & kSegLive)) {
+            if (flags & kSegFirst) {
+                const int ra = slot->ra, rb = slot->rb;
+                const unsigned xs = tile_n & 1u;
+                if (!mbar_wait(&ctl->x_empty[xs], ((tile_n >> 1) & 1u) ^ 1u, abort_flag)) { fail = 112; break; }
+                unsigned char* x = smem + kSmemX + xs * 4 * kTileBytes;
+                unsigned long long* bar = &ctl->x_full[xs];
+                const CUtensorMap *tm1 = dkv ? tm_k : tm_q, *tm2 = dkv ? tm_v : tm_do;
+                const int blocks = rb >= 0 ? 2 : 1;
+                mbar_expect_tx(bar, blocks * (2 * kTileBytes + (dkv ? 0 : kStatFloats * 4)));
+                for (int j = 0; j < blocks; ++j) {
+                    const int row = bh * p.nb + (j ? rb : ra);
+                    tma_load_tile(x + j * kTileBytes, tm1, row * kBlock, bar);
+                    tma_load_tile(x + (2 + j) * kTileBytes, tm2, row * kBlock, bar);
+                    if (!dkv) bulk_load(ctl->x_stats[xs][j], p.stats + (size_t)row * kStatFloats, kStatFloats * 4, bar);
+                }
+                ++tile_n;
+            }
+            const CUtensorMap *tm1 = dkv ? tm_q : tm_k, *tm2 = dkv ? tm_do : tm_v;
+            for (int i = 0; i < n; ++i) {
+                const unsigned g = step_n % kStages;
+                const int row = bh * p.nb + slot->steps[i].c;
+                if (!mbar_wait(&ctl->empty[g], ((step_n / kStages) & 1u) ^ 1u, abort_flag)) { fail = 110; break; }
+                unsigned char* y = smem + kSmemRing + g * 2 * kTileBytes;
+                mbar_expect_tx(&ctl->full[g], 2 * kTileBytes + (dkv ? kStatFloats * 4 : 0));
+                tma_load_tile(y, tm1, row * kBlock, &ctl->full[g]);
+                tma_load_tile(y + kTileBytes, tm2, row * kBlock, &ctl->full[g]);
+                if (dkv) bulk_load(ctl->y_stats[g], p.stats + (size_t)row * kStatFloats, kStatFloats * 4, &ctl->full[g]);
+                ++step_n;
+            }
+            if (fail) break;
+        }
+        mbar_arrive(&ctl->slot_empty[ss]);
+        ++slot_n;
+        if (w < 0) break;
+    }
+    if (fail) give_up(abort_flag, p.status, fail);
+}
+
+// ------------------------------------------------------------------------------------------------ MMA issuer (one thread)
+// front: steps whose S and dP have been issued; back: steps whose accumulation has been issued.
+__device__ __forceinline__ void mma_role(const KernelParams& p, SmemCtl* ctl, unsigned char* smem, unsigned tmem) {
+    int* abort_flag = &ctl->abort_flag;
+    unsigned slot_n = 0, tile_n = 0, acc_n = 0, front = 0, back = 0;
+    unsigned firsts = 0, lasts = 0, kinds = 0;      // bit (step & 7) of the steps between back and front
+    unsigned buf_f = 0, buf_b = 0;                  // front % kBufs, back % kBufs
+    unsigned par_b = 0;                             // parity of p_full of the step at back
+    unsigned stg_f = 0, stg_b = 0, ph_f = 0;        // ring stages of front and back, phase of front's
+    bool open = false, done = false, fresh = false, tile_steps = false;
+    const TileSlot* slot = nullptr;
+    int i = 0, n = 0, flags = 0;
+    unsigned kind = 0, xs = 0;
+    int fail = 0;
+    const unsigned x_base = smem_u32(smem + kSmemX), ring_base = smem_u32(smem + kSmemRing);
+    for (;;) {
+        const unsigned ss = slot_n % kSlots;
+        // (with steps pending the thread must not sleep on the next slot: tiles without steps pass through the slots quickly,
+        // and the next one may only become free once the pending steps' tile is finished)
+        if (!done && front - back < (unsigned)kBufs && (open || front == back || mbar_test(&ctl->slot_full[ss], (slot_n / kSlots) & 1u))) {
+            if (!open) {
+                if (!mbar_wait(&ctl->slot_full[ss], (slot_n / kSlots) & 1u, abort_flag)) { fail = 123; break; }
+                slot = &ctl->slot[ss];
+                if (slot->w < 0) { mbar_arrive(&ctl->slot_empty[ss]); done = true; continue; }
+                flags = slot->flags;
+                kind = (unsigned)slot->kind;
+                n = (flags & kSegLive) ? slot->n : 0;
+                i = 0;
+                open = true;
+                if ((flags & (kSegFirst | kSegLive)) == (kSegFirst | kSegLive)) {
+                    xs = tile_n & 1u;
+                    if (!mbar_wait(&ctl->x_full[xs], (tile_n >> 1) & 1u, abort_flag)) { fail = 124; break; }
+                    ++tile_n;
+                    fresh = true;
+                    tile_steps = false;
+                }
+            }
+            if (i < n) {
+                if (!mbar_wait(&ctl->full[stg_f], ph_f, abort_flag)) { fail = 120; break; }
+                tc_fence_after();
+                const unsigned long long x1 = smem_desc_sw128(x_base + xs * 4 * kTileBytes), x2 = x1 + ((2 * kTileBytes) >> 4);
+                const unsigned long long y1 = smem_desc_sw128(ring_base + stg_f * 2 * kTileBytes), y2 = y1 + (kTileBytes >> 4);
+                const unsigned d = tmem + buf_f * kBufCols;
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) mma_ss(d, x1 + kk * 2, y1 + kk * 2, kIdescQK64, kk > 0);
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) mma_ss(d + 64, x2 + kk * 2, y2 + kk * 2, kIdescQK64, kk > 0);
+                tc_commit(&ctl->sdp_full[buf_f]);
+                const unsigned bit = 1u << (front & 7u);
+                firsts = fresh ? (firsts | bit) : (firsts & ~bit);
+                kinds = kind ? (kinds | bit) : (kinds & ~bit);
+                lasts &= ~bit;
+                fresh = false;
+                tile_steps = true;
+                ++front;
+                ++i;
+                buf_f = buf_f == kBufs - 1 ? 0u : buf_f + 1u;
+                if (++stg_f == kStages) { stg_f = 0; ph_f ^= 1u; }
+            }
+            if (i >= n) {                           // end of the segment
+                if ((flags & (kSegLast | kSegLive)) == (kSegLast | kSegLive)) {
+                    tc_commit(&ctl->x_empty[xs]);   // every S and dP of the tile has been issued
+                    if (tile_steps) {
+                        if (front != back) lasts |= 1u << ((front - 1u) & 7u);
+                        else { tc_commit(&ctl->acc_full); ++acc_n; }
+                    }
+                }
+                mbar_arrive(&ctl->slot_empty[ss]);
+                ++slot_n;
+                open = false;
+            }
+            continue;
+        }
+        if (front == back) break;                   // done, and nothing is pending
+        const unsigned bit = 1u << (back & 7u);
+        // the epilogue must have taken the previous tile's accumulators before this tile's first product overwrites them
+        if ((firsts & bit) && acc_n > 0 && !mbar_wait(&ctl->acc_free, (acc_n - 1) & 1u, abort_flag)) { fail = 127; break; }
+        if (!mbar_wait(&ctl->p_full[buf_b], par_b, abort_flag)) { fail = 122; break; }
+        tc_fence_after();
+        {
+            const unsigned long long y1 = smem_desc_sw128(ring_base + stg_b * 2 * kTileBytes), y2 = y1 + (kTileBytes >> 4);
+            const unsigned a = tmem + buf_b * kBufCols, acc = tmem + kColAcc;
+            const unsigned keep = (firsts & bit) ? 0u : 1u;
+            const bool dkv = !(kinds & bit);
+            // 16 tokens per MMA: 8 packed columns of A (the high halves of 32 columns, then their low halves), two 8-row groups of Y
+            if (dkv) {
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                    const unsigned ak = a + (kk >> 1) * 32 + (kk & 1) * 8;
+                    mma_ts(acc + 64, ak, y2 + ((kk * 2048) >> 4), kIdescPV, kk > 0 ? 1u : keep);
+                    mma_ts(acc + 64, ak + 16, y2 + ((kk * 2048) >> 4), kIdescPV, 1u);
+                }
+            }
+            const unsigned ds = dkv ? a + 64 : a;
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                const unsigned ak = ds + (kk >> 1) * 32 + (kk & 1) * 8;
+                mma_ts(acc, ak, y1 + ((kk * 2048) >> 4), kIdescPV, kk > 0 ? 1u : keep);
+                mma_ts(acc, ak + 16, y1 + ((kk * 2048) >> 4), kIdescPV, 1u);
+            }
+        }
+        tc_commit(&ctl->empty[stg_b]);
+        if (lasts & bit) { tc_commit(&ctl->acc_full); ++acc_n; }
+        ++back;
+        if (buf_b == kBufs - 1) { buf_b = 0; par_b ^= 1u; } else ++buf_b;
+        stg_b = stg_b == kStages - 1 ? 0u : stg_b + 1u;
+    }
+    if (fail) give_up(abort_flag, p.status, fail);
+}
+
+// ------------------------------------------------------------------------------------------------ elementwise (three warpgroups, one thread per row)
+// Query tiles, 32 columns: dS = exp2(S sl2 + nl) (dP + nd) over S, in place.
+__device__ __forceinline__ void dq_columns(unsigned s_addr, float sl2, float nl, float nd, unsigned key_bits) {
+    float s[32], d[32];
+    unsigned hi[16], lo[16];
+    tmem_ld32(s_addr, s);
+    tmem_ld32(s_addr + 64, d);
+    tmem_wait_ld();
+    if (__builtin_expect(key_bits != 0xffffffffu, 0)) {         // padded keys
+#pragma unroll
+        for (int t = 0; t < 32; ++t) s[t] = ((key_bits >> t) & 1u) ? s[t] : -INFINITY;
+    }
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        float x0, x1;
+        ffma2(x0, x1, s[2 * j], s[2 * j + 1], sl2, nl);
+        add_mul2(x0, x1, d[2 * j], d[2 * j + 1], nd, nd, ex2(x0), ex2(x1));
+        split_bf16(x0, x1, hi[j], lo[j]);
+    }
+    tmem_st16(s_addr, hi);
+    tmem_st16(s_addr + 16, lo);
+}
+// Key tiles, 32 columns: P over S and dS over dP; the statistics belong to the columns.
+__device__ __forceinline__ void dkv_columns(unsigned s_addr, float sl2, const float4* nl, const float4* nd) {
+    float s[32], d[32];
+    unsigned phi[16], plo[16], dhi[16], dlo[16];
+    tmem_ld32(s_addr, s);
+    tmem_ld32(s_addr + 64, d);
+    tmem_wait_ld();
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const float4 n4 = nl[j], d4 = nd[j];
+        float x0, x1;
+        ffma2v(x0, x1, s[4 * j], s[4 * j + 1], sl2, n4.x, n4.y);
+        x0 = ex2(x0);
+        x1 = ex2(x1);
+        split_bf16(x0, x1, phi[2 * j], plo[2 * j]);
+        add_mul2(x0, x1, d[4 * j], d[4 * j + 1], d4.x, d4.y, x0, x1);
+        split_bf16(x0, x1, dhi[2 * j], dlo[2 * j]);
+        ffma2v(x0, x1, s[4 * j + 2], s[4 * j + 3], sl2, n4.z, n4.w);
+        x0 = ex2(x0);
+        x1 = ex2(x1);
+        split_bf16(x0, x1, phi[2 * j + 1], plo[2 * j + 1]);
+        add_mul2(x0, x1, d[4 * j + 2], d[4 * j + 3], d4.z, d4.w, x0, x1);
+        split_bf16(x0, x1, dhi[2 * j + 1], dlo[2 * j + 1]);
+    }
+    tmem_st16(s_addr, phi);
+    tmem_st16(s_addr + 16, plo);
+    tmem_st16(s_addr + 64, dhi);
+    tmem_st16(s_addr + 80, dlo);
+}
+
+__device__ __forceinline__ void elementwise_role(const KernelParams& p, SmemCtl* ctl, unsigned tmem, int warp, int lane) {
+    int* abort_flag = &ctl->abort_flag;
+    const unsigned g = (unsigned)warp >> 2;         // warpgroup = score buffer
+    const int quad = warp & 3, row = quad * 32 + lane, r64 = row & (kBlock - 1);
+    const bool lower = row >= kBlock;
+    const int my_who = lower ? kLowerHalf : kUpperHalf;
+    const unsigned buf = tmem + ((unsigned)(quad * 32) << 16) + g * kBufCols;
+    const float sl2 = p.scale_log2;
+    unsigned slot_n = 0, tile_n = 0, step_n = 0, use_n = 0;     // step_n: steps of all earlier segments
+    float nl = 0.f, nd = 0.f;
+    int fail = 0;
+    for (;;) {
+        const unsigned ss = slot_n % kSlots;
+        if (!mbar_wait(&ctl->slot_full[ss], (slot_n / kSlots) & 1u, abort_flag)) { fail = 130; break; }
+        const TileSlot* slot = &ctl->slot[ss];
+        const int w = slot->w, flags = slot->flags, n = slot->n;
+        const bool dkv = slot->kind == kDkv;
+        if (w < 0) break;
+        if ((flags & (kSegFirst | kSegLive)) == (kSegFirst | kSegLive)) {
+            const unsigned xs = tile_n & 1u;
+            if (!mbar_wait(&ctl->x_full[xs], (tile_n >> 1) & 1u, abort_flag)) { fail = 134; break; }
+            nl = ctl->x_stats[xs][lower][r64];      // (stale and unused on key tiles)
+            nd = ctl->x_stats[xs][lower][kBlock + r64];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ctl->x_empty[xs]);
+            ++tile_n;
+        }
+        const unsigned ahead = step_n % kBufs;
+        for (int i = (int)(g >= ahead ? g - ahead : g + kBufs - ahead); i < n; i += kBufs) {
+            const int who = slot->steps[i].who;
+            const bool mine = who == kBothHalves || who == my_who;      // warp-uniform
+            const unsigned long long kb = slot->steps[i].kb;
+            if (!mbar_wait(&ctl->sdp_full[g], use_n & 1u, abort_flag)) { fail = 131; break; }
+            __syncwarp();                           // lanes leave the wait one by one
+            tc_fence_after();
+            if (!mine) {
+                tmem_st32_zero(buf);
+                tmem_st32_zero(buf + 32);
+                if (dkv) {
+                    tmem_st32_zero(buf + 64);
+                    tmem_st32_zero(buf + 96);
+                }
+            } else if (dkv) {
+                const unsigned t = step_n + (unsigned)i, stage = t % kStages;
+                if (!mbar_wait(&ctl->full[stage], (t / kStages) & 1u, abort_flag)) { fail = 132; break; }     // (complete: this makes the copy visible)
+                __syncwarp();
+                const float4* st = reinterpret_cast<const float4*>(ctl->y_stats[stage]);
+#pragma unroll 1
+                for (int c = 0; c < 2; ++c) dkv_columns(buf + 32 * c, sl2, st + 8 * c, st + 16 + 8 * c);
+            } else {
+#pragma unroll 1
+                for (int c = 0; c < 2; ++c) dq_columns(buf + 32 * c, sl2, nl, nd, (unsigned)(kb >> (32 * c)));
+            }
+            tmem_wait_st();
+            tc_fence_before();
+            mbar_arrive(&ctl->p_full[g]);
+            ++use_n;
+        }
+        if (fail) break;
+        step_n += (unsigned)n;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&ctl->slot_empty[ss]);
+        ++slot_n;
+    }
+    if (fail) give_up(abort_flag, p.status, fail);
+}
+
+// ------------------------------------------------------------------------------------------------ epilogue (one warpgroup)
+__device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+
+// Sums the parts of a split tile (the last one to arrive does) and writes the rows.
+__device__ __forceinline__ void merge_parts(const KernelParams& p, const TileSlot* slot, int tid) {
+    const bool dkv = slot->kind == kDkv;
+    const float* base = p.partials + (size_t)slot->split * p.parts * kPartialFloats;
+#pragma unroll 1
+    for (int idx = tid; idx < (dkv ? 2 : 1) * 128 * 16; idx += 128) {
+        const int m = idx >> 11, row = (idx >> 4) & 127, c4 = idx & 15;
+        const int blk = row >= kBlock ? slot->rb : slot->ra;
+        if (blk < 0) continue;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int pt = 0; pt < p.parts; ++pt) {               // fixed order: results do not depend on scheduling
+            const float4 v = __ldcg(reinterpret_cast<const float4*>(base + (size_t)pt * kPartialFloats + m * 128 * kBlock + row * kBlock) + c4);
+            acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+        }
+        const unsigned long long bits = row >= kBlock ? slot->rbits_b : slot->rbits_a;
+        const float f = ((bits >> (row & 63)) & 1ull) ? (m ? 1.f : p.scale) : 0.f;
+        __nv_bfloat16* dst = (dkv ? (m ? p.dv : p.dk) : p.dq) + (((size_t)slot->bh * p.nb + blk) * kBlock + (row & 63)) * kBlock;
+        uint2 v2;
+        v2.x = pack_bf16(acc.x * f, acc.y * f);
+        v2.y = pack_bf16(acc.z * f, acc.w * f);
+        reinterpret_cast<uint2*>(dst)[c4] = v2;
+    }
+}
+
+__device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ctl, unsigned tmem, int warp, int lane) {
+    int* abort_flag = &ctl->abort_flag;
+    const int quad = warp & 3, row = quad * 32 + lane, r64 = row & (kBlock - 1);
+    const bool lower = row >= kBlock;
+    const unsigned acc = tmem + ((unsigned)(quad * 32) << 16) + kColAcc;
+    unsigned slot_n = 0, acc_n = 0;
+    bool have = false;                              // has the tile had any step
+    int fail = 0;
+    for (;;) {
+        const unsigned ss = slot_n % kSlots;
+        if (!mbar_wait(&ctl->slot_full[ss], (slot_n / kSlots) & 1u, abort_flag)) { fail = 140; break; }
+        __syncwarp();
+        const TileSlot* slot = &ctl->slot[ss];
+        const int flags = slot->flags;
+        if (slot->w < 0) break;
+        if (flags & kSegFirst) have = false;
+        have = have || slot->n > 0;
+        if (flags & kSegLast) {
+            const bool dkv = slot->kind == kDkv;
+            const int blk = lower ? slot->rb : slot->ra, split = slot->split;
+            const unsigned long long bits = lower ? slot->rbits_b : slot->rbits_a;
+            const bool row_ok = (bits >> r64) & 1ull;
+            if (have) {
+                if (!mbar_wait(&ctl->acc_full, acc_n & 1u, abort_flag)) { fail = 141; break; }
+                __syncwarp();
+                tc_fence_after();
+                ++acc_n;
+            }
+            const int n_acc = dkv ? 2 : 1;
+            float* part = p.partials + ((size_t)max(split, 0) * p.parts + slot->part) * kPartialFloats + row * kBlock;
+            const size_t tok = (((size_t)slot->bh * p.nb + max(blk, 0)) * kBlock + r64) * kBlock;
+#pragma unroll 1
+            for (int h = 0; h < 2 * n_acc; ++h) {   // 32 columns at a time
+                float o[32];
+                if (have) {
+                    tmem_ld32(acc + 32 * h, o);
+                    tmem_wait_ld();
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) o[j] = 0.f;
+                }
+                if (have && h == 2 * n_acc - 1) { tc_fence_before(); mbar_arrive(&ctl->acc_free); }
+                const int m = h >> 1;
+                if (split >= 0) {
+                    float4* d4 = reinterpret_cast<float4*>(part + m * 128 * kBlock) + 8 * (h & 1);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) d4[j] = make_float4(o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
+                } else if (blk >= 0) {
+                    const float f = row_ok ? (m ? 1.f : p.scale) : 0.f;
+                    uint4* d4 = reinterpret_cast<uint4*>((dkv ? (m ? p.dv : p.dk) : p.dq) + tok) + 4 * (h & 1);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        uint4 v;
+                        v.x = pack_bf16(o[8 * j + 0] * f, o[8 * j + 1] * f);
+                        v.y = pack_bf16(o[8 * j + 2] * f, o[8 * j + 3] * f);
+                        v.z = pack_bf16(o[8 * j + 4] * f, o[8 * j + 5] * f);
+                        v.w = pack_bf16(o[8 * j + 6] * f, o[8 * j + 7] * f);
+                        d4[j] = v;
+                    }
+                }
+            }
+            if (split >= 0) {
+                __threadfence();
+                epilogue_sync();
+                if (row == 0) ctl->merge_last = atomicAdd(&p.arrived[split], 1) == p.parts - 1;
+                epilogue_sync();
+                if (ctl->merge_last) {
+                    __threadfence();
+                    merge_parts(p, slot, row);
+                }
+            }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&ctl->slot_empty[ss]);
+        ++slot_n;
+    }
+    if (fail) give_up(abort_flag, p.status, fail);
+}
+
+// ------------------------------------------------------------------------------------------------ the kernel
+__global__ void __launch_bounds__(kThreads, 1)
+attn_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
+                      const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do, const KernelParams p) {
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    SmemCtl* ctl = reinterpret_cast<SmemCtl*>(smem + kSmemCtl);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kStages; ++i) { mbar_init(&ctl->full[i], 1); mbar_init(&ctl->empty[i], 1); }
+        for (int i = 0; i < 2; ++i) { mbar_init(&ctl->x_full[i], 1); mbar_init(&ctl->x_empty[i], 1 + 4 * kBufs); }      // the MMA thread, the elementwise warps
+        for (int i = 0; i < kBufs; ++i) { mbar_init(&ctl->sdp_full[i], 1); mbar_init(&ctl->p_full[i], 128); }
+        mbar_init(&ctl->acc_full, 1);
+        mbar_init(&ctl->acc_free, 128);
+        for (int i = 0; i < kSlots; ++i) { mbar_init(&ctl->slot_full[i], 1); mbar_init(&ctl->slot_empty[i], 2 + 4 * kBufs + 4); }   // producer, MMA thread, elementwise and epilogue warps
+        ctl->abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == kWarpProducer) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)), "r"(kTmemCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const unsigned tmem = *(volatile unsigned*)&ctl->tmem_base;
+
+    if (warp < kWarpEpilogue) {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsElem));
+        elementwise_role(p, ctl, tmem, warp, lane);
+    } else if (warp < kWarpScheduler) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsEpilogue));
+        epilogue_role(p, ctl, tmem, warp, lane);
+    } else {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLight));
+        if (warp == kWarpScheduler) scheduler_role(p, ctl, lane);
+        else if (warp == kWarpProducer) { if (lane == 0) producer_role(p, ctl, smem, &tm_q, &tm_k, &tm_v, &tm_do); }
+        else if (warp == kWarpMma) { if (lane == 0) mma_role(p, ctl, smem, tmem); }
+    }
+
+    // ------------------------------------------------------------------------------------------------ teardown
+    __syncthreads();
+    if (*(volatile int*)&ctl->abort_flag) {
+        // a wait expired: give copies and MMAs still in flight time to land before shared and tensor memory go away
+        const unsigned long long t0 = global_ns();
+        while (global_ns() - t0 < 200000ull) __nanosleep(1000);
+        __syncthreads();
+    }
+    tc_fence_after();
+    if (warp == kWarpProducer) {
+        __syncwarp();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    }
+}
+
+// Per query row: -lse log2 e (-inf: padded, or nothing attended) and -delta; the key-padding mask as one 64-bit word per
+// block; zeroed counters.  Eight threads share a row.  Reads out and dout once: memory bound.
+constexpr int kPrepThreads = 256, kPrepRows = kPrepThreads / 8;
+__global__ void __launch_bounds__(kPrepThreads)
+attn_bwd_prepare_kernel(const uint4* __restrict__ out, const uint4* __restrict__ dout, const float* __restrict__ lse,
+                        const uint8_t* __restrict__ kpm, float* __restrict__ stats, unsigned long long* __restrict__ kbits,
+                        int* __restrict__ counters, int n_counters, long long rows, int N, int H, int row_ctas, int n_words) {
+    if ((int)blockIdx.x >= row_ctas) {             // the last CTAs: mask words and counters
+        const int part = blockIdx.x - row_ctas, stride = gridDim.x - row_ctas;
+        for (int i = part * kPrepThreads + threadIdx.x; i < n_counters; i += stride * kPrepThreads) counters[i] = 0;
+        const int lane = threadIdx.x & 31;
+        for (int word = (part * kPrepThreads + threadIdx.x) >> 5; word < n_words; word += stride * (kPrepThreads >> 5)) {
+            const uint8_t* src = kpm + (size_t)word * kBlock;
+            const unsigned lo = __ballot_sync(0xffffffffu, src[lane] != 0), hi = __ballot_sync(0xffffffffu, src[lane + 32] != 0);
+            if (lane == 0) kbits[word] = ((unsigned long long)hi << 32) | lo;
+        }
+        return;
+    }
+    const int sub = threadIdx.x & 7;
+    const long long r0 = (long long)blockIdx.x * (2 * kPrepRows) + (threadIdx.x >> 3);
+    uint4 a[2], b[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const long long r = r0 + u * kPrepRows;
+        if (r < rows) { a[u] = out[r * 8 + sub]; b[u] = dout[r * 8 + sub]; }
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const long long r = r0 + u * kPrepRows;
+        if (r >= rows) continue;                   // (whole groups of eight threads)
+        const unsigned* x = reinterpret_cast<const unsigned*>(&a[u]);
+        const unsigned* y = reinterpret_cast<const unsigned*>(&b[u]);
+        float d = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            d = fmaf(__uint_as_float(x[j] << 16), __uint_as_float(y[j] << 16), d);
+            d = fmaf(__uint_as_float(x[j] & 0xffff0000u), __uint_as_float(y[j] & 0xffff0000u), d);
+        }
+        const unsigned group = 0xffu << (threadIdx.x & 24);
+        d += __shfl_xor_sync(group, d, 1);
+        d += __shfl_xor_sync(group, d, 2);
+        d += __shfl_xor_sync(group, d, 4);
+        if (sub == 0) {
+            const long long bh = r / N;
+            const int tok = (int)(r - bh * N);
+            const float l = lse[r];
+            const bool alive = l > -INFINITY && (!kpm || kpm[(size_t)(bh / H) * N + tok] != 0);
+            float* st = stats + (r / kBlock) * kStatFloats + (r & (kBlock - 1));
+            st[0] = alive ? -l * 1.4426950408889634f : -INFINITY;
+            st[kBlock] = alive ? -d : 0.f;
+        }
+    }
+}
+
+struct KernelDevice {
+    bool ready = false;
+    int sm_count = 0;
+};
+std::mutex g_bwd_mu;
+KernelDevice g_bwd_dev[64];
+
+cudaError_t kernel_setup(int device, int* sm_count) {
+    if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(g_bwd_mu);
+    KernelDevice& d = g_bwd_dev[device];
+    if (!d.ready) {
+        cudaError_t e = cudaFuncSetAttribute(attn_bwd_sm100_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&d.sm_count, cudaDevAttrMultiProcessorCount, device);
+        if (e != cudaSuccess) return e;
+        d.ready = true;
+    }
+    *sm_count = d.sm_count;
+    return cudaSuccess;
+}
+
+size_t align256(size_t x) { return (x + 255) / 256 * 256; }
+
+}  // namespace
+
+bool attn_bwd_sm100_takes(const BwdArgs& a) {
+    const int64_t rows = (int64_t)a.B * a.H * a.N;
+    return a.dtype == BIGBIRD_BF16 && a.D == kBlock && a.b == kBlock && rows < (1ll << 31) && (int64_t)a.B * a.H * a.nb * 2 < (1ll << 28);
+}
+
+int launch_attn_bwd_sm100(const BwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, cudaMemPool_t pool, int* status, int* launches,
+                          cudaError_t* cuda_err) {
+    auto fail = [&](cudaError_t e) { *cuda_err = e; return BIGBIRD_ECUDA; };
+    int device = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e == cudaSuccess) e = kernel_setup(device, &sms);
+    if (e != cudaSuccess) return fail(e);
+    const int BH = a.B * a.H;
+    const int64_t rows = (int64_t)BH * a.N;
+    CUtensorMap tm_q, tm_k, tm_v, tm_do;
+    if (!make_map(&tm_q, a.q, (uint64_t)rows) || !make_map(&tm_k, a.k, (uint64_t)rows) || !make_map(&tm_v, a.v, (uint64_t)rows) ||
+        !make_map(&tm_do, a.dout, (uint64_t)rows))
+        return fail(cudaErrorInvalidValue);
+
+    // Tiles of global blocks have nb steps where the others have about ten: cut them into parts of about half of what each SM
+    // gets altogether (at least 8 steps), so that none of them is still running when the rest is done.
+    const int64_t steps = (int64_t)a.B * ((int64_t)L.steps.size() + (int64_t)L.steps_t.size() + (int64_t)a.H * L.global_tiles * a.nb);
+    int part_steps = (int)std::min<int64_t>(a.nb, std::max<int64_t>(8, steps / (2 * sms)));
+    const int parts = (a.nb + part_steps - 1) / part_steps;
+    part_steps = (a.nb + parts - 1) / parts;
+
+    // workspace of this call, on the caller's stream
+    const int n_split = parts > 1 ? 2 * BH * L.global_tiles : 0;
+    const size_t n_words = a.kpm ? (size_t)a.B * a.nb : 0, n_counters = 1 + (size_t)n_split;
+    const size_t off_bits = align256((size_t)BH * a.nb * kStatFloats * sizeof(float));
+    const size_t off_cnt = off_bits + align256(n_words * sizeof(unsigned long long));
+    const size_t off_part = off_cnt + align256(n_counters * sizeof(int));
+    const size_t bytes = off_part + (size_t)n_split * parts * kPartialFloats * sizeof(float);
+    unsigned char* ws = nullptr;
+    e = cudaMallocFromPoolAsync((void**)&ws, bytes, pool, a.stream);
+    if (e != cudaSuccess) return fail(e);
+
+    KernelParams p{};
+    p.dq = (__nv_bfloat16*)a.dq;
+    p.dk = (__nv_bfloat16*)a.dk;
+    p.dv = (__nv_bfloat16*)a.dv;
+    p.stats = (const float*)ws;
+    p.kbits = a.kpm ? (const unsigned long long*)(ws + off_bits) : nullptr;
+    p.counter = (int*)(ws + off_cnt);
+    p.arrived = p.counter + 1;
+    p.partials = (float*)(ws + off_part);
+    p.status = status;
+    p.items_q = dl.items + L.heavy_items_per_head;
+    p.q_stride = L.items_per_head;
+    p.items_k = dl.items_t;
+    p.steps_q = dl.steps;
+    p.steps_k = dl.steps_t;
+    p.global_pairs = dl.global_pairs;
+    p.sparse_tiles = L.sparse_tiles_per_head;
+    p.global_tiles = L.global_tiles;
+    p.parts = parts;
+    p.part_steps = part_steps;
+    p.BH = BH;
+    p.H = a.H;
+    p.nb = a.nb;
+    p.total_work = 2 * BH * (L.global_tiles * parts + L.sparse_tiles_per_head);
+    p.scale = a.scale;
+    p.scale_log2 = a.scale * 1.4426950408889634f;
+
+    const int row_ctas = (int)((rows + 2 * kPrepRows - 1) / (2 * kPrepRows));
+    const int extra = (int)std::min<size_t>(64, 1 + n_words / 64 + n_counters / 2048);
+    attn_bwd_prepare_kernel<<<row_ctas + extra, kPrepThreads, 0, a.stream>>>((const uint4*)a.out, (const uint4*)a.dout, a.lse, a.kpm, (float*)ws,
+        (unsigned long long*)(ws + off_bits), p.counter, (int)n_counters, rows, (int)a.N, a.H, row_ctas, (int)n_words);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) {
+        ++*launches;
+        attn_bwd_sm100_kernel<<<std::min(sms, p.total_work), kThreads, kSmemBytes, a.stream>>>(tm_q, tm_k, tm_v, tm_do, p);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) ++*launches;
+    }
+    const cudaError_t ef = cudaFreeAsync(ws, a.stream);
+    if (e == cudaSuccess) e = ef;
+    return e == cudaSuccess ? BIGBIRD_OK : fail(e);
+}
+
+}  // namespace bigbird

@@ -57,6 +57,12 @@ cudaError_t launch_attn_fwd_simt(const FwdArgs& a, const DeviceLayout& dl, int* 
 // CUDA-core gradient kernels (fp32 arithmetic): dq by query block, dk and dv by key block over the transposed lists.
 cudaError_t launch_attn_bwd_simt(const BwdArgs& a, const DeviceLayout& dl, int* launches);
 
+// tcgen05 gradient kernels (bf16 tensors, b = D = 64).  The workspace of a call comes from `pool`, in stream order.  Returns a
+// BIGBIRD_* code; *cuda_err receives the cudaError_t on BIGBIRD_ECUDA.
+bool attn_bwd_sm100_takes(const BwdArgs& a);
+int launch_attn_bwd_sm100(const BwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, cudaMemPool_t pool, int* status,
+                          int* launches, cudaError_t* cuda_err);
+
 // tcgen05 kernel (bf16 operands).  Returns a BIGBIRD_* code; *cuda_err receives the cudaError_t on BIGBIRD_ECUDA.
 int launch_attn_fwd_sm100(const FwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, DeviceScratch& sc,
                           int* launches, cudaError_t* cuda_err);

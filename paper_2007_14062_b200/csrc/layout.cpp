@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <atomic>
 #include <new>
+#include <utility>
 
 #include "../../include/bigbird.h"
 
@@ -38,38 +39,116 @@ void global_flags(const bigbird_layout& L, std::vector<uint8_t>& is_global) {
 }
 
 // Key blocks of one non-global query block: window (App. D item 2), global columns (item 3), random (item 1).
-void sparse_row(const bigbird_layout& L, const std::vector<uint8_t>& is_global, int h, int j,
-                std::vector<uint8_t>& mark, std::vector<int32_t>& cand, std::vector<int32_t>& out) {
+// Works on the few blocks of the row and not on all nb of them: position i of the ascending candidate list (the blocks that
+// are neither in the window nor global) is i plus the excluded blocks before it, and of the shuffled list only the entries
+// that a swap has moved are kept.
+// (Rows with many random blocks write the list out: finding an entry among the moved ones is a search.)
+struct RowScratch {
+    std::vector<int32_t> taken;                            // window and global blocks, ascending
+    std::vector<int32_t> all;                              // the candidate list, if written out
+    std::vector<std::pair<uint64_t, int32_t>> moved;       // (position, block) of the entries that differ from the ascending list
+};
+void sparse_row(const bigbird_layout& L, const std::vector<int32_t>& globals, int h, int j, RowScratch& s, std::vector<int32_t>& out) {
     const int nb = L.nb, hw = (L.w - 1) / 2;
-    std::fill(mark.begin(), mark.end(), 0);
-    for (int c = std::max(0, j - hw); c <= std::min(nb - 1, j + hw); ++c) mark[c] = 1;
-    for (int c = 0; c < nb; ++c)
-        if (is_global[c]) mark[c] = 1;
-    if (L.r > 0) {
-        cand.clear();
-        for (int c = 0; c < nb; ++c)
-            if (!mark[c]) cand.push_back(c);
-        const uint64_t m = cand.size();
-        const uint64_t take = std::min<uint64_t>((uint64_t)L.r, m);
-        SplitMix64 gen((L.seed << 40) ^ ((uint64_t)h << 20) ^ (uint64_t)j);
-        for (uint64_t t = 0; t < take; ++t) {
-            const uint64_t p = t + gen.below(m - t);
-            std::swap(cand[t], cand[p]);
+    const int lo = std::max(0, j - hw), hi = std::min(nb - 1, j + hw);
+    std::vector<int32_t>& taken = s.taken;
+    taken.clear();
+    for (size_t i = 0;; ++i) {                             // merge of the window with the ascending global blocks
+        if (i == globals.size() || globals[i] >= lo) {
+            for (int c = lo; c <= hi; ++c) taken.push_back(c);
+            for (; i < globals.size(); ++i)
+                if (globals[i] > hi) taken.push_back(globals[i]);
+            break;
         }
-        for (uint64_t t = 0; t < take; ++t) mark[cand[t]] = 1;
+        taken.push_back(globals[i]);
     }
-    out.clear();
-    for (int c = 0; c < nb; ++c)
-        if (mark[c]) out.push_back(c);
+    const size_t row_begin = out.size();
+    out.insert(out.end(), taken.begin(), taken.end());
+    const uint64_t m = (uint64_t)nb - taken.size(), take = std::min<uint64_t>((uint64_t)L.r, m);
+    if (take == 0) return;
+    auto ascending = [&](uint64_t i) {
+        int32_t c = (int32_t)i;
+        for (int32_t e : taken) {
+            if (e > c) break;
+            ++c;
+        }
+        return c;
+    };
+    SplitMix64 gen((L.seed << 40) ^ ((uint64_t)h << 20) ^ (uint64_t)j);
+    if (take > 32) {
+        s.all.clear();
+        size_t i = 0;
+        for (int32_t c = 0; c < nb; ++c) {
+            if (i < taken.size() && taken[i] == c) ++i;
+            else s.all.push_back(c);
+        }
+        for (uint64_t t = 0; t < take; ++t) std::swap(s.all[t], s.all[t + gen.below(m - t)]);
+        out.insert(out.end(), s.all.begin(), s.all.begin() + take);
+        std::sort(out.begin() + row_begin, out.end());
+        return;
+    }
+    s.moved.clear();
+    auto entry = [&](uint64_t i) -> std::pair<uint64_t, int32_t>* {
+        for (auto& e : s.moved)
+            if (e.first == i) return &e;
+        return nullptr;
+    };
+    for (uint64_t t = 0; t < take; ++t) {                  // swap entries t and p; entry t is final afterwards
+        const uint64_t p = t + gen.below(m - t);
+        auto *et = entry(t), *ep = entry(p);
+        const int32_t ct = et ? et->second : ascending(t), cp = ep ? ep->second : ascending(p);
+        out.push_back(cp);
+        if (p != t) {
+            if (ep) ep->second = ct;
+            else s.moved.emplace_back(p, ct);
+        }
+    }
+    std::sort(out.begin() + row_begin, out.end());
+}
+
+// Steps of a tile that stacks rows qa (upper half) and qb (lower half, or kNoBlock) of one head's lists: the merge of the
+// two ascending lists.
+struct TileScratch {
+    std::vector<int32_t> both, pa, pb;
+};
+void sparse_tile(const std::vector<int32_t>& ptr, const std::vector<int32_t>& idx, size_t row0, int qa, int qb, TileScratch& t,
+                 std::vector<Step>& steps) {
+    const int32_t ea = ptr[row0 + qa + 1];
+    int32_t ia = ptr[row0 + qa];
+    if (qb == kNoBlock) {
+        for (; ia < ea; ++ia) steps.push_back(Step{idx[ia], kBothHalves});
+        return;
+    }
+    const int32_t eb = ptr[row0 + qb + 1];
+    int32_t ib = ptr[row0 + qb];
+    t.both.clear();
+    t.pa.clear();
+    t.pb.clear();
+    while (ia < ea || ib < eb) {
+        if (ib == eb || (ia < ea && idx[ia] < idx[ib])) t.pa.push_back(idx[ia++]);
+        else if (ia == ea || idx[ib] < idx[ia]) t.pb.push_back(idx[ib++]);
+        else { t.both.push_back(idx[ia]); ++ia; ++ib; }
+    }
+    // shared, upper-only and lower-only key blocks take turns, so that any run of three consecutive steps gives both
+    // halves of the tile about the same amount of work
+    const size_t ns = std::max(t.both.size(), std::max(t.pa.size(), t.pb.size()));
+    for (size_t s = 0; s < ns; ++s) {
+        if (s < t.both.size()) steps.push_back(Step{t.both[s], kBothHalves});
+        if (s < t.pa.size()) steps.push_back(Step{t.pa[s], kUpperHalf});
+        if (s < t.pb.size()) steps.push_back(Step{t.pb[s], kLowerHalf});
+    }
 }
 
 }  // namespace
 
 int build_layout_host(bigbird_layout* L, int chunk_steps) {
     const int nb = L->nb, H = L->H;
-    std::vector<uint8_t> is_global, mark(nb);
-    std::vector<int32_t> cand, row;
+    std::vector<uint8_t> is_global;
+    std::vector<int32_t> globals;
+    RowScratch row_scratch;
     global_flags(*L, is_global);
+    for (int c = 0; c < nb; ++c)
+        if (is_global[c]) globals.push_back(c);
 
     // ---- CSR ------------------------------------------------------------------------------------
     L->row_ptr.assign(1, 0);
@@ -79,8 +158,7 @@ int build_layout_host(bigbird_layout* L, int chunk_steps) {
             if (is_global[j]) {
                 for (int c = 0; c < nb; ++c) L->col_idx.push_back(c);       // global rows attend everything
             } else {
-                sparse_row(*L, is_global, h, j, mark, cand, row);
-                L->col_idx.insert(L->col_idx.end(), row.begin(), row.end());
+                sparse_row(*L, globals, h, j, row_scratch, L->col_idx);
             }
             if (L->col_idx.size() > (size_t)INT32_MAX) return BIGBIRD_EUNSUPPORTED;
             L->row_ptr.push_back((int32_t)L->col_idx.size());
@@ -126,7 +204,7 @@ int build_layout_host(bigbird_layout* L, int chunk_steps) {
         L->split_tile_q.push_back(gq[2 * t]);
         L->split_tile_q.push_back(2 * t + 1 < (int)gq.size() ? gq[2 * t + 1] : kNoBlock);
     }
-    std::vector<int32_t> la, lb, both, pa, pb;
+    TileScratch tmp;
     for (int h = 0; h < H; ++h) {
         const int32_t base = (int32_t)L->steps.size();
         L->step_base.push_back(base);
@@ -153,33 +231,7 @@ int build_layout_host(bigbird_layout* L, int chunk_steps) {
             it.step_begin = rel();
             it.part = -1;
             it.nparts = 1;
-            const int32_t* ra = &L->col_idx[L->row_ptr[(size_t)h * nb + it.qa]];
-            const int na = L->row_ptr[(size_t)h * nb + it.qa + 1] - L->row_ptr[(size_t)h * nb + it.qa];
-            la.assign(ra, ra + na);
-            if (it.qb == kNoBlock) {
-                for (int32_t c : la) L->steps.push_back(Step{c, kBothHalves});
-            } else {
-                const int32_t* rb = &L->col_idx[L->row_ptr[(size_t)h * nb + it.qb]];
-                const int nbk = L->row_ptr[(size_t)h * nb + it.qb + 1] - L->row_ptr[(size_t)h * nb + it.qb];
-                lb.assign(rb, rb + nbk);
-                both.clear();
-                pa.clear();
-                pb.clear();
-                size_t ia = 0, ib = 0;
-                while (ia < la.size() || ib < lb.size()) {                   // merge of two ascending lists
-                    if (ib == lb.size() || (ia < la.size() && la[ia] < lb[ib])) pa.push_back(la[ia++]);
-                    else if (ia == la.size() || lb[ib] < la[ia]) pb.push_back(lb[ib++]);
-                    else { both.push_back(la[ia]); ++ia; ++ib; }
-                }
-                // shared, upper-only and lower-only key blocks take turns, so that any run of three
-                // consecutive steps gives both halves of the tile about the same amount of work
-                const size_t ns = std::max(both.size(), std::max(pa.size(), pb.size()));
-                for (size_t s = 0; s < ns; ++s) {
-                    if (s < both.size()) L->steps.push_back(Step{both[s], kBothHalves});
-                    if (s < pa.size()) L->steps.push_back(Step{pa[s], kUpperHalf});
-                    if (s < pb.size()) L->steps.push_back(Step{pb[s], kLowerHalf});
-                }
-            }
+            sparse_tile(L->row_ptr, L->col_idx, (size_t)h * nb, it.qa, it.qb, tmp, L->steps);
             it.step_count = rel() - it.step_begin;
             L->items.push_back(it);
         }
@@ -187,6 +239,29 @@ int build_layout_host(bigbird_layout* L, int chunk_steps) {
     L->items_abs = L->items;
     for (int h = 0; h < H; ++h)
         for (int i = 0; i < L->items_per_head; ++i) L->items_abs[(size_t)h * L->items_per_head + i].step_begin += L->step_base[h];
+
+    // ---- what the tensor-core gradients walk besides: pairs of key blocks with the query blocks that attend them ----
+    // (the global key blocks are attended by every query block, so their tiles need no list)
+    L->sparse_tiles_per_head = n_stiles;
+    L->global_tiles = n_gtiles;
+    L->global_pairs.assign(2 * (size_t)n_gtiles, kNoBlock);
+    for (size_t i = 0; i < gq.size(); ++i) L->global_pairs[i] = gq[i];
+    L->items_t.clear();
+    L->steps_t.clear();
+    if (L->b == 64) {
+        for (int h = 0; h < H; ++h)
+            for (int t = 0; t < n_stiles; ++t) {
+                Item it{};
+                it.qa = sq[2 * t];
+                it.qb = 2 * t + 1 < (int)sq.size() ? sq[2 * t + 1] : kNoBlock;
+                it.step_begin = (int32_t)L->steps_t.size();
+                it.part = -1;
+                it.nparts = 1;
+                sparse_tile(L->col_ptr, L->row_idx, (size_t)h * nb, it.qa, it.qb, tmp, L->steps_t);
+                it.step_count = (int32_t)L->steps_t.size() - it.step_begin;
+                L->items_t.push_back(it);
+            }
+    }
     return BIGBIRD_OK;
 }
 

@@ -38,6 +38,10 @@ struct DeviceLayout {
     Item* items = nullptr;
     Step* steps = nullptr;
     int32_t* split_tile_q = nullptr;   // [split_tiles_per_head * 2]
+    Item* items_t = nullptr;           // tiles of key blocks over the transposed lists
+    Step* steps_t = nullptr;
+    int32_t* global_pairs = nullptr;   // [global_tiles * 2]
+    void* block = nullptr;             // the one allocation that holds the arrays above
 };
 
 }  // namespace bigbird
@@ -64,6 +68,13 @@ struct bigbird_layout {
     std::vector<int32_t> step_base;            // [H] offset of the head's steps in `steps`
     std::vector<bigbird::Step> steps;
     std::vector<int32_t> split_tile_q;         // [split_tiles_per_head * 2] query blocks (qa, qb) of each split tile
+    // the same for tiles that stack two key blocks and walk the query blocks that attend them (b == 64 only); global
+    // key blocks have no list, every query block attends them
+    int sparse_tiles_per_head = 0;
+    int global_tiles = 0;                      // tiles of two global blocks
+    std::vector<int32_t> global_pairs;         // [global_tiles * 2], the last entry kNoBlock if their number is odd
+    std::vector<bigbird::Item> items_t;        // [H * sparse_tiles_per_head], step_begin absolute
+    std::vector<bigbird::Step> steps_t;
     // device copies, made on first use
     mutable std::mutex mu;
     mutable bigbird::DeviceLayout dev;

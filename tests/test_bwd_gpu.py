@@ -80,3 +80,19 @@ def test_bad_arguments_are_refused_without_a_launch():
     assert bb.lib().bigbird_attn_bwd(*args(N=1024)) == -1       # layout built for another N
     assert bb.lib().bigbird_attn_bwd(*args(D=48)) == -2
     L.close()
+
+
+# The tensor-core gradient kernels (bf16, b = D = 64) where their schedule can go wrong.  Tolerances as above.
+EDGES = [
+    _case("bf16", 1, 1, 1, g=1, r=0),                           # one block, one tile without a lower half
+    _case("bf16", 1, 1, 4, g=4, r=0),                           # every block global: no sparse tile
+    _case("bf16", 1, 2, 7, g=0, r=1),                           # no global block, an unpaired tile
+    _case("bf16", 1, 1, 40, g=3, r=2),                          # few heads: tiles of global blocks cut into parts, one of them half empty
+    _case("bf16", 1, 1, 120, w=101, lengths="fixed:7000"),      # lists longer than one posted segment
+    _case("bf16", 6, 2, 40, lengths="ragged:1:700"),            # mostly padding: many tiles and parts without any step
+]
+
+
+@pytest.mark.parametrize("wl", EDGES, ids=lambda w: f"{w.name}_{w.lengths}_{w.B}_{w.g}{w.r}{w.w}")
+def test_tensor_core_gradients_at_the_edges_of_the_schedule(wl):
+    test_gradients_match_the_oracle(wl)
