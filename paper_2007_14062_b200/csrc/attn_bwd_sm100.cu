@@ -14,10 +14,9 @@
 // results, at twice the number of the accumulating MMAs.
 //
 // Nothing carries over from step to step but the accumulators, so the steps of a tile are dealt in turn to three warpgroups
-// with a 128-column score buffer each.  One thread issues every MMA: S and dP of a step up to three steps ahead of the step
-// whose accumulation is issued.  A buffer needs no barrier to become free: the MMAs that overwrite it are issued behind the
-// ones that read it, and the tensor pipe keeps their order.  An epilogue warpgroup takes a finished tile's accumulators while
-// the next tile's scores are being computed.
+// with a 128-column score buffer each.  One thread issues the scores of a step as soon as its buffer is free, another the
+// accumulation of the steps in turn.  An epilogue warpgroup takes a finished tile's accumulators while the next tile's scores
+// are being computed.
 // CTAs are persistent; a scheduler warp draws work from a counter: the tiles of global blocks first, cut along their (full)
 // lists into parts where they would outlast the rest, then per (batch, head) the key tiles and the query tiles.  A part
 // leaves its fp32 accumulators in scratch; whichever part is done last sums all of them in a fixed order.  No float atomics:
@@ -41,9 +40,10 @@ constexpr int kBufs = 3;                   // score buffers, each served by one 
 constexpr int kStages = 6;                 // ring of Y1 | Y2 pairs
 constexpr int kSlots = 3;                  // tiles (or segments of long ones) posted by the scheduler
 constexpr int kSegSteps = 96;              // steps per posted segment
-// warps 0..11: the three elementwise warpgroups; 12..15: epilogue; 16: scheduler; 17: TMA producer; 18: MMA issuer
+// warps 0..11: the three elementwise warpgroups; 12..15: epilogue; 16: scheduler; 17: TMA producer; 18, 19: MMA issuers (scores,
+// accumulations)
 constexpr int kThreads = 640;
-constexpr int kWarpEpilogue = 12, kWarpScheduler = 16, kWarpProducer = 17, kWarpMma = 18;
+constexpr int kWarpEpilogue = 12, kWarpScheduler = 16, kWarpProducer = 17, kWarpScore = 18;
 // 640 threads start with 96 registers each; a sub-partition's five warps share 480: three elementwise warps x 120 (32 columns
 // of S and of dP and what becomes of them), an epilogue warp x 64 and a light warp x 56.
 constexpr int kRegsElem = 120, kRegsEpilogue = 64, kRegsLight = 56;
@@ -55,7 +55,8 @@ static_assert(kColAcc + 128 <= kTmemCols, "tensor memory");
 constexpr int kStatFloats = 2 * kBlock;    // per block of query rows: 64 x (-lse log2 e), 64 x (-delta)
 constexpr int kPartialFloats = 2 * 128 * kBlock;   // one part of a split tile: acc0, acc1
 enum { kDkv = 0, kDq = 1 };
-enum { kSegFirst = 1, kSegLast = 2, kSegLive = 4 };
+enum { kSegFirst = 1, kSegLast = 2 };
+enum { kInfoDkv = 1, kInfoFirst = 2, kInfoLast = 4, kInfoEnd = 8 };   // what the issuing threads have to know about a step
 
 struct __align__(16) StepEntry {
     int c;                         // block of the column side
@@ -82,6 +83,7 @@ struct __align__(16) SmemCtl {
     TileSlot slot[kSlots];
     float x_stats[2][2][kStatFloats];      // query tiles: statistics of the rows
     float y_stats[kStages][kStatFloats];   // key tiles: of the step's query block
+    unsigned info[kStages];
     unsigned tmem_base;
     int abort_flag;
     int merge_last;
@@ -156,16 +158,21 @@ __device__ __forceinline__ void scheduler_role(const KernelParams& p, SmemCtl* c
         }
         const int batch = bh / p.H;
         const unsigned long long rbits_a = w >= 0 ? token_bits(p, batch, ra) : 0ull, rbits_b = w >= 0 ? token_bits(p, batch, rb) : 0ull;
-        const bool live = (rbits_a | rbits_b) != 0ull;       // a tile without any valid row needs no steps
-        if (!live) n_raw = 0;
+        if ((rbits_a | rbits_b) == 0ull) n_raw = 0;          // a tile without any valid row needs no steps
         int i0 = 0;
         bool first = true;
+        StepEntry held{-1, 0, 0ull};               // last step of a full segment: kept for the next one, so that no tile's last
+        bool holding = false;                      // segment turns out to be empty
         do {
             const unsigned ss = slot_n % kSlots;
             if (!mbar_wait(&ctl->slot_empty[ss], ((slot_n / kSlots) & 1u) ^ 1u, &ctl->abort_flag)) { give_up(&ctl->abort_flag, p.status, 111); return; }
             __syncwarp();
             TileSlot* slot = &ctl->slot[ss];
             int count = 0;
+            if (holding) {
+                if (lane == 0) slot->steps[0] = held;
+                count = 1;
+            }
 #pragma unroll 1
             while (i0 < n_raw && count <= kSegSteps - 32) {
                 const int i = i0 + lane;
@@ -185,6 +192,9 @@ __device__ __forceinline__ void scheduler_role(const KernelParams& p, SmemCtl* c
                 count += __popc(bal);
                 i0 += 32;
             }
+            __syncwarp();
+            holding = i0 < n_raw && count > 0;
+            if (holding) held = slot->steps[--count];
             if (lane == 0) {
                 slot->w = w;
                 slot->kind = kind;
@@ -192,7 +202,7 @@ __device__ __forceinline__ void scheduler_role(const KernelParams& p, SmemCtl* c
                 slot->ra = ra;
                 slot->rb = rb;
                 slot->n = count;
-                slot->flags = (first ? kSegFirst : 0) | (i0 >= n_raw ? kSegLast : 0) | (live ? kSegLive : 0);
+                slot->flags = (first ? kSegFirst : 0) | (i0 >= n_raw ? kSegLast : 0);
                 slot->split = split;
                 slot->part = part;
                 slot->rbits_a = rbits_a;
@@ -213,6 +223,7 @@ __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ct
                                               const CUtensorMap* tm_k, const CUtensorMap* tm_v, const CUtensorMap* tm_do) {
     int* abort_flag = &ctl->abort_flag;
     unsigned slot_n = 0, tile_n = 0, step_n = 0;
+    bool fresh = false;                             // no step of the tile has been loaded yet
     int fail = 0;
     for (;;) {
         const unsigned ss = slot_n % kSlots;
@@ -220,205 +231,198 @@ __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ct
         const TileSlot* slot = &ctl->slot[ss];
         const int w = slot->w, flags = slot->flags, n = slot->n, bh = slot->bh;
         const bool dkv = slot->kind == kDkv;
-        if (w >= 0 && (flags & kSegLive)) {
-            if (flags & kSegFirst) {
+        if (w < 0) {                                // the last entry of the ring
+            const unsigned g = step_n % kStages;
+            if (!mbar_wait(&ctl->empty[g], ((step_n / kStages) & 1u) ^ 1u, abort_flag)) { fail = 110; break; }
+            ctl->info[g] = kInfoEnd;
+            mbar_arrive(&ctl->full[g]);
+            break;
+        }
+        if (flags & kSegFirst) fresh = true;
+        const CUtensorMap *tm1 = dkv ? tm_q : tm_k, *tm2 = dkv ? tm_do : tm_v;
+        for (int i = 0; i < n; ++i) {
+            unsigned info = (dkv ? kInfoDkv : 0) | (i == n - 1 && (flags & kSegLast) ? kInfoLast : 0);
+            if (fresh) {
                 const int ra = slot->ra, rb = slot->rb;
                 const unsigned xs = tile_n & 1u;
                 if (!mbar_wait(&ctl->x_empty[xs], ((tile_n >> 1) & 1u) ^ 1u, abort_flag)) { fail = 112; break; }
                 unsigned char* x = smem + kSmemX + xs * 4 * kTileBytes;
                 unsigned long long* bar = &ctl->x_full[xs];
-                const CUtensorMap *tm1 = dkv ? tm_k : tm_q, *tm2 = dkv ? tm_v : tm_do;
+                const CUtensorMap *xm1 = dkv ? tm_k : tm_q, *xm2 = dkv ? tm_v : tm_do;
                 const int blocks = rb >= 0 ? 2 : 1;
                 mbar_expect_tx(bar, blocks * (2 * kTileBytes + (dkv ? 0 : kStatFloats * 4)));
                 for (int j = 0; j < blocks; ++j) {
                     const int row = bh * p.nb + (j ? rb : ra);
-                    tma_load_tile(x + j * kTileBytes, tm1, row * kBlock, bar);
-                    tma_load_tile(x + (2 + j) * kTileBytes, tm2, row * kBlock, bar);
+                    tma_load_tile(x + j * kTileBytes, xm1, row * kBlock, bar);
+                    tma_load_tile(x + (2 + j) * kTileBytes, xm2, row * kBlock, bar);
                     if (!dkv) bulk_load(ctl->x_stats[xs][j], p.stats + (size_t)row * kStatFloats, kStatFloats * 4, bar);
                 }
                 ++tile_n;
+                fresh = false;
+                info |= kInfoFirst;
             }
-            const CUtensorMap *tm1 = dkv ? tm_q : tm_k, *tm2 = dkv ? tm_do : tm_v;
-            for (int i = 0; i < n; ++i) {
-                const unsigned g = step_n % kStages;
-                const int row = bh * p.nb + slot->steps[i].c;
-                if (!mbar_wait(&ctl->empty[g], ((step_n / kStages) & 1u) ^ 1u, abort_flag)) { fail = 110; break; }
-                unsigned char* y = smem + kSmemRing + g * 2 * kTileBytes;
-                mbar_expect_tx(&ctl->full[g], 2 * kTileBytes + (dkv ? kStatFloats * 4 : 0));
-                tma_load_tile(y, tm1, row * kBlock, &ctl->full[g]);
-                tma_load_tile(y + kTileBytes, tm2, row * kBlock, &ctl->full[g]);
-                if (dkv) bulk_load(ctl->y_stats[g], p.stats + (size_t)row * kStatFloats, kStatFloats * 4, &ctl->full[g]);
-                ++step_n;
-            }
-            if (fail) break;
+            const unsigned g = step_n % kStages;
+            const int row = bh * p.nb + slot->steps[i].c;
+            if (!mbar_wait(&ctl->empty[g], ((step_n / kStages) & 1u) ^ 1u, abort_flag)) { fail = 110; break; }
+            unsigned char* y = smem + kSmemRing + g * 2 * kTileBytes;
+            ctl->info[g] = info;
+            mbar_expect_tx(&ctl->full[g], 2 * kTileBytes + (dkv ? kStatFloats * 4 : 0));
+            tma_load_tile(y, tm1, row * kBlock, &ctl->full[g]);
+            tma_load_tile(y + kTileBytes, tm2, row * kBlock, &ctl->full[g]);
+            if (dkv) bulk_load(ctl->y_stats[g], p.stats + (size_t)row * kStatFloats, kStatFloats * 4, &ctl->full[g]);
+            ++step_n;
         }
+        if (fail) break;
         mbar_arrive(&ctl->slot_empty[ss]);
         ++slot_n;
-        if (w < 0) break;
     }
     if (fail) give_up(abort_flag, p.status, fail);
 }
 
-// ------------------------------------------------------------------------------------------------ MMA issuer (one thread)
-// front: steps whose S and dP have been issued; back: steps whose accumulation has been issued.
-__device__ __forceinline__ void mma_role(const KernelParams& p, SmemCtl* ctl, unsigned char* smem, unsigned tmem) {
+// ------------------------------------------------------------------------------------------------ MMA issuers (two threads)
+// Each is alone in its warp, so nothing hides the latency of its instructions: an MMA takes some 30 cycles to issue, a barrier
+// test 45, a test behind a commit 200.  One thread that issued everything and walked the posted tiles needed 1740 cycles a step.
+// So one issues the scores (S and dP) and one the accumulations, and both see the ring only, where each entry comes with a word
+// that says what there is to know about the step.  full[] tells both of a loaded entry, empty[] (committed behind a step's
+// accumulation) frees the ring entry for the producer and, three steps on, the score buffer for the first thread.
+__device__ __forceinline__ void score_role(const KernelParams& p, SmemCtl* ctl, unsigned char* smem, unsigned tmem) {
     int* abort_flag = &ctl->abort_flag;
-    unsigned slot_n = 0, tile_n = 0, acc_n = 0, front = 0, back = 0;
-    unsigned firsts = 0, lasts = 0, kinds = 0;      // bit (step & 7) of the steps between back and front
-    unsigned buf_f = 0, buf_b = 0;                  // front % kBufs, back % kBufs
-    unsigned par_b = 0;                             // parity of p_full of the step at back
-    unsigned stg_f = 0, stg_b = 0, ph_f = 0;        // ring stages of front and back, phase of front's
-    bool open = false, done = false, fresh = false, tile_steps = false;
-    const TileSlot* slot = nullptr;
-    int i = 0, n = 0, flags = 0;
-    unsigned kind = 0, xs = 0;
+    constexpr unsigned kStageDesc = (2 * kTileBytes) >> 4, kTileDesc = kTileBytes >> 4;
+    const unsigned ring0 = smem_desc_lo(smem_u32(smem + kSmemRing)), x0 = smem_desc_lo(smem_u32(smem + kSmemX));
+    unsigned stg = 0, ph = 0, buf = 0;              // this step's ring entry (and its phase) and score buffer
+    unsigned old = 0, old_ph = 0, n = 0;            // ring entry and phase of the step three back; steps issued, up to kBufs
+    unsigned xs = 0, x_par = 0, x1 = x0;            // row buffer of the tile
     int fail = 0;
-    const unsigned x_base = smem_u32(smem + kSmemX), ring_base = smem_u32(smem + kSmemRing);
     for (;;) {
-        const unsigned ss = slot_n % kSlots;
-        // (with steps pending the thread must not sleep on the next slot: tiles without steps pass through the slots quickly,
-        // and the next one may only become free once the pending steps' tile is finished)
-        if (!done && front - back < (unsigned)kBufs && (open || front == back || mbar_test(&ctl->slot_full[ss], (slot_n / kSlots) & 1u))) {
-            if (!open) {
-                if (!mbar_wait(&ctl->slot_full[ss], (slot_n / kSlots) & 1u, abort_flag)) { fail = 123; break; }
-                slot = &ctl->slot[ss];
-                if (slot->w < 0) { mbar_arrive(&ctl->slot_empty[ss]); done = true; continue; }
-                flags = slot->flags;
-                kind = (unsigned)slot->kind;
-                n = (flags & kSegLive) ? slot->n : 0;
-                i = 0;
-                open = true;
-                if ((flags & (kSegFirst | kSegLive)) == (kSegFirst | kSegLive)) {
-                    xs = tile_n & 1u;
-                    if (!mbar_wait(&ctl->x_full[xs], (tile_n >> 1) & 1u, abort_flag)) { fail = 124; break; }
-                    ++tile_n;
-                    fresh = true;
-                    tile_steps = false;
-                }
-            }
-            if (i < n) {
-                if (!mbar_wait(&ctl->full[stg_f], ph_f, abort_flag)) { fail = 120; break; }
-                tc_fence_after();
-                const unsigned long long x1 = smem_desc_sw128(x_base + xs * 4 * kTileBytes), x2 = x1 + ((2 * kTileBytes) >> 4);
-                const unsigned long long y1 = smem_desc_sw128(ring_base + stg_f * 2 * kTileBytes), y2 = y1 + (kTileBytes >> 4);
-                const unsigned d = tmem + buf_f * kBufCols;
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) mma_ss(d, x1 + kk * 2, y1 + kk * 2, kIdescQK64, kk > 0);
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) mma_ss(d + 64, x2 + kk * 2, y2 + kk * 2, kIdescQK64, kk > 0);
-                tc_commit(&ctl->sdp_full[buf_f]);
-                const unsigned bit = 1u << (front & 7u);
-                firsts = fresh ? (firsts | bit) : (firsts & ~bit);
-                kinds = kind ? (kinds | bit) : (kinds & ~bit);
-                lasts &= ~bit;
-                fresh = false;
-                tile_steps = true;
-                ++front;
-                ++i;
-                buf_f = buf_f == kBufs - 1 ? 0u : buf_f + 1u;
-                if (++stg_f == kStages) { stg_f = 0; ph_f ^= 1u; }
-            }
-            if (i >= n) {                           // end of the segment
-                if ((flags & (kSegLast | kSegLive)) == (kSegLast | kSegLive)) {
-                    tc_commit(&ctl->x_empty[xs]);   // every S and dP of the tile has been issued
-                    if (tile_steps) {
-                        if (front != back) lasts |= 1u << ((front - 1u) & 7u);
-                        else { tc_commit(&ctl->acc_full); ++acc_n; }
-                    }
-                }
-                mbar_arrive(&ctl->slot_empty[ss]);
-                ++slot_n;
-                open = false;
-            }
-            continue;
+        if (!mbar_wait(&ctl->full[stg], ph, abort_flag)) { fail = 120; break; }
+        const unsigned info = ctl->info[stg];
+        if (info & kInfoEnd) break;
+        if (n == (unsigned)kBufs) {                 // the buffer's last user must have been accumulated
+            if (!mbar_wait(&ctl->empty[old], old_ph, abort_flag)) { fail = 121; break; }
+            if (++old == kStages) { old = 0; old_ph ^= 1u; }
+        } else ++n;
+        if (info & kInfoFirst) {
+            if (!mbar_wait(&ctl->x_full[xs], x_par, abort_flag)) { fail = 124; break; }
+            x1 = x0 + xs * 4 * kTileDesc;
         }
-        if (front == back) break;                   // done, and nothing is pending
-        const unsigned bit = 1u << (back & 7u);
-        // the epilogue must have taken the previous tile's accumulators before this tile's first product overwrites them
-        if ((firsts & bit) && acc_n > 0 && !mbar_wait(&ctl->acc_free, (acc_n - 1) & 1u, abort_flag)) { fail = 127; break; }
-        if (!mbar_wait(&ctl->p_full[buf_b], par_b, abort_flag)) { fail = 122; break; }
         tc_fence_after();
-        {
-            const unsigned long long y1 = smem_desc_sw128(ring_base + stg_b * 2 * kTileBytes), y2 = y1 + (kTileBytes >> 4);
-            const unsigned a = tmem + buf_b * kBufCols, acc = tmem + kColAcc;
-            const unsigned keep = (firsts & bit) ? 0u : 1u;
-            const bool dkv = !(kinds & bit);
-            // 16 tokens per MMA: 8 packed columns of A (the high halves of 32 columns, then their low halves), two 8-row groups of Y
-            if (dkv) {
+        const unsigned y1 = ring0 + stg * kStageDesc, d = tmem + buf * kBufCols;
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    const unsigned ak = a + (kk >> 1) * 32 + (kk & 1) * 8;
-                    mma_ts(acc + 64, ak, y2 + ((kk * 2048) >> 4), kIdescPV, kk > 0 ? 1u : keep);
-                    mma_ts(acc + 64, ak + 16, y2 + ((kk * 2048) >> 4), kIdescPV, 1u);
-                }
-            }
-            const unsigned ds = dkv ? a + 64 : a;
+        for (int kk = 0; kk < 4; ++kk) mma_ss_lo(d, x1 + kk * 2, y1 + kk * 2, kIdescQK64, kk > 0);
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) mma_ss_lo(d + 64, x1 + 2 * kTileDesc + kk * 2, y1 + kTileDesc + kk * 2, kIdescQK64, kk > 0);
+        tc_commit(&ctl->sdp_full[buf]);
+        if (info & kInfoLast) {                     // every S and dP of the tile has been issued
+            tc_commit(&ctl->x_empty[xs]);
+            x_par ^= xs;
+            xs ^= 1u;
+        }
+        if (++buf == kBufs) buf = 0;
+        if (++stg == kStages) { stg = 0; ph ^= 1u; }
+    }
+    if (fail) give_up(abort_flag, p.status, fail);
+}
+
+__device__ __forceinline__ void accumulate_role(const KernelParams& p, SmemCtl* ctl, unsigned char* smem, unsigned tmem) {
+    int* abort_flag = &ctl->abort_flag;
+    constexpr unsigned kStageDesc = (2 * kTileBytes) >> 4, kTileDesc = kTileBytes >> 4;
+    const unsigned ring0 = smem_desc_lo(smem_u32(smem + kSmemRing)), acc = tmem + kColAcc;
+    unsigned stg = 0, ph = 0, buf = 0, par = 0;     // ring entry and its phase, score buffer and the parity of its p_full
+    unsigned acc_n = 0;                             // tiles handed to the epilogue
+    int fail = 0;
+    for (;;) {
+        if (!mbar_wait(&ctl->full[stg], ph, abort_flag)) { fail = 125; break; }
+        const unsigned info = ctl->info[stg];
+        if (info & kInfoEnd) break;
+        // the epilogue must have taken the previous tile's accumulators before this tile's first product overwrites them
+        if ((info & kInfoFirst) && acc_n > 0 && !mbar_wait(&ctl->acc_free, (acc_n - 1) & 1u, abort_flag)) { fail = 127; break; }
+        if (!mbar_wait(&ctl->p_full[buf], par, abort_flag)) { fail = 122; break; }
+        tc_fence_after();
+        const unsigned y1 = ring0 + stg * kStageDesc, y2 = y1 + kTileDesc;
+        const unsigned keep = (info & kInfoFirst) ? 0u : 1u;
+        unsigned a = tmem + buf * kBufCols;
+        // 16 tokens per MMA: 8 packed columns of A (the high halves, then the low halves), two 8-row groups of Y
+        if (info & kInfoDkv) {
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
-                const unsigned ak = ds + (kk >> 1) * 32 + (kk & 1) * 8;
-                mma_ts(acc, ak, y1 + ((kk * 2048) >> 4), kIdescPV, kk > 0 ? 1u : keep);
-                mma_ts(acc, ak + 16, y1 + ((kk * 2048) >> 4), kIdescPV, 1u);
+                mma_ts_lo(acc + 64, a + kk * 16, y2 + ((kk * 2048) >> 4), kIdescPV, kk > 0 ? 1u : keep);
+                mma_ts_lo(acc + 64, a + kk * 16 + 8, y2 + ((kk * 2048) >> 4), kIdescPV, 1u);
             }
+            a += 64;
         }
-        tc_commit(&ctl->empty[stg_b]);
-        if (lasts & bit) { tc_commit(&ctl->acc_full); ++acc_n; }
-        ++back;
-        if (buf_b == kBufs - 1) { buf_b = 0; par_b ^= 1u; } else ++buf_b;
-        stg_b = stg_b == kStages - 1 ? 0u : stg_b + 1u;
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            mma_ts_lo(acc, a + kk * 16, y1 + ((kk * 2048) >> 4), kIdescPV, kk > 0 ? 1u : keep);
+            mma_ts_lo(acc, a + kk * 16 + 8, y1 + ((kk * 2048) >> 4), kIdescPV, 1u);
+        }
+        tc_commit(&ctl->empty[stg]);
+        if (info & kInfoLast) { tc_commit(&ctl->acc_full); ++acc_n; }
+        if (++buf == kBufs) { buf = 0; par ^= 1u; }
+        if (++stg == kStages) { stg = 0; ph ^= 1u; }
     }
     if (fail) give_up(abort_flag, p.status, fail);
 }
 
 // ------------------------------------------------------------------------------------------------ elementwise (three warpgroups, one thread per row)
-// Query tiles, 32 columns: dS = exp2(S sl2 + nl) (dP + nd) over S, in place.
-__device__ __forceinline__ void dq_columns(unsigned s_addr, float sl2, float nl, float nd, unsigned key_bits) {
-    float s[32], d[32];
-    unsigned hi[16], lo[16];
-    tmem_ld32(s_addr, s);
-    tmem_ld32(s_addr + 64, d);
-    tmem_wait_ld();
-    if (__builtin_expect(key_bits != 0xffffffffu, 0)) {         // padded keys
+// The 64 columns of a step, 16 at a time, the next 16 on their way out of tensor memory meanwhile.  What takes the place of 16
+// columns of fp32 is 8 columns of packed high halves and 8 of low halves.
+// Query tiles: dS = exp2(S sl2 + nl) (dP + nd) over S.
+__device__ __forceinline__ void dq_columns(unsigned buf, float sl2, float nl, float nd, unsigned long long kb) {
+    float s[2][16], d[2][16];
+    tmem_ld16(buf, s[0]);
+    tmem_ld16(buf + 64, d[0]);
 #pragma unroll
-        for (int t = 0; t < 32; ++t) s[t] = ((key_bits >> t) & 1u) ? s[t] : -INFINITY;
-    }
+    for (int c = 0; c < 4; ++c) {
+        float *sc = s[c & 1], *dc = d[c & 1];
+        tmem_wait_ld();
+        if (c < 3) {
+            tmem_ld16(buf + 16 * (c + 1), s[(c + 1) & 1]);
+            tmem_ld16(buf + 64 + 16 * (c + 1), d[(c + 1) & 1]);
+        }
+        if (__builtin_expect(kb != ~0ull, 0)) {                 // padded keys
+            const unsigned bits = (unsigned)(kb >> (16 * c));
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        float x0, x1;
-        ffma2(x0, x1, s[2 * j], s[2 * j + 1], sl2, nl);
-        add_mul2(x0, x1, d[2 * j], d[2 * j + 1], nd, nd, ex2(x0), ex2(x1));
-        split_bf16(x0, x1, hi[j], lo[j]);
+            for (int t = 0; t < 16; ++t) sc[t] = ((bits >> t) & 1u) ? sc[t] : -INFINITY;
+        }
+        unsigned o[16];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            float x0, x1;
+            ffma2(x0, x1, sc[2 * j], sc[2 * j + 1], sl2, nl);
+            add_mul2(x0, x1, dc[2 * j], dc[2 * j + 1], nd, nd, ex2(x0), ex2(x1));
+            split_bf16(x0, x1, o[j], o[8 + j]);
+        }
+        tmem_st16(buf + 16 * c, o);
     }
-    tmem_st16(s_addr, hi);
-    tmem_st16(s_addr + 16, lo);
 }
-// Key tiles, 32 columns: P over S and dS over dP; the statistics belong to the columns.
-__device__ __forceinline__ void dkv_columns(unsigned s_addr, float sl2, const float4* nl, const float4* nd) {
-    float s[32], d[32];
-    unsigned phi[16], plo[16], dhi[16], dlo[16];
-    tmem_ld32(s_addr, s);
-    tmem_ld32(s_addr + 64, d);
-    tmem_wait_ld();
+// Key tiles: P over S and dS over dP; the statistics belong to the columns.
+__device__ __forceinline__ void dkv_columns(unsigned buf, float sl2, const float2* nl, const float2* nd) {
+    float s[2][16], d[2][16];
+    tmem_ld16(buf, s[0]);
+    tmem_ld16(buf + 64, d[0]);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const float4 n4 = nl[j], d4 = nd[j];
-        float x0, x1;
-        ffma2v(x0, x1, s[4 * j], s[4 * j + 1], sl2, n4.x, n4.y);
-        x0 = ex2(x0);
-        x1 = ex2(x1);
-        split_bf16(x0, x1, phi[2 * j], plo[2 * j]);
-        add_mul2(x0, x1, d[4 * j], d[4 * j + 1], d4.x, d4.y, x0, x1);
-        split_bf16(x0, x1, dhi[2 * j], dlo[2 * j]);
-        ffma2v(x0, x1, s[4 * j + 2], s[4 * j + 3], sl2, n4.z, n4.w);
-        x0 = ex2(x0);
-        x1 = ex2(x1);
-        split_bf16(x0, x1, phi[2 * j + 1], plo[2 * j + 1]);
-        add_mul2(x0, x1, d[4 * j + 2], d[4 * j + 3], d4.z, d4.w, x0, x1);
-        split_bf16(x0, x1, dhi[2 * j + 1], dlo[2 * j + 1]);
+    for (int c = 0; c < 4; ++c) {
+        float *sc = s[c & 1], *dc = d[c & 1];
+        tmem_wait_ld();
+        if (c < 3) {
+            tmem_ld16(buf + 16 * (c + 1), s[(c + 1) & 1]);
+            tmem_ld16(buf + 64 + 16 * (c + 1), d[(c + 1) & 1]);
+        }
+        unsigned o[16], u[16];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float2 n2 = nl[8 * c + j], d2 = nd[8 * c + j];
+            float x0, x1;
+            ffma2v(x0, x1, sc[2 * j], sc[2 * j + 1], sl2, n2.x, n2.y);
+            x0 = ex2(x0);
+            x1 = ex2(x1);
+            split_bf16(x0, x1, o[j], o[8 + j]);
+            add_mul2(x0, x1, dc[2 * j], dc[2 * j + 1], d2.x, d2.y, x0, x1);
+            split_bf16(x0, x1, u[j], u[8 + j]);
+        }
+        tmem_st16(buf + 16 * c, o);
+        tmem_st16(buf + 64 + 16 * c, u);
     }
-    tmem_st16(s_addr, phi);
-    tmem_st16(s_addr + 16, plo);
-    tmem_st16(s_addr + 64, dhi);
-    tmem_st16(s_addr + 80, dlo);
 }
 
 __device__ __forceinline__ void elementwise_role(const KernelParams& p, SmemCtl* ctl, unsigned tmem, int warp, int lane) {
@@ -431,6 +435,7 @@ __device__ __forceinline__ void elementwise_role(const KernelParams& p, SmemCtl*
     const float sl2 = p.scale_log2;
     unsigned slot_n = 0, tile_n = 0, step_n = 0, use_n = 0;     // step_n: steps of all earlier segments
     float nl = 0.f, nd = 0.f;
+    bool fresh = false;                             // no step of the tile has been seen yet
     int fail = 0;
     for (;;) {
         const unsigned ss = slot_n % kSlots;
@@ -439,7 +444,9 @@ __device__ __forceinline__ void elementwise_role(const KernelParams& p, SmemCtl*
         const int w = slot->w, flags = slot->flags, n = slot->n;
         const bool dkv = slot->kind == kDkv;
         if (w < 0) break;
-        if ((flags & (kSegFirst | kSegLive)) == (kSegFirst | kSegLive)) {
+        if (flags & kSegFirst) fresh = true;
+        if (fresh && n > 0) {
+            fresh = false;
             const unsigned xs = tile_n & 1u;
             if (!mbar_wait(&ctl->x_full[xs], (tile_n >> 1) & 1u, abort_flag)) { fail = 134; break; }
             nl = ctl->x_stats[xs][lower][r64];      // (stale and unused on key tiles)
@@ -467,12 +474,10 @@ __device__ __forceinline__ void elementwise_role(const KernelParams& p, SmemCtl*
                 const unsigned t = step_n + (unsigned)i, stage = t % kStages;
                 if (!mbar_wait(&ctl->full[stage], (t / kStages) & 1u, abort_flag)) { fail = 132; break; }     // (complete: this makes the copy visible)
                 __syncwarp();
-                const float4* st = reinterpret_cast<const float4*>(ctl->y_stats[stage]);
-#pragma unroll 1
-                for (int c = 0; c < 2; ++c) dkv_columns(buf + 32 * c, sl2, st + 8 * c, st + 16 + 8 * c);
+                const float2* st = reinterpret_cast<const float2*>(ctl->y_stats[stage]);
+                dkv_columns(buf, sl2, st, st + 32);
             } else {
-#pragma unroll 1
-                for (int c = 0; c < 2; ++c) dq_columns(buf + 32 * c, sl2, nl, nd, (unsigned)(kb >> (32 * c)));
+                dq_columns(buf, sl2, nl, nd, kb);
             }
             tmem_wait_st();
             tc_fence_before();
@@ -601,7 +606,7 @@ attn_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     SmemCtl* ctl = reinterpret_cast<SmemCtl*>(smem + kSmemCtl);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;      // (uniform, and known to be)
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; ++i) { mbar_init(&ctl->full[i], 1); mbar_init(&ctl->empty[i], 1); }
@@ -609,7 +614,7 @@ attn_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         for (int i = 0; i < kBufs; ++i) { mbar_init(&ctl->sdp_full[i], 1); mbar_init(&ctl->p_full[i], 128); }
         mbar_init(&ctl->acc_full, 1);
         mbar_init(&ctl->acc_free, 128);
-        for (int i = 0; i < kSlots; ++i) { mbar_init(&ctl->slot_full[i], 1); mbar_init(&ctl->slot_empty[i], 2 + 4 * kBufs + 4); }   // producer, MMA thread, elementwise and epilogue warps
+        for (int i = 0; i < kSlots; ++i) { mbar_init(&ctl->slot_full[i], 1); mbar_init(&ctl->slot_empty[i], 1 + 4 * kBufs + 4); }   // producer, elementwise and epilogue warps
         ctl->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -632,8 +637,9 @@ attn_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLight));
         if (warp == kWarpScheduler) scheduler_role(p, ctl, lane);
-        else if (warp == kWarpProducer) { if (lane == 0) producer_role(p, ctl, smem, &tm_q, &tm_k, &tm_v, &tm_do); }
-        else if (warp == kWarpMma) { if (lane == 0) mma_role(p, ctl, smem, tmem); }
+        else if (warp == kWarpProducer) { if (elect_one()) producer_role(p, ctl, smem, &tm_q, &tm_k, &tm_v, &tm_do); }
+        else if (warp == kWarpScore) { if (elect_one()) score_role(p, ctl, smem, tmem); }
+        else if (elect_one()) accumulate_role(p, ctl, smem, tmem);
     }
 
     // ------------------------------------------------------------------------------------------------ teardown

@@ -699,7 +699,7 @@ attn_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     SmemCtl* ctl = reinterpret_cast<SmemCtl*>(smem + kSmemCtl);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;      // (uniform, and known to be)
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStreams; ++s) {
@@ -739,7 +739,7 @@ attn_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLight));
         if (warp == kWarpScheduler) scheduler_role(p, ctl, lane);
         else if (warp == kWarpProducer) { if (lane < 2 * kStreams) producer_role(p, ctl, (lane & 1) ? s1 : s0, lane >= kStreams, &tm_q, &tm_k, &tm_v); }
-        else if (lane == 0) mma_role(p, ctl, warp == kWarpMma ? s0 : s1);
+        else if (elect_one()) mma_role(p, ctl, warp == kWarpMma ? s0 : s1);
     }
 
     // ------------------------------------------------------------------------------------------------ teardown

@@ -55,6 +55,14 @@ __device__ __forceinline__ bool mbar_test(unsigned long long* bar, unsigned pari
     return ok != 0;
 }
 
+// One thread of a converged warp.  (With "lane == 0" instead the compiler does not know that a single thread is left, keeps the
+// operands of MMAs in ordinary registers and moves them to uniform ones in a loop over the active lanes at every MMA.)
+__device__ __forceinline__ bool elect_one() {
+    unsigned e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e != 0;
+}
+
 // Bounded wait, small enough to sit inline at every site (the kernel's hot code has to fit the SM's instruction
 // cache, measured at between 32 and 48 KB: a loop with a clock read and its own give-up code per site did not).  A
 // failing try keeps the thread suspended for about 1.4 us on this part (measured); after kWaitTries of them, about
@@ -173,6 +181,21 @@ __device__ __forceinline__ unsigned long long smem_desc_sw128(unsigned addr) {
          | ((unsigned long long)(1024 >> 4) << 32)   // stride byte offset: next group of 8 rows
          | (1ull << 46)                       // descriptor version of sm_100
          | (2ull << 61);                      // SWIZZLE_128B
+}
+// The same by its low word (the high word is the same for every such tile).
+constexpr unsigned kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ unsigned smem_desc_lo(unsigned addr) { return ((addr & 0x3FFFFu) >> 4) | (1u << 16); }
+__device__ __forceinline__ void mma_ss_lo(unsigned d_tmem, unsigned a_lo, unsigned b_lo, unsigned idesc, unsigned accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\tmov.b64 a, {%1, %5};\n\tmov.b64 b, {%2, %5};\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(kDescHi) : "memory");
+}
+__device__ __forceinline__ void mma_ts_lo(unsigned d_tmem, unsigned a_tmem, unsigned b_lo, unsigned idesc, unsigned accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 b;\n\tmov.b64 b, {%2, %5};\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(kDescHi) : "memory");
 }
 // Instruction descriptor: bf16 x bf16 -> fp32, M = 128, N = 64 (Q K^T adds 64 per further key block); B is K-major (K^T) or MN-major (V).
 constexpr unsigned kIdescQK64 = (1u << 4) | (1u << 7) | (1u << 10) | ((64u >> 3) << 17) | ((128u >> 4) << 24);   // N field (bits 17..22) = N / 8
