@@ -23,8 +23,11 @@
 // results are bit-reproducible.
 //
 // Measured (gradients of the base workload [8, 12, 4096, 64]): CUDA-core kernels 16.3 ms; one thread issuing all MMAs 857 us,
-// the same from one elected thread 557, columns 16 at a time with the next 16 on their way 527, two issuing threads 497 us
-// ([1, 12, 16384, 64] with 13000 valid tokens 338 -> 196 us from the first of these to the last).
+// the same from one elected thread 557, columns 16 at a time with the next 16 on their way 527, two issuing threads 505, all
+// roles on the ring, tests ahead of the commits and rows written by TMA 497 us ([1, 12, 16384, 64] with 13000 valid tokens
+// 338 -> 193 us from the second of these to the last).  A step takes 1400 cycles; its MMAs need 650 of the tensor pipe, without
+// any elementwise work it takes 1100, without any MMAs 1150: what is left is the way of a step through the hands of four
+// warps with three steps in flight, which is all that tensor memory holds.  Two threads per row (24 warps) were no faster.
 //
 // A first kernel makes, per query row, -lse * log2 e (-inf for rows without probabilities) and -delta, packs the key-padding
 // mask and zeroes the counters.
@@ -36,7 +39,7 @@ namespace bigbird {
 namespace {
 
 constexpr int kBufs = 3;                   // score buffers, each served by one warpgroup
-constexpr int kStages = 6;                 // ring of Y1 | Y2 pairs
+constexpr int kStages = 2 * kBufs;         // ring of Y1 | Y2 pairs
 constexpr int kSlots = 3;                  // tiles (or segments of long ones) posted by the scheduler
 constexpr int kSegSteps = 96;              // steps per posted segment
 // warps 0..11: the three elementwise warpgroups; 12..15: epilogue; 16: scheduler; 17: TMA producer; 18, 19: MMA issuers (scores,
@@ -55,7 +58,9 @@ constexpr int kStatFloats = 2 * kBlock;    // per block of query rows: 64 x (-ls
 constexpr int kPartialFloats = 2 * 128 * kBlock;   // one part of a split tile: acc0, acc1
 enum { kDkv = 0, kDq = 1 };
 enum { kSegFirst = 1, kSegLast = 2 };
-enum { kInfoDkv = 1, kInfoFirst = 2, kInfoLast = 4, kInfoEnd = 8 };   // what the issuing threads have to know about a step
+// what there is to know about a ring entry: bits 0..1 the step's kBothHalves / kUpperHalf / kLowerHalf, kind, first and last step of
+// its tile, the tile's row buffer and the parity of that buffer's phase; kInfoEnd: no more steps
+enum { kInfoWho = 3, kInfoDkv = 4, kInfoFirst = 8, kInfoLast = 16, kInfoX = 32, kInfoXPar = 64, kInfoEnd = 128 };
 
 struct __align__(16) StepEntry {
     int c;                         // block of the column side
@@ -77,19 +82,21 @@ struct __align__(16) SmemCtl {
     unsigned long long full[kStages], empty[kStages];
     unsigned long long x_full[2], x_empty[2];
     unsigned long long sdp_full[kBufs], p_full[kBufs];
-    unsigned long long acc_full, acc_free;
+    unsigned long long acc_full, acc_free, epi_sync;
     unsigned long long slot_full[kSlots], slot_empty[kSlots];
     TileSlot slot[kSlots];
     float x_stats[2][2][kStatFloats];      // query tiles: statistics of the rows
     float y_stats[kStages][kStatFloats];   // key tiles: of the step's query block
     unsigned info[kStages];
+    unsigned long long bits[kStages];      // the step's valid-token bits
     unsigned tmem_base;
     int abort_flag;
     int merge_last;
 };
 constexpr int kSmemX = 0;                                      // two buffers of X1a X1b X2a X2b
 constexpr int kSmemRing = 2 * 4 * kTileBytes;
-constexpr int kSmemCtl = kSmemRing + kStages * 2 * kTileBytes;
+constexpr int kSmemOut = kSmemRing + kStages * 2 * kTileBytes;    // four tiles on their way out
+constexpr int kSmemCtl = kSmemOut + 4 * kTileBytes;
 constexpr int kSmemBytes = kSmemCtl + (int)sizeof(SmemCtl) + 1024;   // + slack for the 1024-byte alignment
 static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
 
@@ -230,17 +237,19 @@ __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ct
         const TileSlot* slot = &ctl->slot[ss];
         const int w = slot->w, flags = slot->flags, n = slot->n, bh = slot->bh;
         const bool dkv = slot->kind == kDkv;
-        if (w < 0) {                                // the last entry of the ring
-            const unsigned g = step_n % kStages;
-            if (!mbar_wait(&ctl->empty[g], ((step_n / kStages) & 1u) ^ 1u, abort_flag)) { fail = 110; break; }
-            ctl->info[g] = kInfoEnd;
-            mbar_arrive(&ctl->full[g]);
+        if (w < 0) {                                // the last entries of the ring, one for each score buffer's warps
+            for (int i = 0; i < kBufs; ++i, ++step_n) {
+                const unsigned g = step_n % kStages;
+                if (!mbar_wait(&ctl->empty[g], ((step_n / kStages) & 1u) ^ 1u, abort_flag)) { fail = 110; break; }
+                ctl->info[g] = kInfoEnd;
+                mbar_arrive(&ctl->full[g]);
+            }
             break;
         }
         if (flags & kSegFirst) fresh = true;
         const CUtensorMap *tm1 = dkv ? tm_q : tm_k, *tm2 = dkv ? tm_do : tm_v;
         for (int i = 0; i < n; ++i) {
-            unsigned info = (dkv ? kInfoDkv : 0) | (i == n - 1 && (flags & kSegLast) ? kInfoLast : 0);
+            unsigned info = (unsigned)slot->steps[i].who | (dkv ? kInfoDkv : 0) | (i == n - 1 && (flags & kSegLast) ? kInfoLast : 0);
             if (fresh) {
                 const int ra = slot->ra, rb = slot->rb;
                 const unsigned xs = tile_n & 1u;
@@ -260,11 +269,13 @@ __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ct
                 fresh = false;
                 info |= kInfoFirst;
             }
+            info |= (((tile_n - 1) & 1u) ? kInfoX : 0) | ((((tile_n - 1) >> 1) & 1u) ? kInfoXPar : 0);
             const unsigned g = step_n % kStages;
             const int row = bh * p.nb + slot->steps[i].c;
             if (!mbar_wait(&ctl->empty[g], ((step_n / kStages) & 1u) ^ 1u, abort_flag)) { fail = 110; break; }
             unsigned char* y = smem + kSmemRing + g * 2 * kTileBytes;
             ctl->info[g] = info;
+            ctl->bits[g] = slot->steps[i].kb;
             mbar_expect_tx(&ctl->full[g], 2 * kTileBytes + (dkv ? kStatFloats * 4 : 0));
             tma_load_tile(y, tm1, row * kBlock, &ctl->full[g]);
             tma_load_tile(y + kTileBytes, tm2, row * kBlock, &ctl->full[g]);
@@ -283,25 +294,31 @@ __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ct
 // test 45, a test behind a commit 200.  One thread that issued everything and walked the posted tiles needed 1740 cycles a step.
 // So one issues the scores (S and dP) and one the accumulations, and both see the ring only, where each entry comes with a word
 // that says what there is to know about the step.  full[] tells both of a loaded entry, empty[] (committed behind a step's
-// accumulation) frees the ring entry for the producer and, three steps on, the score buffer for the first thread.
+// accumulation) frees the ring entry for the producer and, three steps on, the score buffer for the first thread.  The tests for
+// the next step come before a step's commit: behind it they cost four times as much.
 __device__ __forceinline__ void score_role(const KernelParams& p, SmemCtl* ctl, unsigned char* smem, unsigned tmem) {
     int* abort_flag = &ctl->abort_flag;
     constexpr unsigned kStageDesc = (2 * kTileBytes) >> 4, kTileDesc = kTileBytes >> 4;
     const unsigned ring0 = smem_desc_lo(smem_u32(smem + kSmemRing)), x0 = smem_desc_lo(smem_u32(smem + kSmemX));
     unsigned stg = 0, ph = 0, buf = 0;              // this step's ring entry (and its phase) and score buffer
     unsigned old = 0, old_ph = 0, n = 0;            // ring entry and phase of the step three back; steps issued, up to kBufs
-    unsigned xs = 0, x_par = 0, x1 = x0;            // row buffer of the tile
+    unsigned x1 = x0;                               // row buffer of the tile
+    bool have_f = false, have_e = false;            // the tests made ahead
+    unsigned info = 0;
     int fail = 0;
     for (;;) {
-        if (!mbar_wait(&ctl->full[stg], ph, abort_flag)) { fail = 120; break; }
-        const unsigned info = ctl->info[stg];
+        if (!have_f) {
+            if (!mbar_wait(&ctl->full[stg], ph, abort_flag)) { fail = 120; break; }
+            info = ctl->info[stg];
+        }
         if (info & kInfoEnd) break;
         if (n == (unsigned)kBufs) {                 // the buffer's last user must have been accumulated
-            if (!mbar_wait(&ctl->empty[old], old_ph, abort_flag)) { fail = 121; break; }
+            if (!have_e && !mbar_wait(&ctl->empty[old], old_ph, abort_flag)) { fail = 121; break; }
             if (++old == kStages) { old = 0; old_ph ^= 1u; }
         } else ++n;
         if (info & kInfoFirst) {
-            if (!mbar_wait(&ctl->x_full[xs], x_par, abort_flag)) { fail = 124; break; }
+            const unsigned xs = (info & kInfoX) ? 1u : 0u;
+            if (!mbar_wait(&ctl->x_full[xs], (info & kInfoXPar) ? 1u : 0u, abort_flag)) { fail = 124; break; }
             x1 = x0 + xs * 4 * kTileDesc;
         }
         tc_fence_after();
@@ -310,14 +327,13 @@ __device__ __forceinline__ void score_role(const KernelParams& p, SmemCtl* ctl, 
         for (int kk = 0; kk < 4; ++kk) mma_ss_lo(d, x1 + kk * 2, y1 + kk * 2, kIdescQK64, kk > 0);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) mma_ss_lo(d + 64, x1 + 2 * kTileDesc + kk * 2, y1 + kTileDesc + kk * 2, kIdescQK64, kk > 0);
-        tc_commit(&ctl->sdp_full[buf]);
-        if (info & kInfoLast) {                     // every S and dP of the tile has been issued
-            tc_commit(&ctl->x_empty[xs]);
-            x_par ^= xs;
-            xs ^= 1u;
-        }
+        unsigned long long* const done = &ctl->sdp_full[buf];
         if (++buf == kBufs) buf = 0;
         if (++stg == kStages) { stg = 0; ph ^= 1u; }
+        have_f = mbar_test(&ctl->full[stg], ph);
+        have_e = mbar_test(&ctl->empty[old], old_ph);
+        info = ctl->info[stg];                      // (read again if the entry is not there yet)
+        tc_commit(done);
     }
     if (fail) give_up(abort_flag, p.status, fail);
 }
@@ -328,14 +344,18 @@ __device__ __forceinline__ void accumulate_role(const KernelParams& p, SmemCtl* 
     const unsigned ring0 = smem_desc_lo(smem_u32(smem + kSmemRing)), acc = tmem + kColAcc;
     unsigned stg = 0, ph = 0, buf = 0, par = 0;     // ring entry and its phase, score buffer and the parity of its p_full
     unsigned acc_n = 0;                             // tiles handed to the epilogue
+    bool have_f = false, have_p = false;            // the tests made ahead
+    unsigned info = 0;
     int fail = 0;
     for (;;) {
-        if (!mbar_wait(&ctl->full[stg], ph, abort_flag)) { fail = 125; break; }
-        const unsigned info = ctl->info[stg];
+        if (!have_f) {
+            if (!mbar_wait(&ctl->full[stg], ph, abort_flag)) { fail = 125; break; }
+            info = ctl->info[stg];
+        }
         if (info & kInfoEnd) break;
         // the epilogue must have taken the previous tile's accumulators before this tile's first product overwrites them
         if ((info & kInfoFirst) && acc_n > 0 && !mbar_wait(&ctl->acc_free, (acc_n - 1) & 1u, abort_flag)) { fail = 127; break; }
-        if (!mbar_wait(&ctl->p_full[buf], par, abort_flag)) { fail = 122; break; }
+        if (!have_p && !mbar_wait(&ctl->p_full[buf], par, abort_flag)) { fail = 122; break; }
         tc_fence_after();
         const unsigned y1 = ring0 + stg * kStageDesc, y2 = y1 + kTileDesc;
         const unsigned keep = (info & kInfoFirst) ? 0u : 1u;
@@ -354,10 +374,19 @@ __device__ __forceinline__ void accumulate_role(const KernelParams& p, SmemCtl* 
             mma_ts_lo(acc, a + kk * 16, y1 + ((kk * 2048) >> 4), kIdescPV, kk > 0 ? 1u : keep);
             mma_ts_lo(acc, a + kk * 16 + 8, y1 + ((kk * 2048) >> 4), kIdescPV, 1u);
         }
-        tc_commit(&ctl->empty[stg]);
-        if (info & kInfoLast) { tc_commit(&ctl->acc_full); ++acc_n; }
+        const unsigned now = info;
+        unsigned long long* const done = &ctl->empty[stg];
         if (++buf == kBufs) { buf = 0; par ^= 1u; }
         if (++stg == kStages) { stg = 0; ph ^= 1u; }
+        have_f = mbar_test(&ctl->full[stg], ph);
+        have_p = mbar_test(&ctl->p_full[buf], par);
+        info = ctl->info[stg];                      // (read again if the entry is not there yet)
+        tc_commit(done);
+        if (now & kInfoLast) {                      // (the tile's scores and elementwise work are done as well: its rows may go)
+            tc_commit(&ctl->acc_full);
+            tc_commit(&ctl->x_empty[(now & kInfoX) ? 1 : 0]);
+            ++acc_n;
+        }
     }
     if (fail) give_up(abort_flag, p.status, fail);
 }
@@ -424,76 +453,64 @@ __device__ __forceinline__ void dkv_columns(unsigned buf, float sl2, const float
     }
 }
 
+// Like the issuing threads they walk the ring only: every third entry is theirs.
 __device__ __forceinline__ void elementwise_role(const KernelParams& p, SmemCtl* ctl, unsigned tmem, int warp, int lane) {
     int* abort_flag = &ctl->abort_flag;
     const unsigned g = (unsigned)warp >> 2;         // warpgroup = score buffer
-    const int quad = warp & 3, row = quad * 32 + lane, r64 = row & (kBlock - 1);
-    const bool lower = row >= kBlock;
-    const int my_who = lower ? kLowerHalf : kUpperHalf;
-    const unsigned buf = tmem + ((unsigned)(quad * 32) << 16) + g * kBufCols;
-    const float sl2 = p.scale_log2;
-    unsigned slot_n = 0, tile_n = 0, step_n = 0, use_n = 0;     // step_n: steps of all earlier segments
-    float nl = 0.f, nd = 0.f;
-    bool fresh = false;                             // no step of the tile has been seen yet
+    const int row = (warp & 3) * 32 + lane;
+    const unsigned other = row >= kBlock ? kUpperHalf : kLowerHalf;
+    const unsigned buf = tmem + ((unsigned)((warp & 3) * 32) << 16) + g * kBufCols;
+    const float* x_stats = &ctl->x_stats[0][row >= kBlock][row & (kBlock - 1)];
+    unsigned stage = g, par = 0, full_par = 0;      // par: of this buffer's use; the ring has twice as many entries as there are buffers
     int fail = 0;
     for (;;) {
-        const unsigned ss = slot_n % kSlots;
-        if (!mbar_wait(&ctl->slot_full[ss], (slot_n / kSlots) & 1u, abort_flag)) { fail = 130; break; }
-        const TileSlot* slot = &ctl->slot[ss];
-        const int w = slot->w, flags = slot->flags, n = slot->n;
-        const bool dkv = slot->kind == kDkv;
-        if (w < 0) break;
-        if (flags & kSegFirst) fresh = true;
-        if (fresh && n > 0) {
-            fresh = false;
-            const unsigned xs = tile_n & 1u;
-            if (!mbar_wait(&ctl->x_full[xs], (tile_n >> 1) & 1u, abort_flag)) { fail = 134; break; }
-            nl = ctl->x_stats[xs][lower][r64];      // (stale and unused on key tiles)
-            nd = ctl->x_stats[xs][lower][kBlock + r64];
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&ctl->x_empty[xs]);
-            ++tile_n;
+        if (!mbar_wait(&ctl->full[stage], full_par, abort_flag)) { fail = 132; break; }
+        const unsigned info = ctl->info[stage];
+        if (info & kInfoEnd) break;
+        const bool dkv = info & kInfoDkv;
+        const bool mine = (info & kInfoWho) != other;       // warp-uniform
+        float nl = 0.f, nd = 0.f;
+        if (!dkv) {
+            const unsigned xs = (info & kInfoX) ? 1u : 0u;
+            if (!mbar_wait(&ctl->x_full[xs], (info & kInfoXPar) ? 1u : 0u, abort_flag)) { fail = 134; break; }
+            nl = x_stats[xs * 2 * kStatFloats];
+            nd = x_stats[xs * 2 * kStatFloats + kBlock];
         }
-        const unsigned ahead = step_n % kBufs;
-        for (int i = (int)(g >= ahead ? g - ahead : g + kBufs - ahead); i < n; i += kBufs) {
-            const int who = slot->steps[i].who;
-            const bool mine = who == kBothHalves || who == my_who;      // warp-uniform
-            const unsigned long long kb = slot->steps[i].kb;
-            if (!mbar_wait(&ctl->sdp_full[g], use_n & 1u, abort_flag)) { fail = 131; break; }
-            __syncwarp();                           // lanes leave the wait one by one
-            tc_fence_after();
-            if (!mine) {
-                tmem_st32_zero(buf);
-                tmem_st32_zero(buf + 32);
-                if (dkv) {
-                    tmem_st32_zero(buf + 64);
-                    tmem_st32_zero(buf + 96);
-                }
-            } else if (dkv) {
-                const unsigned t = step_n + (unsigned)i, stage = t % kStages;
-                if (!mbar_wait(&ctl->full[stage], (t / kStages) & 1u, abort_flag)) { fail = 132; break; }     // (complete: this makes the copy visible)
-                __syncwarp();
-                const float2* st = reinterpret_cast<const float2*>(ctl->y_stats[stage]);
-                dkv_columns(buf, sl2, st, st + 32);
-            } else {
-                dq_columns(buf, sl2, nl, nd, kb);
+        if (!mbar_wait(&ctl->sdp_full[g], par, abort_flag)) { fail = 131; break; }
+        __syncwarp();                               // lanes leave the wait one by one
+        tc_fence_after();
+        if (!mine) {
+            tmem_st32_zero(buf);
+            tmem_st32_zero(buf + 32);
+            if (dkv) {
+                tmem_st32_zero(buf + 64);
+                tmem_st32_zero(buf + 96);
             }
-            tmem_wait_st();
-            tc_fence_before();
-            mbar_arrive(&ctl->p_full[g]);
-            ++use_n;
+        } else if (dkv) {
+            const float2* st = reinterpret_cast<const float2*>(ctl->y_stats[stage]);
+            dkv_columns(buf, p.scale_log2, st, st + 32);
+        } else {
+            dq_columns(buf, p.scale_log2, nl, nd, ctl->bits[stage]);
         }
-        if (fail) break;
-        step_n += (unsigned)n;
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&ctl->slot_empty[ss]);
-        ++slot_n;
+        tmem_wait_st();
+        tc_fence_before();
+        mbar_arrive(&ctl->p_full[g]);
+        par ^= 1u;
+        if (stage == g) stage = g + kBufs;
+        else { stage = g; full_par ^= 1u; }
     }
     if (fail) give_up(abort_flag, p.status, fail);
 }
 
 // ------------------------------------------------------------------------------------------------ epilogue (one warpgroup)
-__device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+// All epilogue threads (a bounded wait like every other: a warp that has given up must not leave the others in a hardware barrier).
+__device__ __forceinline__ bool epilogue_sync(SmemCtl* ctl, unsigned& n) {
+    mbar_arrive(&ctl->epi_sync);
+    const bool ok = mbar_wait(&ctl->epi_sync, n & 1u, &ctl->abort_flag);
+    ++n;
+    __syncwarp();
+    return ok;
+}
 
 // Sums the parts of a split tile (the last one to arrive does) and writes the rows.
 __device__ __forceinline__ void merge_parts(const KernelParams& p, const TileSlot* slot, int tid) {
@@ -519,12 +536,15 @@ __device__ __forceinline__ void merge_parts(const KernelParams& p, const TileSlo
     }
 }
 
-__device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ctl, unsigned tmem, int warp, int lane) {
+__device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ctl, unsigned char* smem, unsigned tmem, int warp, int lane,
+                                              const CUtensorMap* tm_dq, const CUtensorMap* tm_dk, const CUtensorMap* tm_dv) {
     int* abort_flag = &ctl->abort_flag;
     const int quad = warp & 3, row = quad * 32 + lane, r64 = row & (kBlock - 1);
     const bool lower = row >= kBlock;
     const unsigned acc = tmem + ((unsigned)(quad * 32) << 16) + kColAcc;
-    unsigned slot_n = 0, acc_n = 0;
+    unsigned char* const stage = smem + kSmemOut;   // [accumulator][half of the tile]: 64 x 64 bf16, swizzled
+    const unsigned my_row = smem_u32(stage) + (lower ? kTileBytes : 0) + r64 * 128;
+    unsigned slot_n = 0, acc_n = 0, sync_n = 0;
     bool have = false;                              // has the tile had any step
     int fail = 0;
     for (;;) {
@@ -538,53 +558,63 @@ __device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ct
         have = have || slot->n > 0;
         if (flags & kSegLast) {
             const bool dkv = slot->kind == kDkv;
-            const int blk = lower ? slot->rb : slot->ra, split = slot->split;
-            const unsigned long long bits = lower ? slot->rbits_b : slot->rbits_a;
-            const bool row_ok = (bits >> r64) & 1ull;
+            const int split = slot->split, n_chunks = dkv ? 8 : 4;     // of 16 columns
+            const bool row_ok = ((lower ? slot->rbits_b : slot->rbits_a) >> r64) & 1ull;
+            if (row == 0) bulk_wait_read();         // the previous tile has left the staging tiles
+            if (!epilogue_sync(ctl, sync_n)) { fail = 142; break; }
             if (have) {
                 if (!mbar_wait(&ctl->acc_full, acc_n & 1u, abort_flag)) { fail = 141; break; }
                 __syncwarp();
                 tc_fence_after();
                 ++acc_n;
             }
-            const int n_acc = dkv ? 2 : 1;
             float* part = p.partials + ((size_t)max(split, 0) * p.parts + slot->part) * kPartialFloats + row * kBlock;
-            const size_t tok = (((size_t)slot->bh * p.nb + max(blk, 0)) * kBlock + r64) * kBlock;
 #pragma unroll 1
-            for (int h = 0; h < 2 * n_acc; ++h) {   // 32 columns at a time
-                float o[32];
+            for (int c = 0; c < n_chunks; ++c) {
+                float o[16];
                 if (have) {
-                    tmem_ld32(acc + 32 * h, o);
+                    tmem_ld16(acc + 16 * c, o);
                     tmem_wait_ld();
+                    if (c == n_chunks - 1) { tc_fence_before(); mbar_arrive(&ctl->acc_free); }
                 } else {
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) o[j] = 0.f;
+                    for (int j = 0; j < 16; ++j) o[j] = 0.f;
                 }
-                if (have && h == 2 * n_acc - 1) { tc_fence_before(); mbar_arrive(&ctl->acc_free); }
-                const int m = h >> 1;
+                const int m = c >> 2;
                 if (split >= 0) {
-                    float4* d4 = reinterpret_cast<float4*>(part + m * 128 * kBlock) + 8 * (h & 1);
+                    float4* d4 = reinterpret_cast<float4*>(part + m * 128 * kBlock) + 4 * (c & 3);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) d4[j] = make_float4(o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
-                } else if (blk >= 0) {
+                    for (int j = 0; j < 4; ++j) d4[j] = make_float4(o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
+                } else {
                     const float f = row_ok ? (m ? 1.f : p.scale) : 0.f;
-                    uint4* d4 = reinterpret_cast<uint4*>((dkv ? (m ? p.dv : p.dk) : p.dq) + tok) + 4 * (h & 1);
+                    const unsigned base = my_row + m * 2 * kTileBytes;
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        uint4 v;
-                        v.x = pack_bf16(o[8 * j + 0] * f, o[8 * j + 1] * f);
-                        v.y = pack_bf16(o[8 * j + 2] * f, o[8 * j + 3] * f);
-                        v.z = pack_bf16(o[8 * j + 4] * f, o[8 * j + 5] * f);
-                        v.w = pack_bf16(o[8 * j + 6] * f, o[8 * j + 7] * f);
-                        d4[j] = v;
-                    }
+                    for (int j = 0; j < 2; ++j)     // 16 bytes of a row; the swizzle keeps the rows of a store in different banks
+                        st_shared16(base + (((2 * (c & 3) + j) ^ (r64 & 7)) << 4), pack_bf16(o[8 * j] * f, o[8 * j + 1] * f),
+                                    pack_bf16(o[8 * j + 2] * f, o[8 * j + 3] * f), pack_bf16(o[8 * j + 4] * f, o[8 * j + 5] * f),
+                                    pack_bf16(o[8 * j + 6] * f, o[8 * j + 7] * f));
                 }
             }
-            if (split >= 0) {
+            if (split < 0) {
+                proxy_fence();
+                if (!epilogue_sync(ctl, sync_n)) { fail = 142; break; }
+                if (row == 0) {
+                    const int first = slot->bh * p.nb, ra = (first + slot->ra) * kBlock, rb = (first + slot->rb) * kBlock;
+                    const bool two = slot->rb >= 0;
+                    const CUtensorMap* tm0 = dkv ? tm_dk : tm_dq;
+                    tma_store_tile(tm0, ra, stage);
+                    if (two) tma_store_tile(tm0, rb, stage + kTileBytes);
+                    if (dkv) {
+                        tma_store_tile(tm_dv, ra, stage + 2 * kTileBytes);
+                        if (two) tma_store_tile(tm_dv, rb, stage + 3 * kTileBytes);
+                    }
+                    bulk_commit();
+                }
+            } else {
                 __threadfence();
-                epilogue_sync();
+                if (!epilogue_sync(ctl, sync_n)) { fail = 142; break; }
                 if (row == 0) ctl->merge_last = atomicAdd(&p.arrived[split], 1) == p.parts - 1;
-                epilogue_sync();
+                if (!epilogue_sync(ctl, sync_n)) { fail = 142; break; }
                 if (ctl->merge_last) {
                     __threadfence();
                     merge_parts(p, slot, row);
@@ -595,13 +625,16 @@ __device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ct
         if (lane == 0) mbar_arrive(&ctl->slot_empty[ss]);
         ++slot_n;
     }
+    if (row == 0) bulk_wait_all();
     if (fail) give_up(abort_flag, p.status, fail);
 }
 
 // ------------------------------------------------------------------------------------------------ the kernel
 __global__ void __launch_bounds__(kThreads, 1)
 attn_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                      const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do, const KernelParams p) {
+                      const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do,
+                      const __grid_constant__ CUtensorMap tm_dq, const __grid_constant__ CUtensorMap tm_dk,
+                      const __grid_constant__ CUtensorMap tm_dv, const KernelParams p) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     SmemCtl* ctl = reinterpret_cast<SmemCtl*>(smem + kSmemCtl);
@@ -609,11 +642,12 @@ attn_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; ++i) { mbar_init(&ctl->full[i], 1); mbar_init(&ctl->empty[i], 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(&ctl->x_full[i], 1); mbar_init(&ctl->x_empty[i], 1 + 4 * kBufs); }      // the MMA thread, the elementwise warps
+        for (int i = 0; i < 2; ++i) { mbar_init(&ctl->x_full[i], 1); mbar_init(&ctl->x_empty[i], 1); }
         for (int i = 0; i < kBufs; ++i) { mbar_init(&ctl->sdp_full[i], 1); mbar_init(&ctl->p_full[i], 128); }
         mbar_init(&ctl->acc_full, 1);
         mbar_init(&ctl->acc_free, 128);
-        for (int i = 0; i < kSlots; ++i) { mbar_init(&ctl->slot_full[i], 1); mbar_init(&ctl->slot_empty[i], 1 + 4 * kBufs + 4); }   // producer, elementwise and epilogue warps
+        mbar_init(&ctl->epi_sync, 128);
+        for (int i = 0; i < kSlots; ++i) { mbar_init(&ctl->slot_full[i], 1); mbar_init(&ctl->slot_empty[i], 1 + 4); }   // producer, epilogue warps
         ctl->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -632,7 +666,7 @@ attn_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         elementwise_role(p, ctl, tmem, warp, lane);
     } else if (warp < kWarpScheduler) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsEpilogue));
-        epilogue_role(p, ctl, tmem, warp, lane);
+        epilogue_role(p, ctl, smem, tmem, warp, lane, &tm_dq, &tm_dk, &tm_dv);
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLight));
         if (warp == kWarpScheduler) scheduler_role(p, ctl, lane);
@@ -749,9 +783,10 @@ int launch_attn_bwd_sm100(const BwdArgs& a, const bigbird_layout& L, const Devic
     if (e != cudaSuccess) return fail(e);
     const int BH = a.B * a.H;
     const int64_t rows = (int64_t)BH * a.N;
-    CUtensorMap tm_q, tm_k, tm_v, tm_do;
+    CUtensorMap tm_q, tm_k, tm_v, tm_do, tm_dq, tm_dk, tm_dv;
     if (!make_map(&tm_q, a.q, (uint64_t)rows) || !make_map(&tm_k, a.k, (uint64_t)rows) || !make_map(&tm_v, a.v, (uint64_t)rows) ||
-        !make_map(&tm_do, a.dout, (uint64_t)rows))
+        !make_map(&tm_do, a.dout, (uint64_t)rows) || !make_map(&tm_dq, a.dq, (uint64_t)rows) || !make_map(&tm_dk, a.dk, (uint64_t)rows) ||
+        !make_map(&tm_dv, a.dv, (uint64_t)rows))
         return fail(cudaErrorInvalidValue);
 
     // Tiles of global blocks have nb steps where the others have about ten: cut them into parts of about half of what each SM
@@ -806,7 +841,7 @@ int launch_attn_bwd_sm100(const BwdArgs& a, const bigbird_layout& L, const Devic
     e = cudaGetLastError();
     if (e == cudaSuccess) {
         ++*launches;
-        attn_bwd_sm100_kernel<<<std::min(sms, p.total_work), kThreads, kSmemBytes, a.stream>>>(tm_q, tm_k, tm_v, tm_do, p);
+        attn_bwd_sm100_kernel<<<std::min(sms, p.total_work), kThreads, kSmemBytes, a.stream>>>(tm_q, tm_k, tm_v, tm_do, tm_dq, tm_dk, tm_dv, p);
         e = cudaGetLastError();
         if (e == cudaSuccess) ++*launches;
     }
