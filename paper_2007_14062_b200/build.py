@@ -11,7 +11,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libbigbird.so")
 LIB_DEBUG = os.path.join(HERE, "libbigbird_debug.so")      # the same library compiled with -DBB_DEBUG (index checks inside the kernels)
 SOURCES = ["layout.cpp", "api.cu", "attn_fwd_simt.cu", "attn_bwd_simt.cu", "attn_fwd_sm100.cu", "attn_bwd_sm100.cu"]
-HEADERS = ["layout.h", "kernels.h", "sm100.cuh", os.path.join("..", "..", "include", "bigbird.h")]
+HEADERS = ["layout.h", "kernels.h", "sm100.cuh", "simt.cuh", os.path.join("..", "..", "include", "bigbird.h")]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
     "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden", "--expt-relaxed-constexpr",

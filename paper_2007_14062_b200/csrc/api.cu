@@ -111,6 +111,7 @@ cudaError_t upload_layout(const bigbird_layout* L, DeviceLayout& d) {
     put(&d.items_t, L->items_t);
     put(&d.steps_t, L->steps_t);
     put(&d.global_pairs, L->global_pairs);
+    put(&d.block_order, L->block_order);
     cudaError_t e = cudaMalloc(&d.block, host.size() + 256);
     if (e == cudaSuccess) e = cudaMemcpy(d.block, host.data(), host.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return e;
@@ -136,6 +137,18 @@ int get_device_layout(const bigbird_layout* L, int device, DeviceLayout* out) {
         d.device = device;
     }
     *out = d;
+    return BIGBIRD_OK;
+}
+
+int get_sms(int device, int* sms) {
+    static int counts[kMaxDevices];
+    if (device < 0 || device >= kMaxDevices) return BIGBIRD_EUNSUPPORTED;
+    std::lock_guard<std::mutex> lock(g_mu);
+    if (!counts[device]) {
+        const cudaError_t e = cudaDeviceGetAttribute(&counts[device], cudaDevAttrMultiProcessorCount, device);
+        if (e != cudaSuccess) return cuda_fail(e);
+    }
+    *sms = counts[device];
     return BIGBIRD_OK;
 }
 
@@ -170,7 +183,10 @@ int fwd(bool force_simt, const void* q, const void* k, const void* v, const bigb
     if (rc != BIGBIRD_OK) return rc;
     FwdArgs a{q, k, v, kpm, out, lse, B, H, D, b, L->nb, N, scale, dtype, (cudaStream_t)stream};
     if (simt) {
-        e = launch_attn_fwd_simt(a, dl, &t_last_launches);
+        int sms = 0;
+        rc = get_sms(device, &sms);
+        if (rc != BIGBIRD_OK) return rc;
+        e = launch_attn_fwd_simt(a, *L, dl, sms, &t_last_launches);
         return e == cudaSuccess ? BIGBIRD_OK : cuda_fail(e);
     }
     DeviceScratch* sc = nullptr;

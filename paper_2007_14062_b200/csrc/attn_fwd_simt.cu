@@ -1,187 +1,211 @@
 // CUDA-core BigBird attention forward (arXiv 2007.14062, Eq. (AT) over the block lists of App. D).
 // fp32 arithmetic throughout; the path for fp32 tensors and an independent check for the tensor-core kernel.
 //
-// One CTA per (batch*head, query block, group of 8 query rows).  A warp shares a query row: for the scores each lane
-// takes a thirty-second of a chunk's keys (and the whole dot product of each), for the output a thirty-second of the head
-// dimension.  Key blocks are staged through shared memory (64 keys at a time for D <= 64, 32 for D = 128) and folded
-// into a running (max, sum, output) triple per row (online softmax).  The next chunk's K and V are already on their
-// way into registers while the current one is being used.
-#include <cuda_bf16.h>
-#include <math_constants.h>
-
-#include "kernels.h"
-#include "../../include/bigbird.h"
+// A CTA keeps its rows of q in shared memory and walks the rows' key blocks in chunks: scores in registers, online softmax over
+// the 16 threads that share a row, probabilities to shared memory (read back by the same 16 threads), output sums in registers.
+// The next chunk's K is on its way while the probabilities and sums are made, the next V while the scores are.  See simt.cuh for
+// the tile shapes and for how clusters share the long tiles.
+// Bound by the FMA pipes.  Measured (a warp per row before, no reuse of K and V in registers): [2, 12, 52 x 84, 64] with three
+// global blocks 3740 -> 691 us, [2, 8, 2560, 128] padded 1547 -> 331 us, [1, 2, 512, 64] 22.6 -> 18.5 us.
+#include "simt.cuh"
 
 namespace bigbird {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kLanesPerRow = 32;
-constexpr int kRowsPerCta = kThreads / kLanesPerRow;
-
-__device__ __forceinline__ float to_float(float x) { return x; }
-__device__ __forceinline__ float to_float(__nv_bfloat16 x) { return __bfloat162float(x); }
-__device__ __forceinline__ void store_val(float* p, float x) { *p = x; }
-__device__ __forceinline__ void store_val(__nv_bfloat16* p, float x) { *p = __float2bfloat16_rn(x); }
-
-template <typename T, int D>
-__global__ void __launch_bounds__(kThreads)
-attn_fwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
-                     const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
-                     const uint8_t* __restrict__ kpm, T* __restrict__ out, float* __restrict__ lse,
-                     int H, int64_t N, int b, int nb, float scale) {
-    constexpr int DL = D / kLanesPerRow;           // head dims per lane for the output: d = DL*sub .. DL*sub + DL - 1
-    constexpr int KC = D <= 64 ? 64 : 32;          // keys per staged chunk
-    constexpr int PF = KC * D / kThreads;          // elements of K (and of V) each thread moves per chunk
-    // rows padded by four floats: 16-byte aligned for vector loads, and the keys a warp reads at once fall
-    // into different banks
-    __shared__ __align__(16) float sk[KC][D + 4];
-    __shared__ __align__(16) float sv[KC][D + 4];
-    __shared__ uint8_t svalid[KC];
-
-    const int groups = (b + kRowsPerCta - 1) / kRowsPerCta;
-    const int j = blockIdx.x / groups;
-    const int row = (blockIdx.x % groups) * kRowsPerCta + threadIdx.x / kLanesPerRow;
-    const int bh = blockIdx.y;
-    const int h = bh % H, batch = bh / H;
-    const int sub = threadIdx.x % kLanesPerRow;
-    const int64_t base = (int64_t)bh * N * D;
-    const int list_begin = row_ptr[(int64_t)h * nb + j], list_end = row_ptr[(int64_t)h * nb + j + 1];
-    const uint8_t* mask = kpm ? kpm + (int64_t)batch * N : nullptr;
-    const bool row_ok = row < b;
-    const int64_t tok = (int64_t)j * b + row;
-
-    // Scores: lane t of a row takes the keys t, t + 32, ... of a chunk and the whole dot product of each (no
-    // exchange between lanes per key).  Output: lane t accumulates the head dims DL t .. DL t + DL - 1 over every key of
-    // the chunk; the probabilities pass from the first layout to the second through shared memory.
-    constexpr int KL = KC / kLanesPerRow;           // keys per lane per chunk
-    __shared__ float sp[kRowsPerCta][KC];
-    const int rloc = threadIdx.x / kLanesPerRow;
-    float qr[D], o[DL];
-#pragma unroll
-    for (int d = 0; d < D; ++d) qr[d] = row_ok ? to_float(q[base + tok * D + d]) * scale : 0.f;
-#pragma unroll
-    for (int i = 0; i < DL; ++i) o[i] = 0.f;
-    float m = -CUDART_INF_F, l = 0.f;               // l: this lane's keys only, summed over the lanes at the end
-
-    // chunks of the key sweep: (list entry, offset inside the key block)
-    const int chunks_per_block = (b + KC - 1) / KC;
-    const int n_chunks = (list_end - list_begin) * chunks_per_block;
-    float pk[PF], pv[PF];
-    uint8_t pm = 1;
-    auto fetch = [&](int ci) {                      // chunk ci from global memory into registers
-        const int64_t key0 = (int64_t)col_idx[list_begin + ci / chunks_per_block] * b + (ci % chunks_per_block) * KC;
-        const int nk = min(KC, b - (ci % chunks_per_block) * KC);
-#pragma unroll
-        for (int t = 0; t < PF; ++t) {
-            const int idx = threadIdx.x + t * kThreads, kk = idx / D, d = idx % D;
-            const bool in = kk < nk;
-            pk[t] = in ? to_float(k[base + (key0 + kk) * D + d]) : 0.f;
-            pv[t] = in ? to_float(v[base + (key0 + kk) * D + d]) : 0.f;
-        }
-        if (threadIdx.x < KC) pm = (threadIdx.x < nk && (mask ? mask[key0 + threadIdx.x] != 0 : true)) ? 1 : 0;
-    };
-    if (n_chunks > 0) fetch(0);
-    for (int ci = 0; ci < n_chunks; ++ci) {
-        __syncthreads();                            // the previous chunk has been used
-#pragma unroll
-        for (int t = 0; t < PF; ++t) {
-            const int idx = threadIdx.x + t * kThreads, kk = idx / D, d = idx % D;
-            sk[kk][d] = pk[t];
-            sv[kk][d] = pv[t];
-        }
-        if (threadIdx.x < KC) svalid[threadIdx.x] = pm;
-        __syncthreads();
-        if (ci + 1 < n_chunks) fetch(ci + 1);       // in flight while this chunk is being used
-        float s[KL];
-        float cmax = -CUDART_INF_F;
-#pragma unroll
-        for (int u = 0; u < KL; ++u) {
-            const int kk = sub + kLanesPerRow * u;
-            float acc = 0.f;
-#pragma unroll
-            for (int d = 0; d < D; d += 4) {
-                const float4 k4 = *reinterpret_cast<const float4*>(&sk[kk][d]);
-                acc = fmaf(qr[d], k4.x, acc);
-                acc = fmaf(qr[d + 1], k4.y, acc);
-                acc = fmaf(qr[d + 2], k4.z, acc);
-                acc = fmaf(qr[d + 3], k4.w, acc);
-            }
-            s[u] = svalid[kk] ? acc : -CUDART_INF_F;         // keys beyond the block's end were staged as invalid
-            cmax = fmaxf(cmax, s[u]);
-        }
-        cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, 1));
-        cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, 2));
-        cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, 4));
-        cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, 8));
-        cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, 16));
-        if (cmax == -CUDART_INF_F) continue;        // whole chunk masked (uniform across the CTA: the mask is per key)
-        const float m_new = fmaxf(m, cmax);
-        const float alpha = expf(m - m_new);        // m = -inf on the first chunk gives 0
-        l *= alpha;
-#pragma unroll
-        for (int i = 0; i < DL; ++i) o[i] *= alpha;
-#pragma unroll
-        for (int u = 0; u < KL; ++u) {
-            const float p = expf(s[u] - m_new);     // exp(-inf) = 0 for masked keys
-            l += p;
-            sp[rloc][sub + kLanesPerRow * u] = p;
-        }
-        __syncwarp();                               // a row is one warp
-#pragma unroll
-        for (int kk = 0; kk < KC; ++kk) {
-            const float p = sp[rloc][kk];
-            if constexpr (DL >= 2) {
-#pragma unroll
-                for (int i = 0; i < DL; i += 2) {
-                    const float2 v2 = *reinterpret_cast<const float2*>(&sv[kk][DL * sub + i]);
-                    o[i] = fmaf(p, v2.x, o[i]);
-                    o[i + 1] = fmaf(p, v2.y, o[i + 1]);
-                }
-            } else {
-                o[0] = fmaf(p, sv[kk][sub], o[0]);
-            }
-        }
-        __syncwarp();
-        m = m_new;
+template <int D>
+struct FwdShape {
+    static constexpr int KC = 64;                  // tokens per chunk
+    static constexpr int LD = D + 4, LDP = KC + 4; // padded rows: 16-byte aligned, and what a warp reads at once falls into different banks
+    static constexpr bool kAlias = D == 128;       // P takes the place of K (which then cannot be fetched ahead): two CTAs fit an SM
+    static size_t smem(int rows_pad) {
+        const size_t k = (size_t)KC * LD, p = (size_t)rows_pad * LDP;
+        return sizeof(float) * ((size_t)rows_pad * LD + (kAlias ? std::max(k, p) : k + p) + (size_t)KC * D);
     }
-    l += __shfl_xor_sync(0xffffffffu, l, 1);
-    l += __shfl_xor_sync(0xffffffffu, l, 2);
-    l += __shfl_xor_sync(0xffffffffu, l, 4);
-    l += __shfl_xor_sync(0xffffffffu, l, 8);
-    l += __shfl_xor_sync(0xffffffffu, l, 16);
-    if (row_ok) {
-        const bool q_valid = mask ? mask[tok] != 0 : true;
-        const bool any = q_valid && l > 0.f;
-        const float inv = any ? 1.f / l : 0.f;
+};
+
+// dynamic shared memory: Q [rows][LD] | K [KC][LD] | P [rows][LDP] (in K's place for D = 128) | V [KC][D]
+template <typename T, int D, int TM>
+__global__ void __launch_bounds__(256, 2)
+attn_fwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, const int32_t* __restrict__ row_ptr,
+                     const int32_t* __restrict__ col_idx, const uint8_t* __restrict__ kpm, T* __restrict__ out, float* __restrict__ lse,
+                     Tiling tiling, int64_t N, float scale) {
+    using S = FwdShape<D>;
+    using C = Cols<D>;
+    constexpr int KC = S::KC, LD = S::LD, LDP = S::LDP, TN = KC / 16;
+    __shared__ uint8_t svalid[KC];
+    extern __shared__ __align__(16) float smem[];
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4, rows_pad = (blockDim.x >> 4) * TM;
+    float* const sq = smem;
+    float* const sk = sq + rows_pad * LD;
+    float* const sp = S::kAlias ? sk : sk + KC * LD;
+    float* const sv = S::kAlias ? sk + max(KC * LD, rows_pad * LDP) : sp + rows_pad * LDP;
+
+    Tile tile;
+    if (!find_tile(tiling, tile)) return;          // (a CTA without a tile belongs to a cluster that shares none)
+    const int b = tiling.b, batch = tile.bh / tiling.H;
+    const int64_t base = (int64_t)tile.bh * N * D;
+    const int have = min(tiling.rows, b - tile.row0);
+    const int tok0 = tile.blk * b + tile.row0;     // first row
+    const uint8_t* mask = kpm ? kpm + (int64_t)batch * N : nullptr;
+    const Walk w = share_walk(tiling, row_ptr, col_idx, tile, KC);
+    const T *kb = k + base, *vb = v + base;
+    // whether a chunk's tokens are keys: threads 0 .. 63 (a CTA of one warp: two each) look one chunk ahead
+    auto key_valid = [&](int i) -> unsigned { return i < w.last && (!mask || mask[w.token(i)] != 0) ? 1u : 0u; };
+    auto chunk_valid = [&](int i0) -> unsigned {
+        unsigned f = threadIdx.x < KC ? key_valid(i0 + threadIdx.x) : 0u;
+        if (blockDim.x < KC) f |= key_valid(i0 + 32 + threadIdx.x) << 1;
+        return f;
+    };
+    // is any row of the tile a token (a thread per row: there are at least as many)
+    const bool row_live = __syncthreads_or((int)threadIdx.x < have && (!mask || mask[tok0 + threadIdx.x] != 0));
+    if (row_live) {
+        stage_rows<D>(sq, LD, q + base + (int64_t)tok0 * D, rows_pad, have);
+        stage_chunk<D>(sk, LD, kb, w, w.first, KC);
+        stage_chunk<D>(sv, D, vb, w, w.first, KC);
+    }
+    unsigned vf = row_live ? chunk_valid(w.first) : 0u;
+
+    const float* qrow = sq + ty * TM * LD;
+    float* prow = sp + ty * TM * LDP;
+    float o[TM][C::N], m[TM], l[TM];
 #pragma unroll
-        for (int i = 0; i < DL; ++i) store_val(&out[base + tok * D + DL * sub + i], o[i] * inv);
-        if (lse && sub == 0) lse[(int64_t)bh * N + tok] = any ? m + logf(l) : -CUDART_INF_F;
+    for (int i = 0; i < TM; ++i) {
+        m[i] = -CUDART_INF_F;
+        l[i] = 0.f;                                // this thread's keys only
+#pragma unroll
+        for (int c = 0; c < C::N; ++c) o[i][c] = 0.f;
+    }
+    for (int i0 = w.first; i0 < w.last && row_live; i0 += KC) {
+        if (threadIdx.x < KC) svalid[threadIdx.x] = (uint8_t)(vf & 1u);
+        if (blockDim.x < KC) svalid[32 + threadIdx.x] = (uint8_t)(vf >> 1);
+        copy_wait();
+        const bool any = __syncthreads_or(vf != 0u);
+        if (i0 + KC < w.last) vf = chunk_valid(i0 + KC);
+        if (any) {
+            float s[TM][TN];
+            dot_tile<TM, TN, D>(s, qrow, LD, sk + tx * LD, LD);
+            bool valid[TN];
+#pragma unroll
+            for (int j = 0; j < TN; ++j) valid[j] = svalid[tx + 16 * j] != 0;
+            __syncthreads();                       // K has been read
+            if (!S::kAlias && i0 + KC < w.last) stage_chunk<D>(sk, LD, kb, w, i0 + KC, KC);
+#pragma unroll
+            for (int i = 0; i < TM; ++i) {
+                float mx = -CUDART_INF_F;
+#pragma unroll
+                for (int j = 0; j < TN; ++j) {
+                    s[i][j] = valid[j] ? s[i][j] * scale : -CUDART_INF_F;
+                    mx = fmaxf(mx, s[i][j]);
+                }
+                mx = fmaxf(m[i], row_max16(mx));   // finite: the chunk has a valid key
+                const float alpha = expf(m[i] - mx);        // 0 on the first one
+                m[i] = mx;
+                l[i] *= alpha;
+#pragma unroll
+                for (int c = 0; c < C::N; ++c) o[i][c] *= alpha;
+#pragma unroll
+                for (int j = 0; j < TN; ++j) {
+                    const float p = expf(s[i][j] - mx);
+                    l[i] += p;
+                    prow[i * LDP + tx + 16 * j] = p;
+                }
+            }
+            __syncwarp();                          // a row's probabilities are read by the half-warp that wrote them
+            sum_tile<TM, D>(o, prow, LDP, sv, D, KC, tx);
+        }
+        __syncthreads();                           // V (and K, or P in its place) has been read
+        if (i0 + KC < w.last) {
+            if (S::kAlias || !any) stage_chunk<D>(sk, LD, kb, w, i0 + KC, KC);
+            stage_chunk<D>(sv, D, vb, w, i0 + KC, KC);
+        }
+    }
+    copy_wait();
+#pragma unroll
+    for (int i = 0; i < TM; ++i) l[i] = row_sum16(l[i]);
+
+    if (tile.shares > 1) {
+        // every CTA of the cluster leaves its (O, m, l) in its shared memory; each then adds up its share of the rows
+        constexpr int LDO = D + 4;
+        cg::cluster_group cluster = cg::this_cluster();
+        __syncthreads();
+        float* const so = smem;                    // [rows][LDO], columns D, D + 1: m, l
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+            float* row = so + (ty * TM + i) * LDO;
+            store_cols<D>(row, o[i], 1.f, tx);
+            if (tx == 0) { row[D] = m[i]; row[D + 1] = l[i]; }
+        }
+        cluster.sync();
+        auto part = [&](int s) -> const float* { return cluster.map_shared_rank(so, s); };
+        const int per = (have + tile.shares - 1) / tile.shares, r_end = min(have, per * (tile.rank + 1));
+        for (int r = per * tile.rank + ty; r < r_end; r += blockDim.x >> 4) {
+            float mx = -CUDART_INF_F;
+            for (int s = 0; s < tile.shares; ++s) mx = fmaxf(mx, part(s)[r * LDO + D]);
+            float sum = 0.f, acc[C::N];
+#pragma unroll
+            for (int c = 0; c < C::N; ++c) acc[c] = 0.f;
+            for (int s = 0; s < tile.shares; ++s) {
+                const float* row = part(s) + r * LDO;
+                const float ms = row[D];
+                if (ms == -CUDART_INF_F) continue;
+                const float f = expf(ms - mx);
+                sum = fmaf(f, row[D + 1], sum);
+#pragma unroll
+                for (int g = 0; g < C::NG; ++g)
+#pragma unroll
+                    for (int c = 0; c < C::G; c += 2) {
+                        const float2 x = *reinterpret_cast<const float2*>(row + C::at(tx, g) + c);
+                        acc[C::G * g + c] = fmaf(f, x.x, acc[C::G * g + c]);
+                        acc[C::G * g + c + 1] = fmaf(f, x.y, acc[C::G * g + c + 1]);
+                    }
+            }
+            const int tok = tok0 + r;
+            const bool good = sum > 0.f && (!mask || mask[tok] != 0);
+            store_cols<D>(out + base + (int64_t)tok * D, acc, good ? 1.f / sum : 0.f, tx);
+            if (lse && tx == 0) lse[(int64_t)tile.bh * N + tok] = good ? mx + logf(sum) : -CUDART_INF_F;
+        }
+        cluster.sync();                            // nobody leaves while its shared memory is being read
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+        const int r = ty * TM + i, tok = tok0 + r;
+        if (r >= have) continue;
+        const bool good = l[i] > 0.f && (!mask || mask[tok] != 0);
+        store_cols<D>(out + base + (int64_t)tok * D, o[i], good ? 1.f / l[i] : 0.f, tx);
+        if (lse && tx == 0) lse[(int64_t)tile.bh * N + tok] = good ? m[i] + logf(l[i]) : -CUDART_INF_F;
     }
 }
 
+template <typename T, int D, int TM>
+cudaError_t launch_tm(const FwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, int sms) {
+    static std::once_flag once[64];
+    const cudaError_t e = allow_smem((const void*)attn_fwd_simt_kernel<T, D, TM>, FwdShape<D>::smem(16 * TM), once);
+    if (e != cudaSuccess) return e;
+    const Shape s = make_shape(TM, L, dl, a.B * a.H, 2 * sms, FwdShape<D>::KC);
+    return launch_clusters(attn_fwd_simt_kernel<T, D, TM>, s, FwdShape<D>::smem(s.threads / 16 * TM), a.stream, (const T*)a.q, (const T*)a.k, (const T*)a.v,
+                           (const int32_t*)dl.row_ptr, (const int32_t*)dl.col_idx, a.kpm, (T*)a.out, a.lse, s.t, a.N, a.scale);
+}
+template <typename T, int D>
+cudaError_t launch_d(const FwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, int sms) {
+    if constexpr (D <= 64)
+        if (rows_per_thread(a.b, D) == 6) return launch_tm<T, D, 6>(a, L, dl, sms);
+    return launch_tm<T, D, 4>(a, L, dl, sms);
+}
 template <typename T>
-cudaError_t launch_t(const FwdArgs& a, const DeviceLayout& dl) {
-    dim3 grid((unsigned)(a.nb * ((a.b + kRowsPerCta - 1) / kRowsPerCta)), (unsigned)(a.B * a.H));
-    dim3 block(kThreads);
-#define BB_LAUNCH(DD)                                                                                     \
-    attn_fwd_simt_kernel<T, DD><<<grid, block, 0, a.stream>>>((const T*)a.q, (const T*)a.k, (const T*)a.v, \
-        dl.row_ptr, dl.col_idx, a.kpm, (T*)a.out, a.lse, a.H, a.N, a.b, a.nb, a.scale)
+cudaError_t launch_t(const FwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, int sms) {
     switch (a.D) {
-        case 32: BB_LAUNCH(32); break;
-        case 64: BB_LAUNCH(64); break;
-        case 128: BB_LAUNCH(128); break;
+        case 32: return launch_d<T, 32>(a, L, dl, sms);
+        case 64: return launch_d<T, 64>(a, L, dl, sms);
+        case 128: return launch_d<T, 128>(a, L, dl, sms);
         default: return cudaErrorInvalidValue;
     }
-#undef BB_LAUNCH
-    return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_attn_fwd_simt(const FwdArgs& a, const DeviceLayout& dl, int* launches) {
-    if ((int64_t)a.B * a.H > 65535) return cudaErrorInvalidValue;
-    cudaError_t e = a.dtype == BIGBIRD_BF16 ? launch_t<__nv_bfloat16>(a, dl) : launch_t<float>(a, dl);
+cudaError_t launch_attn_fwd_simt(const FwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, int sms, int* launches) {
+    const cudaError_t e = a.dtype == BIGBIRD_BF16 ? launch_t<__nv_bfloat16>(a, L, dl, sms) : launch_t<float>(a, L, dl, sms);
     if (e == cudaSuccess) ++*launches;
     return e;
 }

@@ -244,6 +244,9 @@ int build_layout_host(bigbird_layout* L, int chunk_steps) {
     // (the global key blocks are attended by every query block, so their tiles need no list)
     L->sparse_tiles_per_head = n_stiles;
     L->global_tiles = n_gtiles;
+    L->n_globals = (int)gq.size();
+    L->block_order = gq;
+    L->block_order.insert(L->block_order.end(), sq.begin(), sq.end());
     L->global_pairs.assign(2 * (size_t)n_gtiles, kNoBlock);
     for (size_t i = 0; i < gq.size(); ++i) L->global_pairs[i] = gq[i];
     L->items_t.clear();

@@ -41,6 +41,7 @@ struct DeviceLayout {
     Item* items_t = nullptr;           // tiles of key blocks over the transposed lists
     Step* steps_t = nullptr;
     int32_t* global_pairs = nullptr;   // [global_tiles * 2]
+    int32_t* block_order = nullptr;    // [nb]
     void* block = nullptr;             // the one allocation that holds the arrays above
 };
 
@@ -73,6 +74,8 @@ struct bigbird_layout {
     int sparse_tiles_per_head = 0;
     int global_tiles = 0;                      // tiles of two global blocks
     std::vector<int32_t> global_pairs;         // [global_tiles * 2], the last entry kNoBlock if their number is odd
+    int n_globals = 0;                         // global blocks, and all blocks with the global ones first
+    std::vector<int32_t> block_order;
     std::vector<bigbird::Item> items_t;        // [H * sparse_tiles_per_head], step_begin absolute
     std::vector<bigbird::Step> steps_t;
     // device copies, made on first use

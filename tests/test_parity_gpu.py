@@ -147,6 +147,22 @@ def test_paper_etc_block_sizes_on_the_cuda_core_path(name, wl, g_tokens):
         L.close()
 
 
+# Tile shapes of the CUDA-core kernels: blocks of one token, one row of threads more or less than a tile, six rows per thread,
+# several tiles per block; tiles shared by a cluster (few tiles; global blocks of a longer layout) and not.  Tolerances as above.
+SHAPES = [(b, 12, 1, D, 1) for b, D in [(1, 32), (5, 64), (16, 128), (33, 64), (84, 32), (96, 64), (97, 64), (130, 64)]] + \
+         [(16, 100, 4, 32, 2), (24, 60, 4, 64, 2), (84, 9, 20, 32, 3)]
+
+
+@pytest.mark.parametrize("b,nb,B,D,g", SHAPES)
+def test_tile_shapes_of_the_cuda_core_path(b, nb, B, D, g):
+    wl = synth.Workload(f"shape_{b}_{nb}", "fp32", B, 2, nb * b, D, b, 3, g, 2, 0, seed=17)
+    q, k, v = synth.make_qkv(wl)
+    kpm = torch.ones(B, wl.N, dtype=torch.uint8)
+    kpm[0, wl.N * 2 // 3:] = 0
+    out, lse = _run(wl, q, k, v, kpm, "fwd")
+    _compare(wl, q, k, v, kpm, out, lse, slices=[(0, 0), (B - 1, 1)])
+
+
 @pytest.mark.parametrize("impl", ["fwd", "simt"])
 def test_fully_padded_sequence_and_no_lse(impl):
     wl = _small("bf16", 2, 2, 8)
