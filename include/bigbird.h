@@ -156,8 +156,8 @@ BIGBIRD_API int bigbird_attn_fwd_simt(const void* q, const void* k, const void* 
  *   dq, dk, dv  device, [B, H, N, D], same dtype; every element is written.  A padded QUERY row gets dq = 0 and gives
  *             nothing to dk, dv; a padded key gets dk = dv = 0.
  * D in {32, 64, 128}, any b.  BIGBIRD_BF16 with D == b == 64 runs on tensor cores (bf16 operands; P and dS enter the products
- * as sums of two bf16 numbers; fp32 accumulation), everything else on CUDA cores in fp32 arithmetic.  The tensor-core path
- * takes its workspace (statistics per query row, packed mask, partial results) in stream order from a memory pool that lives
+ * as sums of two bf16 numbers; fp32 accumulation), everything else on CUDA cores in fp32 arithmetic.  The workspace
+ * (statistics per query row, packed mask, partial results) is taken in stream order from a memory pool that lives
  * as long as any layout is in use on the device: calls on different streams or threads may overlap.  Only enqueues work.
  * Errors: BIGBIRD_EINVAL, BIGBIRD_EUNSUPPORTED, BIGBIRD_ECUDA.
  */

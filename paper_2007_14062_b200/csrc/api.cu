@@ -234,17 +234,21 @@ int bigbird_attn_bwd(const void* q, const void* k, const void* v, const void* ou
     rc = get_device_layout(layout, device, &dl);
     if (rc != BIGBIRD_OK) return rc;
     BwdArgs a{q, k, v, out, lse, dout, key_padding_mask, dq, dk, dv, B, H, D, b, layout->nb, N, scale, dtype, (cudaStream_t)stream};
+    cudaMemPool_t pool = nullptr;
+    rc = get_pool(device, &pool);
+    if (rc != BIGBIRD_OK) return rc;
     if (attn_bwd_sm100_takes(a)) {
         DeviceScratch* sc = nullptr;
-        cudaMemPool_t pool = nullptr;
         rc = get_scratch(device, &sc);
-        if (rc == BIGBIRD_OK) rc = get_pool(device, &pool);
         if (rc != BIGBIRD_OK) return rc;
         rc = launch_attn_bwd_sm100(a, *layout, dl, pool, sc->status, &t_last_launches, &e);
         if (rc == BIGBIRD_ECUDA) t_last_cuda_error = (int)e;
         return rc;
     }
-    e = launch_attn_bwd_simt(a, dl, &t_last_launches);
+    int sms = 0;
+    rc = get_sms(device, &sms);
+    if (rc != BIGBIRD_OK) return rc;
+    e = launch_attn_bwd_simt(a, *layout, dl, pool, sms, &t_last_launches);
     return e == cudaSuccess ? BIGBIRD_OK : cuda_fail(e);
 }
 

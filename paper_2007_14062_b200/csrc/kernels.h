@@ -55,7 +55,8 @@ constexpr int kCounterSlots = 64;
 cudaError_t launch_attn_fwd_simt(const FwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, int sms, int* launches);
 
 // CUDA-core gradient kernels (fp32 arithmetic): dq by query block, dk and dv by key block over the transposed lists.
-cudaError_t launch_attn_bwd_simt(const BwdArgs& a, const DeviceLayout& dl, int* launches);
+// The workspace of a call comes from `pool`, in stream order.
+cudaError_t launch_attn_bwd_simt(const BwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, cudaMemPool_t pool, int sms, int* launches);
 
 // tcgen05 gradient kernels (bf16 tensors, b = D = 64).  The workspace of a call comes from `pool`, in stream order.  Returns a
 // BIGBIRD_* code; *cuda_err receives the cudaError_t on BIGBIRD_ECUDA.

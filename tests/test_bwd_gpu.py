@@ -96,3 +96,14 @@ EDGES = [
 @pytest.mark.parametrize("wl", EDGES, ids=lambda w: f"{w.name}_{w.lengths}_{w.B}_{w.g}{w.r}{w.w}")
 def test_tensor_core_gradients_at_the_edges_of_the_schedule(wl):
     test_gradients_match_the_oracle(wl)
+
+
+# Tile shapes of the CUDA-core gradient kernels: see the forward kernel's in test_parity_gpu.py.  Tolerances as above.
+SHAPES = [_case("fp32", B, 2, nb, b=b, D=D, g=g, r=2, lengths=f"ragged:{nb * b // 2}:{nb * b}")
+          for b, nb, B, D, g in [(1, 12, 1, 32, 1), (5, 12, 1, 64, 1), (16, 12, 1, 128, 1), (33, 12, 1, 64, 1), (96, 12, 1, 64, 1), (97, 12, 1, 32, 1),
+                                 (130, 12, 1, 64, 1), (16, 100, 4, 32, 2), (24, 60, 4, 64, 2), (84, 9, 20, 32, 3)]]
+
+
+@pytest.mark.parametrize("wl", SHAPES, ids=lambda w: f"{w.b}_{w.N // w.b}_{w.B}_{w.D}")
+def test_tile_shapes_of_the_cuda_core_gradients(wl):
+    test_gradients_match_the_oracle(wl)
