@@ -122,11 +122,9 @@ BIGBIRD_API int bigbird_layout_destroy(bigbird_layout* layout);
  *   stream    cudaStream_t (NULL = default stream).  The call only enqueues work; it never synchronises.
  *
  * Supported: D == 64 and b == 64 for BIGBIRD_BF16; D in {32, 64, 128} and any b for BIGBIRD_FP32.
- * The first call on a device (and the first call with a larger B, N or a new layout) allocates device
- * scratch owned by the library; later calls allocate nothing.  That scratch (packed mask bits, partial results
- * of split global tiles) is per device: calls that use a key-padding mask or a layout with N/b > 96 must not
- * overlap on the GPU with other such calls (put them on one stream).  Host threads may call concurrently: the
- * library serialises its own bookkeeping.
+ * The first call on a device and the first call with a new layout allocate device memory owned by the library.  Scratch of
+ * a call (packed mask bits, partial results of split global tiles) is taken in stream order from a memory pool that lives as
+ * long as any layout is in use on the device: calls on different streams or threads may overlap.
  * Errors: BIGBIRD_EINVAL, BIGBIRD_EUNSUPPORTED, BIGBIRD_ECUDA, BIGBIRD_ENOMEM.  There is no CPU path.
  */
 BIGBIRD_API int bigbird_attn_fwd(const void* q, const void* k, const void* v, const bigbird_layout* layout,
@@ -175,7 +173,7 @@ BIGBIRD_API int bigbird_attn_bwd(const void* q, const void* k, const void* v, co
  * whose memory is owned by a pool the application sized up front, in a latency-critical serving loop where an
  * implicit device synchronisation is unacceptable, or in a process that has handed all remaining GPU memory to
  * another component.  This entry point calls no cudaMalloc, cudaFree or other allocating routine.  Its scratch
- * is one fixed array of about 1.4 MB that is part of the library image: every GPU that loads the library
+ * is one fixed array of about 5.8 MB that is part of the library image: every GPU that loads the library
  * holds it until the process exits.
  *
  * Arguments, layouts, results and asynchrony are those of bigbird_attn_fwd, with these differences:

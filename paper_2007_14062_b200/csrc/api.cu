@@ -193,7 +193,10 @@ int fwd(bool force_simt, const void* q, const void* k, const void* v, const bigb
     rc = get_scratch(device, &sc);
     if (rc != BIGBIRD_OK) return rc;
     cudaError_t ce = cudaSuccess;
-    rc = launch_attn_fwd_sm100(a, *L, dl, *sc, &t_last_launches, &ce);
+    cudaMemPool_t pool = nullptr;
+    rc = get_pool(device, &pool);
+    if (rc != BIGBIRD_OK) return rc;
+    rc = launch_attn_fwd_sm100(a, *L, dl, *sc, pool, &t_last_launches, &ce);
     if (rc == BIGBIRD_ECUDA) t_last_cuda_error = (int)ce;
     return rc;
 }

@@ -32,6 +32,7 @@
 //     first, then the sparse tiles in (batch, head)-major order.
 //
 // Every wait on an mbarrier is bounded: on expiry the kernel records BIGBIRD_ETIMEOUT and returns.
+#include <algorithm>
 #include <mutex>
 
 #include "sm100.cuh"
@@ -131,12 +132,13 @@ struct KernelParams {
     const Step* steps;
     int* counter;                      // [2]: next work index, finished CTAs
     int* status;                       // [2]: code, detail
-    int items_per_head, heavy_per_head;
+    int items_per_head, heavy_per_head, layout_parts;   // of the layout's schedule, whose global tiles may be cut otherwise
+    int global_tiles;                  // per head
+    int parts, part_steps;             // how this launch cuts them (part_steps: key blocks)
     int BH, H, nb;
     int total_work;
     float scale_log2;
-    float* partials;                   // [BH * split_tiles_per_head * max_parts][kPartialFloats] or nullptr
-    int split_tiles_per_head, max_parts;
+    float* partials;                   // [BH * global_tiles * parts][kPartialFloats], if parts > 1
 };
 
 // ------------------------------------------------------------------------------------------------ helpers
@@ -201,19 +203,29 @@ __device__ __forceinline__ int schedule_one(const KernelParams& p, SmemCtl* ctl,
     if (lane == 0) w = atomicAdd(&p.counter[0], 1);
     w = __shfl_sync(0xffffffffu, w, 0);
     if (w >= p.total_work) w = -1;
-    // decode the work index: global-row tiles of every (batch, head) first, then the sparse tiles
-    int bh = 0, it = 0, batch = 0;
+    // decode the work index: the parts of the global-row tiles of every (batch, head) first, then the sparse tiles
+    int bh = 0, batch = 0, part_slot = -1;
+    bool heavy = false;
     Item item{};
     if (w >= 0) {
-        const int heavy_total = p.BH * p.heavy_per_head;
-        const bool heavy = w < heavy_total;
-        const unsigned per_head = heavy ? p.heavy_per_head : p.items_per_head - p.heavy_per_head;
+        const unsigned heavy_total = (unsigned)(p.BH * p.global_tiles * p.parts);
+        heavy = (unsigned)w < heavy_total;
+        const unsigned per_head = heavy ? p.global_tiles * p.parts : p.items_per_head - p.heavy_per_head;
         const unsigned x = heavy ? w : w - heavy_total;
         bh = (int)(x / per_head);                   // (one division for either kind of item: this code is kept small)
-        it = (int)(x - bh * per_head) + (heavy ? 0 : p.heavy_per_head);
+        int it = (int)(x - bh * per_head), part = 0;
         batch = (int)((unsigned)bh / (unsigned)p.H);
+        if (heavy) {
+            part = it % p.parts;
+            it = it / p.parts * p.layout_parts;
+            if (p.parts > 1) part_slot = (int)x;
+        } else it += p.heavy_per_head;
         if (BB_CHECK(bh >= 0 && bh < p.BH && it >= 0 && it < p.items_per_head, 71)) item = p.items[(size_t)(bh - batch * p.H) * p.items_per_head + it];
         else w = -1;
+        if (heavy) {                                // its list is every block of the sequence
+            item.step_begin = part * p.part_steps;
+            item.step_count = min(p.part_steps, p.nb - item.step_begin);
+        }
         if (!BB_CHECK(item.step_count >= 0 && item.step_begin >= 0 && item.qa >= 0 && item.qa < p.nb && item.qb < p.nb, 72)) w = -1;
     }
     const unsigned long long qbits_a = w >= 0 ? key_bits(p, batch, item.qa) : 0ull;
@@ -234,7 +246,7 @@ __device__ __forceinline__ int schedule_one(const KernelParams& p, SmemCtl* ctl,
             ChunkEntry e{-1, 0, 0ull};
             bool alive = false;
             if (i < n_raw) {
-                const Step s = p.steps[item.step_begin + i];
+                const Step s = heavy ? Step{item.step_begin + i, kBothHalves} : p.steps[item.step_begin + i];
                 // halves whose query rows are all padding do not attend anything
                 const bool ua = s.who != kLowerHalf && qbits_a != 0ull;
                 const bool ub = s.who != kUpperHalf && qbits_b != 0ull;
@@ -259,7 +271,7 @@ __device__ __forceinline__ int schedule_one(const KernelParams& p, SmemCtl* ctl,
             slot->flags = (first ? kSegFirst : 0) | (i0 >= n_raw ? kSegLast : 0) | (tile_live ? kSegLive : 0);
             slot->qbits_a = qbits_a;
             slot->qbits_b = qbits_b;
-            slot->part_slot = (w >= 0 && item.nparts > 1) ? ((bh * p.split_tiles_per_head + item.tile) * p.max_parts + item.part) : -1;
+            slot->part_slot = w >= 0 ? part_slot : -1;
         }
         __threadfence_block();
         __syncwarp();
@@ -656,7 +668,7 @@ __device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ct
             unsigned char* dst = partial ? reinterpret_cast<unsigned char*>(p.partials + (size_t)part_slot * kPartialFloats + row * 64)
                                          : reinterpret_cast<unsigned char*>(p.out + (((size_t)bh * p.nb + (my_q >= 0 ? my_q : 0)) * kBlock + r64) * kBlock);
             bool write = partial || my_q >= 0;              // warp-uniform
-            if (!BB_CHECK(bh >= 0 && bh < p.BH && my_q < p.nb && part_slot < p.BH * max(p.split_tiles_per_head, 1) * p.max_parts, 74)) write = false;
+            if (!BB_CHECK(bh >= 0 && bh < p.BH && my_q < p.nb && part_slot < p.BH * max(p.global_tiles, 1) * p.parts, 74)) write = false;
 #pragma unroll 1
             for (int c = 0; c < 2; ++c) {
                 float o[32];
@@ -725,6 +737,8 @@ attn_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    grid_dependency_release();
+    grid_dependency_wait();
     const unsigned tmem = *(volatile unsigned*)&ctl->tmem_base;
     const StreamRef s0{&ctl->st[0], smem, tmem};
     const StreamRef s1{&ctl->st[1], smem + kStreamSmemBytes, tmem + kStreamCols};
@@ -767,39 +781,40 @@ attn_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     }
 }
 
-// Combines the parts of the split tiles: one CTA per (batch*head, split tile, group of 16 rows); 16 threads share
-// a row, each owning 4 of its 64 output columns.
+// Adds up the parts of the split tiles, in a fixed order: results do not depend on scheduling.  One CTA per (batch*head, split
+// tile, group of 16 rows); 16 threads share a row, each owning 4 of its 64 output columns.
 __global__ void __launch_bounds__(256)
-merge_split_tiles_kernel(const float* __restrict__ partials, const int* __restrict__ tile_q, const unsigned long long* __restrict__ kbits,
-                         __nv_bfloat16* __restrict__ out, float* __restrict__ lse, int H, int nb, int tiles_per_head, int nparts) {
+merge_split_tiles_kernel(const float* __restrict__ partials, const Item* __restrict__ items, const unsigned long long* __restrict__ kbits,
+                         __nv_bfloat16* __restrict__ out, float* __restrict__ lse, int H, int nb, int items_per_head, int layout_parts, int tiles_per_head,
+                         int nparts) {
+    grid_dependency_release();
     const int rgrp = blockIdx.x & 7, tile = (blockIdx.x >> 3) % tiles_per_head, bh = (blockIdx.x >> 3) / tiles_per_head;
     const int row = rgrp * 16 + (threadIdx.x >> 4), c4 = threadIdx.x & 15, r64 = row & (kBlock - 1);
-    const int q = tile_q[2 * tile + (row >> 6)];
+    const Item& item = items[(size_t)(bh % H) * items_per_head + tile * layout_parts];
+    const int q = row >= kBlock ? item.qb : item.qa;
+    grid_dependency_wait();
     if (q < 0) return;
     const unsigned long long qb = kbits ? kbits[(size_t)(bh / H) * nb + q] : ~0ull;
     const float* base = partials + (size_t)(bh * tiles_per_head + tile) * nparts * kPartialFloats;
+    const float* stats = base + 128 * 64 + row;
     float m = -INFINITY;
-    for (int pt = 0; pt < nparts; ++pt) m = fmaxf(m, base[(size_t)pt * kPartialFloats + 128 * 64 + row]);
+#pragma unroll 4
+    for (int pt = 0; pt < nparts; ++pt) m = fmaxf(m, stats[(size_t)pt * kPartialFloats]);
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     float l = 0.f;
-    if (m > -INFINITY) {
-        for (int pt = 0; pt < nparts; ++pt) {            // fixed order: results do not depend on scheduling
-            const float* part = base + (size_t)pt * kPartialFloats;
-            const float lp = part[128 * 64 + 128 + row];
-            if (!(lp > 0.f)) continue;
-            const float wgt = exp2f(part[128 * 64 + row] - m);
-            l += wgt * lp;
-            const float4 v = reinterpret_cast<const float4*>(part + row * 64)[c4];
-            acc.x += wgt * v.x; acc.y += wgt * v.y; acc.z += wgt * v.z; acc.w += wgt * v.w;
-        }
+#pragma unroll 4
+    for (int pt = 0; pt < nparts; ++pt) {
+        const float mp = stats[(size_t)pt * kPartialFloats], lp = stats[(size_t)pt * kPartialFloats + 128];
+        const float4 v = reinterpret_cast<const float4*>(base + (size_t)pt * kPartialFloats)[row * 16 + c4];
+        if (!(lp > 0.f)) continue;                   // (such a part has left no accumulator)
+        const float wgt = exp2f(mp - m);
+        l += wgt * lp;
+        acc.x += wgt * v.x; acc.y += wgt * v.y; acc.z += wgt * v.z; acc.w += wgt * v.w;
     }
     const bool good = ((qb >> r64) & 1ull) && l > 0.f;
     const float inv = good ? 1.f / l : 0.f;
     const size_t tok = ((size_t)bh * nb + q) * kBlock + r64;
-    uint2 v2;
-    v2.x = pack_bf16(acc.x * inv, acc.y * inv);
-    v2.y = pack_bf16(acc.z * inv, acc.w * inv);
-    reinterpret_cast<uint2*>(out + tok * kBlock)[c4] = v2;
+    reinterpret_cast<uint2*>(out + tok * kBlock)[c4] = make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
     if (lse && c4 == 0) lse[tok] = good ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
 }
 
@@ -818,9 +833,10 @@ __global__ void wait_expiry_selftest_kernel(int* status) {
 }
 
 // One 64-bit word per (batch, key block): bit t = key_padding_mask[batch, block*64 + t] != 0.
-__global__ void pack_mask_kernel(const uint8_t* __restrict__ kpm, unsigned long long* __restrict__ kbits, int n_words) {
-    const int word = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(256) pack_mask_kernel(const uint8_t* __restrict__ kpm, unsigned long long* __restrict__ kbits, int n_words) {
+    grid_dependency_release();
+    grid_dependency_wait();
+    const int word = (blockIdx.x * 256 + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (word >= n_words) return;
     const uint8_t* src = kpm + (size_t)word * kBlock;
     const unsigned lo = __ballot_sync(0xffffffffu, src[lane] != 0);
@@ -863,26 +879,74 @@ cudaError_t kernel_setup(int device, int* sm_count) {
     return cudaSuccess;
 }
 
-// One CTA per SM, each running kStreams tile streams.
-int grid_size(int sm_count, int total_work) {
-    int grid = sm_count;
-    const int needed = (total_work + kStreams - 1) / kStreams;
-    if (grid > needed) grid = needed;
-    return grid < 1 ? 1 : grid;
+// How a launch cuts the tiles of global blocks: their lists are as long as the sequence, the other tiles' a dozen blocks, so that
+// they outlast everything else unless the GPU has a lot to do.  A part is three quarters of what each stream gets altogether, but
+// no shorter than the other tiles are.  Measured, uncut (or in parts of 32) -> cut like this: one sequence of 3001 tokens in 4096,
+// 12 heads 60 -> 42 us (the chain of a global tile was 50 of them); [2, 12, 1024] stays uncut.
+struct Cut {
+    int parts, part_steps;
+};
+Cut cut_global_tiles(const bigbird_layout& L, int B, int sms, int max_parts) {
+    if (L.global_tiles == 0) return Cut{1, L.nb};
+    const int64_t per_stream = (int64_t)B * (int64_t)L.steps.size() / (kStreams * sms);
+    const int64_t sparse = L.sparse_tiles_per_head
+        ? ((int64_t)L.steps.size() - (int64_t)L.H * L.global_tiles * L.nb) / ((int64_t)L.H * L.sparse_tiles_per_head) : 0;
+    const int64_t want = std::max<int64_t>({8, sparse, per_stream * 3 / 4});
+    if (L.nb < 2 * want) return Cut{1, L.nb};           // (adding up the parts costs as much as what is left to gain)
+    int parts = (int)std::min<int64_t>((L.nb + want - 1) / want, std::max(1, max_parts));
+    const int part_steps = ((L.nb + parts - 1) / parts + kStepChunks - 1) / kStepChunks * kStepChunks;
+    parts = (L.nb + part_steps - 1) / part_steps;
+    return Cut{parts, part_steps};
+}
+
+void set_shape(KernelParams& p, const bigbird_layout& L, int B, Cut cut, float scale) {
+    p.items_per_head = L.items_per_head;
+    p.heavy_per_head = L.heavy_items_per_head;
+    p.layout_parts = L.max_parts;
+    p.global_tiles = L.global_tiles;
+    p.parts = cut.parts;
+    p.part_steps = cut.part_steps;
+    p.BH = B * L.H;
+    p.H = L.H;
+    p.nb = L.nb;
+    p.total_work = p.BH * (L.global_tiles * cut.parts + L.sparse_tiles_per_head);
+    p.scale_log2 = scale * 1.4426950408889634f;
+}
+
+// One CTA per SM, each running kStreams tile streams; every SM gets work before any stream gets its second tile.
+int grid_size(int sm_count, int total_work) { return std::max(1, std::min(sm_count, total_work)); }
+
+// The kernels of a call, in the order of the stream, each allowed to begin before the one in front of it has drained: they wait for
+// it (grid_dependency_wait) before they touch memory that it may use.
+cudaError_t enqueue(const KernelParams& p, const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
+                    const uint8_t* kpm, unsigned long long* kbits, int n_words, int sm_count, cudaStream_t stream, int* launches) {
+    cudaError_t e = cudaSuccess;
+    if (n_words) {
+        e = launch_chained(pack_mask_kernel, (unsigned)((n_words * 32 + 255) / 256), 256, 0, stream, kpm, kbits, n_words);
+        if (e != cudaSuccess) return e;
+        ++*launches;
+    }
+    e = launch_chained(attn_fwd_sm100_kernel, (unsigned)grid_size(sm_count, p.total_work), kThreads, kSmemBytes, stream, tm_q, tm_k, tm_v, p);
+    if (e != cudaSuccess) return e;
+    ++*launches;
+    if (p.parts > 1) {
+        e = launch_chained(merge_split_tiles_kernel, (unsigned)(p.BH * p.global_tiles * 8), 256, 0, stream, (const float*)p.partials, p.items, p.kbits, p.out, p.lse,
+                           p.H, p.nb, p.items_per_head, p.layout_parts, p.global_tiles, p.parts);
+        if (e != cudaSuccess) return e;
+        ++*launches;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace
 
-int launch_attn_fwd_sm100(const FwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, DeviceScratch& sc,
+int launch_attn_fwd_sm100(const FwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, DeviceScratch& sc, cudaMemPool_t pool,
                           int* launches, cudaError_t* cuda_err) {
     *cuda_err = cudaSuccess;
     if (!(a.scale > 0.f) || !(a.scale < INFINITY)) return BIGBIRD_EINVAL;
     const int64_t rows = (int64_t)a.B * a.H * a.N;
     if (rows >= (1ll << 31) || (int64_t)a.B * a.H * L.items_per_head >= (1ll << 31)) return BIGBIRD_EUNSUPPORTED;
 
-    // One host thread at a time past this point: the per-device scratch bookkeeping below (counter slots, grown
-    // buffers) is plain data.
-    std::lock_guard<std::mutex> launch_lock(g_launch_mu);
     int device = 0, sm_count = 0;
     cudaError_t de = cudaGetDevice(&device);
     if (de == cudaSuccess) de = kernel_setup(device, &sm_count);
@@ -894,70 +958,39 @@ int launch_attn_fwd_sm100(const FwdArgs& a, const bigbird_layout& L, const Devic
         return BIGBIRD_ECUDA;
     }
 
-    const unsigned long long* kbits = nullptr;
-    if (a.kpm) {
-        const size_t words = (size_t)a.B * a.nb;
-        if (words > sc.kbits_cap) {                      // grows only when a larger B * N/b shows up
-            cudaFree(sc.kbits);
-            sc.kbits = nullptr;
-            sc.kbits_cap = 0;
-            cudaError_t e = cudaMalloc(&sc.kbits, words * sizeof(unsigned long long));
-            if (e != cudaSuccess) { *cuda_err = e; return BIGBIRD_ECUDA; }
-            sc.kbits_cap = words;
-        }
-        const int threads = 256, blocks = (int)((words * 32 + threads - 1) / threads);
-        pack_mask_kernel<<<blocks, threads, 0, a.stream>>>(a.kpm, sc.kbits, (int)words);
-        cudaError_t e = cudaGetLastError();
+    // scratch of this call, on the caller's stream: parts of split tiles, packed mask bits
+    const Cut cut = cut_global_tiles(L, a.B, sm_count, 1 << 20);
+    const size_t words = a.kpm ? (size_t)a.B * a.nb : 0;
+    const size_t off_bits = cut.parts > 1 ? (size_t)a.B * a.H * L.global_tiles * cut.parts * kPartialFloats * sizeof(float) : 0;
+    unsigned char* ws = nullptr;
+    if (off_bits + words) {
+        cudaError_t e = cudaMallocFromPoolAsync((void**)&ws, off_bits + words * sizeof(unsigned long long), pool, a.stream);
         if (e != cudaSuccess) { *cuda_err = e; return BIGBIRD_ECUDA; }
-        ++*launches;
-        kbits = sc.kbits;
-    }
-
-    const bool split = L.split_tiles_per_head > 0 && L.max_parts > 1;
-    if (split) {
-        const size_t need = (size_t)a.B * a.H * L.split_tiles_per_head * L.max_parts * kPartialFloats;
-        if (need > sc.partials_cap) {                    // grows only when a larger problem shows up
-            cudaFree(sc.partials);
-            sc.partials = nullptr;
-            sc.partials_cap = 0;
-            cudaError_t e = cudaMalloc(&sc.partials, need * sizeof(float));
-            if (e != cudaSuccess) { *cuda_err = e; return BIGBIRD_ECUDA; }
-            sc.partials_cap = need;
-        }
     }
 
     KernelParams p{};
     p.out = (__nv_bfloat16*)a.out;
     p.lse = a.lse;
-    p.kbits = kbits;
-    p.partials = split ? sc.partials : nullptr;
-    p.split_tiles_per_head = L.split_tiles_per_head;
-    p.max_parts = L.max_parts;
+    p.kbits = words ? (const unsigned long long*)(ws + off_bits) : nullptr;
+    p.partials = (float*)ws;
     p.items = dl.items;
     p.steps = dl.steps;
-    p.counter = sc.counters + 2 * (sc.next_slot++ % kCounterSlots);
-    p.status = sc.status;
-    p.items_per_head = L.items_per_head;
-    p.heavy_per_head = L.heavy_items_per_head;
-    p.BH = a.B * a.H;
-    p.H = a.H;
-    p.nb = a.nb;
-    p.total_work = p.BH * L.items_per_head;
-    p.scale_log2 = a.scale * 1.4426950408889634f;
-
-    const int grid = grid_size(sm_count, p.total_work);
-    attn_fwd_sm100_kernel<<<grid, kThreads, kSmemBytes, a.stream>>>(tm_q, tm_k, tm_v, p);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) { *cuda_err = e; return BIGBIRD_ECUDA; }
-    ++*launches;
-    if (split) {
-        merge_split_tiles_kernel<<<p.BH * L.split_tiles_per_head * 8, 256, 0, a.stream>>>(sc.partials, dl.split_tile_q, kbits, p.out, p.lse, a.H,
-                                                                                     a.nb, L.split_tiles_per_head, L.max_parts);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) { *cuda_err = e; return BIGBIRD_ECUDA; }
-        ++*launches;
+    unsigned slot;
+    {
+        std::lock_guard<std::mutex> lock(g_launch_mu);
+        slot = sc.next_slot++ % kCounterSlots;
     }
-    return BIGBIRD_OK;
+    p.counter = sc.counters + 2 * slot;
+    p.status = sc.status;
+    set_shape(p, L, a.B, cut, a.scale);
+
+    cudaError_t e = enqueue(p, tm_q, tm_k, tm_v, a.kpm, (unsigned long long*)(ws + off_bits), (int)words, sm_count, a.stream, launches);
+    if (ws) {
+        const cudaError_t ef = cudaFreeAsync(ws, a.stream);
+        if (e == cudaSuccess) e = ef;
+    }
+    *cuda_err = e;
+    return e == cudaSuccess ? BIGBIRD_OK : BIGBIRD_ECUDA;
 }
 
 }  // namespace bigbird
@@ -973,10 +1006,12 @@ namespace {
 constexpr size_t kStaticMaskWords = 16384;      // B * N/b
 constexpr size_t kStaticItems = 8192;           // H * tiles per head
 constexpr size_t kStaticSteps = 131072;         // (key block, halves) entries summed over heads
+constexpr size_t kStaticParts = 128;            // parts of split global tiles
 constexpr size_t kStaticOffMask = 256;          // bytes 0..15: status[2], counter[2]
 constexpr size_t kStaticOffItems = kStaticOffMask + kStaticMaskWords * sizeof(unsigned long long);
 constexpr size_t kStaticOffSteps = kStaticOffItems + kStaticItems * sizeof(Item);
-constexpr size_t kStaticBytes = kStaticOffSteps + kStaticSteps * sizeof(Step);      // about 1.4 MB per GPU
+constexpr size_t kStaticOffParts = kStaticOffSteps + kStaticSteps * sizeof(Step);
+constexpr size_t kStaticBytes = kStaticOffParts + kStaticParts * kPartialFloats * sizeof(float);     // about 5.8 MB per GPU
 
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
 
@@ -1062,32 +1097,22 @@ extern "C" int bigbird_attn_fwd_static(const void* q, const void* k, const void*
         static_remember_schedule(device, L->uid);
     }
 
-    const unsigned long long* kbits = nullptr;
-    if (key_padding_mask) {
-        const int threads = 256, blocks = (int)((words * 32 + threads - 1) / threads);
-        pack_mask_kernel<<<blocks, threads, 0, stream>>>(key_padding_mask, kbits_dev, (int)words);
-        if (cudaGetLastError() != cudaSuccess) return BIGBIRD_ECUDA;
-        kbits = kbits_dev;
-    }
+    const size_t tiles = (size_t)B * H * L->global_tiles;
+    const Cut cut = cut_global_tiles(*L, B, sd.sm_count, tiles ? (int)std::min<size_t>(kStaticParts / tiles, 1 << 20) : 1);
 
     KernelParams p{};
     p.out = (__nv_bfloat16*)out;
     p.lse = lse;
-    p.kbits = kbits;
+    p.kbits = key_padding_mask ? kbits_dev : nullptr;
+    p.partials = reinterpret_cast<float*>(sd.base + kStaticOffParts);
     p.items = items_dev;
     p.steps = steps_dev;
     p.status = words4;
     p.counter = words4 + 2;
-    p.items_per_head = L->items_per_head;
-    p.heavy_per_head = L->heavy_items_per_head;
-    p.BH = B * H;
-    p.H = H;
-    p.nb = L->nb;
-    p.total_work = p.BH * L->items_per_head;
-    p.scale_log2 = scale * 1.4426950408889634f;
-    const int grid = grid_size(sd.sm_count, p.total_work);
-    attn_fwd_sm100_kernel<<<grid, kThreads, kSmemBytes, stream>>>(tm_q, tm_k, tm_v, p);
-    if (cudaGetLastError() != cudaSuccess) return BIGBIRD_ECUDA;
+    set_shape(p, *L, B, cut, scale);
+    int launches = 0;
+    if (enqueue(p, tm_q, tm_k, tm_v, key_padding_mask, kbits_dev, key_padding_mask ? (int)words : 0, sd.sm_count, stream, &launches) != cudaSuccess)
+        return BIGBIRD_ECUDA;
     return BIGBIRD_OK;
 }
 

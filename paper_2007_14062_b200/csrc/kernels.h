@@ -44,10 +44,6 @@ struct DeviceScratch {
     int* status = nullptr;          // [2]: code, detail
     int* counters = nullptr;        // [kCounterSlots * 2] work counters of the dynamic scheduler
     unsigned next_slot = 0;
-    unsigned long long* kbits = nullptr;   // [B * nb] one bit per key of a 64-token block (1 = valid)
-    size_t kbits_cap = 0;
-    float* partials = nullptr;      // partial (O, m, l) of split tiles
-    size_t partials_cap = 0;
 };
 constexpr int kCounterSlots = 64;
 
@@ -65,7 +61,8 @@ int launch_attn_bwd_sm100(const BwdArgs& a, const bigbird_layout& L, const Devic
                           int* launches, cudaError_t* cuda_err);
 
 // tcgen05 kernel (bf16 operands).  Returns a BIGBIRD_* code; *cuda_err receives the cudaError_t on BIGBIRD_ECUDA.
-int launch_attn_fwd_sm100(const FwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, DeviceScratch& sc,
+// Scratch of a call comes from `pool`, in stream order.
+int launch_attn_fwd_sm100(const FwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, DeviceScratch& sc, cudaMemPool_t pool,
                           int* launches, cudaError_t* cuda_err);
 
 // One-thread kernel whose bounded wait is left to expire (about two seconds); sets the device status word.

@@ -321,7 +321,27 @@ __device__ __forceinline__ void split_bf16(float x0, float x1, unsigned& hi, uns
     lo = pack_bf16(x0 - h0, x1 - h1);
 }
 
+// Chained launches (launch_chained): lets the next kernel of the stream begin when it finds room; waits until the kernels in front
+// have finished and their writes are visible.
+__device__ __forceinline__ void grid_dependency_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------------------------------------------ host side
+// A launch that may begin before the kernel in front of it in the stream has drained; the kernel waits for it itself.
+template <typename... Ps, typename... As>
+cudaError_t launch_chained(void (*kernel)(Ps...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream, const As&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, Ps(args)...);
+}
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                   const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -339,13 +359,13 @@ EncodeTiledFn get_encode_fn() {
     return fn;
 }
 
-// [rows, 64] bf16 row-major tensor read in 64 x 64 boxes with the 128-byte swizzle.
-bool make_map(CUtensorMap* tm, const void* base, uint64_t rows) {
+// [rows, 64] bf16 row-major tensor read (or written) in boxes of 64 (or box_rows) rows with the 128-byte swizzle.
+inline bool make_map(CUtensorMap* tm, const void* base, uint64_t rows, int box_rows = kBlock) {
     EncodeTiledFn enc = get_encode_fn();
     if (!enc) return false;
     cuuint64_t dims[2] = {(cuuint64_t)kBlock, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)(kBlock * 2)};
-    cuuint32_t box[2] = {(cuuint32_t)kBlock, (cuuint32_t)kBlock};
+    cuuint32_t box[2] = {(cuuint32_t)kBlock, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     return enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,

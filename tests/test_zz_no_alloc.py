@@ -135,3 +135,28 @@ def test_static_entry_point_refuses_what_does_not_fit():
                                             None, 1, 2, 512, 64, 64, 0.125, bb.BIGBIRD_FP32, None)
     assert code == -2
     L.close()
+
+
+def test_static_entry_point_splits_global_tiles_like_the_allocating_one():
+    """One sequence: the global tiles are cut into parts whose partial results live in the fixed array (and in scratch of the
+    allocating entry point).  Then as many heads as leave the array room for one part per tile only."""
+    for wl in (synth.Workload("noalloc_e", "bf16", 1, 3, 80 * 64, 64, 64, 3, 3, 2, 0, seed=15, lengths="fixed:4001"),
+               synth.Workload("noalloc_f", "bf16", 1, 70, 80 * 64, 64, 64, 3, 2, 0, 1, seed=16)):
+        L = bb.bigbird_build_layout(wl.N, wl.b, wl.w, wl.g, wl.r, wl.seed, wl.H, wl.mode)
+        dev = torch.device("cuda:0")
+        q, k, v = (t.to(dev) for t in synth.make_qkv(wl))
+        kpm = synth.key_padding_mask(wl)
+        md = None if kpm is None else kpm.to(dev)
+        res = []
+        for fn in (bb.bigbird_attn_fwd_simt, bb.bigbird_attn_fwd, bb.bigbird_attn_fwd_static):
+            out = torch.full_like(q, float("nan"))
+            lse = torch.full(q.shape[:3], float("nan"), device=dev, dtype=torch.float32)
+            fn(q, k, v, L, md, out, lse, wl.scale)
+            res.append((out.float(), lse))
+        torch.cuda.synchronize()
+        assert bb.bigbird_last_status() == (0, 0) and bb.bigbird_last_status_static() == (0, 0)
+        for out, lse in res[1:]:
+            assert (out - res[0][0]).abs().max() <= TOL_OUT
+            fin = torch.isfinite(res[0][1])
+            assert torch.equal(fin, torch.isfinite(lse)) and (lse[fin] - res[0][1][fin]).abs().max() <= TOL_LSE
+        L.close()
