@@ -113,13 +113,13 @@ attn_bwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* 
 
     const float *r1 = x1 + ty * TM * LD, *r2 = x2 + ty * TM * LD;
     float* const prow = sp + ty * TM * LDP;
-    float acc[NA][TM][C::N];
+    f32x2 acc[NA][TM][C::N];
 #pragma unroll
     for (int a = 0; a < NA; ++a)
 #pragma unroll
         for (int i = 0; i < TM; ++i)
 #pragma unroll
-            for (int c = 0; c < C::N; ++c) acc[a][i][c] = 0.f;
+            for (int c = 0; c < C::N; ++c) acc[a][i][c] = 0;
     for (int i0 = w.first; i0 < w.last && live; i0 += KC) {
         if ((int)threadIdx.x < KC) { sbias[threadIdx.x] = next_bias[0]; sdelta[threadIdx.x] = next_delta[0]; }
         if (blockDim.x < KC) { sbias[32 + threadIdx.x] = next_bias[1]; sdelta[32 + threadIdx.x] = next_delta[1]; }
@@ -171,19 +171,15 @@ attn_bwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* 
         for (int r = per * tile.rank + ty; r < r_end; r += blockDim.x >> 4)
 #pragma unroll
             for (int a = 0; a < NA; ++a) {
-                float sum[C::N];
+                f32x2 sum[C::N];
 #pragma unroll
-                for (int c = 0; c < C::N; ++c) sum[c] = 0.f;
-                for (int s = 0; s < tile.shares; ++s) {
+                for (int c = 0; c < C::N; ++c) sum[c] = 0;
+#pragma unroll
+                for (int s = 0; s < 8; ++s) {      // (at most eight shares; their loads are in flight together)
+                    if (s >= tile.shares) continue;
                     const float* part = cluster.map_shared_rank(smem, s) + (a * rows_pad + r) * LD;
 #pragma unroll
-                    for (int g = 0; g < C::NG; ++g)
-#pragma unroll
-                        for (int c = 0; c < C::G; c += 2) {
-                            const float2 x = *reinterpret_cast<const float2*>(part + C::at(tx, g) + c);
-                            sum[C::G * g + c] += x.x;
-                            sum[C::G * g + c + 1] += x.y;
-                        }
+                    for (int c = 0; c < C::N; ++c) fma2(sum[c], pair(1.f, 1.f), *reinterpret_cast<const f32x2*>(part + C::at(tx, c)));
                 }
                 store_cols<D>((a ? g1 : g0) + base + (int64_t)(tok0 + r) * D, sum, a ? 1.f : scale, tx);
             }

@@ -67,13 +67,14 @@ attn_fwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* 
 
     const float* qrow = sq + ty * TM * LD;
     float* prow = sp + ty * TM * LDP;
-    float o[TM][C::N], m[TM], l[TM];
+    f32x2 o[TM][C::N];
+    float m[TM], l[TM];
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
         m[i] = -CUDART_INF_F;
         l[i] = 0.f;                                // this thread's keys only
 #pragma unroll
-        for (int c = 0; c < C::N; ++c) o[i][c] = 0.f;
+        for (int c = 0; c < C::N; ++c) o[i][c] = 0;
     }
     for (int i0 = w.first; i0 < w.last && row_live; i0 += KC) {
         if (threadIdx.x < KC) svalid[threadIdx.x] = (uint8_t)(vf & 1u);
@@ -102,7 +103,7 @@ attn_fwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* 
                 m[i] = mx;
                 l[i] *= alpha;
 #pragma unroll
-                for (int c = 0; c < C::N; ++c) o[i][c] *= alpha;
+                for (int c = 0; c < C::N; ++c) mul2(o[i][c], pair(alpha, alpha));
 #pragma unroll
                 for (int j = 0; j < TN; ++j) {
                     const float p = expf(s[i][j] - mx);
@@ -136,28 +137,26 @@ attn_fwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* 
             if (tx == 0) { row[D] = m[i]; row[D + 1] = l[i]; }
         }
         cluster.sync();
-        auto part = [&](int s) -> const float* { return cluster.map_shared_rank(so, s); };
         const int per = (have + tile.shares - 1) / tile.shares, r_end = min(have, per * (tile.rank + 1));
         for (int r = per * tile.rank + ty; r < r_end; r += blockDim.x >> 4) {
-            float mx = -CUDART_INF_F;
-            for (int s = 0; s < tile.shares; ++s) mx = fmaxf(mx, part(s)[r * LDO + D]);
-            float sum = 0.f, acc[C::N];
+            // (at most eight shares; all remote loads of a row are in flight together)
+            float ms[8], mx = -CUDART_INF_F, sum = 0.f;
+            f32x2 acc[C::N];
 #pragma unroll
-            for (int c = 0; c < C::N; ++c) acc[c] = 0.f;
-            for (int s = 0; s < tile.shares; ++s) {
-                const float* row = part(s) + r * LDO;
-                const float ms = row[D];
-                if (ms == -CUDART_INF_F) continue;
-                const float f = expf(ms - mx);
+            for (int s = 0; s < 8; ++s) {
+                ms[s] = s < tile.shares ? cluster.map_shared_rank(so, s)[r * LDO + D] : -CUDART_INF_F;
+                mx = fmaxf(mx, ms[s]);
+            }
+#pragma unroll
+            for (int c = 0; c < C::N; ++c) acc[c] = 0;
+#pragma unroll
+            for (int s = 0; s < 8; ++s) {
+                if (ms[s] == -CUDART_INF_F) continue;
+                const float* row = cluster.map_shared_rank(so, s) + r * LDO;
+                const float f = expf(ms[s] - mx);
                 sum = fmaf(f, row[D + 1], sum);
 #pragma unroll
-                for (int g = 0; g < C::NG; ++g)
-#pragma unroll
-                    for (int c = 0; c < C::G; c += 2) {
-                        const float2 x = *reinterpret_cast<const float2*>(row + C::at(tx, g) + c);
-                        acc[C::G * g + c] = fmaf(f, x.x, acc[C::G * g + c]);
-                        acc[C::G * g + c + 1] = fmaf(f, x.y, acc[C::G * g + c + 1]);
-                    }
+                for (int c = 0; c < C::N; ++c) fma2(acc[c], pair(f, f), *reinterpret_cast<const f32x2*>(row + C::at(tx, c)));
             }
             const int tok = tok0 + r;
             const bool good = sum > 0.f && (!mask || mask[tok] != 0);
