@@ -11,7 +11,7 @@
 // memory between the 16 threads that share a row.  See simt.cuh for the tile shapes and for how clusters share the long tiles.
 // Padded query rows get dq = 0 and give nothing to dk, dv; padded keys get dk = dv = 0.
 // Bound by the FMA pipes (three products per pair of tokens by query, four by key).  Measured (four lanes per row with two
-// exchanges per score before): [2, 12, 52 x 84, 64] with three global blocks 12.16 -> 2.28 ms.
+// exchanges per score before): [2, 12, 52 x 84, 64] with three global blocks 12.16 -> 2.22 ms.
 #include "simt.cuh"
 
 namespace bigbird {
@@ -45,6 +45,8 @@ attn_bwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* 
     float* const row_bias = sp + rows_pad * LDP;
     float* const row_delta = row_bias + rows_pad;
 
+    grid_dependency_release();
+    grid_dependency_wait();
     Tile tile;
     if (!find_tile(tiling, tile)) return;          // (a CTA without a tile belongs to a cluster that shares none)
     const int b = tiling.b, batch = tile.bh / tiling.H;
@@ -213,8 +215,10 @@ cudaError_t launch_tm(const BwdArgs& a, const bigbird_layout& L, const DeviceLay
 }
 template <typename T, int D>
 cudaError_t launch_d(const BwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, int sms, float* ws) {
+    const int tm = rows_per_thread(L, a.B * a.H, D, 2 * sms);
+    if (tm == 2) return launch_tm<T, D, 2>(a, L, dl, sms, ws);
     if constexpr (D <= 64)
-        if (rows_per_thread(a.b, D) == 6) return launch_tm<T, D, 6>(a, L, dl, sms, ws);
+        if (tm == 6) return launch_tm<T, D, 6>(a, L, dl, sms, ws);
     return launch_tm<T, D, 4>(a, L, dl, sms, ws);
 }
 template <typename T>

@@ -659,6 +659,8 @@ attn_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    grid_dependency_release();
+    grid_dependency_wait();
     const unsigned tmem = *(volatile unsigned*)&ctl->tmem_base;
 
     if (warp < kWarpEpilogue) {
@@ -697,6 +699,8 @@ __global__ void __launch_bounds__(kPrepThreads)
 attn_bwd_prepare_kernel(const uint4* __restrict__ out, const uint4* __restrict__ dout, const float* __restrict__ lse,
                         const uint8_t* __restrict__ kpm, float* __restrict__ stats, unsigned long long* __restrict__ kbits,
                         int* __restrict__ counters, int n_counters, long long rows, int N, int H, int row_ctas, int n_words) {
+    grid_dependency_release();
+    grid_dependency_wait();
     if ((int)blockIdx.x >= row_ctas) {             // the last CTAs: mask words and counters
         const int part = blockIdx.x - row_ctas, stride = gridDim.x - row_ctas;
         for (int i = part * kPrepThreads + threadIdx.x; i < n_counters; i += stride * kPrepThreads) counters[i] = 0;
@@ -836,13 +840,11 @@ int launch_attn_bwd_sm100(const BwdArgs& a, const bigbird_layout& L, const Devic
 
     const int row_ctas = (int)((rows + 2 * kPrepRows - 1) / (2 * kPrepRows));
     const int extra = (int)std::min<size_t>(64, 1 + n_words / 64 + n_counters / 2048);
-    attn_bwd_prepare_kernel<<<row_ctas + extra, kPrepThreads, 0, a.stream>>>((const uint4*)a.out, (const uint4*)a.dout, a.lse, a.kpm, (float*)ws,
-        (unsigned long long*)(ws + off_bits), p.counter, (int)n_counters, rows, (int)a.N, a.H, row_ctas, (int)n_words);
-    e = cudaGetLastError();
+    e = launch_chained(attn_bwd_prepare_kernel, (unsigned)(row_ctas + extra), kPrepThreads, 0, a.stream, (const uint4*)a.out, (const uint4*)a.dout, a.lse, a.kpm,
+                       (float*)ws, (unsigned long long*)(ws + off_bits), p.counter, (int)n_counters, (long long)rows, (int)a.N, a.H, row_ctas, (int)n_words);
     if (e == cudaSuccess) {
         ++*launches;
-        attn_bwd_sm100_kernel<<<std::min(sms, p.total_work), kThreads, kSmemBytes, a.stream>>>(tm_q, tm_k, tm_v, tm_do, tm_dq, tm_dk, tm_dv, p);
-        e = cudaGetLastError();
+        e = launch_chained(attn_bwd_sm100_kernel, (unsigned)std::min(sms, p.total_work), kThreads, kSmemBytes, a.stream, tm_q, tm_k, tm_v, tm_do, tm_dq, tm_dk, tm_dv, p);
         if (e == cudaSuccess) ++*launches;
     }
     const cudaError_t ef = cudaFreeAsync(ws, a.stream);

@@ -6,7 +6,8 @@
 // The next chunk's K is on its way while the probabilities and sums are made, the next V while the scores are.  See simt.cuh for
 // the tile shapes and for how clusters share the long tiles.
 // Bound by the FMA pipes.  Measured (a warp per row before, no reuse of K and V in registers): [2, 12, 52 x 84, 64] with three
-// global blocks 3740 -> 691 us, [2, 8, 2560, 128] padded 1547 -> 331 us, [1, 2, 512, 64] 22.6 -> 18.5 us.
+// global blocks 3740 -> 655 us, [2, 8, 2560, 128] padded 1547 -> 305 us, [1, 2, 512, 64] 22.6 -> 13.7 us (18.5 with four rows per
+// thread and launches that wait for the kernel in front to drain).
 #include "simt.cuh"
 
 namespace bigbird {
@@ -40,6 +41,8 @@ attn_fwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* 
     float* const sp = S::kAlias ? sk : sk + KC * LD;
     float* const sv = S::kAlias ? sk + max(KC * LD, rows_pad * LDP) : sp + rows_pad * LDP;
 
+    grid_dependency_release();
+    grid_dependency_wait();
     Tile tile;
     if (!find_tile(tiling, tile)) return;          // (a CTA without a tile belongs to a cluster that shares none)
     const int b = tiling.b, batch = tile.bh / tiling.H;
@@ -187,8 +190,10 @@ cudaError_t launch_tm(const FwdArgs& a, const bigbird_layout& L, const DeviceLay
 }
 template <typename T, int D>
 cudaError_t launch_d(const FwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, int sms) {
+    const int tm = rows_per_thread(L, a.B * a.H, D, 2 * sms);
+    if (tm == 2) return launch_tm<T, D, 2>(a, L, dl, sms);
     if constexpr (D <= 64)
-        if (rows_per_thread(a.b, D) == 6) return launch_tm<T, D, 6>(a, L, dl, sms);
+        if (tm == 6) return launch_tm<T, D, 6>(a, L, dl, sms);
     return launch_tm<T, D, 4>(a, L, dl, sms);
 }
 template <typename T>

@@ -68,4 +68,11 @@ int launch_attn_fwd_sm100(const FwdArgs& a, const bigbird_layout& L, const Devic
 // One-thread kernel whose bounded wait is left to expire (about two seconds); sets the device status word.
 cudaError_t launch_wait_expiry_selftest(DeviceScratch& sc, cudaStream_t stream);
 
+#ifdef __CUDACC__
+// Every kernel of the library is launched so that it may begin before the kernel in front of it in the stream has drained: it lets
+// the next one begin as soon as there is room, and waits for those in front before it touches memory that they may use.
+__device__ __forceinline__ void grid_dependency_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+#endif
+
 }  // namespace bigbird

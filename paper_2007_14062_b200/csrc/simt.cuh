@@ -226,13 +226,16 @@ struct Shape {
     Tiling t;
     int threads, grid;
 };
-// Six rows per thread where that covers a block with no more padding than four would (the larger micro-tile reads less shared
+// Two rows per thread where four would leave half of the GPU idle; else six where that covers a block with no more padding than four would (the larger micro-tile reads less shared
 // memory per FMA); four for D = 128, whose sums take twice the registers.
 inline int padded_rows(int tm, int b) {
     const int tiles = (b + 16 * tm - 1) / (16 * tm), rows = (b + tiles - 1) / tiles;
     return tiles * std::max(2, ((rows + tm - 1) / tm + 1) / 2 * 2) * tm;
 }
-inline int rows_per_thread(int b, int D) { return D <= 64 && padded_rows(6, b) <= padded_rows(4, b) ? 6 : 4; }
+inline int rows_per_thread(const bigbird_layout& L, int BH, int D, int slots) {
+    if (2 * (int64_t)BH * L.nb * ((L.b + 63) / 64) <= slots) return 2;
+    return D <= 64 && padded_rows(6, L.b) <= padded_rows(4, L.b) ? 6 : 4;
+}
 
 // tm: rows per thread; kc: tokens per chunk; slots: CTAs that fit the GPU at a time.
 inline Shape make_shape(int tm, const bigbird_layout& L, const DeviceLayout& dl, int BH, int slots, int kc) {
@@ -286,12 +289,14 @@ cudaError_t launch_clusters(void (*kernel)(Ps...), const Shape& s, size_t smem, 
     cfg.blockDim = dim3((unsigned)s.threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = (unsigned)s.t.cluster;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)s.t.cluster;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = s.t.cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 

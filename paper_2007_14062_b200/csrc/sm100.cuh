@@ -321,11 +321,6 @@ __device__ __forceinline__ void split_bf16(float x0, float x1, unsigned& hi, uns
     lo = pack_bf16(x0 - h0, x1 - h1);
 }
 
-// Chained launches (launch_chained): lets the next kernel of the stream begin when it finds room; waits until the kernels in front
-// have finished and their writes are visible.
-__device__ __forceinline__ void grid_dependency_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // ------------------------------------------------------------------------------------------------ host side
 // A launch that may begin before the kernel in front of it in the stream has drained; the kernel waits for it itself.
 template <typename... Ps, typename... As>
