@@ -185,7 +185,7 @@ BIGBIRD_API int bigbird_attn_bwd(const void* q, const void* k, const void* v, co
  *   - the array holds the device copy of one layout's schedule.  A call with another layout than the previous
  *     call on that device first copies the new schedule from the handle's host arrays (two cudaMemcpyAsync on
  *     `stream` from pageable memory: the host may wait until they have been staged); later calls with the same
- *     layout enqueue only a 16-byte cudaMemsetAsync and the kernels.  `layout` must not be destroyed while a
+ *     layout enqueue only the kernels (and a 16-byte cudaMemsetAsync if there is no mask).  `layout` must not be destroyed while a
  *     call that uses it is being enqueued;
  *   - the first call on a device looks up the array's device address and sets a kernel attribute; make that
  *     first call outside any stream capture;

@@ -197,11 +197,16 @@ struct StreamRef {
 // Fetches the next work item for a stream, drops the key blocks that are entirely padding and posts the live
 // list.  Returns the work index (-1: the stream has been told that there is no more work), or -2 after an
 // expired wait.
-__device__ __forceinline__ int schedule_one(const KernelParams& p, SmemCtl* ctl, StreamCtl* sc, unsigned& sched_n, int lane) {
+__device__ __forceinline__ int schedule_one(const KernelParams& p, SmemCtl* ctl, StreamCtl* sc, int stream, unsigned& sched_n, int lane) {
     const unsigned lt_mask = (1u << lane) - 1u;
-    int w = 0;
-    if (lane == 0) w = atomicAdd(&p.counter[0], 1);
-    w = __shfl_sync(0xffffffffu, w, 0);
+    // A stream's first item is its own, which spreads the global tiles over the SMs (the second streams in the opposite order, so
+    // that with little work a CTA with a global tile has nothing else); after that they are drawn.
+    int w = stream == 0 ? (int)blockIdx.x : (int)(2 * gridDim.x - 1 - blockIdx.x);
+    static_assert(kStreams == 2, "first items");
+    if (sched_n > 0) {
+        if (lane == 0) w = (int)gridDim.x * kStreams + atomicAdd(&p.counter[0], 1);
+        w = __shfl_sync(0xffffffffu, w, 0);
+    }
     if (w >= p.total_work) w = -1;
     // decode the work index: the parts of the global-row tiles of every (batch, head) first, then the sparse tiles
     int bh = 0, batch = 0, part_slot = -1;
@@ -295,7 +300,7 @@ __device__ __forceinline__ void scheduler_role(const KernelParams& p, SmemCtl* c
             unsigned n = s == 0 ? sched_n0 : sched_n1;
             const unsigned ss = n % kSchedSlots, sp = (n / kSchedSlots) & 1u;
             if (!__all_sync(0xffffffffu, mbar_test(&sc->sched_empty[ss], sp ^ 1u))) continue;
-            const int w = schedule_one(p, ctl, sc, n, lane);
+            const int w = schedule_one(p, ctl, sc, s, n, lane);
             if (s == 0) sched_n0 = n; else sched_n1 = n;
             if (w == -2) return;
             if (w < 0) done |= 1u << s;
@@ -797,19 +802,32 @@ merge_split_tiles_kernel(const float* __restrict__ partials, const Item* __restr
     const unsigned long long qb = kbits ? kbits[(size_t)(bh / H) * nb + q] : ~0ull;
     const float* base = partials + (size_t)(bh * tiles_per_head + tile) * nparts * kPartialFloats;
     const float* stats = base + 128 * 64 + row;
-    float m = -INFINITY;
-#pragma unroll 4
-    for (int pt = 0; pt < nparts; ++pt) m = fmaxf(m, stats[(size_t)pt * kPartialFloats]);
+    float m = -INFINITY, l = 0.f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    float l = 0.f;
-#pragma unroll 4
-    for (int pt = 0; pt < nparts; ++pt) {
-        const float mp = stats[(size_t)pt * kPartialFloats], lp = stats[(size_t)pt * kPartialFloats + 128];
-        const float4 v = reinterpret_cast<const float4*>(base + (size_t)pt * kPartialFloats)[row * 16 + c4];
-        if (!(lp > 0.f)) continue;                   // (such a part has left no accumulator)
-        const float wgt = exp2f(mp - m);
-        l += wgt * lp;
-        acc.x += wgt * v.x; acc.y += wgt * v.y; acc.z += wgt * v.z; acc.w += wgt * v.w;
+    for (int p0 = 0; p0 < nparts; p0 += 8) {         // eight parts at a time, all of their loads in flight together
+        float mp[8], lp[8], mx = m;
+        float4 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const size_t off = (size_t)min(p0 + u, nparts - 1) * kPartialFloats;
+            mp[u] = stats[off];
+            lp[u] = p0 + u < nparts ? stats[off + 128] : 0.f;
+            v[u] = reinterpret_cast<const float4*>(base + off)[row * 16 + c4];
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) mx = fmaxf(mx, lp[u] > 0.f ? mp[u] : -INFINITY);
+        if (mx == -INFINITY) continue;
+        const float scale = exp2f(m - mx);           // 0 on the first parts that have anything
+        m = mx;
+        l *= scale;
+        acc.x *= scale; acc.y *= scale; acc.z *= scale; acc.w *= scale;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if (!(lp[u] > 0.f)) continue;            // (such a part has left no accumulator)
+            const float wgt = exp2f(mp[u] - mx);
+            l += wgt * lp[u];
+            acc.x += wgt * v[u].x; acc.y += wgt * v[u].y; acc.z += wgt * v[u].z; acc.w += wgt * v[u].w;
+        }
     }
     const bool good = ((qb >> r64) & 1ull) && l > 0.f;
     const float inv = good ? 1.f / l : 0.f;
@@ -832,10 +850,11 @@ __global__ void wait_expiry_selftest_kernel(int* status) {
     }
 }
 
-// One 64-bit word per (batch, key block): bit t = key_padding_mask[batch, block*64 + t] != 0.
-__global__ void __launch_bounds__(256) pack_mask_kernel(const uint8_t* __restrict__ kpm, unsigned long long* __restrict__ kbits, int n_words) {
+// One 64-bit word per (batch, key block): bit t = key_padding_mask[batch, block*64 + t] != 0; and four words to be cleared, if any.
+__global__ void __launch_bounds__(256) pack_mask_kernel(const uint8_t* __restrict__ kpm, unsigned long long* __restrict__ kbits, int n_words, int* __restrict__ zero4) {
     grid_dependency_release();
     grid_dependency_wait();
+    if (zero4 && blockIdx.x == 0 && threadIdx.x < 4) zero4[threadIdx.x] = 0;
     const int word = (blockIdx.x * 256 + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (word >= n_words) return;
     const uint8_t* src = kpm + (size_t)word * kBlock;
@@ -919,10 +938,10 @@ int grid_size(int sm_count, int total_work) { return std::max(1, std::min(sm_cou
 // The kernels of a call, in the order of the stream, each allowed to begin before the one in front of it has drained: they wait for
 // it (grid_dependency_wait) before they touch memory that it may use.
 cudaError_t enqueue(const KernelParams& p, const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
-                    const uint8_t* kpm, unsigned long long* kbits, int n_words, int sm_count, cudaStream_t stream, int* launches) {
+                    const uint8_t* kpm, unsigned long long* kbits, int n_words, int* zero4, int sm_count, cudaStream_t stream, int* launches) {
     cudaError_t e = cudaSuccess;
     if (n_words) {
-        e = launch_chained(pack_mask_kernel, (unsigned)((n_words * 32 + 255) / 256), 256, 0, stream, kpm, kbits, n_words);
+        e = launch_chained(pack_mask_kernel, (unsigned)((n_words * 32 + 255) / 256), 256, 0, stream, kpm, kbits, n_words, zero4);
         if (e != cudaSuccess) return e;
         ++*launches;
     }
@@ -984,7 +1003,7 @@ int launch_attn_fwd_sm100(const FwdArgs& a, const bigbird_layout& L, const Devic
     p.status = sc.status;
     set_shape(p, L, a.B, cut, a.scale);
 
-    cudaError_t e = enqueue(p, tm_q, tm_k, tm_v, a.kpm, (unsigned long long*)(ws + off_bits), (int)words, sm_count, a.stream, launches);
+    cudaError_t e = enqueue(p, tm_q, tm_k, tm_v, a.kpm, (unsigned long long*)(ws + off_bits), (int)words, nullptr, sm_count, a.stream, launches);
     if (ws) {
         const cudaError_t ef = cudaFreeAsync(ws, a.stream);
         if (e == cudaSuccess) e = ef;
@@ -1086,8 +1105,10 @@ extern "C" int bigbird_attn_fwd_static(const void* q, const void* k, const void*
 
     // The array keeps what the last call left: status and work counter must start at zero, and the schedule of
     // this call's layout replaces the previous one (step offsets made absolute, as the kernel expects).
-    e = cudaMemsetAsync(words4, 0, 16, stream);
-    if (e != cudaSuccess) return BIGBIRD_ECUDA;
+    if (!key_padding_mask) {                    // (else the kernel that packs the mask does it)
+        e = cudaMemsetAsync(words4, 0, 16, stream);
+        if (e != cudaSuccess) return BIGBIRD_ECUDA;
+    }
     // The schedule is sent only when the array does not hold this layout's already (copies from the handle's own
     // host arrays, which live as long as the handle).
     if (sd.schedule_uid != L->uid) {
@@ -1111,7 +1132,7 @@ extern "C" int bigbird_attn_fwd_static(const void* q, const void* k, const void*
     p.counter = words4 + 2;
     set_shape(p, *L, B, cut, scale);
     int launches = 0;
-    if (enqueue(p, tm_q, tm_k, tm_v, key_padding_mask, kbits_dev, key_padding_mask ? (int)words : 0, sd.sm_count, stream, &launches) != cudaSuccess)
+    if (enqueue(p, tm_q, tm_k, tm_v, key_padding_mask, kbits_dev, key_padding_mask ? (int)words : 0, words4, sd.sm_count, stream, &launches) != cudaSuccess)
         return BIGBIRD_ECUDA;
     return BIGBIRD_OK;
 }
