@@ -107,7 +107,6 @@ cudaError_t upload_layout(const bigbird_layout* L, DeviceLayout& d) {
     put(&d.row_idx, L->row_idx);
     put(&d.items, L->items_abs);
     put(&d.steps, L->steps);
-    put(&d.split_tile_q, L->split_tile_q);
     put(&d.items_t, L->items_t);
     put(&d.steps_t, L->steps_t);
     put(&d.global_pairs, L->global_pairs);

@@ -25,7 +25,8 @@
 // Measured (gradients of the base workload [8, 12, 4096, 64]): CUDA-core kernels 16.3 ms; one thread issuing all MMAs 857 us,
 // the same from one elected thread 557, columns 16 at a time with the next 16 on their way 527, two issuing threads 505, all
 // roles on the ring, tests ahead of the commits and rows written by TMA 497 us ([1, 12, 16384, 64] with 13000 valid tokens
-// 338 -> 193 us from the second of these to the last).  A step takes 1400 cycles; its MMAs need 650 of the tensor pipe, without
+// 338 -> 193 us from the second of these to the last), and 189 with the parts of
+// a cut tile fetched together ([2, 12, 1024] 54 -> 39.5 us, there no longer cut).  A step takes 1400 cycles; its MMAs need 650 of the tensor pipe, without
 // any elementwise work it takes 1100, without any MMAs 1150: what is left is the way of a step through the hands of four
 // warps with three steps in flight, which is all that tensor memory holds.  Two threads per row (24 warps) were no faster.
 //
@@ -126,10 +127,14 @@ __device__ __forceinline__ unsigned long long token_bits(const KernelParams& p, 
 __device__ __forceinline__ void scheduler_role(const KernelParams& p, SmemCtl* ctl, int lane) {
     const unsigned lt_mask = (1u << lane) - 1u;
     unsigned slot_n = 0;
+    bool first_item = true;
     for (;;) {
-        int w = 0;
-        if (lane == 0) w = atomicAdd(p.counter, 1);
-        w = __shfl_sync(0xffffffffu, w, 0);
+        int w = (int)blockIdx.x;                    // the first item is the CTA's own, the others are drawn
+        if (!first_item) {
+            if (lane == 0) w = (int)gridDim.x + atomicAdd(p.counter, 1);
+            w = __shfl_sync(0xffffffffu, w, 0);
+        }
+        first_item = false;
         if (w >= p.total_work) w = -1;
         int kind = 0, bh = 0, ra = kNoBlock, rb = kNoBlock, begin = 0, n_raw = 0, split = -1, part = 0;
         const Step* steps = nullptr;               // nullptr: blocks begin, begin + 1, ... attended by both halves
@@ -516,23 +521,31 @@ __device__ __forceinline__ bool epilogue_sync(SmemCtl* ctl, unsigned& n) {
 __device__ __forceinline__ void merge_parts(const KernelParams& p, const TileSlot* slot, int tid) {
     const bool dkv = slot->kind == kDkv;
     const float* base = p.partials + (size_t)slot->split * p.parts * kPartialFloats;
+    // four columns of four rows at a time, so that their loads are in flight together
 #pragma unroll 1
-    for (int idx = tid; idx < (dkv ? 2 : 1) * 128 * 16; idx += 128) {
-        const int m = idx >> 11, row = (idx >> 4) & 127, c4 = idx & 15;
-        const int blk = row >= kBlock ? slot->rb : slot->ra;
-        if (blk < 0) continue;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int pt = 0; pt < p.parts; ++pt) {               // fixed order: results do not depend on scheduling
-            const float4 v = __ldcg(reinterpret_cast<const float4*>(base + (size_t)pt * kPartialFloats + m * 128 * kBlock + row * kBlock) + c4);
-            acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+    for (int i0 = tid; i0 < (dkv ? 2 : 1) * 128 * 16; i0 += 4 * 128) {
+        const float4* src = reinterpret_cast<const float4*>(base) + i0;       // rows of 16 float4, the accumulators one behind the other
+        float4 acc[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+        for (int pt = 0; pt < p.parts; ++pt, src += kPartialFloats / 4) {     // fixed order: results do not depend on scheduling
+            float4 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = __ldcg(src + 128 * u);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) { acc[u].x += v[u].x; acc[u].y += v[u].y; acc[u].z += v[u].z; acc[u].w += v[u].w; }
         }
-        const unsigned long long bits = row >= kBlock ? slot->rbits_b : slot->rbits_a;
-        const float f = ((bits >> (row & 63)) & 1ull) ? (m ? 1.f : p.scale) : 0.f;
-        __nv_bfloat16* dst = (dkv ? (m ? p.dv : p.dk) : p.dq) + (((size_t)slot->bh * p.nb + blk) * kBlock + (row & 63)) * kBlock;
-        uint2 v2;
-        v2.x = pack_bf16(acc.x * f, acc.y * f);
-        v2.y = pack_bf16(acc.z * f, acc.w * f);
-        reinterpret_cast<uint2*>(dst)[c4] = v2;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int idx = i0 + 128 * u, m = idx >> 11, row = (idx >> 4) & 127, c4 = idx & 15;
+            const int blk = row >= kBlock ? slot->rb : slot->ra;
+            if (blk < 0) continue;
+            const unsigned long long bits = row >= kBlock ? slot->rbits_b : slot->rbits_a;
+            const float f = ((bits >> (row & 63)) & 1ull) ? (m ? 1.f : p.scale) : 0.f;
+            __nv_bfloat16* dst = (dkv ? (m ? p.dv : p.dk) : p.dq) + (((size_t)slot->bh * p.nb + blk) * kBlock + (row & 63)) * kBlock;
+            reinterpret_cast<uint2*>(dst)[c4] = make_uint2(pack_bf16(acc[u].x * f, acc[u].y * f), pack_bf16(acc[u].z * f, acc[u].w * f));
+        }
     }
 }
 
@@ -793,12 +806,16 @@ int launch_attn_bwd_sm100(const BwdArgs& a, const bigbird_layout& L, const Devic
         !make_map(&tm_dv, a.dv, (uint64_t)rows))
         return fail(cudaErrorInvalidValue);
 
-    // Tiles of global blocks have nb steps where the others have about ten: cut them into parts of about half of what each SM
-    // gets altogether (at least 8 steps), so that none of them is still running when the rest is done.
+    // Tiles of global blocks have nb steps where the others have about ten: cut them into parts of about a third of what each
+    // SM gets altogether, so that none of them is still running when the rest is done, of 16 steps or more, and not at all up
+    // to 32 steps: adding the parts up takes about 5 us on the path of the last one (it was 24 when a thread fetched one value
+    // after the other).  Measured, gradients of B, 12 heads, nb blocks in us: [2, nb 16] 39.5 uncut, 43.7 in two, 52 in four;
+    // [1, 32] 56.9 uncut, 54.6 in two; four heads [1, 32] 34.6, 38.2; [1, 64] 93.7 uncut, 79.7 in two, 74.6 in three, 75.2 in
+    // four, 78.5 in eight; [1, 256] 200 uncut, 190 in two, 191 in three; [3, 16 heads, 96] 212 uncut, 221 in two.
     const int64_t steps = (int64_t)a.B * ((int64_t)L.steps.size() + (int64_t)L.steps_t.size() + (int64_t)a.H * L.global_tiles * a.nb);
-    int part_steps = (int)std::min<int64_t>(a.nb, std::max<int64_t>(8, steps / (2 * sms)));
-    const int parts = (a.nb + part_steps - 1) / part_steps;
-    part_steps = (a.nb + parts - 1) / parts;
+    const int64_t want = std::max<int64_t>(16, steps / (3 * sms));
+    const int want_parts = a.nb <= 32 ? 1 : (int)((a.nb + want - 1) / want);
+    const int part_steps = (a.nb + want_parts - 1) / want_parts, parts = (a.nb + part_steps - 1) / part_steps;
 
     // workspace of this call, on the caller's stream
     const int n_split = parts > 1 ? 2 * BH * L.global_tiles : 0;

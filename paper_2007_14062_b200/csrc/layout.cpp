@@ -193,17 +193,11 @@ int build_layout_host(bigbird_layout* L, int chunk_steps) {
     if (chunk_steps <= 0) chunk_steps = nb <= 96 ? nb : 32;
     const int parts = (nb + chunk_steps - 1) / chunk_steps;
     L->max_parts = parts;
-    L->split_tiles_per_head = parts > 1 ? n_gtiles : 0;
     L->heavy_items_per_head = n_gtiles * parts;
     L->items_per_head = L->heavy_items_per_head + n_stiles;
     L->items.clear();
     L->steps.clear();
     L->step_base.clear();
-    L->split_tile_q.clear();
-    for (int t = 0; t < n_gtiles && parts > 1; ++t) {
-        L->split_tile_q.push_back(gq[2 * t]);
-        L->split_tile_q.push_back(2 * t + 1 < (int)gq.size() ? gq[2 * t + 1] : kNoBlock);
-    }
     TileScratch tmp;
     for (int h = 0; h < H; ++h) {
         const int32_t base = (int32_t)L->steps.size();

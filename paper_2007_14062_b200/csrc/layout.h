@@ -37,7 +37,6 @@ struct DeviceLayout {
     int32_t* row_idx = nullptr;
     Item* items = nullptr;
     Step* steps = nullptr;
-    int32_t* split_tile_q = nullptr;   // [split_tiles_per_head * 2]
     Item* items_t = nullptr;           // tiles of key blocks over the transposed lists
     Step* steps_t = nullptr;
     int32_t* global_pairs = nullptr;   // [global_tiles * 2]
@@ -62,13 +61,11 @@ struct bigbird_layout {
     // tile schedule: per head the same number of items, heavy (global) items first
     int items_per_head = 0;
     int heavy_items_per_head = 0;   // leading items of each head that belong to global tiles
-    int split_tiles_per_head = 0;   // global tiles cut into chunks (each needs a merge)
     int max_parts = 1;
     std::vector<bigbird::Item> items;          // [H * items_per_head], step_begin relative to the head's first step
     std::vector<bigbird::Item> items_abs;      // the same with step_begin made absolute (what the kernel reads)
     std::vector<int32_t> step_base;            // [H] offset of the head's steps in `steps`
     std::vector<bigbird::Step> steps;
-    std::vector<int32_t> split_tile_q;         // [split_tiles_per_head * 2] query blocks (qa, qb) of each split tile
     // the same for tiles that stack two key blocks and walk the query blocks that attend them (b == 64 only); global
     // key blocks have no list, every query block attends them
     int sparse_tiles_per_head = 0;
