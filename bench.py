@@ -213,8 +213,8 @@ def run_reference(args, wl):
 
 
 def run_backward(args, wl):
-    """`--direction bwd`: the gradient kernels (CUDA cores, fp32 arithmetic) on the same workload, one GPU.  Their
-    FLOPs are counted like the forward pass's: five b x b x D products per attended block pair (the scores again,
+    """`--direction bwd`: the gradient kernels on the same workload, one GPU (tensor cores for bf16 tensors with 64-token
+    blocks and 64-wide heads, CUDA cores in fp32 otherwise).  Their FLOPs are counted like the forward pass's: five b x b x D products per attended block pair (the scores again,
     dP, dV, dQ, dK) against the forward pass's two."""
     import paper_2007_14062_b200 as bb
     if not torch.cuda.is_available():
@@ -256,19 +256,24 @@ def run_backward(args, wl):
     ms_per_step = ev0.elapsed_time(ev1) / steps
     tflops = flops_per_step / (ms_per_step * 1e-3) / 1e12
     clocks = sampler.summary()
-    # fp32 FMA peak of the CUDA cores from unit counts and the clock: SMs x 128 lanes x 2 FLOP x max SM clock
-    sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    alu_peak = sms * 128 * 2 * (clocks["sm_max_mhz"] or 1965) * 1e6 / 1e12
+    tensor = wl.dtype == "bf16" and wl.b == 64 and wl.D == 64
+    if tensor:
+        peaks = measured_peaks()
+        peak, source, kernel = peaks["bf16_tflops"], f"{peaks['source']} bf16 burst", "attn_bwd_sm100_kernel"
+    else:
+        # fp32 FMA peak of the CUDA cores from unit counts and the clock: SMs x 128 lanes x 2 FLOP x max SM clock
+        sms = torch.cuda.get_device_properties(dev).multi_processor_count
+        peak, source, kernel = sms * 128 * 2 * (clocks["sm_max_mhz"] or 1965) * 1e6 / 1e12, "fp32 FMA lanes x clock (derived)", "attn_bwd_simt_kernel"
     elt = q.element_size()
     min_bytes = wl.B * wl.H * wl.N * (8 * wl.D * elt + 4)          # q, k, v, out, dout read, dq, dk, dv written, lse read
     line = {"metric": "block-sparse attn bwd TFLOP/s (counted FLOPs)", "value": tflops, "unit": UNIT, "n_gpus": 1, "steps": steps,
             "warmup": warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": "f32", "data": "synthetic", "direction": "bwd",
+            "dtype": "bf16" if tensor else "f32", "data": "synthetic", "direction": "bwd",
             "config": dict(workload_config(wl, pairs), counted_gflop_per_step_bwd=flops_per_step / 1e9,
                            l2=f"one set of eight tensors ({8 * q.numel() * elt / 1e6:.0f} MB)"),
             "gpu_launches": launches * steps, "clocks": clocks,
-            "roofline": {"bound": "alu", "achieved": tflops, "peak": alu_peak, "unit": "TFLOP/s", "frac": tflops / alu_peak,
-                         "traffic": None, "peak_source": "fp32 FMA lanes x clock (derived)", "kernel": "attn_bwd_dq_kernel + attn_bwd_dkv_kernel",
+            "roofline": {"bound": "tensor" if tensor else "alu", "achieved": tflops, "peak": peak, "unit": "TFLOP/s", "frac": tflops / peak,
+                         "traffic": None, "peak_source": source, "kernel": kernel,
                          "min_hbm_bytes_per_launch": min_bytes, "achieved_hbm_gbs_on_min_bytes": min_bytes / (ms_per_step * 1e-3) / 1e9}}
     if not args.no_cpu_baseline:
         from oracle import bigbird_oracle as O
