@@ -542,9 +542,11 @@ __device__ __forceinline__ void merge_parts(const KernelParams& p, const TileSlo
             const int blk = row >= kBlock ? slot->rb : slot->ra;
             if (blk < 0) continue;
             const unsigned long long bits = row >= kBlock ? slot->rbits_b : slot->rbits_a;
-            const float f = ((bits >> (row & 63)) & 1ull) ? (m ? 1.f : p.scale) : 0.f;
+            const bool row_ok = (bits >> (row & 63)) & 1ull;     // (a select: see the epilogue)
+            const float f = m ? 1.f : p.scale;
             __nv_bfloat16* dst = (dkv ? (m ? p.dv : p.dk) : p.dq) + (((size_t)slot->bh * p.nb + blk) * kBlock + (row & 63)) * kBlock;
-            reinterpret_cast<uint2*>(dst)[c4] = make_uint2(pack_bf16(acc[u].x * f, acc[u].y * f), pack_bf16(acc[u].z * f, acc[u].w * f));
+            reinterpret_cast<uint2*>(dst)[c4] = row_ok ? make_uint2(pack_bf16(acc[u].x * f, acc[u].y * f), pack_bf16(acc[u].z * f, acc[u].w * f))
+                                                       : make_uint2(0u, 0u);
         }
     }
 }
@@ -599,13 +601,16 @@ __device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ct
 #pragma unroll
                     for (int j = 0; j < 4; ++j) d4[j] = make_float4(o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
                 } else {
-                    const float f = row_ok ? (m ? 1.f : p.scale) : 0.f;
+                    // A padded row is zeroed by a select and not by a factor: a padded key takes part like any other up to here, and
+                    // since its scores are not in lse, its sums may be infinite or NaN.
+                    const float f = m ? 1.f : p.scale;
                     const unsigned base = my_row + m * 2 * kTileBytes;
+                    unsigned w[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) w[j] = row_ok ? pack_bf16(o[2 * j] * f, o[2 * j + 1] * f) : 0u;
 #pragma unroll
                     for (int j = 0; j < 2; ++j)     // 16 bytes of a row; the swizzle keeps the rows of a store in different banks
-                        st_shared16(base + (((2 * (c & 3) + j) ^ (r64 & 7)) << 4), pack_bf16(o[8 * j] * f, o[8 * j + 1] * f),
-                                    pack_bf16(o[8 * j + 2] * f, o[8 * j + 3] * f), pack_bf16(o[8 * j + 4] * f, o[8 * j + 5] * f),
-                                    pack_bf16(o[8 * j + 6] * f, o[8 * j + 7] * f));
+                        st_shared16(base + (((2 * (c & 3) + j) ^ (r64 & 7)) << 4), w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
                 }
             }
             if (split < 0) {

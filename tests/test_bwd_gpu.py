@@ -107,3 +107,40 @@ SHAPES = [_case("fp32", B, 2, nb, b=b, D=D, g=g, r=2, lengths=f"ragged:{nb * b /
 @pytest.mark.parametrize("wl", SHAPES, ids=lambda w: f"{w.b}_{w.N // w.b}_{w.B}_{w.D}")
 def test_tile_shapes_of_the_cuda_core_gradients(wl):
     test_gradients_match_the_oracle(wl)
+
+
+# What stands in padded rows must leave no trace, however large (finite: a padded row of k, v, q or dout takes part in tensor-core
+# products with probability zero).  Tensor-core gradients, tiles of global blocks whole and cut; the last case pads the tail of a
+# global key block.  1e3: scores of a padded key row exceed the row's lse by far more than exp can hold.
+PADDED = [(_case("bf16", 2, 2, 12), 197, 0), (_case("bf16", 1, 1, 40, g=3, r=2), 2001, 0), (_case("bf16", 2, 2, 9, mode=1, g=2, r=0), 500, 100),
+          (_case("bf16", 1, 1, 40, mode=1, g=3, r=2), 2560, 130)]
+
+
+@pytest.mark.parametrize("what,size", [("k", 1e3), ("q", 1e3), ("v", 1e3), ("dout", 1e3)])
+@pytest.mark.parametrize("wl,valid,gtok", PADDED, ids=lambda x: getattr(x, "name", x))
+def test_padded_rows_of_any_finite_size_leave_no_trace(wl, valid, gtok, what, size):
+    dev = torch.device("cuda:0")
+    kpm = torch.zeros(wl.B, wl.N, dtype=torch.uint8)
+    kpm[:, :valid] = 1
+    if gtok:
+        kpm[:, gtok:wl.g * wl.b] = 0
+    pad = (kpm == 0)[:, None, :, None].to(dev)
+    t = dict(zip("qkv", (x.to(dev).masked_fill(pad, 0) for x in synth.make_qkv(wl))))
+    t["dout"] = torch.randn(t["q"].shape, generator=torch.Generator(dev).manual_seed(3), device=dev).to(torch.bfloat16).masked_fill(pad, 0)
+    L = bb.bigbird_build_layout(wl.N, wl.b, wl.w, wl.g, wl.r, wl.seed, wl.H, wl.mode)
+    out = torch.empty_like(t["q"])
+    lse = torch.empty(out.shape[:3], device=dev, dtype=torch.float32)
+    bb.bigbird_attn_fwd(t["q"], t["k"], t["v"], L, kpm.to(dev), out, lse, wl.scale)
+    res = []
+    for dirty in (False, True):
+        if dirty:
+            sign = 1 - 2 * (torch.arange(wl.N * wl.D, device=dev).reshape(wl.N, wl.D) % 3 % 2)        # both signs in every row
+            t[what] = torch.where(pad, (sign * size).to(torch.bfloat16), t[what])
+        grads = [torch.full_like(out, float("nan")) for _ in range(3)]
+        bb.bigbird_attn_bwd(t["q"], t["k"], t["v"], out, lse, t["dout"], L, kpm.to(dev), *grads, wl.scale)
+        res.append(grads)
+    assert bb.bigbird_last_status() == (0, 0)
+    for clean, dirty in zip(*res):
+        assert torch.equal(clean, dirty)
+        assert (dirty.masked_select(pad) == 0).all()
+    L.close()
