@@ -60,12 +60,13 @@ constexpr int kPartialFloats = 2 * 128 * kBlock;   // one part of a split tile: 
 enum { kDkv = 0, kDq = 1 };
 enum { kSegFirst = 1, kSegLast = 2 };
 // what there is to know about a ring entry: bits 0..1 the step's kBothHalves / kUpperHalf / kLowerHalf, kind, first and last step of
-// its tile, the tile's row buffer and the parity of that buffer's phase; kInfoEnd: no more steps
-enum { kInfoWho = 3, kInfoDkv = 4, kInfoFirst = 8, kInfoLast = 16, kInfoX = 32, kInfoXPar = 64, kInfoEnd = 128 };
+// its tile, the tile's row buffer and the parity of that buffer's phase; kInfoEnd: no more steps; kInfoPadded: some of the block's
+// tokens are padding
+enum { kInfoWho = 3, kInfoDkv = 4, kInfoFirst = 8, kInfoLast = 16, kInfoX = 32, kInfoXPar = 64, kInfoEnd = 128, kInfoPadded = 256 };
 
 struct __align__(16) StepEntry {
     int c;                         // block of the column side
-    int who;                       // kBothHalves, kUpperHalf or kLowerHalf
+    int who;                       // kBothHalves, kUpperHalf or kLowerHalf, and kInfoPadded
     unsigned long long kb;         // its valid-token bits (never 0)
 };
 struct __align__(16) TileSlot {
@@ -196,6 +197,7 @@ __device__ __forceinline__ void scheduler_role(const KernelParams& p, SmemCtl* c
                     e.who = (ua && ub) ? kBothHalves : (ua ? kUpperHalf : kLowerHalf);
                     alive = BB_CHECK(s.c >= 0 && s.c < p.nb, 170);
                     if (alive) e.kb = token_bits(p, batch, s.c);
+                    if (e.kb != ~0ull) e.who |= kInfoPadded;
                     alive = alive && e.kb != 0ull && (ua || ub);
                 }
                 const unsigned bal = __ballot_sync(0xffffffffu, alive);
@@ -399,8 +401,24 @@ __device__ __forceinline__ void accumulate_role(const KernelParams& p, SmemCtl* 
 // ------------------------------------------------------------------------------------------------ elementwise (three warpgroups, one thread per row)
 // The 64 columns of a step, 16 at a time, the next 16 on their way out of tensor memory meanwhile.  What takes the place of 16
 // columns of fp32 is 8 columns of packed high halves and 8 of low halves.
+// -inf over the scores of a step's padded tokens, in tensor memory.  (Rare: the blocks that hold a sequence's end.  Key tiles need
+// it although their padded queries have -inf for their statistics: that makes P zero only where S is below infinity.  A test per
+// 16 columns in dq_columns and dkv_columns cost training 5%.)
+__device__ __forceinline__ void mask_scores(unsigned buf, unsigned long long bits64) {
+#pragma unroll 1
+    for (int c = 0; c < 4; ++c) {
+        float s[16];
+        const unsigned bits = (unsigned)(bits64 >> (16 * c));
+        tmem_ld16(buf + 16 * c, s);
+        tmem_wait_ld();
+#pragma unroll
+        for (int t = 0; t < 16; ++t) s[t] = ((bits >> t) & 1u) ? s[t] : -INFINITY;
+        tmem_st16(buf + 16 * c, reinterpret_cast<unsigned*>(s));
+    }
+    tmem_wait_st();
+}
 // Query tiles: dS = exp2(S sl2 + nl) (dP + nd) over S.
-__device__ __forceinline__ void dq_columns(unsigned buf, float sl2, float nl, float nd, unsigned long long kb) {
+__device__ __forceinline__ void dq_columns(unsigned buf, float sl2, float nl, float nd) {
     float s[2][16], d[2][16];
     tmem_ld16(buf, s[0]);
     tmem_ld16(buf + 64, d[0]);
@@ -411,11 +429,6 @@ __device__ __forceinline__ void dq_columns(unsigned buf, float sl2, float nl, fl
         if (c < 3) {
             tmem_ld16(buf + 16 * (c + 1), s[(c + 1) & 1]);
             tmem_ld16(buf + 64 + 16 * (c + 1), d[(c + 1) & 1]);
-        }
-        if (__builtin_expect(kb != ~0ull, 0)) {                 // padded keys
-            const unsigned bits = (unsigned)(kb >> (16 * c));
-#pragma unroll
-            for (int t = 0; t < 16; ++t) sc[t] = ((bits >> t) & 1u) ? sc[t] : -INFINITY;
         }
         unsigned o[16];
 #pragma unroll
@@ -484,6 +497,7 @@ __device__ __forceinline__ void elementwise_role(const KernelParams& p, SmemCtl*
         if (!mbar_wait(&ctl->sdp_full[g], par, abort_flag)) { fail = 131; break; }
         __syncwarp();                               // lanes leave the wait one by one
         tc_fence_after();
+        if (__builtin_expect((info & kInfoPadded) != 0, 0) && mine) mask_scores(buf, ctl->bits[stage]);
         if (!mine) {
             tmem_st32_zero(buf);
             tmem_st32_zero(buf + 32);
@@ -495,7 +509,7 @@ __device__ __forceinline__ void elementwise_role(const KernelParams& p, SmemCtl*
             const float2* st = reinterpret_cast<const float2*>(ctl->y_stats[stage]);
             dkv_columns(buf, p.scale_log2, st, st + 32);
         } else {
-            dq_columns(buf, p.scale_log2, nl, nd, ctl->bits[stage]);
+            dq_columns(buf, p.scale_log2, nl, nd);
         }
         tmem_wait_st();
         tc_fence_before();
