@@ -214,8 +214,8 @@ BIGBIRD_API int bigbird_last_status_static(void* stream, int* status, int* detai
  * BIGBIRD_OK, or BIGBIRD_ETIMEOUT if a bounded wait inside a kernel gave up (the kernel then returned early and
  * its outputs are invalid).  *detail (may be NULL) receives a code naming the wait.  Clears the word.
  * The word is one per device, shared by every bigbird_attn_fwd launch on it, so a timeout cannot be attributed to
- * one call among several in flight; after a timeout the function also resets the work counters of every launch
- * slot on that device (with a blocking cudaMemset), which is only safe once all attention kernels on the device
+ * one call among several in flight; after a timeout the function also resets the work counters of every stream
+ * on that device (with a blocking cudaMemset), which is only safe once all attention kernels on the device
  * have finished.  A debugging facility: call it with the device otherwise idle.
  */
 BIGBIRD_API int bigbird_last_status(void* stream, int* status, int* detail);

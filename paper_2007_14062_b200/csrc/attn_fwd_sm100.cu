@@ -850,11 +850,12 @@ __global__ void wait_expiry_selftest_kernel(int* status) {
     }
 }
 
-// One 64-bit word per (batch, key block): bit t = key_padding_mask[batch, block*64 + t] != 0; and four words to be cleared, if any.
-__global__ void __launch_bounds__(256) pack_mask_kernel(const uint8_t* __restrict__ kpm, unsigned long long* __restrict__ kbits, int n_words, int* __restrict__ zero4) {
+// One 64-bit word per (batch, key block): bit t = key_padding_mask[batch, block*64 + t] != 0; and n_zero words to be cleared.
+__global__ void __launch_bounds__(256) pack_mask_kernel(const uint8_t* __restrict__ kpm, unsigned long long* __restrict__ kbits, int n_words, int* __restrict__ zero,
+                                                        int n_zero) {
     grid_dependency_release();
     grid_dependency_wait();
-    if (zero4 && blockIdx.x == 0 && threadIdx.x < 4) zero4[threadIdx.x] = 0;
+    if (blockIdx.x == 0 && (int)threadIdx.x < n_zero) zero[threadIdx.x] = 0;
     const int word = (blockIdx.x * 256 + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (word >= n_words) return;
     const uint8_t* src = kpm + (size_t)word * kBlock;
@@ -935,13 +936,30 @@ void set_shape(KernelParams& p, const bigbird_layout& L, int B, Cut cut, float s
 // One CTA per SM, each running kStreams tile streams; every SM gets work before any stream gets its second tile.
 int grid_size(int sm_count, int total_work) { return std::max(1, std::min(sm_count, total_work)); }
 
+// The work counter of the calls on one stream, or null.  Calls on one stream take turns and the last CTA of each leaves the pair at
+// zero, so they can share one that the library keeps; calls on different streams cannot, and neither can a captured call, which
+// runs on whatever stream its graph is launched on: those count in their own workspace, and a kernel has to zero it first.  (A call
+// with a mask always does: the kernel that packs the mask is there anyway.)  No stream gets an id that another one has had.  Under
+// the lock.
+int* stream_counter(DeviceScratch& sc, cudaStream_t stream) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamIsCapturing(stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) return nullptr;
+    if (cudaStreamGetId(stream, &id) != cudaSuccess) return nullptr;
+    int i = 0;
+    while (i < sc.streams && sc.stream_ids[i] != id) ++i;
+    if (i == kCounterSlots) return nullptr;
+    if (i == sc.streams) sc.stream_ids[sc.streams++] = id;
+    return sc.counters + 2 * i;
+}
+
 // The kernels of a call, in the order of the stream, each allowed to begin before the one in front of it has drained: they wait for
 // it (grid_dependency_wait) before they touch memory that it may use.
 cudaError_t enqueue(const KernelParams& p, const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
-                    const uint8_t* kpm, unsigned long long* kbits, int n_words, int* zero4, int sm_count, cudaStream_t stream, int* launches) {
+                    const uint8_t* kpm, unsigned long long* kbits, int n_words, int* zero, int n_zero, int sm_count, cudaStream_t stream, int* launches) {
     cudaError_t e = cudaSuccess;
-    if (n_words) {
-        e = launch_chained(pack_mask_kernel, (unsigned)((n_words * 32 + 255) / 256), 256, 0, stream, kpm, kbits, n_words, zero4);
+    if (n_words || n_zero) {
+        e = launch_chained(pack_mask_kernel, (unsigned)std::max(1, (n_words * 32 + 255) / 256), 256, 0, stream, kpm, kbits, n_words, zero, n_zero);
         if (e != cudaSuccess) return e;
         ++*launches;
     }
@@ -977,13 +995,21 @@ int launch_attn_fwd_sm100(const FwdArgs& a, const bigbird_layout& L, const Devic
         return BIGBIRD_ECUDA;
     }
 
-    // scratch of this call, on the caller's stream: parts of split tiles, packed mask bits
+    // scratch of this call, on the caller's stream: parts of split tiles, packed mask bits, work counter (where the kernel that packs
+    // the mask can zero it)
+    int* counter = nullptr;
+    if (!a.kpm) {
+        std::lock_guard<std::mutex> lock(g_launch_mu);
+        counter = stream_counter(sc, a.stream);
+    }
+    const int own_counter = counter ? 0 : 2;
     const Cut cut = cut_global_tiles(L, a.B, sm_count, 1 << 20);
     const size_t words = a.kpm ? (size_t)a.B * a.nb : 0;
     const size_t off_bits = cut.parts > 1 ? (size_t)a.B * a.H * L.global_tiles * cut.parts * kPartialFloats * sizeof(float) : 0;
     unsigned char* ws = nullptr;
-    if (off_bits + words) {
-        cudaError_t e = cudaMallocFromPoolAsync((void**)&ws, off_bits + words * sizeof(unsigned long long), pool, a.stream);
+    const size_t off_counter = off_bits + words * sizeof(unsigned long long), bytes = off_counter + own_counter * sizeof(int);
+    if (bytes) {
+        cudaError_t e = cudaMallocFromPoolAsync((void**)&ws, bytes, pool, a.stream);
         if (e != cudaSuccess) { *cuda_err = e; return BIGBIRD_ECUDA; }
     }
 
@@ -994,16 +1020,11 @@ int launch_attn_fwd_sm100(const FwdArgs& a, const bigbird_layout& L, const Devic
     p.partials = (float*)ws;
     p.items = dl.items;
     p.steps = dl.steps;
-    unsigned slot;
-    {
-        std::lock_guard<std::mutex> lock(g_launch_mu);
-        slot = sc.next_slot++ % kCounterSlots;
-    }
-    p.counter = sc.counters + 2 * slot;
+    p.counter = counter ? counter : (int*)(ws + off_counter);
     p.status = sc.status;
     set_shape(p, L, a.B, cut, a.scale);
 
-    cudaError_t e = enqueue(p, tm_q, tm_k, tm_v, a.kpm, (unsigned long long*)(ws + off_bits), (int)words, nullptr, sm_count, a.stream, launches);
+    cudaError_t e = enqueue(p, tm_q, tm_k, tm_v, a.kpm, (unsigned long long*)(ws + off_bits), (int)words, p.counter, own_counter, sm_count, a.stream, launches);
     if (ws) {
         const cudaError_t ef = cudaFreeAsync(ws, a.stream);
         if (e == cudaSuccess) e = ef;
@@ -1132,7 +1153,7 @@ extern "C" int bigbird_attn_fwd_static(const void* q, const void* k, const void*
     p.counter = words4 + 2;
     set_shape(p, *L, B, cut, scale);
     int launches = 0;
-    if (enqueue(p, tm_q, tm_k, tm_v, key_padding_mask, kbits_dev, key_padding_mask ? (int)words : 0, words4, sd.sm_count, stream, &launches) != cudaSuccess)
+    if (enqueue(p, tm_q, tm_k, tm_v, key_padding_mask, kbits_dev, key_padding_mask ? (int)words : 0, words4, key_padding_mask ? 4 : 0, sd.sm_count, stream, &launches) != cudaSuccess)
         return BIGBIRD_ECUDA;
     return BIGBIRD_OK;
 }

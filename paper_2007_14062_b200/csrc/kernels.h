@@ -40,12 +40,13 @@ struct BwdArgs {
 };
 
 // Per-device scratch owned by the library.
+constexpr int kCounterSlots = 64;
 struct DeviceScratch {
     int* status = nullptr;          // [2]: code, detail
-    int* counters = nullptr;        // [kCounterSlots * 2] work counters of the dynamic scheduler
-    unsigned next_slot = 0;
+    int* counters = nullptr;        // [kCounterSlots * 2] work counters of the dynamic scheduler, a pair per stream, zero between calls
+    unsigned long long stream_ids[kCounterSlots] = {};     // the streams that own them
+    int streams = 0;
 };
-constexpr int kCounterSlots = 64;
 
 // CUDA-core kernel (fp32 arithmetic).  Returns a cudaError_t.  *launches is incremented per kernel enqueued.
 cudaError_t launch_attn_fwd_simt(const FwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, int sms, int* launches);

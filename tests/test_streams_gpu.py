@@ -1,0 +1,100 @@
+"""The library under several streams: what include/bigbird.h says about overlap."""
+import ctypes
+
+import pytest
+import torch
+
+import paper_2007_14062_b200 as bb
+from paper_2007_14062_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+class Problem:
+    """Inputs of one call on the GPU, and its results on the default stream."""
+
+    def __init__(self, dtype, B, H, nb, seed, lengths=None, mode=0, g=2, r=3):
+        wl = self.wl = synth.Workload("streams", dtype, B, H, nb * 64, 64, 64, 3, g, r, mode, seed=seed)
+        dev = torch.device("cuda:0")
+        gen = torch.Generator(dev).manual_seed(seed)
+        self.q, self.k, self.v, self.dout = (torch.randn((B, H, wl.N, 64), generator=gen, device=dev).to(synth.torch_dtype(dtype)) for _ in range(4))
+        self.mask = None
+        if lengths is not None:
+            self.mask = (torch.arange(wl.N)[None, :] < torch.tensor(lengths)[:, None]).to(torch.uint8).to(dev)
+        self.layout = bb.bigbird_build_layout(wl.N, 64, 3, g, r, seed, H, mode)
+
+    def outputs(self, bwd=False):
+        nan = [torch.full_like(self.q, float("nan")), torch.full(self.q.shape[:3], float("nan"), device=self.q.device)]
+        return nan + [torch.full_like(self.q, float("nan")) for _ in range(3 if bwd else 0)]
+
+    def run(self, o, stream=None, fwd=bb.bigbird_attn_fwd):
+        fwd(self.q, self.k, self.v, self.layout, self.mask, o[0], o[1], self.wl.scale, stream)
+        if len(o) > 2:
+            bb.bigbird_attn_bwd(self.q, self.k, self.v, o[0], o[1], self.dout, self.layout, self.mask, *o[2:], self.wl.scale, stream)
+
+    def expected(self, bwd=False):
+        o = self.outputs(bwd)
+        self.run(o)
+        torch.cuda.synchronize()
+        return o
+
+
+def same(a, b):
+    return all(torch.equal(x, y) for x, y in zip(a, b))
+
+
+# More tiles than the GPU has tile streams, so that a call draws work from its counter.
+BUSY = [dict(dtype="bf16", B=3, H=12, nb=32, seed=5), dict(dtype="bf16", B=3, H=12, nb=32, seed=6, lengths=[2048, 1999, 777])]
+
+
+@pytest.mark.parametrize("kw", BUSY, ids=["full", "padded"])
+def test_many_calls_queued_on_two_streams(kw):
+    """More calls in flight on each of two streams than the library has counters of its own, the second stream's queued behind
+    all of the first's; the same bits as one call at a time."""
+    p = Problem(**kw)
+    want = p.expected()
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    outs = [[p.outputs() for _ in range(80)] for _ in streams]
+    torch.cuda.synchronize()
+    for s, os_ in zip(streams, outs):
+        for o in os_:
+            p.run(o, s.cuda_stream)
+    torch.cuda.synchronize()
+    assert bb.bigbird_last_status() == (0, 0)
+    assert all(same(want, o) for os_ in outs for o in os_)
+
+
+def test_training_steps_queued_on_two_streams():
+    ps = [Problem(**kw) for kw in BUSY]
+    want = [p.expected(bwd=True) for p in ps]
+    streams = [torch.cuda.Stream() for _ in ps]
+    outs = [[p.outputs(bwd=True) for _ in range(20)] for p in ps]
+    torch.cuda.synchronize()
+    for i in range(20):
+        for p, s, os_ in zip(ps, streams, outs):
+            p.run(os_[i], s.cuda_stream)
+    torch.cuda.synchronize()
+    assert bb.bigbird_last_status() == (0, 0)
+    assert all(same(w, o) for w, os_ in zip(want, outs) for o in os_)
+
+
+def test_more_streams_than_the_library_has_counters():
+    p = Problem(**BUSY[0])
+    want = p.expected()
+    rt = torch.cuda.cudart()
+    handles = []
+    for _ in range(70):
+        h = ctypes.c_uint64(0)
+        assert int(rt.cudaStreamCreate(ctypes.addressof(h))) == 0
+        handles.append(h.value)
+    outs = [p.outputs() for _ in handles]
+    torch.cuda.synchronize()
+    for _ in range(2):
+        for h, o in zip(handles, outs):
+            p.run(o, h)
+    torch.cuda.synchronize()
+    for h in handles:
+        assert int(rt.cudaStreamDestroy(h)) == 0
+    assert bb.bigbird_last_status() == (0, 0)
+    assert all(same(want, o) for o in outs)
