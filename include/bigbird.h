@@ -157,7 +157,7 @@ BIGBIRD_API int bigbird_attn_fwd_simt(const void* q, const void* k, const void* 
  * as sums of two bf16 numbers; fp32 accumulation), everything else on CUDA cores in fp32 arithmetic.  The workspace
  * (statistics per query row, packed mask, partial results) is taken in stream order from a memory pool that lives
  * as long as any layout is in use on the device: calls on different streams or threads may overlap.  Only enqueues work.
- * Errors: BIGBIRD_EINVAL, BIGBIRD_EUNSUPPORTED, BIGBIRD_ECUDA.
+ * Errors: BIGBIRD_EINVAL, BIGBIRD_EUNSUPPORTED, BIGBIRD_ECUDA, BIGBIRD_ENOMEM.
  */
 BIGBIRD_API int bigbird_attn_bwd(const void* q, const void* k, const void* v, const void* out, const float* lse, const void* dout,
                      const bigbird_layout* layout, const uint8_t* key_padding_mask, void* dq, void* dk, void* dv,

@@ -2,10 +2,10 @@
 // scratch, kernel dispatch.  See include/bigbird.h for the contract of each function.
 #include <cuda_runtime.h>
 
+#include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
-#include <utility>
-#include <vector>
 
 #include "kernels.h"
 #include "../../include/bigbird.h"
@@ -91,31 +91,32 @@ void free_device_layout(DeviceLayout& d) {
     d = DeviceLayout{};
 }
 
-// Device copy of the layout: one allocation, one copy.
-cudaError_t upload_layout(const bigbird_layout* L, DeviceLayout& d) {
-    std::vector<unsigned char> host;
-    std::vector<std::pair<void**, size_t>> at;               // where each array's device address goes, and its offset
-    auto put = [&](auto** dst, const auto& v) {
-        host.resize((host.size() + 255) / 256 * 256);
-        at.emplace_back((void**)dst, host.size());
-        const unsigned char* src = reinterpret_cast<const unsigned char*>(v.data());
-        host.insert(host.end(), src, src + v.size() * sizeof(v[0]));
+// Device copy of the layout: one allocation, one copy.  (Nothing here throws: the callers are C entry points.)
+int upload_layout(const bigbird_layout* L, DeviceLayout& d) {
+    struct Array {
+        void** dst;            // where its device address goes
+        const void* src;
+        size_t bytes;
     };
-    put(&d.row_ptr, L->row_ptr);
-    put(&d.col_idx, L->col_idx);
-    put(&d.col_ptr, L->col_ptr);
-    put(&d.row_idx, L->row_idx);
-    put(&d.items, L->items_abs);
-    put(&d.steps, L->steps);
-    put(&d.items_t, L->items_t);
-    put(&d.steps_t, L->steps_t);
-    put(&d.global_pairs, L->global_pairs);
-    put(&d.block_order, L->block_order);
-    cudaError_t e = cudaMalloc(&d.block, host.size() + 256);
-    if (e == cudaSuccess) e = cudaMemcpy(d.block, host.data(), host.size(), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return e;
-    for (auto& [dst, off] : at) *dst = (unsigned char*)d.block + off;
-    return cudaSuccess;
+    auto array = [](auto** dst, const auto& v) { return Array{(void**)dst, v.data(), v.size() * sizeof(v[0])}; };
+    const Array arrays[] = {array(&d.row_ptr, L->row_ptr), array(&d.col_idx, L->col_idx), array(&d.col_ptr, L->col_ptr), array(&d.row_idx, L->row_idx),
+                            array(&d.items, L->items_abs), array(&d.steps, L->steps), array(&d.items_t, L->items_t), array(&d.steps_t, L->steps_t),
+                            array(&d.global_pairs, L->global_pairs), array(&d.block_order, L->block_order)};
+    auto align256 = [](size_t x) { return (x + 255) / 256 * 256; };
+    size_t total = 256;
+    for (const Array& a : arrays) total += align256(a.bytes);
+    std::unique_ptr<unsigned char[]> host(new (std::nothrow) unsigned char[total]);
+    if (!host) return BIGBIRD_ENOMEM;
+    cudaError_t e = cudaMalloc(&d.block, total);
+    if (e != cudaSuccess) return cuda_fail(e);
+    size_t at = 0;
+    for (const Array& a : arrays) {
+        if (a.bytes) std::memcpy(host.get() + at, a.src, a.bytes);
+        *a.dst = (unsigned char*)d.block + at;
+        at += align256(a.bytes);
+    }
+    e = cudaMemcpy(d.block, host.get(), at, cudaMemcpyHostToDevice);
+    return e == cudaSuccess ? BIGBIRD_OK : cuda_fail(e);
 }
 
 // Device copy of the layout on the current device (made on first use, remade if the device changes).
@@ -129,9 +130,9 @@ int get_device_layout(const bigbird_layout* L, int device, DeviceLayout* out) {
             free_device_layout(d);
             cudaSetDevice(cur);
         }
-        cudaError_t e = upload_layout(L, d);
-        if (e != cudaSuccess) { free_device_layout(d); return cuda_fail(e); }
-        const int rc = hold_pool(device);
+        int rc = upload_layout(L, d);
+        if (rc != BIGBIRD_OK) { free_device_layout(d); return rc; }
+        rc = hold_pool(device);
         if (rc != BIGBIRD_OK) { free_device_layout(d); return rc; }
         d.device = device;
     }

@@ -1,5 +1,10 @@
-"""The library under several streams: what include/bigbird.h says about overlap."""
+"""The library under several streams and with a host that is out of memory: what include/bigbird.h says
+about overlap and error codes."""
 import ctypes
+import os
+import subprocess
+import sys
+import textwrap
 
 import pytest
 import torch
@@ -8,6 +13,7 @@ import paper_2007_14062_b200 as bb
 from paper_2007_14062_b200 import synth
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 class Problem:
@@ -98,3 +104,54 @@ def test_more_streams_than_the_library_has_counters():
         assert int(rt.cudaStreamDestroy(h)) == 0
     assert bb.bigbird_last_status() == (0, 0)
     assert all(same(want, o) for o in outs)
+
+
+def test_running_out_of_host_memory_is_an_error_code(tmp_path):
+    """A call that cannot get the host memory for the device copy of its layout returns BIGBIRD_ENOMEM: nothing is thrown
+    through the C entry point, and the next call is fine."""
+    src = tmp_path / "no_memory.cpp"
+    src.write_text(textwrap.dedent("""
+        #include <cstdlib>
+        #include <new>
+        static thread_local bool armed = false;
+        extern "C" void arm(int on) { armed = on != 0; }
+        void* operator new(std::size_t n) {
+            void* p = armed && n >= 65536 ? nullptr : std::malloc(n ? n : 1);
+            if (!p) throw std::bad_alloc();
+            return p;
+        }
+        void* operator new[](std::size_t n) { return operator new(n); }
+        void* operator new(std::size_t n, const std::nothrow_t&) noexcept { return armed && n >= 65536 ? nullptr : std::malloc(n ? n : 1); }
+        void* operator new[](std::size_t n, const std::nothrow_t& t) noexcept { return operator new(n, t); }
+        void operator delete(void* p) noexcept { std::free(p); }
+        void operator delete[](void* p) noexcept { std::free(p); }
+        void operator delete(void* p, std::size_t) noexcept { std::free(p); }
+        void operator delete[](void* p, std::size_t) noexcept { std::free(p); }
+    """))
+    so = tmp_path / "no_memory.so"
+    subprocess.run(["g++", "-O1", "-shared", "-fPIC", "-o", str(so), str(src)], check=True)
+    code = textwrap.dedent(f"""
+        import ctypes, torch
+        import paper_2007_14062_b200 as bb
+        arm = ctypes.CDLL({str(so)!r}).arm
+        q = torch.randn(1, 12, 4096, 64, device="cuda", dtype=torch.bfloat16)
+        out = torch.empty_like(q)
+        L = bb.bigbird_build_layout(4096, 64, 3, 2, 3, 0, 12)
+        L2 = bb.bigbird_build_layout(4096, 64, 3, 2, 3, 0, 12)
+        bb.bigbird_attn_fwd(q, q, q, L, None, out, None, 0.125)
+        torch.cuda.synchronize()
+        arm(1)
+        try:
+            bb.bigbird_attn_fwd(q, q, q, L2, None, torch.empty_like(q), None, 0.125)
+            code = 0
+        except bb.BigBirdError as e:
+            code = e.code
+        arm(0)
+        assert code in (0, -5), code
+        again = torch.empty_like(q)
+        bb.bigbird_attn_fwd(q, q, q, L2, None, again, None, 0.125)
+        assert torch.equal(out, again)
+        print("fine", code)
+    """)
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, LD_PRELOAD=str(so)), capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "fine -5" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
