@@ -35,6 +35,7 @@ int get_scratch(int device, DeviceScratch** out) {
         cudaError_t e = cudaMalloc(&p, sizeof(int) * (2 + 2 * kCounterSlots));
         if (e != cudaSuccess) return cuda_fail(e);
         e = cudaMemset(p, 0, sizeof(int) * (2 + 2 * kCounterSlots));
+        if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);        // see upload_layout
         if (e != cudaSuccess) { cudaFree(p); return cuda_fail(e); }
         s.status = p;
         s.counters = p + 2;
@@ -115,7 +116,10 @@ int upload_layout(const bigbird_layout* L, DeviceLayout& d) {
         *a.dst = (unsigned char*)d.block + at;
         at += align256(a.bytes);
     }
-    e = cudaMemcpy(d.block, host.get(), at, cudaMemcpyHostToDevice);
+    // Waited for: a copy's call may return while it is on its way from the driver's staging memory, and a stream that does not
+    // synchronise with the legacy one (torch's streams do not) would not wait for it.
+    e = cudaMemcpyAsync(d.block, host.get(), at, cudaMemcpyHostToDevice, cudaStreamLegacy);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
     return e == cudaSuccess ? BIGBIRD_OK : cuda_fail(e);
 }
 

@@ -106,6 +106,19 @@ def test_more_streams_than_the_library_has_counters():
     assert all(same(want, o) for o in outs)
 
 
+def test_first_calls_of_layouts_on_a_side_stream():
+    """The device copy of a layout is complete before any stream can reach it."""
+    side = torch.cuda.Stream()
+    for seed in range(30):
+        p = Problem("bf16", 1, 2, 40, seed=100 + seed)
+        o = p.outputs()
+        torch.cuda.synchronize()
+        p.run(o, side.cuda_stream)
+        torch.cuda.synchronize()
+        assert same(o, p.expected())
+        p.layout.close()
+
+
 def test_running_out_of_host_memory_is_an_error_code(tmp_path):
     """A call that cannot get the host memory for the device copy of its layout returns BIGBIRD_ENOMEM: nothing is thrown
     through the C entry point, and the next call is fine."""
