@@ -24,6 +24,17 @@ struct FwdShape {
     }
 };
 
+// V of padded keys becomes zero: a chunk may hold the end of one block and the beginning of another that is all padding, uninitialised
+// perhaps, and 0 * NaN is not 0.  Rare, and not inline: it shares no registers with the loop then.  ([2, 8, 2560, 128] padded 305.8 us
+// without it, 307.5 like this, 313.5 inline.)
+template <int D, int KC>
+__device__ __noinline__ void zero_padded(float* sv, const uint8_t* svalid) {
+#pragma unroll 1
+    for (int r = threadIdx.x >> 5; r < KC; r += blockDim.x >> 5)
+        if (!svalid[r])
+            for (int c = threadIdx.x & 31; c < D / 4; c += 32) *reinterpret_cast<float4*>(sv + r * D + 4 * c) = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
 // dynamic shared memory: Q [rows][LD] | K [KC][LD] | P [rows][LDP] (in K's place for D = 128) | V [KC][D]
 template <typename T, int D, int TM>
 __global__ void __launch_bounds__(256, 2)
@@ -83,9 +94,11 @@ attn_fwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* 
         if (threadIdx.x < KC) svalid[threadIdx.x] = (uint8_t)(vf & 1u);
         if (blockDim.x < KC) svalid[32 + threadIdx.x] = (uint8_t)(vf >> 1);
         copy_wait();
-        const bool any = __syncthreads_or(vf != 0u);
+        const int with_keys = __syncthreads_count(vf != 0u);       // threads, of those that look, that have seen a key
+        const bool any = with_keys != 0;
         if (i0 + KC < w.last) vf = chunk_valid(i0 + KC);
         if (any) {
+            if (mask && with_keys < KC) zero_padded<D, KC>(sv, svalid);       // (every thread of a one-warp CTA looks at two keys: always)
             float s[TM][TN];
             dot_tile<TM, TN, D>(s, qrow, LD, sk + tx * LD, LD);
             bool valid[TN];

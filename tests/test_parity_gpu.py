@@ -232,6 +232,22 @@ def test_bounded_wait_expires_with_a_status_and_the_context_stays_usable():
     _compare(wl, q, k, v, None, out, lse, slices=None)
 
 
+@pytest.mark.parametrize("b,nb,D,valid", [(84, 9, 64, 420), (16, 20, 64, 176), (24, 12, 128, 168)])
+def test_contents_of_padded_key_blocks_do_not_matter_on_the_cuda_core_path(b, nb, D, valid):
+    """The kernel walks 64 keys at a time whatever the block size, so that a chunk may hold the end of the last block with tokens
+    and the beginning of one without: uninitialised memory there (NaN) must not reach the rows that attend the former."""
+    wl = synth.Workload(f"padblocks_{b}", "fp32", 1, 2, nb * b, D, b, 3, 2, 2, 1, seed=19)
+    q, k, v = synth.make_qkv(wl)
+    kpm = torch.ones((1, wl.N), dtype=torch.uint8)
+    kpm[:, valid:] = 0
+    clean = _run(wl, q, k, v, kpm)
+    _compare(wl, q, k, v, kpm, *clean, slices=None)
+    for t in (q, k, v):
+        t[:, :, valid:] = float("nan")
+    dirty = _run(wl, q, k, v, kpm)
+    assert np.array_equal(clean[0], dirty[0]) and np.array_equal(clean[1], dirty[1])
+
+
 # ------------------------------------------------------------------------------------------------ full-size workloads
 def _sample_slices(wl, n, seed=0):
     rng = np.random.default_rng(seed)
