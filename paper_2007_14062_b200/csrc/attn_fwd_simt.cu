@@ -114,9 +114,10 @@ attn_fwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* 
                     s[i][j] = valid[j] ? s[i][j] * scale : -CUDART_INF_F;
                     mx = fmaxf(mx, s[i][j]);
                 }
-                mx = fmaxf(m[i], row_max16(mx));   // finite: the chunk has a valid key
-                const float alpha = expf(m[i] - mx);        // 0 on the first one
-                m[i] = mx;
+                const float m_old = m[i];
+                m[i] = mx = fmaxf(m_old, row_max16(mx));
+                if (mx == -CUDART_INF_F) mx = 0.f;          // nothing so far but scores that overflowed to -inf: probabilities of zero
+                const float alpha = expf(m_old - mx);       // 0 on the first chunk
                 l[i] *= alpha;
 #pragma unroll
                 for (int c = 0; c < C::N; ++c) mul2(o[i][c], pair(alpha, alpha));

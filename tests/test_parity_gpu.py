@@ -248,6 +248,23 @@ def test_contents_of_padded_key_blocks_do_not_matter_on_the_cuda_core_path(b, nb
     assert np.array_equal(clean[0], dirty[0]) and np.array_equal(clean[1], dirty[1])
 
 
+def test_scores_of_minus_infinity_on_the_cuda_core_path():
+    """Products that overflow fp32 to -inf have probability zero, also where a row's first keys are all of them; a row that has
+    nothing else comes out as one without keys."""
+    wl = _small("fp32", 12, 2, 8)                                 # (enough tiles that each has a CTA of its own)
+    shape = (wl.B, 2, wl.N, 64)
+    q, v = torch.full(shape, 1e30), torch.ones(shape)
+    k = torch.full(shape, 1e-30)
+    k[:, :, :64] = -1e30                                          # the first global block: first in every row's list
+    out, lse = _run(wl, q, k, v, None)
+    rows = _graph(wl)
+    cnt = np.stack([O.build_mask(rows, h)[:, 64:].sum(axis=1) for h in range(wl.H)])
+    assert np.abs(out - 1).max() <= 4e-6                          # (as in the closed forms above)
+    assert np.abs(lse - (np.log(cnt) + 8)).max() <= 1e-4          # every other score is 64 * 1e30 * 1e-30 / sqrt(64) = 8
+    out, lse = _run(wl, q, torch.full(shape, -1e30), v, None)
+    assert (out == 0).all() and np.isneginf(lse).all()
+
+
 # ------------------------------------------------------------------------------------------------ full-size workloads
 def _sample_slices(wl, n, seed=0):
     rng = np.random.default_rng(seed)
