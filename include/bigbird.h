@@ -188,7 +188,9 @@ BIGBIRD_API int bigbird_attn_bwd(const void* q, const void* k, const void* v, co
  *     layout enqueue only the kernels (and a 16-byte cudaMemsetAsync if there is no mask).  `layout` must not be destroyed while a
  *     call that uses it is being enqueued;
  *   - the first call on a device looks up the array's device address and sets a kernel attribute; make that
- *     first call outside any stream capture;
+ *     first call outside any stream capture.  A call that is captured sends the schedule whenever its graph runs if the array
+ *     held another one at the time of the capture (`layout` must then live as long as the graph, and every later call on the
+ *     device sends its own); if the array held it already, the graph does not send it, and may only run while the array does;
  *   - all calls on a device share the array, which keeps the contents of the last call: the entry point
  *     re-initialises what must start at zero, but two calls whose kernels overlap on the GPU (different
  *     streams, or different threads) race on it and give undefined results.  Serialise them;

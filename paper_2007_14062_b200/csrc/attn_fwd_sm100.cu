@@ -1059,6 +1059,7 @@ struct StaticDevice {
     unsigned char* base = nullptr;              // device address of g_static_scratch on this device
     int sm_count = 0;
     uint64_t schedule_uid = 0;                  // layout whose schedule the array holds (0: none)
+    bool graphs_send = false;                   // a captured call sends a schedule: the array may hold that one at any time from then on
 };
 std::mutex g_static_mu;
 StaticDevice g_static_dev[64];
@@ -1082,11 +1083,11 @@ cudaError_t static_setup(int device, StaticDevice* out) {
     return cudaSuccess;
 }
 
-void static_remember_schedule(int device, uint64_t uid) {
+void static_remember_schedule(int device, uint64_t uid, bool captured = false) {
     std::lock_guard<std::mutex> lock(g_static_mu);
     g_static_dev[device].schedule_uid = uid;
+    if (captured) g_static_dev[device].graphs_send = true;
 }
-void static_forget_schedule(int device) { static_remember_schedule(device, 0); }
 
 }  // namespace
 }  // namespace bigbird
@@ -1131,12 +1132,16 @@ extern "C" int bigbird_attn_fwd_static(const void* q, const void* k, const void*
         if (e != cudaSuccess) return BIGBIRD_ECUDA;
     }
     // The schedule is sent only when the array does not hold this layout's already (copies from the handle's own
-    // host arrays, which live as long as the handle).
-    if (sd.schedule_uid != L->uid) {
-        e = cudaMemcpyAsync(items_dev, L->items_abs.data(), n_items * sizeof(Item), cudaMemcpyHostToDevice, stream);
+    // host arrays, which live as long as the handle).  Copies that are captured have not been made, and are made whenever the
+    // graph runs.
+    if (sd.schedule_uid != L->uid || sd.graphs_send) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        e = cudaStreamIsCapturing(stream, &capture);
+        const bool captured = capture != cudaStreamCaptureStatusNone;
+        if (e == cudaSuccess) e = cudaMemcpyAsync(items_dev, L->items_abs.data(), n_items * sizeof(Item), cudaMemcpyHostToDevice, stream);
         if (e == cudaSuccess && n_steps) e = cudaMemcpyAsync(steps_dev, L->steps.data(), n_steps * sizeof(Step), cudaMemcpyHostToDevice, stream);
-        if (e != cudaSuccess) { static_forget_schedule(device); return BIGBIRD_ECUDA; }
-        static_remember_schedule(device, L->uid);
+        static_remember_schedule(device, e == cudaSuccess && !captured ? L->uid : 0, captured);
+        if (e != cudaSuccess) return BIGBIRD_ECUDA;
     }
 
     const size_t tiles = (size_t)B * H * L->global_tiles;

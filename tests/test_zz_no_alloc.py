@@ -119,6 +119,43 @@ def test_static_entry_point_reuses_the_uploaded_schedule():
     L.close()
 
 
+def test_static_entry_point_does_not_take_a_captured_schedule_for_a_sent_one():
+    """Capturing a call with a layout whose schedule the array does not hold sends nothing: calls outside the graph with that
+    layout, before the graph has run and after, and with another one between its runs, all send their own."""
+    dev = torch.device("cuda:0")
+    cases = []
+    for seed, nb, H in ((17, 12, 2), (18, 20, 3)):
+        wl = synth.Workload("noalloc_g", "bf16", 2, H, nb * 64, 64, 64, 3, 2, 3, 0, seed=seed)
+        q, k, v = (t.to(dev) for t in synth.make_qkv(wl))
+        L = bb.bigbird_build_layout(wl.N, wl.b, wl.w, wl.g, wl.r, wl.seed, wl.H, wl.mode)
+        want, out = torch.empty_like(q), torch.empty_like(q)
+        bb.bigbird_attn_fwd(q, k, v, L, None, want, None, wl.scale)
+        cases.append((q, k, v, L, out, want, wl.scale))
+
+    def call(case):
+        q, k, v, L, out, _, scale = case
+        bb.bigbird_attn_fwd_static(q, k, v, L, None, out, None, scale)
+
+    def check(case, run=call):
+        case[4].fill_(float("nan"))
+        run(case)
+        torch.cuda.synchronize()
+        assert torch.equal(case[4], case[5])
+
+    first, second = cases
+    check(first)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call(second)
+    replay = lambda case: graph.replay()
+    for case, run in ((second, call), (first, call), (second, replay), (second, call), (first, call), (second, replay), (first, call)):
+        check(case, run)
+    assert bb.bigbird_last_status_static() == (0, 0)
+    del graph
+    for case in cases:
+        case[3].close()
+
+
 def test_static_entry_point_refuses_what_does_not_fit():
     # 131072 schedule steps is the limit of the fixed array; this layout needs more.  Nothing is launched.
     L = bb.bigbird_build_layout(1024 * 64, 64, 3, 2, 3, 0, 20, 0)
