@@ -122,9 +122,12 @@ BIGBIRD_API int bigbird_layout_destroy(bigbird_layout* layout);
  *   stream    cudaStream_t (NULL = default stream).  The call only enqueues work; it never synchronises.
  *
  * Supported: D == 64 and b == 64 for BIGBIRD_BF16; D in {32, 64, 128} and any b for BIGBIRD_FP32.
- * The first call on a device and the first call with a new layout allocate device memory owned by the library.  Scratch of
- * a call (packed mask bits, partial results of split global tiles) is taken in stream order from a memory pool that lives as
- * long as any layout is in use on the device: calls on different streams or threads may overlap.
+ * The first call on a device and the first call with a new layout allocate device memory owned by the library: make them
+ * outside any stream capture.  Scratch of a call (packed mask bits, partial results of split global tiles) is taken in stream
+ * order from a memory pool that lives as long as any layout is in use on the device: calls on different streams or threads may
+ * overlap.  A captured call puts an allocation node and a free node around its kernels, so that its scratch belongs to the
+ * graph; the graph may run beside calls outside it, and is subject to CUDA's limits for graphs with such nodes (one
+ * executable of it at a time, no child graph).  The layout must live as long as the graph.
  * Errors: BIGBIRD_EINVAL, BIGBIRD_EUNSUPPORTED, BIGBIRD_ECUDA, BIGBIRD_ENOMEM.  There is no CPU path.
  */
 BIGBIRD_API int bigbird_attn_fwd(const void* q, const void* k, const void* v, const bigbird_layout* layout,
@@ -156,7 +159,8 @@ BIGBIRD_API int bigbird_attn_fwd_simt(const void* q, const void* k, const void* 
  * D in {32, 64, 128}, any b.  BIGBIRD_BF16 with D == b == 64 runs on tensor cores (bf16 operands; P and dS enter the products
  * as sums of two bf16 numbers; fp32 accumulation), everything else on CUDA cores in fp32 arithmetic.  The workspace
  * (statistics per query row, packed mask, partial results) is taken in stream order from a memory pool that lives
- * as long as any layout is in use on the device: calls on different streams or threads may overlap.  Only enqueues work.
+ * as long as any layout is in use on the device: calls on different streams or threads may overlap, and a captured call
+ * behaves as one of bigbird_attn_fwd does.  Only enqueues work.
  * Errors: BIGBIRD_EINVAL, BIGBIRD_EUNSUPPORTED, BIGBIRD_ECUDA, BIGBIRD_ENOMEM.
  */
 BIGBIRD_API int bigbird_attn_bwd(const void* q, const void* k, const void* v, const void* out, const float* lse, const void* dout,

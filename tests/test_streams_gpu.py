@@ -1,5 +1,5 @@
-"""The library under several streams and with a host that is out of memory: what include/bigbird.h says
-about overlap and error codes."""
+"""The library under several streams, in CUDA graphs and with a host that is out of memory: what include/bigbird.h says
+about overlap, capture and error codes."""
 import ctypes
 import os
 import subprocess
@@ -104,6 +104,43 @@ def test_more_streams_than_the_library_has_counters():
         assert int(rt.cudaStreamDestroy(h)) == 0
     assert bb.bigbird_last_status() == (0, 0)
     assert all(same(want, o) for o in outs)
+
+
+# Calls with and without a mask, with and without scratch for the parts of global tiles; the gradients of each; CUDA cores.
+CAPTURED = [dict(dtype="bf16", B=3, H=12, nb=32, seed=5), dict(dtype="bf16", B=2, H=2, nb=12, seed=8, lengths=[768, 197]),
+            dict(dtype="bf16", B=1, H=2, nb=100, seed=9, lengths=[4000]), dict(dtype="bf16", B=1, H=4, nb=64, seed=10),
+            dict(dtype="fp32", B=1, H=2, nb=10, seed=11, lengths=[600])]
+
+
+@pytest.mark.parametrize("kw", CAPTURED, ids=lambda kw: f"{kw['dtype']}_{kw['B']}_{kw['H']}_{kw['nb']}")
+def test_captured_forward_and_backward_replay_on_new_inputs(kw):
+    """A training step in a CUDA graph, replayed on other inputs while the same layout is used outside the graph."""
+    p = Problem(**kw)
+    other = Problem(**dict(kw, seed=kw["seed"] + 50))
+    p.expected(bwd=True)                                          # the layout goes to the device outside capture
+    o = p.outputs(bwd=True)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        p.run(o)
+    side = torch.cuda.Stream()
+    for data in (p, other, p):
+        q = [t.clone() for t in (p.q, p.k, p.v, p.dout)]
+        for dst, src in zip((p.q, p.k, p.v, p.dout), (data.q, data.k, data.v, data.dout)):
+            dst.copy_(src)
+        want = p.expected(bwd=True)
+        for t in o:
+            t.fill_(float("nan"))
+        torch.cuda.synchronize()
+        eager = p.outputs(bwd=True)
+        torch.cuda.synchronize()
+        graph.replay()
+        p.run(eager, side.cuda_stream)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert same(want, o) and same(want, eager)
+        for dst, src in zip((p.q, p.k, p.v, p.dout), q):
+            dst.copy_(src)
+    assert bb.bigbird_last_status() == (0, 0)
 
 
 def test_first_calls_of_layouts_on_a_side_stream():
