@@ -1,4 +1,4 @@
-"""Parity of bigbird_attn_bwd (CUDA-core gradient kernels) with the fp64 oracle's gradients, through the C-ABI.
+"""Parity of bigbird_attn_bwd (tensor-core and CUDA-core gradient kernels) with the fp64 oracle's gradients, through the C-ABI.
 
 Tolerances (max-abs): 1e-4 for fp32 tensors (fp32 arithmetic, sums over up to a few hundred rows); 3e-2 for bf16 tensors
 (the gradients are rounded to bf16 on output; |dq|, |dk|, |dv| reach a few units)."""
@@ -31,7 +31,7 @@ CASES = [
 
 
 @pytest.mark.parametrize("wl", CASES, ids=lambda w: f"{w.name}_{w.lengths}_{w.mode}_{w.b}")
-def test_gradients_match_the_oracle(wl):
+def test_gradients_match_the_oracle(wl, forward=bb.bigbird_attn_fwd_simt):
     dev = torch.device("cuda:0")
     q, k, v = synth.make_qkv(wl)
     gen = torch.Generator().manual_seed(wl.seed + 100)
@@ -45,7 +45,7 @@ def test_gradients_match_the_oracle(wl):
     md = None if kpm is None else kpm.to(dev)
     out = torch.empty_like(qd)
     lse = torch.empty(q.shape[:3], device=dev, dtype=torch.float32)
-    bb.bigbird_attn_fwd_simt(qd, kd, vd, L, md, out, lse, wl.scale)
+    forward(qd, kd, vd, L, md, out, lse, wl.scale)
     dq, dk, dv = (torch.full_like(qd, float("nan")) for _ in range(3))
     bb.bigbird_attn_bwd(qd, kd, vd, out, lse, dod, L, md, dq, dk, dv, wl.scale)
     torch.cuda.synchronize()
@@ -96,6 +96,41 @@ EDGES = [
 @pytest.mark.parametrize("wl", EDGES, ids=lambda w: f"{w.name}_{w.lengths}_{w.B}_{w.g}{w.r}{w.w}")
 def test_tensor_core_gradients_at_the_edges_of_the_schedule(wl):
     test_gradients_match_the_oracle(wl)
+
+
+@pytest.mark.parametrize("wl", [w for w in CASES if w.dtype == "bf16"] + EDGES, ids=lambda w: f"{w.name}_{w.lengths}_{w.B}_{w.g}{w.r}{w.w}")
+def test_tensor_core_forward_and_backward_in_a_row(wl):
+    """What a training step does: the gradients of the tensor-core forward pass, queued behind it.  (Its out and lse are as close to
+    the oracle's as those of the CUDA-core pass above, so the same tolerance holds.)"""
+    test_gradients_match_the_oracle(wl, bb.bigbird_attn_fwd)
+
+
+@pytest.mark.parametrize("wl", [_case("bf16", 1, 2, 24), _case("bf16", 1, 1, 40, g=3, r=2), _case("bf16", 1, 2, 14, mode=1, r=0)],
+                         ids=lambda w: f"{w.name}_{w.mode}")
+def test_tensor_core_gradients_keep_sixteen_bits_of_p_and_ds(wl):
+    """Against the header's formulas in fp64 from the same bf16 inputs, out and lse.  P and dS enter the products as two bf16
+    numbers, 2^-17 of the value off at most, so that nearly all results round to the same bf16 number as the formulas': the formulas
+    themselves with P and dS cut to two numbers miss it for 0.25 % of them, 1.2e-4 of the norm, and the kernel 1.3e-4.  Four times
+    that is allowed; with one number each it is 42 % and 2.6e-3."""
+    dev = torch.device("cuda:0")
+    q, k, v = (t.to(dev) for t in synth.make_qkv(wl))
+    dout = torch.randn(q.shape, generator=torch.Generator(dev).manual_seed(5), device=dev).to(torch.bfloat16)
+    L = bb.bigbird_build_layout(wl.N, wl.b, wl.w, wl.g, wl.r, wl.seed, wl.H, wl.mode)
+    out, grads = torch.empty_like(q), [torch.empty_like(q) for _ in range(3)]
+    lse = torch.empty(q.shape[:3], device=dev, dtype=torch.float32)
+    bb.bigbird_attn_fwd(q, k, v, L, None, out, lse, wl.scale)
+    bb.bigbird_attn_bwd(q, k, v, out, lse, dout, L, None, *grads, wl.scale)
+    gr = O.Graph(wl.N, wl.b, wl.w, wl.g, wl.r, wl.seed, wl.H, wl.mode)
+    A = torch.from_numpy(np.stack([O.build_mask(gr, h) for h in range(wl.H)])).to(dev)
+    q, k, v, out, dout, lse = (t.double() for t in (q, k, v, out, dout, lse))
+    P = torch.exp(wl.scale * q @ k.mT - lse[..., None]) * A
+    dS = P * (dout @ v.mT - (dout * out).sum(-1, keepdim=True))
+    for got, want in zip(grads, (wl.scale * dS @ k, wl.scale * dS.mT @ q, P.mT @ dout)):
+        rounded = want.to(torch.bfloat16).double()
+        off = ((got.double() - rounded).norm() / want.norm()).item()
+        assert off <= 5e-4
+        assert ((got.double() - want).norm() / want.norm()).item() <= 2e-3     # bf16's rounding itself is 1.7e-3
+    L.close()
 
 
 # Tile shapes of the CUDA-core gradient kernels: see the forward kernel's in test_parity_gpu.py.  Tolerances as above.
