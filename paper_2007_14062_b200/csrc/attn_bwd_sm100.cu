@@ -265,6 +265,7 @@ __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ct
                 unsigned long long* bar = &ctl->x_full[xs];
                 const CUtensorMap *xm1 = dkv ? tm_k : tm_q, *xm2 = dkv ? tm_v : tm_do;
                 const int blocks = rb >= 0 ? 2 : 1;
+                if (!BB_CHECK(bh >= 0 && bh < p.BH && ra >= 0 && ra < p.nb && rb < p.nb && rb >= kNoBlock, 172)) return;
                 mbar_expect_tx(bar, blocks * (2 * kTileBytes + (dkv ? 0 : kStatFloats * 4)));
                 for (int j = 0; j < blocks; ++j) {
                     const int row = bh * p.nb + (j ? rb : ra);
@@ -279,6 +280,7 @@ __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ct
             info |= (((tile_n - 1) & 1u) ? kInfoX : 0) | ((((tile_n - 1) >> 1) & 1u) ? kInfoXPar : 0);
             const unsigned g = step_n % kStages;
             const int row = bh * p.nb + slot->steps[i].c;
+            if (!BB_CHECK(n <= kSegSteps && slot->steps[i].c >= 0 && slot->steps[i].c < p.nb, 173)) return;
             if (!mbar_wait(&ctl->empty[g], ((step_n / kStages) & 1u) ^ 1u, abort_flag)) { fail = 110; break; }
             unsigned char* y = smem + kSmemRing + g * 2 * kTileBytes;
             ctl->info[g] = info;
@@ -588,6 +590,8 @@ __device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ct
         if (flags & kSegLast) {
             const bool dkv = slot->kind == kDkv;
             const int split = slot->split, n_chunks = dkv ? 8 : 4;     // of 16 columns
+            if (!BB_CHECK(slot->bh >= 0 && slot->bh < p.BH && slot->ra >= 0 && slot->ra < p.nb && slot->rb < p.nb &&
+                          split < 2 * p.BH * p.global_tiles && slot->part >= 0 && slot->part < p.parts, 174)) break;
             const bool row_ok = ((lower ? slot->rbits_b : slot->rbits_a) >> r64) & 1ull;
             if (row == 0) bulk_wait_read();         // the previous tile has left the staging tiles
             if (!epilogue_sync(ctl, sync_n)) { fail = 142; break; }
