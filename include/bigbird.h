@@ -93,9 +93,9 @@ BIGBIRD_API int bigbird_layout_export_transposed(const bigbird_layout* layout, i
  * The tensor-core kernel stacks two query blocks into one 2b-row tile (upper half, lower half) and walks a
  * list of steps; a step is one key block together with the halves of the tile that attend it.
  *   sizes   host int32[4]: items per head, leading "heavy" (global-tile) items per head, total steps, heads
- *   items   host int32[H * items_per_head * 8] or NULL: per item (qa, qb, step_begin, step_count, part, nparts, tile, 0),
+ *   items   host int32[H * items_per_head * 8] or NULL: per item (qa, qb, step_begin, step_count, -1, 1, tile, 0),
  *           qa / qb the query blocks of the upper / lower half (qb == -1: none), step_begin relative to the
- *           head's first step
+ *           head's first step, tile counting a head's global tiles, which are whole here: launches may cut them
  *   step_base host int32[H] or NULL: first step of each head
  *   steps   host int32[total_steps * 2] or NULL: (key block, who) with who = 0 both halves, 1 upper half only,
  *           2 lower half only
@@ -183,9 +183,9 @@ BIGBIRD_API int bigbird_attn_bwd(const void* q, const void* k, const void* v, co
  * Arguments, layouts, results and asynchrony are those of bigbird_attn_fwd, with these differences:
  *   - BIGBIRD_BF16 with D == 64 and b == 64 only (the tensor-core kernel); anything else is BIGBIRD_EUNSUPPORTED;
  *   - limits set by the fixed array: B * N/b <= 16384, H * (tiles per head) <= 8192 and at most 131072 schedule
- *     steps summed over heads (bigbird_layout_schedule reports both), and N/b <= 96 (longer sequences have
- *     their global tiles split into parts whose partial results need scratch that grows with B * H); beyond
- *     them the call does nothing and returns BIGBIRD_ELIMIT;
+ *     steps summed over heads (bigbird_layout_schedule reports both), and N/b <= 96 (the tiles of global
+ *     blocks of longer sequences want to be cut into more parts than the array has room for, and outlast everything
+ *     else where they are not); beyond them the call does nothing and returns BIGBIRD_ELIMIT;
  *   - the array holds the device copy of one layout's schedule.  A call with another layout than the previous
  *     call on that device first copies the new schedule from the handle's host arrays (two cudaMemcpyAsync on
  *     `stream` from pageable memory: the host may wait until they have been staged); later calls with the same

@@ -830,9 +830,10 @@ int launch_attn_bwd_sm100(const BwdArgs& a, const bigbird_layout& L, const Devic
         return fail(cudaErrorInvalidValue);
 
     // Tiles of global blocks have nb steps where the others have about ten: cut them into parts of about a third of what each
-    // SM gets altogether, so that none of them is still running when the rest is done, of 16 steps or more, and not at all up
-    // to 32 steps: adding the parts up takes about 5 us on the path of the last one (it was 24 when a thread fetched one value
-    // after the other).  Measured, gradients of B, 12 heads, nb blocks in us: [2, nb 16] 39.5 uncut, 43.7 in two, 52 in four;
+    // SM gets altogether, so that none of them is still running when the rest is done, but no more than one for every 16 steps
+    // (rounded up: parts of 11 steps or more), and not at all up to 32 steps: adding the parts up takes about 5 us on the path of
+    // the last one (it was 24 when a thread fetched one value after the other), and at 32 steps that is more than a cut gains with
+    // few heads, less with many.  Measured, gradients of B, 12 heads, nb blocks in us: [2, nb 16] 39.5 uncut, 43.7 in two, 52 in four;
     // [1, 32] 56.9 uncut, 54.6 in two; four heads [1, 32] 34.6, 38.2; [1, 64] 93.7 uncut, 79.7 in two, 74.6 in three, 75.2 in
     // four, 78.5 in eight; [1, 256] 200 uncut, 190 in two, 191 in three; [3, 16 heads, 96] 212 uncut, 221 in two.
     const int64_t steps = (int64_t)a.B * ((int64_t)L.steps.size() + (int64_t)L.steps_t.size() + (int64_t)a.H * L.global_tiles * a.nb);
@@ -861,7 +862,7 @@ int launch_attn_bwd_sm100(const BwdArgs& a, const bigbird_layout& L, const Devic
     p.arrived = p.counter + 1;
     p.partials = (float*)(ws + off_part);
     p.status = status;
-    p.items_q = dl.items + L.heavy_items_per_head;
+    p.items_q = dl.items + L.global_tiles;
     p.q_stride = L.items_per_head;
     p.items_k = dl.items_t;
     p.steps_q = dl.steps;

@@ -132,8 +132,7 @@ struct KernelParams {
     const Step* steps;
     int* counter;                      // [2]: next work index, finished CTAs
     int* status;                       // [2]: code, detail
-    int items_per_head, heavy_per_head, layout_parts;   // of the layout's schedule, whose global tiles may be cut otherwise
-    int global_tiles;                  // per head
+    int items_per_head, global_tiles;  // of the layout's schedule, the global tiles first
     int parts, part_steps;             // how this launch cuts them (part_steps: key blocks)
     int BH, H, nb;
     int total_work;
@@ -215,16 +214,16 @@ __device__ __forceinline__ int schedule_one(const KernelParams& p, SmemCtl* ctl,
     if (w >= 0) {
         const unsigned heavy_total = (unsigned)(p.BH * p.global_tiles * p.parts);
         heavy = (unsigned)w < heavy_total;
-        const unsigned per_head = heavy ? p.global_tiles * p.parts : p.items_per_head - p.heavy_per_head;
+        const unsigned per_head = heavy ? p.global_tiles * p.parts : p.items_per_head - p.global_tiles;
         const unsigned x = heavy ? w : w - heavy_total;
         bh = (int)(x / per_head);                   // (one division for either kind of item: this code is kept small)
         int it = (int)(x - bh * per_head), part = 0;
         batch = (int)((unsigned)bh / (unsigned)p.H);
         if (heavy) {
             part = it % p.parts;
-            it = it / p.parts * p.layout_parts;
+            it = it / p.parts;
             if (p.parts > 1) part_slot = (int)x;
-        } else it += p.heavy_per_head;
+        } else it += p.global_tiles;
         if (BB_CHECK(bh >= 0 && bh < p.BH && it >= 0 && it < p.items_per_head, 71)) item = p.items[(size_t)(bh - batch * p.H) * p.items_per_head + it];
         else w = -1;
         if (heavy) {                                // its list is every block of the sequence
@@ -790,12 +789,12 @@ attn_fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
 // tile, group of 16 rows); 16 threads share a row, each owning 4 of its 64 output columns.
 __global__ void __launch_bounds__(256)
 merge_split_tiles_kernel(const float* __restrict__ partials, const Item* __restrict__ items, const unsigned long long* __restrict__ kbits,
-                         __nv_bfloat16* __restrict__ out, float* __restrict__ lse, int H, int nb, int items_per_head, int layout_parts, int tiles_per_head,
+                         __nv_bfloat16* __restrict__ out, float* __restrict__ lse, int H, int nb, int items_per_head, int tiles_per_head,
                          int nparts) {
     grid_dependency_release();
     const int rgrp = blockIdx.x & 7, tile = (blockIdx.x >> 3) % tiles_per_head, bh = (blockIdx.x >> 3) / tiles_per_head;
     const int row = rgrp * 16 + (threadIdx.x >> 4), c4 = threadIdx.x & 15, r64 = row & (kBlock - 1);
-    const Item& item = items[(size_t)(bh % H) * items_per_head + tile * layout_parts];
+    const Item& item = items[(size_t)(bh % H) * items_per_head + tile];
     const int q = row >= kBlock ? item.qb : item.qa;
     grid_dependency_wait();
     if (q < 0) return;
@@ -900,8 +899,8 @@ cudaError_t kernel_setup(int device, int* sm_count) {
 }
 
 // How a launch cuts the tiles of global blocks: their lists are as long as the sequence, the other tiles' a dozen blocks, so that
-// they outlast everything else unless the GPU has a lot to do.  A part is three quarters of what each stream gets altogether, but
-// no shorter than the other tiles are.  Measured, uncut (or in parts of 32) -> cut like this: one sequence of 3001 tokens in 4096,
+// they outlast everything else unless the GPU has a lot to do.  As many parts as there are three quarters of what each stream gets
+// altogether in a list, or lengths of another tile if that is longer, rounded up: a part is at least two thirds as long.  Measured, uncut (or in parts of 32) -> cut like this: one sequence of 3001 tokens in 4096,
 // 12 heads 60 -> 42 us (the chain of a global tile was 50 of them); [2, 12, 1024] stays uncut.
 struct Cut {
     int parts, part_steps;
@@ -921,8 +920,6 @@ Cut cut_global_tiles(const bigbird_layout& L, int B, int sms, int max_parts) {
 
 void set_shape(KernelParams& p, const bigbird_layout& L, int B, Cut cut, float scale) {
     p.items_per_head = L.items_per_head;
-    p.heavy_per_head = L.heavy_items_per_head;
-    p.layout_parts = L.max_parts;
     p.global_tiles = L.global_tiles;
     p.parts = cut.parts;
     p.part_steps = cut.part_steps;
@@ -968,7 +965,7 @@ cudaError_t enqueue(const KernelParams& p, const CUtensorMap& tm_q, const CUtens
     ++*launches;
     if (p.parts > 1) {
         e = launch_chained(merge_split_tiles_kernel, (unsigned)(p.BH * p.global_tiles * 8), 256, 0, stream, (const float*)p.partials, p.items, p.kbits, p.out, p.lse,
-                           p.H, p.nb, p.items_per_head, p.layout_parts, p.global_tiles, p.parts);
+                           p.H, p.nb, p.items_per_head, p.global_tiles, p.parts);
         if (e != cudaSuccess) return e;
         ++*launches;
     }
@@ -1046,7 +1043,10 @@ namespace {
 constexpr size_t kStaticMaskWords = 16384;      // B * N/b
 constexpr size_t kStaticItems = 8192;           // H * tiles per head
 constexpr size_t kStaticSteps = 131072;         // (key block, halves) entries summed over heads
-constexpr size_t kStaticParts = 128;            // parts of split global tiles
+constexpr size_t kStaticParts = 128;            // parts of split global tiles (more tiles than fit stay whole)
+// N/b: the tiles of global blocks of longer sequences outlast everything else if they are not cut, however little room is left for
+// parts, and the allocating entry point cuts them as finely as it pays.
+constexpr int kStaticBlocks = 96;
 constexpr size_t kStaticOffMask = 256;          // bytes 0..15: status[2], counter[2]
 constexpr size_t kStaticOffItems = kStaticOffMask + kStaticMaskWords * sizeof(unsigned long long);
 constexpr size_t kStaticOffSteps = kStaticOffItems + kStaticItems * sizeof(Item);
@@ -1107,7 +1107,7 @@ extern "C" int bigbird_attn_fwd_static(const void* q, const void* k, const void*
     // the fixed scratch bounds the problem
     const size_t words = (size_t)B * L->nb, n_items = L->items.size(), n_steps = L->steps.size();
     if (words > kStaticMaskWords || n_items > kStaticItems || n_steps > kStaticSteps) return BIGBIRD_ELIMIT;
-    if (L->max_parts > 1) return BIGBIRD_ELIMIT;    // split global tiles need scratch for their partial results
+    if (L->nb > kStaticBlocks) return BIGBIRD_ELIMIT;
 
     int device = 0;
     cudaError_t e = cudaGetDevice(&device);

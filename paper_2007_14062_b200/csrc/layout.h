@@ -17,15 +17,16 @@ constexpr int32_t kUpperHalf = 1;
 constexpr int32_t kLowerHalf = 2;
 constexpr int32_t kNoBlock = -1;
 
-// One unit of work for a CTA: a tile of two query blocks and a contiguous range of steps.
+// A tile of two query blocks and a contiguous range of steps, in the form in which bigbird_layout_schedule exports it.  (Launches may
+// cut the tiles of global blocks into parts, by what else there is to do; the layout keeps them whole.)
 struct Item {
     int32_t qa;          // query block of the upper half
     int32_t qb;          // query block of the lower half, or kNoBlock
     int32_t step_begin;  // index into the head's step array
     int32_t step_count;
-    int32_t part;        // >= 0: this item is one chunk of a split tile and writes partial results to slot `part`
-    int32_t nparts;      // number of chunks of the tile (1 = not split)
-    int32_t tile;        // index of the split tile within the head (valid when nparts > 1)
+    int32_t part;        // -1
+    int32_t nparts;      // 1
+    int32_t tile;        // index among the head's global tiles (0 for the others)
     int32_t pad_;
 };
 
@@ -58,10 +59,9 @@ struct bigbird_layout {
     // the same graph by key block: rows h*nb + c list, ascending, the query blocks that attend key block c
     std::vector<int32_t> col_ptr;
     std::vector<int32_t> row_idx;
-    // tile schedule: per head the same number of items, heavy (global) items first
+    // tile schedule: per head the same number of items, the tiles of global blocks first
     int items_per_head = 0;
-    int heavy_items_per_head = 0;   // leading items of each head that belong to global tiles
-    int max_parts = 1;
+    int global_tiles = 0;                      // of two global blocks each
     std::vector<bigbird::Item> items;          // [H * items_per_head], step_begin relative to the head's first step
     std::vector<bigbird::Item> items_abs;      // the same with step_begin made absolute (what the kernel reads)
     std::vector<int32_t> step_base;            // [H] offset of the head's steps in `steps`
@@ -69,7 +69,6 @@ struct bigbird_layout {
     // the same for tiles that stack two key blocks and walk the query blocks that attend them (b == 64 only); global
     // key blocks have no list, every query block attends them
     int sparse_tiles_per_head = 0;
-    int global_tiles = 0;                      // tiles of two global blocks
     std::vector<int32_t> global_pairs;         // [global_tiles * 2], the last entry kNoBlock if their number is odd
     int n_globals = 0;                         // global blocks, and all blocks with the global ones first
     std::vector<int32_t> block_order;
@@ -81,6 +80,6 @@ struct bigbird_layout {
 };
 
 namespace bigbird {
-// Builds CSR and schedule; returns 0 or a negative BIGBIRD_* code.  chunk_steps <= 0 picks the default.
-int build_layout_host(bigbird_layout* L, int chunk_steps);
+// Builds CSR and schedule; returns 0 or a negative BIGBIRD_* code.
+int build_layout_host(bigbird_layout* L);
 }
