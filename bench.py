@@ -36,7 +36,8 @@ NOMINAL_BF16_TFLOPS = 2250.0
 FALLBACK_PEAKS = {"bf16_tflops": 1590.0, "hbm_gbs": 6650.0}
 # dram__bytes_read.sum + dram__bytes_write.sum of one attn_fwd_sm100_kernel launch on this workload, from the
 # ncu capture summarised in profiles/ (None until a capture exists for the current kernel).
-NCU_DRAM_BYTES_PER_LAUNCH = {"c2_base_itc_bf16": 242.1e6}
+NCU_DRAM_BYTES_PER_LAUNCH = {"c2_base_itc_bf16": 241.4e6}
+NCU_DRAM_BYTES_PER_BACKWARD_LAUNCH = {"c2_base_itc_bf16": 530.3e6}     # the same of attn_bwd_sm100_kernel
 
 
 def measured_peaks():
@@ -273,7 +274,7 @@ def run_backward(args, wl):
                            l2=f"one set of eight tensors ({8 * q.numel() * elt / 1e6:.0f} MB)"),
             "gpu_launches": launches * steps, "clocks": clocks,
             "roofline": {"bound": "tensor" if tensor else "alu", "achieved": tflops, "peak": peak, "unit": "TFLOP/s", "frac": tflops / peak,
-                         "traffic": None, "peak_source": source, "kernel": kernel,
+                         "traffic": NCU_DRAM_BYTES_PER_BACKWARD_LAUNCH.get(wl.name), "peak_source": source, "kernel": kernel,
                          "min_hbm_bytes_per_launch": min_bytes, "achieved_hbm_gbs_on_min_bytes": min_bytes / (ms_per_step * 1e-3) / 1e9}}
     if not args.no_cpu_baseline:
         from oracle import bigbird_oracle as O
