@@ -404,19 +404,25 @@ __device__ __forceinline__ void accumulate_role(const KernelParams& p, SmemCtl* 
 // ------------------------------------------------------------------------------------------------ elementwise (three warpgroups, one thread per row)
 // The 64 columns of a step, 16 at a time, the next 16 on their way out of tensor memory meanwhile.  What takes the place of 16
 // columns of fp32 is 8 columns of packed high halves and 8 of low halves.
-// -inf over the scores of a step's padded tokens, in tensor memory.  (Rare: the blocks that hold a sequence's end.  Key tiles need
-// it although their padded queries have -inf for their statistics: that makes P zero only where S is below infinity.  A test per
-// 16 columns in dq_columns and dkv_columns cost training 5%.)
+// -inf over S and zero over dP of a step's padded tokens, in tensor memory: either may have overflowed.  (Rare: the blocks that hold a
+// sequence's end.  Key tiles need it although their padded queries have -inf for their statistics: that makes P zero only where S is
+// below infinity.  A test per 16 columns in dq_columns and dkv_columns cost training 5%.)
 __device__ __forceinline__ void mask_scores(unsigned buf, unsigned long long bits64) {
 #pragma unroll 1
     for (int c = 0; c < 4; ++c) {
-        float s[16];
+        float s[16], d[16];
         const unsigned bits = (unsigned)(bits64 >> (16 * c));
         tmem_ld16(buf + 16 * c, s);
+        tmem_ld16(buf + 64 + 16 * c, d);
         tmem_wait_ld();
 #pragma unroll
-        for (int t = 0; t < 16; ++t) s[t] = ((bits >> t) & 1u) ? s[t] : -INFINITY;
+        for (int t = 0; t < 16; ++t) {
+            const bool token = (bits >> t) & 1u;
+            s[t] = token ? s[t] : -INFINITY;
+            d[t] = token ? d[t] : 0.f;
+        }
         tmem_st16(buf + 16 * c, reinterpret_cast<unsigned*>(s));
+        tmem_st16(buf + 64 + 16 * c, reinterpret_cast<unsigned*>(d));
     }
     tmem_wait_st();
 }
