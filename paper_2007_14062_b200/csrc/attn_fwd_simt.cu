@@ -176,8 +176,8 @@ attn_fwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* 
                 for (int c = 0; c < C::N; ++c) fma2(acc[c], pair(f, f), *reinterpret_cast<const f32x2*>(row + C::at(tx, c)));
             }
             const int tok = tok0 + r;
-            const bool good = sum > 0.f && (!mask || mask[tok] != 0);
-            store_cols<D>(out + base + (int64_t)tok * D, acc, good ? 1.f / sum : 0.f, tx);
+            const bool token = !mask || mask[tok] != 0, good = token && sum > 0.f;
+            store_cols<D>(out + base + (int64_t)tok * D, acc, good ? 1.f / sum : 0.f, tx, !token);
             if (lse && tx == 0) lse[(int64_t)tile.bh * N + tok] = good ? mx + logf(sum) : -CUDART_INF_F;
         }
         cluster.sync();                            // nobody leaves while its shared memory is being read
@@ -187,8 +187,8 @@ attn_fwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* 
     for (int i = 0; i < TM; ++i) {
         const int r = ty * TM + i, tok = tok0 + r;
         if (r >= have) continue;
-        const bool good = l[i] > 0.f && (!mask || mask[tok] != 0);
-        store_cols<D>(out + base + (int64_t)tok * D, o[i], good ? 1.f / l[i] : 0.f, tx);
+        const bool token = !mask || mask[tok] != 0, good = token && l[i] > 0.f;
+        store_cols<D>(out + base + (int64_t)tok * D, o[i], good ? 1.f / l[i] : 0.f, tx, !token);
         if (lse && tx == 0) lse[(int64_t)tile.bh * N + tok] = good ? m[i] + logf(l[i]) : -CUDART_INF_F;
     }
 }

@@ -97,7 +97,7 @@ struct __align__(16) EpiMsg {
     int bh, qa, qb;
     int part_slot;
     int pad_[3];
-    float inv[kSoftmaxThreads];    // per row: 1 / l, or 0 for a row that must come out as zeros
+    float inv[kSoftmaxThreads];    // per row: 1 / l, 0 if there is no such thing, -1 for a padded row, which comes out as zeros
 };
 
 struct __align__(16) StreamCtl {
@@ -602,10 +602,10 @@ __device__ __forceinline__ void softmax_role(const KernelParams& p, SmemCtl* ctl
                 part[128 * 64 + row] = have ? m_ref : -INFINITY;
                 part[128 * 64 + 128 + row] = have ? l_sum : 0.f;
             } else if (my_q >= 0) {                 // warp-uniform
-                const bool good = have && ((qbits >> r64) & 1ull) && l_sum > 0.f;
+                const bool token = (qbits >> r64) & 1ull, good = have && token && l_sum > 0.f;
                 const size_t tok = ((size_t)slot->bh * p.nb + my_q) * kBlock + r64;
                 if (p.lse) p.lse[tok] = good ? (m_ref + __log2f(l_sum)) * 0.6931471805599453f : -INFINITY;
-                inv = good ? __frcp_rn(l_sum) : 0.f;
+                inv = good ? __frcp_rn(l_sum) : (token ? 0.f : -1.f);
                 if (!have) {                        // no key block was attended: the row is zeros, written from here
                     uint4* dst = reinterpret_cast<uint4*>(p.out + tok * kBlock);
                     const uint4 z = make_uint4(0u, 0u, 0u, 0u);
@@ -685,14 +685,16 @@ __device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ct
 #pragma unroll
                     for (int j = 0; j < 8; ++j) d4[j] = make_float4(o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
                 } else {
+                    // (a select for padded rows: what stands in them may be anything, and with it their sums)
+                    const bool token = inv >= 0.f;
                     uint4* d4 = reinterpret_cast<uint4*>(dst) + 4 * c;
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         uint4 v;
-                        v.x = pack_bf16(o[8 * j + 0] * inv, o[8 * j + 1] * inv);
-                        v.y = pack_bf16(o[8 * j + 2] * inv, o[8 * j + 3] * inv);
-                        v.z = pack_bf16(o[8 * j + 4] * inv, o[8 * j + 5] * inv);
-                        v.w = pack_bf16(o[8 * j + 6] * inv, o[8 * j + 7] * inv);
+                        v.x = token ? pack_bf16(o[8 * j + 0] * inv, o[8 * j + 1] * inv) : 0u;
+                        v.y = token ? pack_bf16(o[8 * j + 2] * inv, o[8 * j + 3] * inv) : 0u;
+                        v.z = token ? pack_bf16(o[8 * j + 4] * inv, o[8 * j + 5] * inv) : 0u;
+                        v.w = token ? pack_bf16(o[8 * j + 6] * inv, o[8 * j + 7] * inv) : 0u;
                         d4[j] = v;
                     }
                 }
@@ -828,10 +830,11 @@ merge_split_tiles_kernel(const float* __restrict__ partials, const Item* __restr
             acc.x += wgt * v[u].x; acc.y += wgt * v[u].y; acc.z += wgt * v[u].z; acc.w += wgt * v[u].w;
         }
     }
-    const bool good = ((qb >> r64) & 1ull) && l > 0.f;
+    const bool token = (qb >> r64) & 1ull, good = token && l > 0.f;
     const float inv = good ? 1.f / l : 0.f;
     const size_t tok = ((size_t)bh * nb + q) * kBlock + r64;
-    reinterpret_cast<uint2*>(out + tok * kBlock)[c4] = make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
+    reinterpret_cast<uint2*>(out + tok * kBlock)[c4] = token ? make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv))
+                                                             : make_uint2(0u, 0u);
     if (lse && c4 == 0) lse[tok] = good ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
 }
 

@@ -158,13 +158,14 @@ __device__ __forceinline__ void sum_tile(f32x2 (&acc)[TM][Cols<D>::N], const flo
         }
     }
 }
+// The sums times f, or zeros: a select, since what stands in padded rows may be anything, and with it their sums.
 template <int D, typename T>
-__device__ __forceinline__ void store_cols(T* row, const f32x2* acc, float f, int tx) {
+__device__ __forceinline__ void store_cols(T* row, const f32x2* acc, float f, int tx, bool zero = false) {
     using C = Cols<D>;
 #pragma unroll
     for (int c = 0; c < C::N; ++c) {
         const float2 x = unpair(acc[c]);
-        store2(row + C::at(tx, c), x.x * f, x.y * f);
+        store2(row + C::at(tx, c), zero ? 0.f : x.x * f, zero ? 0.f : x.y * f);
     }
 }
 

@@ -18,7 +18,7 @@ pytestmark = pytest.mark.gpu
 
 TOL_OUT = {"fp32": 1e-5, "bf16": 2e-2}
 TOL_LSE = 1e-3
-IMPLS = {"fwd": bb.bigbird_attn_fwd, "simt": bb.bigbird_attn_fwd_simt}
+IMPLS = {"fwd": bb.bigbird_attn_fwd, "simt": bb.bigbird_attn_fwd_simt, "static": bb.bigbird_attn_fwd_static}
 
 
 def _graph(wl):
@@ -35,7 +35,7 @@ def _run(wl, q, k, v, kpm, impl="fwd", want_lse=True):
     IMPLS[impl](qd, kd, vd, L, md, out, lse, wl.scale)
     st, detail = bb.bigbird_last_status()
     assert st == 0, (st, detail)
-    assert bb.bigbird_last_launch_count() >= 1
+    assert impl == "static" or bb.bigbird_last_launch_count() >= 1
     res = out.float().cpu().numpy(), (None if lse is None else lse.cpu().numpy())
     L.close()
     return res
@@ -246,6 +246,26 @@ def test_contents_of_padded_key_blocks_do_not_matter_on_the_cuda_core_path(b, nb
         t[:, :, valid:] = float("nan")
     dirty = _run(wl, q, k, v, kpm)
     assert np.array_equal(clean[0], dirty[0]) and np.array_equal(clean[1], dirty[1])
+
+
+@pytest.mark.parametrize("dtype,B,nb,lengths,kw,impl",
+                         [("bf16", 2, 12, (768, 197), {}, impl) for impl in ("fwd", "static", "simt")] +
+                         [("bf16", 1, 80, (5001,), dict(mode=1, g=3, r=0), impl) for impl in ("fwd", "static", "simt")] +
+                         [("fp32", 1, 8, (300,), {}, "fwd"), ("fp32", 12, 8, (300,) * 12, {}, "fwd")])
+def test_contents_of_padded_query_rows_do_not_matter(dtype, B, nb, lengths, kw, impl):
+    """NaN in the rows of q behind a sequence's end: out = 0 and lse = -inf there, and the same bits everywhere else (tiles of global
+    blocks whole and cut, the latter with padding in the tail of the last global block; CUDA-core tiles shared by a cluster and not)."""
+    wl = _small(dtype, B, 2, nb, **kw)
+    q, k, v = synth.make_qkv(wl)
+    kpm = (torch.arange(wl.N)[None, :] < torch.tensor(lengths)[:, None]).to(torch.uint8)
+    if kw:
+        kpm[:, 130:192] = 0
+    clean = _run(wl, q, k, v, kpm, impl)
+    q = q.masked_fill((kpm == 0)[:, None, :, None], float("nan"))
+    dirty = _run(wl, q, k, v, kpm, impl)
+    assert np.array_equal(clean[0], dirty[0]) and np.array_equal(clean[1], dirty[1])
+    pad = kpm.numpy() == 0
+    assert (dirty[0].transpose(0, 2, 1, 3)[pad] == 0).all() and np.isneginf(dirty[1].transpose(0, 2, 1)[pad]).all()
 
 
 def test_scores_of_minus_infinity_on_the_cuda_core_path():
