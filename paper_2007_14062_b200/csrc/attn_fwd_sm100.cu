@@ -79,7 +79,7 @@ struct __align__(16) ChunkEntry {
                                    // bit 2 (kHasPadding): some of its keys are padding
     unsigned long long kb;         // valid-key bits (never 0: blocks that are entirely padding are dropped)
 };
-enum { kSegFirst = 1, kSegLast = 2, kSegLive = 4 };
+enum { kSegFirst = 1, kSegLast = 2 };
 enum { kWhoMask = 3, kHasPadding = 4, kNoChunk = 3 };
 struct __align__(16) WorkSlot {
     int w;                         // work index, -1 = no more work
@@ -136,6 +136,7 @@ struct KernelParams {
     int parts, part_steps;             // how this launch cuts them (part_steps: key blocks)
     int BH, H, nb;
     int total_work;
+    int ahead;                         // tiles that a stream has in hand at most, 2 .. kSchedSlots
     float scale_log2;
     float* partials;                   // [BH * global_tiles * parts][kPartialFloats], if parts > 1
 };
@@ -193,49 +194,78 @@ struct StreamRef {
 };
 
 // ------------------------------------------------------------------------------------------------ scheduler (one warp, both streams)
-// Fetches the next work item for a stream, drops the key blocks that are entirely padding and posts the live
-// list.  Returns the work index (-1: the stream has been told that there is no more work), or -2 after an
-// expired wait.
-__device__ __forceinline__ int schedule_one(const KernelParams& p, SmemCtl* ctl, StreamCtl* sc, int stream, unsigned& sched_n, int lane) {
-    const unsigned lt_mask = (1u << lane) - 1u;
-    // A stream's first item is its own, which spreads the global tiles over the SMs (the second streams in the opposite order, so
-    // that with little work a CTA with a global tile has nothing else); after that they are drawn.
-    int w = stream == 0 ? (int)blockIdx.x : (int)(2 * gridDim.x - 1 - blockIdx.x);
-    static_assert(kStreams == 2, "first items");
-    if (sched_n > 0) {
-        if (lane == 0) w = (int)gridDim.x * kStreams + atomicAdd(&p.counter[0], 1);
-        w = __shfl_sync(0xffffffffu, w, 0);
-    }
-    if (w >= p.total_work) w = -1;
-    // decode the work index: the parts of the global-row tiles of every (batch, head) first, then the sparse tiles
-    int bh = 0, batch = 0, part_slot = -1;
-    bool heavy = false;
-    Item item{};
-    if (w >= 0) {
-        const unsigned heavy_total = (unsigned)(p.BH * p.global_tiles * p.parts);
-        heavy = (unsigned)w < heavy_total;
-        const unsigned per_head = heavy ? p.global_tiles * p.parts : p.items_per_head - p.global_tiles;
-        const unsigned x = heavy ? w : w - heavy_total;
-        bh = (int)(x / per_head);                   // (one division for either kind of item: this code is kept small)
-        int it = (int)(x - bh * per_head), part = 0;
-        batch = (int)((unsigned)bh / (unsigned)p.H);
-        if (heavy) {
-            part = it % p.parts;
-            it = it / p.parts;
-            if (p.parts > 1) part_slot = (int)x;
-        } else it += p.global_tiles;
-        if (BB_CHECK(bh >= 0 && bh < p.BH && it >= 0 && it < p.items_per_head, 71)) item = p.items[(size_t)(bh - batch * p.H) * p.items_per_head + it];
-        else w = -1;
-        if (heavy) {                                // its list is every block of the sequence
-            item.step_begin = part * p.part_steps;
-            item.step_count = min(p.part_steps, p.nb - item.step_begin);
+// Zeros and -inf to the rows of a tile that holds no token.  (By the scheduler itself, with nothing in its way but its own stores: such a
+// tile takes no slot and none of its stream's time: [16, 16, 4096] with 1024 to 4096 tokens 213 -> 196 us.)  row_a, row_b: blocks of the
+// B H N / 64 ones; row_b < 0: none.
+__device__ __forceinline__ void clear_tile(__nv_bfloat16* out, float* lse, float* partials, int row_a, int row_b, int part_slot, int lane) {
+    if (part_slot >= 0) {                           // a part: nothing to add; the rows are written when the parts are merged
+        float* stats = partials + (size_t)part_slot * kPartialFloats + 128 * 64;
+#pragma unroll 1
+        for (int r = lane; r < 128; r += 32) {
+            stats[r] = -INFINITY;
+            stats[128 + r] = 0.f;
         }
-        if (!BB_CHECK(item.step_count >= 0 && item.step_begin >= 0 && item.qa >= 0 && item.qa < p.nb && item.qb < p.nb, 72)) w = -1;
+        return;
     }
-    const unsigned long long qbits_a = w >= 0 ? key_bits(p, batch, item.qa) : 0ull;
-    const unsigned long long qbits_b = w >= 0 ? key_bits(p, batch, item.qb) : 0ull;
-    const bool tile_live = (qbits_a | qbits_b) != 0ull;      // a tile whose query rows are all padding is skipped
-    const int n_raw = (w >= 0 && tile_live) ? item.step_count : 0;
+#pragma unroll 1
+    for (int i = lane; i < (row_b >= 0 ? 16 : 8) * kBlock; i += 32) {
+        const size_t tok = (size_t)(i < 8 * kBlock ? row_a : row_b) * kBlock + ((i >> 3) & (kBlock - 1));
+        reinterpret_cast<uint4*>(out + tok * kBlock)[i & 7] = make_uint4(0u, 0u, 0u, 0u);
+        if (lse && (i & 7) == 0) lse[tok] = -INFINITY;
+    }
+}
+
+// Fetches the next work item for a stream that has a token among its rows, drops the key blocks that are entirely padding and posts the
+// live list.  Returns the work index (-1: the stream has been told that there is no more work), or -2 after an expired wait.
+__device__ __forceinline__ int schedule_one(const KernelParams& p, SmemCtl* ctl, StreamCtl* sc, int stream, unsigned& sched_n, bool& drawn, int lane) {
+    const unsigned lt_mask = (1u << lane) - 1u;
+    int w, bh, batch, part_slot;
+    bool heavy;
+    Item item;
+    unsigned long long qbits_a, qbits_b;
+#pragma unroll 1
+    for (;;) {                                      // up to a tile with a token
+        // A stream's first item is its own, which spreads the global tiles over the SMs (the second streams in the opposite order, so
+        // that with little work a CTA with a global tile has nothing else); after that they are drawn.
+        w = stream == 0 ? (int)blockIdx.x : (int)(2 * gridDim.x - 1 - blockIdx.x);
+        static_assert(kStreams == 2, "first items");
+        if (drawn) {
+            if (lane == 0) w = (int)gridDim.x * kStreams + atomicAdd(&p.counter[0], 1);
+            w = __shfl_sync(0xffffffffu, w, 0);
+        }
+        drawn = true;
+        if (w >= p.total_work) w = -1;
+        // decode the work index: the parts of the global-row tiles of every (batch, head) first, then the sparse tiles
+        bh = 0; batch = 0; part_slot = -1;
+        heavy = false;
+        item = Item{};
+        if (w >= 0) {
+            const unsigned heavy_total = (unsigned)(p.BH * p.global_tiles * p.parts);
+            heavy = (unsigned)w < heavy_total;
+            const unsigned per_head = heavy ? p.global_tiles * p.parts : p.items_per_head - p.global_tiles;
+            const unsigned x = heavy ? w : w - heavy_total;
+            bh = (int)(x / per_head);                   // (one division for either kind of item: this code is kept small)
+            int it = (int)(x - bh * per_head), part = 0;
+            batch = (int)((unsigned)bh / (unsigned)p.H);
+            if (heavy) {
+                part = it % p.parts;
+                it = it / p.parts;
+                if (p.parts > 1) part_slot = (int)x;
+            } else it += p.global_tiles;
+            if (BB_CHECK(bh >= 0 && bh < p.BH && it >= 0 && it < p.items_per_head, 71)) item = p.items[(size_t)(bh - batch * p.H) * p.items_per_head + it];
+            else w = -1;
+            if (heavy) {                                // its list is every block of the sequence
+                item.step_begin = part * p.part_steps;
+                item.step_count = min(p.part_steps, p.nb - item.step_begin);
+            }
+            if (!BB_CHECK(item.step_count >= 0 && item.step_begin >= 0 && item.qa >= 0 && item.qa < p.nb && item.qb < p.nb, 72)) w = -1;
+        }
+        qbits_a = w >= 0 ? key_bits(p, batch, item.qa) : 0ull;
+        qbits_b = w >= 0 ? key_bits(p, batch, item.qb) : 0ull;
+        if (w < 0 || (qbits_a | qbits_b) != 0ull) break;
+        clear_tile(p.out, p.lse, p.partials, bh * p.nb + item.qa, item.qb >= 0 ? bh * p.nb + item.qb : -1, part_slot, lane);
+    }
+    const int n_raw = w >= 0 ? item.step_count : 0;
     int i0 = 0;
     bool first = true;
     do {
@@ -272,7 +302,7 @@ __device__ __forceinline__ int schedule_one(const KernelParams& p, SmemCtl* ctl,
             slot->qa = item.qa;
             slot->qb = item.qb;
             slot->n_chunks = count;
-            slot->flags = (first ? kSegFirst : 0) | (i0 >= n_raw ? kSegLast : 0) | (tile_live ? kSegLive : 0);
+            slot->flags = (first ? kSegFirst : 0) | (i0 >= n_raw ? kSegLast : 0);
             slot->qbits_a = qbits_a;
             slot->qbits_b = qbits_b;
             slot->part_slot = w >= 0 ? part_slot : -1;
@@ -288,7 +318,7 @@ __device__ __forceinline__ int schedule_one(const KernelParams& p, SmemCtl* ctl,
 
 __device__ __forceinline__ void scheduler_role(const KernelParams& p, SmemCtl* ctl, int lane) {
     unsigned sched_n0 = 0, sched_n1 = 0;            // slots posted per stream (scalars: an indexed array would live in local memory)
-    unsigned done = 0;                              // bit s: stream s has been told that there is no more work
+    unsigned done = 0, drawn = 0;                   // bit s: stream s has been told that there is no more work; has had an item
     IdleClock idle;
     while (done != (1u << kStreams) - 1u) {
         bool progress = false;
@@ -297,9 +327,12 @@ __device__ __forceinline__ void scheduler_role(const KernelParams& p, SmemCtl* c
             if ((done >> s) & 1u) continue;
             StreamCtl* sc = &ctl->st[s];
             unsigned n = s == 0 ? sched_n0 : sched_n1;
-            const unsigned ss = n % kSchedSlots, sp = (n / kSchedSlots) & 1u;
-            if (!__all_sync(0xffffffffu, mbar_test(&sc->sched_empty[ss], sp ^ 1u))) continue;
-            const int w = schedule_one(p, ctl, sc, s, n, lane);
+            // (the slot posted `ahead` slots ago must have been given back)
+            const unsigned m = n - (unsigned)p.ahead;
+            if (n >= (unsigned)p.ahead && !__all_sync(0xffffffffu, mbar_test(&sc->sched_empty[m % kSchedSlots], (m / kSchedSlots) & 1u))) continue;
+            bool d = (drawn >> s) & 1u;
+            const int w = schedule_one(p, ctl, sc, s, n, d, lane);
+            drawn |= 1u << s;
             if (s == 0) sched_n0 = n; else sched_n1 = n;
             if (w == -2) return;
             if (w < 0) done |= 1u << s;
@@ -334,7 +367,7 @@ __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ct
         if (!poll_wait(&sc->sched_full[ss], sp, idle, abort_flag, p.status, 13)) return;
         const WorkSlot* slot = &sc->slot[ss];
         const int w = slot->w, flags = slot->flags, bh = slot->bh, n = slot->n_chunks;
-        if (w >= 0 && (flags & kSegLive)) {
+        if (w >= 0) {
             if (!v_lane && (flags & kSegFirst)) {
                 const int qa = slot->qa, qb = slot->qb;
                 const unsigned qs = q_n & 1u;
@@ -393,7 +426,7 @@ __device__ __forceinline__ void mma_role(const KernelParams& p, SmemCtl* ctl, co
         if (!mbar_wait(&sc->sched_full[ss], sp, abort_flag)) { fail = 23; break; }
         const WorkSlot* slot = &sc->slot[ss];
         const int w = slot->w, flags = slot->flags, n = slot->n_chunks;
-        const bool work = w >= 0 && (flags & kSegLive);
+        const bool work = w >= 0;
         const bool first = work && (flags & kSegFirst), last = work && (flags & kSegLast);
         if (first) {
             tile_steps = false;
@@ -515,7 +548,6 @@ __device__ __forceinline__ void softmax_role(const KernelParams& p, SmemCtl* ctl
             mbar_arrive(&sc->epi_full[msg_n & 1u]);
             break;
         }
-        const bool live = flags & kSegLive;
         if (flags & kSegFirst) {
             m_ref = -INFINITY;
             l_sum = 0.f;
@@ -592,7 +624,7 @@ __device__ __forceinline__ void softmax_role(const KernelParams& p, SmemCtl* ctl
             // -------------------------------------------------------- end of the tile: lse now, the output rows via the epilogue
             const int my_q = lower ? slot->qb : slot->qa;
             const unsigned long long qbits = lower ? slot->qbits_b : slot->qbits_a;
-            const bool have = live && o_dirty;
+            const bool have = o_dirty;
             const int part_slot = slot->part_slot;
             const int r64 = row & (kBlock - 1);
             float inv = 0.f;
@@ -606,12 +638,7 @@ __device__ __forceinline__ void softmax_role(const KernelParams& p, SmemCtl* ctl
                 const size_t tok = ((size_t)slot->bh * p.nb + my_q) * kBlock + r64;
                 if (p.lse) p.lse[tok] = good ? (m_ref + __log2f(l_sum)) * 0.6931471805599453f : -INFINITY;
                 inv = good ? __frcp_rn(l_sum) : (token ? 0.f : -1.f);
-                if (!have) {                        // no key block was attended: the row is zeros, written from here
-                    uint4* dst = reinterpret_cast<uint4*>(p.out + tok * kBlock);
-                    const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) dst[j] = z;
-                }
+                // (a tile that is no part has a step: one of its rows is a token, and a block is in its own window)
             }
             if (have) {                             // CTA-uniform per stream: every thread of the warpgroup posts
                 EpiMsg* msg = &sc->epi[msg_n & 1u];
@@ -921,7 +948,7 @@ Cut cut_global_tiles(const bigbird_layout& L, int B, int sms, int max_parts) {
     return Cut{parts, part_steps};
 }
 
-void set_shape(KernelParams& p, const bigbird_layout& L, int B, Cut cut, float scale) {
+void set_shape(KernelParams& p, const bigbird_layout& L, int B, Cut cut, float scale, int sm_count) {
     p.items_per_head = L.items_per_head;
     p.global_tiles = L.global_tiles;
     p.parts = cut.parts;
@@ -930,6 +957,10 @@ void set_shape(KernelParams& p, const bigbird_layout& L, int B, Cut cut, float s
     p.H = L.H;
     p.nb = L.nb;
     p.total_work = p.BH * (L.global_tiles * cut.parts + L.sparse_tiles_per_head);
+    // Tiles that a stream has in hand are not drawn by another one that runs dry, so with few tiles in all it should have few: [1, 12,
+    // 16384] with 13000 tokens (5 tiles per stream) 75 us with three, 69 with two; [16, 16, 4096] ragged (28, many of them without a
+    // token) 204 and 210; [8, 12, 4096] (10) 125 with either.
+    p.ahead = p.total_work < 8 * kStreams * sm_count ? 2 : kSchedSlots;
     p.scale_log2 = scale * 1.4426950408889634f;
 }
 
@@ -1022,7 +1053,7 @@ int launch_attn_fwd_sm100(const FwdArgs& a, const bigbird_layout& L, const Devic
     p.steps = dl.steps;
     p.counter = counter ? counter : (int*)(ws + off_counter);
     p.status = sc.status;
-    set_shape(p, L, a.B, cut, a.scale);
+    set_shape(p, L, a.B, cut, a.scale, sm_count);
 
     cudaError_t e = enqueue(p, tm_q, tm_k, tm_v, a.kpm, (unsigned long long*)(ws + off_bits), (int)words, p.counter, own_counter, sm_count, a.stream, launches);
     if (ws) {
@@ -1159,7 +1190,7 @@ extern "C" int bigbird_attn_fwd_static(const void* q, const void* k, const void*
     p.steps = steps_dev;
     p.status = words4;
     p.counter = words4 + 2;
-    set_shape(p, *L, B, cut, scale);
+    set_shape(p, *L, B, cut, scale, sd.sm_count);
     int launches = 0;
     if (enqueue(p, tm_q, tm_k, tm_v, key_padding_mask, kbits_dev, key_padding_mask ? (int)words : 0, words4, key_padding_mask ? 4 : 0, sd.sm_count, stream, &launches) != cudaSuccess)
         return BIGBIRD_ECUDA;

@@ -1,0 +1,71 @@
+"""Tiles without a token, and sequences that end inside, before and at the edges of tiles: what the schedulers of the tensor-core
+kernels clear themselves.  Results and gradients start from NaN, so that rows nobody writes are found."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import paper_2007_14062_b200 as bb
+
+pytestmark = pytest.mark.gpu
+
+# B, H, nb, g, mode, lengths: few tiles per stream and many; an odd number of sparse blocks; global tiles cut into parts or not, with
+# and without tokens; lengths at block and tile edges
+CASES = [
+    (3, 2, 8, 2, 0, [0, 1, 512]),
+    (2, 3, 13, 2, 0, [64, 65]),
+    (3, 4, 70, 3, 1, [0, 4480, 128]),
+    (2, 2, 96, 2, 0, [4097, 191]),
+    (40, 8, 16, 2, 0, None),
+]
+
+
+def _lengths(B, nb, lengths):
+    return np.array(lengths) if lengths else np.random.RandomState(7).randint(0, nb * 64 + 1, B)
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: f"B{c[0]}_H{c[1]}_nb{c[2]}_g{c[3]}_mode{c[4]}")
+@pytest.mark.parametrize("entry", ["fwd", "static"])
+def test_rows_of_tiles_without_tokens(case, entry):
+    B, H, nb, g, mode, lengths = case
+    N = nb * 64
+    lens = _lengths(B, nb, lengths)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    q, k, v, dout = (torch.randn((B, H, N, 64), generator=gen, device="cuda").to(torch.bfloat16) for _ in range(4))
+    mask = torch.from_numpy((np.arange(N)[None] < lens[:, None]).astype(np.uint8)).cuda()
+    rows = mask.bool()[:, None, :].expand(B, H, N)
+    L = bb.bigbird_build_layout(N, 64, 3, g, 3, 5, H, mode)
+    scale = 1.0 / math.sqrt(64)
+
+    def empty():
+        return torch.full_like(q, float("nan")), torch.full((B, H, N), float("nan"), device="cuda")
+
+    out, lse = empty()
+    fwd = bb.bigbird_attn_fwd if entry == "fwd" else bb.bigbird_attn_fwd_static
+    fwd(q, k, v, L, mask, out, lse, scale)
+    ref, ref_lse = empty()
+    bb.bigbird_attn_fwd_simt(q, k, v, L, mask, ref, ref_lse, scale)
+    assert (bb.bigbird_last_status() if entry == "fwd" else bb.bigbird_last_status_static())[0] == 0
+    assert (out[~rows] == 0).all() and (lse[~rows] == -math.inf).all()
+    if rows.any():
+        # bf16 probabilities and results against fp32 arithmetic on the same bf16 inputs: the bounds of the parity tests
+        assert (out[rows].float() - ref[rows].float()).abs().max() <= 2e-2
+        assert (lse[rows] - ref_lse[rows]).abs().max() <= 1e-3
+    if entry == "static":
+        L.close()
+        return
+    grads = [empty()[0] for _ in range(3)]
+    bb.bigbird_attn_bwd(q, k, v, out, lse, dout, L, mask, *grads, scale)
+    assert bb.bigbird_last_status()[0] == 0
+    for x in grads:
+        assert (x[~rows] == 0).all() and torch.isfinite(x[rows].float()).all()
+    # the fp32 gradients of the same inputs
+    f = [t.float() for t in (q, k, v, out, dout)]
+    want = [torch.full_like(f[0], float("nan")) for _ in range(3)]
+    bb.bigbird_attn_bwd(f[0], f[1], f[2], f[3], lse, f[4], L, mask, *want, scale)
+    for x, y in zip(grads, want):
+        # the gradients are rounded to bf16 once (2^-9 of a value) and carry 16 bits of P and dS (the bound of the gradient tests)
+        err = torch.linalg.norm((x[rows].float() - y[rows]).double()) if rows.any() else 0.0
+        assert err <= (2.0 ** -8 + 5e-4) * torch.linalg.norm(y[rows].double())
+    L.close()
