@@ -540,9 +540,11 @@ __device__ __forceinline__ void softmax_role(const KernelParams& p, SmemCtl* ctl
         const WorkSlot* slot = &sc->slot[ss];
         const int w = slot->w, flags = slot->flags, n = slot->n_chunks;
         if (w < 0) {                                // tell the epilogue that this stream is finished
-            // (once it has taken the last tile: only then is it known to have read every earlier message, so that
-            // the entry reused here is free)
-            if (msg_n > 0 && !mbar_wait(&sc->o_free, (msg_n - 1) & 1u, abort_flag)) { fail = 36; break; }
+            // (The entry reused here holds the message of the last tile but one.  That one has been read once the last tile's P V has
+            // been issued, since its first product waits for the accumulator before.  Waiting for the epilogue to take the last tile
+            // would not do: if that tile has one step, the last but one may still be in the accumulator, and its phase of o_free has the
+            // other parity, so that the wait passes at once.)
+            if (msg_n > 0 && !mbar_wait(&sc->pv_done, (grp_n - 1) & 1u, abort_flag)) { fail = 36; break; }
             EpiMsg* msg = &sc->epi[msg_n & 1u];
             if (row == 0) msg->kind = kEpiDone;
             mbar_arrive(&sc->epi_full[msg_n & 1u]);
