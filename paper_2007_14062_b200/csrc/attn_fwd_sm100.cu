@@ -686,14 +686,17 @@ __device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ct
             const unsigned msg_n = st & 0xffffu, tile_n = (st >> 16) & 0x7fffu;
             const unsigned e = msg_n & 1u, eph = (msg_n >> 1) & 1u;
             if (!__all_sync(0xffffffffu, mbar_test(&sc->epi_full[e], eph))) continue;
-            progress = true;
             const EpiMsg* msg = &sc->epi[e];
+            // (The accumulator is polled for as well: a tile's last P V is issued when the stream's next item is there, and for that the
+            // scheduler may have to wait until this warp has served the other stream.)
+            if (msg->kind != kEpiDone && !__all_sync(0xffffffffu, mbar_test(&sc->o_done, tile_n & 1u))) continue;
+            progress = true;
             const unsigned st_next = msg->kind == kEpiDone ? (st | 0x80000000u) : (((msg_n + 1u) & 0xffffu) | (((tile_n + 1u) & 0x7fffu) << 16));
             if (s == 0) state0 = st_next; else state1 = st_next;
             if (st_next >> 31) continue;
             const int bh = msg->bh, my_q = lower ? msg->qb : msg->qa, part_slot = msg->part_slot;
             const float inv = msg->inv[row];
-            if (!mbar_wait(&sc->o_done, tile_n & 1u, abort_flag)) { give_up(abort_flag, p.status, 40); return; }
+            __syncwarp();
             tc_fence_after();
             const unsigned lane_addr = tmem + s * kStreamCols + ((unsigned)(quad * 32) << 16);
             // the row's destination: the output tensor, or (raw fp32) the scratch of a split tile's part
