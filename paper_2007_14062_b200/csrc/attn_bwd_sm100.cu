@@ -13,6 +13,11 @@
 // two bf16 numbers (16 significant bits): the products keep the precision of the fp32 path to below the rounding of the
 // results, at twice the number of the accumulating MMAs.
 //
+// A block of the column side that only the upper rows of a tile attend shares a step with one that only the lower rows attend: each has
+// its products with all 128 rows, the second ones leaving the lanes of the upper half alone (the instruction's vector of disabled lanes).
+// The products are as many as if the two had a step of their own, but the way of a step through the hands of four warps is gone once and
+// not twice: 6312 steps instead of 8740 for the sparse tiles of the base layout, 12 heads, both kinds.
+//
 // Nothing carries over from step to step but the accumulators, so the steps of a tile are dealt in turn to three warpgroups
 // with a 128-column score buffer each.  One thread issues the scores of a step as soon as its buffer is free, another the
 // accumulation of the steps in turn.  An epilogue warpgroup takes a finished tile's accumulators while the next tile's scores
@@ -31,6 +36,10 @@
 // left is the way of a step through the hands of four warps with three steps in flight, which is all that tensor memory holds.  Two
 // threads per row (24 warps) were no faster.
 //
+// With shared steps [8, 12, 4096] takes 419 us at full clocks (430 with a step for each block) and forward and gradients together 628
+// instead of 646 under the power cap; a shared step takes two places in the ring of Y, for which a tile's results leave through its own
+// row buffer and no longer through one of their own.
+//
 // A first kernel makes, per query row, -lse * log2 e (-inf for rows without probabilities) and -delta, packs the key-padding
 // mask and zeroes the counters.
 #include <algorithm>
@@ -41,10 +50,11 @@ namespace bigbird {
 namespace {
 
 constexpr int kBufs = 3;                   // score buffers, each served by one warpgroup
-constexpr int kStages = 2 * kBufs;         // ring of Y1 | Y2 pairs
-constexpr int kSlots = 2;                  // tiles (or segments of long ones) posted by the scheduler (with three, a CTA held work that others
-                                           // ran out of: [1, 12, 16384] with 13000 tokens 185 us, 181 with two)
-constexpr int kSegSteps = 96;              // steps per posted segment
+constexpr int kRing = 2 * kBufs;           // ring of steps
+constexpr int kStages = 9;                 // ring of Y1 | Y2 pairs: one for a step, two if the halves of the tile share it
+constexpr int kSlots = 3;                  // tiles (or segments of long ones) posted by the scheduler (two: [3, 16, 4096] ragged, forward and
+                                           // gradients, 212.5 us against 209.2)
+constexpr int kSegSteps = 64;              // steps per posted segment, at least 33
 // warps 0..11: the three elementwise warpgroups; 12..15: epilogue; 16: scheduler; 17: TMA producer; 18, 19: MMA issuers (scores,
 // accumulations)
 constexpr int kThreads = 640;
@@ -61,15 +71,19 @@ constexpr int kStatFloats = 2 * kBlock;    // per block of query rows: 64 x (-ls
 constexpr int kPartialFloats = 2 * 128 * kBlock;   // one part of a split tile: acc0, acc1
 enum { kDkv = 0, kDq = 1 };
 enum { kSegFirst = 1, kSegLast = 2 };
-// what there is to know about a ring entry: bits 0..1 the step's kBothHalves / kUpperHalf / kLowerHalf, kind, first and last step of
-// its tile, the tile's row buffer and the parity of that buffer's phase; kInfoEnd: no more steps; kInfoPadded: some of the block's
-// tokens are padding
-enum { kInfoWho = 3, kInfoDkv = 4, kInfoFirst = 8, kInfoLast = 16, kInfoX = 32, kInfoXPar = 64, kInfoEnd = 128, kInfoPadded = 256 };
+// A step: one block that both halves of the tile attend or only one of them, or (kSecond) one for the upper half and another for the
+// lower, whose rows are computed with 128-row products that leave the lanes of the other half alone.
+enum { kAttends = 1, kPadded = 2, kSecond = 4 };        // of a half: it attends the step; some of its block's tokens are padding; its block is c1
+// what there is to know about a ring entry: the halves (kLower times the lower one's bits), kind, first and last step of its tile, the
+// tile's row buffer and the parity of that buffer's phase; kInfoEnd: no more steps; from bit kInfoStage the places of Y, 4 bits each
+enum { kLower = 8, kInfoShared = kSecond * kLower, kInfoDkv = 64, kInfoFirst = 128, kInfoLast = 256, kInfoX = 512, kInfoXPar = 1024, kInfoEnd = 2048 };
+constexpr int kInfoStage = 12;
+static_assert(kStages <= 16, "bits of a place");
 
 struct __align__(16) StepEntry {
-    int c;                         // block of the column side
-    int who;                       // kBothHalves, kUpperHalf or kLowerHalf, and kInfoPadded
-    unsigned long long kb;         // its valid-token bits (never 0)
+    int c0, c1;                    // blocks of the column side; c1 < 0: none
+    int half[2];                   // kAttends, kPadded, kSecond of the upper and the lower half
+    unsigned long long kb[2];      // valid-token bits of c0 and c1 (never 0)
 };
 struct __align__(16) TileSlot {
     int w;                         // work index, -1 = no more work
@@ -83,7 +97,7 @@ struct __align__(16) TileSlot {
     StepEntry steps[kSegSteps];
 };
 struct __align__(16) SmemCtl {
-    unsigned long long full[kStages], empty[kStages];
+    unsigned long long full[kRing], empty[kRing];
     unsigned long long x_full[2], x_empty[2];
     unsigned long long sdp_full[kBufs], p_full[kBufs];
     unsigned long long acc_full, acc_free, epi_sync;
@@ -91,16 +105,15 @@ struct __align__(16) SmemCtl {
     TileSlot slot[kSlots];
     float x_stats[2][2][kStatFloats];      // query tiles: statistics of the rows
     float y_stats[kStages][kStatFloats];   // key tiles: of the step's query block
-    unsigned info[kStages];
-    unsigned long long bits[kStages];      // the step's valid-token bits
+    unsigned info[kRing];
+    unsigned long long bits[kRing][2];     // the valid-token bits of the step's blocks
     unsigned tmem_base;
     int abort_flag;
     int merge_last;
 };
-constexpr int kSmemX = 0;                                      // two buffers of X1a X1b X2a X2b
+constexpr int kSmemX = 0;                                      // two buffers of X1a X1b X2a X2b; the tile's results leave through its own
 constexpr int kSmemRing = 2 * 4 * kTileBytes;
-constexpr int kSmemOut = kSmemRing + kStages * 2 * kTileBytes;    // four tiles on their way out
-constexpr int kSmemCtl = kSmemOut + 4 * kTileBytes;
+constexpr int kSmemCtl = kSmemRing + kStages * 2 * kTileBytes;
 constexpr int kSmemBytes = kSmemCtl + (int)sizeof(SmemCtl) + 1024;   // + slack for the 1024-byte alignment
 static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
 
@@ -192,7 +205,7 @@ __device__ __forceinline__ void scheduler_role(const KernelParams& p, SmemCtl* c
         }
         int i0 = 0;
         bool first = true;
-        StepEntry held{-1, 0, 0ull};               // last step of a full segment: kept for the next one, so that no tile's last
+        StepEntry held{};                          // last step of a full segment: kept for the next one, so that no tile's last
         bool holding = false;                      // segment turns out to be empty
         do {
             const unsigned ss = slot_n % kSlots;
@@ -207,21 +220,41 @@ __device__ __forceinline__ void scheduler_role(const KernelParams& p, SmemCtl* c
 #pragma unroll 1
             while (i0 < n_raw && count <= kSegSteps - 32) {
                 const int i = i0 + lane;
-                StepEntry e{-1, 0, 0ull};
-                bool alive = false;
+                int c = -1;
+                unsigned long long kb = 0ull;
+                bool ua = false, ub = false;
                 if (i < n_raw) {
                     const Step s = steps ? steps[begin + i] : Step{begin + i, kBothHalves};
-                    const bool ua = s.who != kLowerHalf && rbits_a != 0ull, ub = s.who != kUpperHalf && rbits_b != 0ull;
-                    e.c = s.c;
-                    e.who = (ua && ub) ? kBothHalves : (ua ? kUpperHalf : kLowerHalf);
-                    alive = BB_CHECK(s.c >= 0 && s.c < p.nb, 170);
-                    if (alive) e.kb = token_bits(p, batch, s.c);
-                    if (e.kb != ~0ull) e.who |= kInfoPadded;
-                    alive = alive && e.kb != 0ull && (ua || ub);
+                    c = s.c;
+                    if (BB_CHECK(c >= 0 && c < p.nb, 170)) kb = token_bits(p, batch, c);
+                    ua = s.who != kLowerHalf && rbits_a != 0ull && kb != 0ull;
+                    ub = s.who != kUpperHalf && rbits_b != 0ull && kb != 0ull;
                 }
-                const unsigned bal = __ballot_sync(0xffffffffu, alive);
-                if (alive) slot->steps[count + __popc(bal & lt_mask)] = e;
-                count += __popc(bal);
+                // In turn a block of both halves and one of the upper half together with one of the lower (what is left of either
+                // by itself): steps of one and of two blocks alternate, so that the ring holds the same number of steps at any time.
+                const unsigned b_both = __ballot_sync(0xffffffffu, ua && ub), b_up = __ballot_sync(0xffffffffu, ua && !ub),
+                               b_lo = __ballot_sync(0xffffffffu, ub && !ua);
+                const int n_both = __popc(b_both), n_up = __popc(b_up), n_lo = __popc(b_lo), n_one = max(n_up, n_lo);
+                if (ua || ub) {
+                    const int rank = __popc((ua ? (ub ? b_both : b_up) : b_lo) & lt_mask);
+                    const int at = ua && ub ? (rank < n_one ? 2 * rank : n_one + rank) : (rank < n_both ? 2 * rank + 1 : n_both + rank);
+                    const bool second = !ua && rank < n_up;
+                    const int flags = kAttends | (kb != ~0ull ? kPadded : 0);
+                    StepEntry* e = &slot->steps[count + at];
+                    e->kb[second ? 1 : 0] = kb;
+                    if (second) {
+                        e->c1 = c;
+                        e->half[1] = flags | kSecond;
+                    } else {
+                        e->c0 = c;
+                        e->half[0] = ua ? flags : 0;
+                        if (ub || rank >= n_lo) {
+                            e->c1 = -1;
+                            e->half[1] = ub ? flags : 0;
+                        }
+                    }
+                }
+                count += n_both + n_one;
                 i0 += 32;
             }
             __syncwarp();
@@ -254,9 +287,19 @@ __device__ __forceinline__ void scheduler_role(const KernelParams& p, SmemCtl* c
 __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ctl, unsigned char* smem, const CUtensorMap* tm_q,
                                               const CUtensorMap* tm_k, const CUtensorMap* tm_v, const CUtensorMap* tm_do) {
     int* abort_flag = &ctl->abort_flag;
-    unsigned slot_n = 0, tile_n = 0, step_n = 0;
+    unsigned slot_n = 0, tile_n = 0, step_n = 0, done_n = 0;      // done_n: steps known to be accumulated
+    unsigned stage = 0, free_stages = kStages, shared_steps = 0;  // bit n mod 32 of shared_steps: step n has two blocks
     bool fresh = false;                             // no step of the tile has been loaded yet
     int fail = 0;
+    // room for a step of `blocks` blocks
+    auto room = [&](unsigned blocks) -> bool {
+        while (free_stages < blocks || step_n - done_n == (unsigned)kRing) {
+            if (!mbar_wait(&ctl->empty[done_n % kRing], (done_n / kRing) & 1u, abort_flag)) return false;
+            free_stages += 1u + ((shared_steps >> (done_n & 31u)) & 1u);
+            ++done_n;
+        }
+        return true;
+    };
     for (;;) {
         const unsigned ss = slot_n % kSlots;
         if (!mbar_wait(&ctl->slot_full[ss], (slot_n / kSlots) & 1u, abort_flag)) { fail = 113; break; }
@@ -265,9 +308,10 @@ __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ct
         const bool dkv = slot->kind == kDkv;
         if (w < 0) {                                // the last entries of the ring, one for each score buffer's warps
             for (int i = 0; i < kBufs; ++i, ++step_n) {
-                const unsigned g = step_n % kStages;
-                if (!mbar_wait(&ctl->empty[g], ((step_n / kStages) & 1u) ^ 1u, abort_flag)) { fail = 110; break; }
+                if (!room(0)) { fail = 110; break; }
+                const unsigned g = step_n % kRing;
                 ctl->info[g] = kInfoEnd;
+                __threadfence_block();              // (nothing is loaded into this entry: its word is on its own ahead of the arrival)
                 mbar_arrive(&ctl->full[g]);
             }
             break;
@@ -275,7 +319,9 @@ __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ct
         if (flags & kSegFirst) fresh = true;
         const CUtensorMap *tm1 = dkv ? tm_q : tm_k, *tm2 = dkv ? tm_do : tm_v;
         for (int i = 0; i < n; ++i) {
-            unsigned info = (unsigned)slot->steps[i].who | (dkv ? kInfoDkv : 0) | (i == n - 1 && (flags & kSegLast) ? kInfoLast : 0);
+            const StepEntry* e = &slot->steps[i];
+            const int c0 = e->c0, c1 = e->c1;
+            unsigned info = (unsigned)(e->half[0] | e->half[1] * kLower) | (dkv ? kInfoDkv : 0) | (i == n - 1 && (flags & kSegLast) ? kInfoLast : 0);
             if (fresh) {
                 const int ra = slot->ra, rb = slot->rb;
                 const unsigned xs = tile_n & 1u;
@@ -297,17 +343,26 @@ __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ct
                 info |= kInfoFirst;
             }
             info |= (((tile_n - 1) & 1u) ? kInfoX : 0) | ((((tile_n - 1) >> 1) & 1u) ? kInfoXPar : 0);
-            const unsigned g = step_n % kStages;
-            const int row = bh * p.nb + slot->steps[i].c;
-            if (!BB_CHECK(n <= kSegSteps && slot->steps[i].c >= 0 && slot->steps[i].c < p.nb, 173)) return;
-            if (!mbar_wait(&ctl->empty[g], ((step_n / kStages) & 1u) ^ 1u, abort_flag)) { fail = 110; break; }
-            unsigned char* y = smem + kSmemRing + g * 2 * kTileBytes;
-            ctl->info[g] = info;
-            ctl->bits[g] = slot->steps[i].kb;
-            mbar_expect_tx(&ctl->full[g], 2 * kTileBytes + (dkv ? kStatFloats * 4 : 0));
-            tma_load_tile(y, tm1, row * kBlock, &ctl->full[g]);
-            tma_load_tile(y + kTileBytes, tm2, row * kBlock, &ctl->full[g]);
-            if (dkv) bulk_load(ctl->y_stats[g], p.stats + (size_t)row * kStatFloats, kStatFloats * 4, &ctl->full[g]);
+            if (!BB_CHECK(n <= kSegSteps && c0 >= 0 && c0 < p.nb && c1 < p.nb && (c1 >= 0) == ((info & kInfoShared) != 0), 173)) return;
+            const unsigned blocks = c1 >= 0 ? 2u : 1u, g = step_n % kRing;
+            if (!room(blocks)) { fail = 110; break; }
+            free_stages -= blocks;
+            const unsigned bit = 1u << (step_n & 31u);
+            shared_steps = c1 >= 0 ? shared_steps | bit : shared_steps & ~bit;
+            const unsigned next = stage + 1 == kStages ? 0u : stage + 1;
+            ctl->info[g] = info | (stage << kInfoStage) | (next << (kInfoStage + 4));
+            ctl->bits[g][0] = e->kb[0];
+            ctl->bits[g][1] = e->kb[1];
+            mbar_expect_tx(&ctl->full[g], blocks * (2 * kTileBytes + (dkv ? kStatFloats * 4 : 0)));
+#pragma unroll 1
+            for (unsigned j = 0; j < blocks; ++j) {
+                const int row = bh * p.nb + (j ? c1 : c0);
+                unsigned char* y = smem + kSmemRing + stage * 2 * kTileBytes;
+                tma_load_tile(y, tm1, row * kBlock, &ctl->full[g]);
+                tma_load_tile(y + kTileBytes, tm2, row * kBlock, &ctl->full[g]);
+                if (dkv) bulk_load(ctl->y_stats[stage], p.stats + (size_t)row * kStatFloats, kStatFloats * 4, &ctl->full[g]);
+                if (++stage == kStages) stage = 0;
+            }
             ++step_n;
         }
         if (fail) break;
@@ -322,7 +377,7 @@ __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ct
 // test 45, a test behind a commit 200.  One thread that issued everything and walked the posted tiles needed 1740 cycles a step.
 // So one issues the scores (S and dP) and one the accumulations, and both see the ring only, where each entry comes with a word
 // that says what there is to know about the step.  full[] tells both of a loaded entry, empty[] (committed behind a step's
-// accumulation) frees the ring entry for the producer and, three steps on, the score buffer for the first thread.  The tests for
+// accumulation) frees the ring entry and its Y for the producer and, three steps on, the score buffer for the first thread.  The tests for
 // the next step come before a step's commit: behind it they cost four times as much.
 __device__ __forceinline__ void score_role(const KernelParams& p, SmemCtl* ctl, unsigned char* smem, unsigned tmem) {
     int* abort_flag = &ctl->abort_flag;
@@ -337,12 +392,12 @@ __device__ __forceinline__ void score_role(const KernelParams& p, SmemCtl* ctl, 
     for (;;) {
         if (!have_f) {
             if (!mbar_wait(&ctl->full[stg], ph, abort_flag)) { fail = 120; break; }
-            info = ctl->info[stg];
+            info = ld_shared(&ctl->info[stg]);
         }
         if (info & kInfoEnd) break;
         if (n == (unsigned)kBufs) {                 // the buffer's last user must have been accumulated
             if (!have_e && !mbar_wait(&ctl->empty[old], old_ph, abort_flag)) { fail = 121; break; }
-            if (++old == kStages) { old = 0; old_ph ^= 1u; }
+            if (++old == kRing) { old = 0; old_ph ^= 1u; }
         } else ++n;
         if (info & kInfoFirst) {
             const unsigned xs = (info & kInfoX) ? 1u : 0u;
@@ -350,17 +405,24 @@ __device__ __forceinline__ void score_role(const KernelParams& p, SmemCtl* ctl, 
             x1 = x0 + xs * 4 * kTileDesc;
         }
         tc_fence_after();
-        const unsigned y1 = ring0 + stg * kStageDesc, d = tmem + buf * kBufCols;
+        const unsigned y1 = ring0 + ((info >> kInfoStage) & 15u) * kStageDesc, d = tmem + buf * kBufCols;
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) mma_ss_lo(d, x1 + kk * 2, y1 + kk * 2, kIdescQK64, kk > 0);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) mma_ss_lo(d + 64, x1 + 2 * kTileDesc + kk * 2, y1 + kTileDesc + kk * 2, kIdescQK64, kk > 0);
+        if (info & kInfoShared) {                   // over the lanes of the lower half: with its own block
+            const unsigned z1 = ring0 + ((info >> (kInfoStage + 4)) & 15u) * kStageDesc;
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) mma_ss_half(d, x1 + kk * 2, z1 + kk * 2, kIdescQK64, kk > 0, ~0u, 0u);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) mma_ss_half(d + 64, x1 + 2 * kTileDesc + kk * 2, z1 + kTileDesc + kk * 2, kIdescQK64, kk > 0, ~0u, 0u);
+        }
         unsigned long long* const done = &ctl->sdp_full[buf];
         if (++buf == kBufs) buf = 0;
-        if (++stg == kStages) { stg = 0; ph ^= 1u; }
+        if (++stg == kRing) { stg = 0; ph ^= 1u; }
         have_f = mbar_test(&ctl->full[stg], ph);
         have_e = mbar_test(&ctl->empty[old], old_ph);
-        info = ctl->info[stg];                      // (read again if the entry is not there yet)
+        info = ld_shared(&ctl->info[stg]);                      // (read again if the entry is not there yet)
         tc_commit(done);
     }
     if (fail) give_up(abort_flag, p.status, fail);
@@ -378,41 +440,48 @@ __device__ __forceinline__ void accumulate_role(const KernelParams& p, SmemCtl* 
     for (;;) {
         if (!have_f) {
             if (!mbar_wait(&ctl->full[stg], ph, abort_flag)) { fail = 125; break; }
-            info = ctl->info[stg];
+            info = ld_shared(&ctl->info[stg]);
         }
         if (info & kInfoEnd) break;
         // the epilogue must have taken the previous tile's accumulators before this tile's first product overwrites them
         if ((info & kInfoFirst) && acc_n > 0 && !mbar_wait(&ctl->acc_free, (acc_n - 1) & 1u, abort_flag)) { fail = 127; break; }
         if (!have_p && !mbar_wait(&ctl->p_full[buf], par, abort_flag)) { fail = 122; break; }
         tc_fence_after();
-        const unsigned y1 = ring0 + stg * kStageDesc, y2 = y1 + kTileDesc;
         const unsigned keep = (info & kInfoFirst) ? 0u : 1u;
-        unsigned a = tmem + buf * kBufCols;
-        // 16 tokens per MMA: 8 packed columns of A (the high halves, then the low halves), two 8-row groups of Y
-        if (info & kInfoDkv) {
+        unsigned y1 = ring0 + ((info >> kInfoStage) & 15u) * kStageDesc, skip_upper = 0u, skip_lower = (info & kInfoShared) ? ~0u : 0u;
+#pragma unroll 1
+        for (;;) {                                  // a shared step: the upper half's block, then the lower half's, each for its lanes
+            unsigned a = tmem + buf * kBufCols;
+            // 16 tokens per MMA: 8 packed columns of A (the high halves, then the low halves), two 8-row groups of Y
+            if (info & kInfoDkv) {
+                const unsigned y2 = y1 + kTileDesc;
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                    mma_ts_half(acc + 64, a + kk * 16, y2 + ((kk * 2048) >> 4), kIdescPV, kk > 0 ? 1u : keep, skip_upper, skip_lower);
+                    mma_ts_half(acc + 64, a + kk * 16 + 8, y2 + ((kk * 2048) >> 4), kIdescPV, 1u, skip_upper, skip_lower);
+                }
+                a += 64;
+            }
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
-                mma_ts_lo(acc + 64, a + kk * 16, y2 + ((kk * 2048) >> 4), kIdescPV, kk > 0 ? 1u : keep);
-                mma_ts_lo(acc + 64, a + kk * 16 + 8, y2 + ((kk * 2048) >> 4), kIdescPV, 1u);
+                mma_ts_half(acc, a + kk * 16, y1 + ((kk * 2048) >> 4), kIdescPV, kk > 0 ? 1u : keep, skip_upper, skip_lower);
+                mma_ts_half(acc, a + kk * 16 + 8, y1 + ((kk * 2048) >> 4), kIdescPV, 1u, skip_upper, skip_lower);
             }
-            a += 64;
-        }
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-            mma_ts_lo(acc, a + kk * 16, y1 + ((kk * 2048) >> 4), kIdescPV, kk > 0 ? 1u : keep);
-            mma_ts_lo(acc, a + kk * 16 + 8, y1 + ((kk * 2048) >> 4), kIdescPV, 1u);
+            if (!skip_lower) break;
+            y1 = ring0 + ((info >> (kInfoStage + 4)) & 15u) * kStageDesc;
+            skip_upper = ~0u;
+            skip_lower = 0u;
         }
         const unsigned now = info;
         unsigned long long* const done = &ctl->empty[stg];
         if (++buf == kBufs) { buf = 0; par ^= 1u; }
-        if (++stg == kStages) { stg = 0; ph ^= 1u; }
+        if (++stg == kRing) { stg = 0; ph ^= 1u; }
         have_f = mbar_test(&ctl->full[stg], ph);
         have_p = mbar_test(&ctl->p_full[buf], par);
-        info = ctl->info[stg];                      // (read again if the entry is not there yet)
+        info = ld_shared(&ctl->info[stg]);                      // (read again if the entry is not there yet)
         tc_commit(done);
-        if (now & kInfoLast) {                      // (the tile's scores and elementwise work are done as well: its rows may go)
+        if (now & kInfoLast) {                      // (the tile's scores and elementwise work are done as well)
             tc_commit(&ctl->acc_full);
-            tc_commit(&ctl->x_empty[(now & kInfoX) ? 1 : 0]);
             ++acc_n;
         }
     }
@@ -503,17 +572,19 @@ __device__ __forceinline__ void elementwise_role(const KernelParams& p, SmemCtl*
     int* abort_flag = &ctl->abort_flag;
     const unsigned g = (unsigned)warp >> 2;         // warpgroup = score buffer
     const int row = (warp & 3) * 32 + lane;
-    const unsigned other = row >= kBlock ? kUpperHalf : kLowerHalf;
+    const unsigned half_shift = row >= kBlock ? 3 : 0;
+    static_assert(kLower == 8, "");
     const unsigned buf = tmem + ((unsigned)((warp & 3) * 32) << 16) + g * kBufCols;
     const float* x_stats = &ctl->x_stats[0][row >= kBlock][row & (kBlock - 1)];
     unsigned stage = g, par = 0, full_par = 0;      // par: of this buffer's use; the ring has twice as many entries as there are buffers
     int fail = 0;
     for (;;) {
         if (!mbar_wait(&ctl->full[stage], full_par, abort_flag)) { fail = 132; break; }
-        const unsigned info = ctl->info[stage];
+        const unsigned info = ld_shared(&ctl->info[stage]);
         if (info & kInfoEnd) break;
         const bool dkv = info & kInfoDkv;
-        const bool mine = (info & kInfoWho) != other;       // warp-uniform
+        const unsigned half = (info >> half_shift) & 7u;        // warp-uniform
+        const bool mine = half & kAttends, second = half & kSecond;
         float nl = 0.f, nd = 0.f;
         if (!dkv) {
             const unsigned xs = (info & kInfoX) ? 1u : 0u;
@@ -524,7 +595,7 @@ __device__ __forceinline__ void elementwise_role(const KernelParams& p, SmemCtl*
         if (!mbar_wait(&ctl->sdp_full[g], par, abort_flag)) { fail = 131; break; }
         __syncwarp();                               // lanes leave the wait one by one
         tc_fence_after();
-        if (__builtin_expect((info & kInfoPadded) != 0, 0) && mine) mask_scores(buf, ctl->bits[stage]);
+        if (__builtin_expect((half & kPadded) != 0, 0)) mask_scores(buf, ctl->bits[stage][second]);
         if (!mine) {
             tmem_st32_zero(buf);
             tmem_st32_zero(buf + 32);
@@ -533,7 +604,7 @@ __device__ __forceinline__ void elementwise_role(const KernelParams& p, SmemCtl*
                 tmem_st32_zero(buf + 96);
             }
         } else if (dkv) {
-            const float2* st = reinterpret_cast<const float2*>(ctl->y_stats[stage]);
+            const float2* st = reinterpret_cast<const float2*>(ctl->y_stats[(info >> (kInfoStage + (second ? 4 : 0))) & 15u]);
             dkv_columns(buf, p.scale_log2, st, st + 32);
         } else {
             dq_columns(buf, p.scale_log2, nl, nd);
@@ -598,8 +669,7 @@ __device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ct
     const int quad = warp & 3, row = quad * 32 + lane, r64 = row & (kBlock - 1);
     const bool lower = row >= kBlock;
     const unsigned acc = tmem + ((unsigned)(quad * 32) << 16) + kColAcc;
-    unsigned char* const stage = smem + kSmemOut;   // [accumulator][half of the tile]: 64 x 64 bf16, swizzled
-    const unsigned my_row = smem_u32(stage) + (lower ? kTileBytes : 0) + r64 * 128;
+    const unsigned my_row = (lower ? kTileBytes : 0) + r64 * 128;     // of a 128 x 64 bf16 tile, swizzled
     unsigned slot_n = 0, acc_n = 0, sync_n = 0;
     bool have = false;                              // has the tile had any step
     int fail = 0;
@@ -618,13 +688,28 @@ __device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ct
             if (!BB_CHECK(slot->bh >= 0 && slot->bh < p.BH && slot->ra >= 0 && slot->ra < p.nb && slot->rb < p.nb &&
                           split < 2 * p.BH * p.global_tiles && slot->part >= 0 && slot->part < p.parts, 174)) break;
             const bool row_ok = ((lower ? slot->rbits_b : slot->rbits_a) >> r64) & 1ull;
-            if (row == 0) bulk_wait_read();         // the previous tile has left the staging tiles
-            if (!epilogue_sync(ctl, sync_n)) { fail = 142; break; }
+            if (!have && split < 0) {               // no steps, so no row buffer either: zeros, straight to the rows
+                const int blk = lower ? slot->rb : slot->ra;
+                if (blk >= 0)
+#pragma unroll 1
+                    for (int m = 0; m < (dkv ? 2 : 1); ++m) {
+                        uint4* dst = reinterpret_cast<uint4*>((dkv ? (m ? p.dv : p.dk) : p.dq) + (((size_t)slot->bh * p.nb + blk) * kBlock + r64) * kBlock);
+#pragma unroll 1
+                        for (int j = 0; j < 8; ++j) dst[j] = make_uint4(0u, 0u, 0u, 0u);
+                    }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&ctl->slot_empty[ss]);
+                ++slot_n;
+                continue;
+            }
+            const unsigned xs = acc_n & 1u;
+            unsigned char* const stage = smem + kSmemX + xs * 4 * kTileBytes;     // the tile's row buffer has been read: [accumulator][half of the tile]
             if (have) {
                 if (!mbar_wait(&ctl->acc_full, acc_n & 1u, abort_flag)) { fail = 141; break; }
                 __syncwarp();
                 tc_fence_after();
                 ++acc_n;
+                if (split >= 0 && row == 0) mbar_arrive(&ctl->x_empty[xs]);
             }
             float* part = p.partials + ((size_t)max(split, 0) * p.parts + slot->part) * kPartialFloats + row * kBlock;
 #pragma unroll 1
@@ -647,7 +732,7 @@ __device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ct
                     // A padded row is zeroed by a select and not by a factor: a padded key takes part like any other up to here, and
                     // since its scores are not in lse, its sums may be infinite or NaN.
                     const float f = m ? 1.f : p.scale;
-                    const unsigned base = my_row + m * 2 * kTileBytes;
+                    const unsigned base = smem_u32(stage) + my_row + m * 2 * kTileBytes;
                     unsigned w[8];
 #pragma unroll
                     for (int j = 0; j < 8; ++j) w[j] = row_ok ? pack_bf16(o[2 * j] * f, o[2 * j + 1] * f) : 0u;
@@ -670,6 +755,8 @@ __device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ct
                         if (two) tma_store_tile(tm_dv, rb, stage + 3 * kTileBytes);
                     }
                     bulk_commit();
+                    bulk_wait_read();               // the row buffer may be filled again
+                    mbar_arrive(&ctl->x_empty[xs]);
                 }
             } else {
                 __threadfence();
@@ -702,7 +789,7 @@ attn_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;      // (uniform, and known to be)
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kStages; ++i) { mbar_init(&ctl->full[i], 1); mbar_init(&ctl->empty[i], 1); }
+        for (int i = 0; i < kRing; ++i) { mbar_init(&ctl->full[i], 1); mbar_init(&ctl->empty[i], 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(&ctl->x_full[i], 1); mbar_init(&ctl->x_empty[i], 1); }
         for (int i = 0; i < kBufs; ++i) { mbar_init(&ctl->sdp_full[i], 1); mbar_init(&ctl->p_full[i], 128); }
         mbar_init(&ctl->acc_full, 1);

@@ -85,3 +85,28 @@ def test_streams_that_end_with_a_tile_of_one_step():
             fwd(q, k, v, L, mask, out, lse, 0.125)
             assert status()[0] == 0
     L.close()
+
+
+@pytest.mark.parametrize("shape", [(9, 1, 1, 0, 0), (33, 3, 0, 5, 0), (24, 5, 3, 0, 1), (120, 101, 2, 3, 0), (16, 3, 2, 40, 0)],
+                         ids=lambda s: "nb%d_w%d_g%d_r%d_mode%d" % s)
+@pytest.mark.parametrize("padded", [False, True])
+def test_gradients_of_steps_that_the_halves_of_a_tile_share(shape, padded):
+    """Tiles whose halves have equally many blocks of their own, unequally many or none, and lists longer than a posted segment."""
+    nb, w, g, r, mode = shape
+    B, H, N = 2, 2, nb * 64
+    gen = torch.Generator(device="cuda").manual_seed(nb)
+    q, k, v, dout = (torch.randn((B, H, N, 64), generator=gen, device="cuda").to(torch.bfloat16) for _ in range(4))
+    lens = np.array([N - 70, max(1, N // 3)])
+    mask = torch.from_numpy((np.arange(N)[None] < lens[:, None]).astype(np.uint8)).cuda() if padded else None
+    L = bb.bigbird_build_layout(N, 64, w, g, r, 5, H, mode)
+    out, lse = torch.empty_like(q), torch.empty((B, H, N), device="cuda")
+    bb.bigbird_attn_fwd(q, k, v, L, mask, out, lse, 0.125)
+    grads = [torch.full_like(q, float("nan")) for _ in range(3)]
+    bb.bigbird_attn_bwd(q, k, v, out, lse, dout, L, mask, *grads, 0.125)
+    assert bb.bigbird_last_status()[0] == 0
+    f = [t.float() for t in (q, k, v, out, dout)]
+    want = [torch.empty_like(f[0]) for _ in range(3)]
+    bb.bigbird_attn_bwd(f[0], f[1], f[2], f[3], lse, f[4], L, mask, *want, 0.125)
+    for x, y in zip(grads, want):               # the bound of the test above
+        assert torch.linalg.norm((x.float() - y).double()) <= (2.0 ** -8 + 5e-4) * torch.linalg.norm(y.double())
+    L.close()
