@@ -26,7 +26,7 @@ struct BwdShape {
 
 // dynamic shared memory: X1, X2 [rows][LD] | Y1, Y2 [KC][LD] | P [rows][LDP] | bias, -delta of the rows
 template <typename T, int D, int TM, bool kDkv>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(max_threads(TM), 2)
 attn_bwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, const T* __restrict__ out,
                      const float* __restrict__ lse, const T* __restrict__ dout, const int32_t* __restrict__ ptr, const int32_t* __restrict__ idx,
                      const uint8_t* __restrict__ kpm, T* __restrict__ g0, T* __restrict__ g1, float* __restrict__ minus_delta, Tiling tiling,
@@ -201,7 +201,7 @@ attn_bwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* 
 template <typename T, int D, int TM, bool kDkv>
 cudaError_t launch_one(const BwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, int sms, float* minus_delta) {
     static std::once_flag once[64];
-    const cudaError_t e = allow_smem((const void*)attn_bwd_simt_kernel<T, D, TM, kDkv>, BwdShape<D>::smem(16 * TM), once);
+    const cudaError_t e = allow_smem((const void*)attn_bwd_simt_kernel<T, D, TM, kDkv>, BwdShape<D>::smem(max_threads(TM) / 16 * TM), once);
     if (e != cudaSuccess) return e;
     const Shape s = make_shape(TM, L, dl, a.B * a.H, 2 * sms, BwdShape<D>::KC);
     return launch_clusters(attn_bwd_simt_kernel<T, D, TM, kDkv>, s, BwdShape<D>::smem(s.threads / 16 * TM), a.stream, (const T*)a.q, (const T*)a.k,
@@ -217,8 +217,10 @@ template <typename T, int D>
 cudaError_t launch_d(const BwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, int sms, float* ws) {
     const int tm = rows_per_thread(L, a.B * a.H, D, 2 * sms);
     if (tm == 2) return launch_tm<T, D, 2>(a, L, dl, sms, ws);
-    if constexpr (D <= 64)
+    if constexpr (D <= 64) {
         if (tm == 6) return launch_tm<T, D, 6>(a, L, dl, sms, ws);
+        if (tm == 7) return launch_tm<T, D, 7>(a, L, dl, sms, ws);
+    }
     return launch_tm<T, D, 4>(a, L, dl, sms, ws);
 }
 template <typename T>

@@ -5,8 +5,8 @@
 // the 16 threads that share a row, probabilities to shared memory (read back by the same 16 threads), output sums in registers.
 // The next chunk's K is on its way while the probabilities and sums are made; its V is requested when the sums are done, and both
 // are waited for at the top of the chunk.  See simt.cuh for the tile shapes and for how clusters share the long tiles.
-// Bound by the FMA pipes.  Measured (a warp per row before, no reuse of K and V in registers): [2, 12, 52 x 84, 64] with three
-// global blocks 3740 -> 655 us, [2, 8, 2560, 128] padded 1547 -> 307 us, [1, 2, 512, 64] 22.6 -> 13.8 us (18.5 with four rows per
+// Bound by shared-memory latency and the FMA pipes.  Measured (a warp per row before, no reuse of K and V in registers): [2, 12, 52 x 84,
+// 64] with three global blocks 3740 -> 655 us, [2, 8, 2560, 128] padded 1547 -> 302 us, [1, 2, 512, 64] 22.6 -> 13.8 us (18.5 with four rows per
 // thread and launches that wait for the kernel in front to drain).
 #include "simt.cuh"
 
@@ -37,7 +37,7 @@ __device__ __noinline__ void zero_padded(float* sv, const uint8_t* svalid) {
 
 // dynamic shared memory: Q [rows][LD] | K [KC][LD] | P [rows][LDP] (in K's place for D = 128) | V [KC][D]
 template <typename T, int D, int TM>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(max_threads(TM), 2)
 attn_fwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, const int32_t* __restrict__ row_ptr,
                      const int32_t* __restrict__ col_idx, const uint8_t* __restrict__ kpm, T* __restrict__ out, float* __restrict__ lse,
                      Tiling tiling, int64_t N, float scale) {
@@ -196,7 +196,7 @@ attn_fwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* 
 template <typename T, int D, int TM>
 cudaError_t launch_tm(const FwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, int sms) {
     static std::once_flag once[64];
-    const cudaError_t e = allow_smem((const void*)attn_fwd_simt_kernel<T, D, TM>, FwdShape<D>::smem(16 * TM), once);
+    const cudaError_t e = allow_smem((const void*)attn_fwd_simt_kernel<T, D, TM>, FwdShape<D>::smem(max_threads(TM) / 16 * TM), once);
     if (e != cudaSuccess) return e;
     const Shape s = make_shape(TM, L, dl, a.B * a.H, 2 * sms, FwdShape<D>::KC);
     return launch_clusters(attn_fwd_simt_kernel<T, D, TM>, s, FwdShape<D>::smem(s.threads / 16 * TM), a.stream, (const T*)a.q, (const T*)a.k, (const T*)a.v,
@@ -206,8 +206,10 @@ template <typename T, int D>
 cudaError_t launch_d(const FwdArgs& a, const bigbird_layout& L, const DeviceLayout& dl, int sms) {
     const int tm = rows_per_thread(L, a.B * a.H, D, 2 * sms);
     if (tm == 2) return launch_tm<T, D, 2>(a, L, dl, sms);
-    if constexpr (D <= 64)
+    if constexpr (D <= 64) {
         if (tm == 6) return launch_tm<T, D, 6>(a, L, dl, sms);
+        if (tm == 7) return launch_tm<T, D, 7>(a, L, dl, sms);
+    }
     return launch_tm<T, D, 4>(a, L, dl, sms);
 }
 template <typename T>
