@@ -31,7 +31,7 @@
 // the same from one elected thread 557, columns 16 at a time with the next 16 on their way 527, two issuing threads 505, all
 // roles on the ring, tests ahead of the commits and rows written by TMA 497 us ([1, 12, 16384, 64] with 13000 valid tokens
 // 338 -> 193 us from the second of these to the last), and 189 with the parts of a cut tile fetched together ([2, 12, 1024]
-// 54 -> 39.5 us, there no longer cut); 430 us at full clocks.  A step takes 1400 cycles; its MMAs need 640 of the tensor pipe
+// 54 -> 39.5 us, there no longer cut); 430 us at full clocks.  A step took 1400 cycles then; its MMAs need 640 of the tensor pipe
 // (51% of the launch by its counter, 555 steps per SM), without any elementwise work it takes 1100, without any MMAs 1150: what is
 // left is the way of a step through the hands of four warps with three steps in flight, which is all that tensor memory holds.  Two
 // threads per row (24 warps) were no faster.
