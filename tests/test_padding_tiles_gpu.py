@@ -87,6 +87,29 @@ def test_streams_that_end_with_a_tile_of_one_step():
     L.close()
 
 
+@pytest.mark.parametrize("entry", ["fwd", "static"])
+def test_parts_without_tokens_leave_nothing_of_their_scratch(entry):
+    """Tiles of global blocks that are cut into parts and hold no token: nothing is written for such a part, and the merge must not let
+    through what an earlier call left in its place."""
+    B, H, nb = 1, 2, 70
+    N = nb * 64
+    L = bb.bigbird_build_layout(N, 64, 3, 4, 3, 5, H, 1)
+    fwd = bb.bigbird_attn_fwd if entry == "fwd" else bb.bigbird_attn_fwd_static
+    q, k, v = (torch.randn((B, H, N, 64), device="cuda").to(torch.bfloat16) for _ in range(3))
+    mask = torch.ones((B, N), dtype=torch.uint8, device="cuda")
+    res = []
+    for dirty in (q, torch.full_like(q, float("nan")), q * 1e19):       # what the earlier call computes: sums, NaN, infinities
+        out, lse = torch.full_like(q, float("nan")), torch.full((B, H, N), float("nan"), device="cuda")
+        mask.fill_(1)
+        fwd(dirty, dirty, v, L, mask, out, lse, 0.125)
+        mask[:, :128] = 0                                                # the first pair of global blocks
+        fwd(q, k, v, L, mask, out, lse, 0.125)
+        assert (out[:, :, :128] == 0).all() and (lse[:, :, :128] == -math.inf).all() and torch.isfinite(out.float()).all()
+        res.append((out, lse))
+    assert all(torch.equal(x, y) for r in res[1:] for x, y in zip(r, res[0]))
+    L.close()
+
+
 @pytest.mark.parametrize("shape", [(9, 1, 1, 0, 0), (33, 3, 0, 5, 0), (24, 5, 3, 0, 1), (120, 101, 2, 3, 0), (16, 3, 2, 40, 0)],
                          ids=lambda s: "nb%d_w%d_g%d_r%d_mode%d" % s)
 @pytest.mark.parametrize("padded", [False, True])
