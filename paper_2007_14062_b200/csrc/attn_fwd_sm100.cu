@@ -962,8 +962,11 @@ void set_shape(KernelParams& p, const bigbird_layout& L, int B, Cut cut, float s
     p.total_work = p.BH * (L.global_tiles * cut.parts + L.sparse_tiles_per_head);
     // Tiles that a stream has in hand are not drawn by another one that runs dry, so with few tiles in all it should have few: [1, 12,
     // 16384] with 13000 tokens (5 tiles per stream) 75 us with three, 69 with two; [16, 16, 4096] ragged (28, many of them without a
-    // token) 204 and 210; [8, 12, 4096] (10) 125 with either.
-    p.ahead = p.total_work < 8 * kStreams * sm_count ? 2 : kSchedSlots;
+    // token) 204 and 210; [8, 12, 4096] (10) 125 with either.  A tile with a list of five key blocks or less, though, is over before the
+    // scheduler has another, so there only fewer than four count as few: [4, 12, 4096] (5.2 tiles per stream) with lists of three 43.9
+    // us with three, 45.8 with two, but with lists of eight 71.8 and 67.0; [4, 16, 2048] (3.5) with lists of five 44.1 and 40.5.
+    const int64_t lists = (int64_t)L.steps.size() - (int64_t)L.H * L.global_tiles * L.nb, tiles = (int64_t)L.H * L.sparse_tiles_per_head;
+    p.ahead = p.total_work < (2 * lists > 11 * tiles ? 8 : 4) * kStreams * sm_count ? 2 : kSchedSlots;
     p.scale_log2 = scale * 1.4426950408889634f;
 }
 
