@@ -37,8 +37,9 @@
 // threads per row (24 warps) were no faster.
 //
 // With shared steps [8, 12, 4096] takes 419 us at full clocks (430 with a step for each block) and forward and gradients together 628
-// instead of 646 under the power cap; a shared step takes two places in the ring of Y, for which a tile's results leave through its own
-// row buffer and no longer through one of their own.
+// instead of 646 under the power cap.  A shared step takes two of the seven places in the ring of Y.  (Nine of them, for which a tile's
+// results left through its own row buffer, were no faster there, and the tile after next waited for that buffer: [8, 12, 4224] ETC 359 us
+// against 345 under the power cap, [1, 2, 384] 13.5 against 13.35.)
 //
 // A first kernel makes, per query row, -lse * log2 e (-inf for rows without probabilities) and -delta, packs the key-padding
 // mask and zeroes the counters.
@@ -51,7 +52,7 @@ namespace {
 
 constexpr int kBufs = 3;                   // score buffers, each served by one warpgroup
 constexpr int kRing = 2 * kBufs;           // ring of steps
-constexpr int kStages = 9;                 // ring of Y1 | Y2 pairs: one for a step, two if the halves of the tile share it
+constexpr int kStages = 7;                 // ring of Y1 | Y2 pairs: one for a step, two if the halves of the tile share it
 constexpr int kSlots = 3;                  // tiles (or segments of long ones) posted by the scheduler (two: [3, 16, 4096] ragged, forward and
                                            // gradients, 212.5 us against 209.2)
 constexpr int kSegSteps = 64;              // steps per posted segment, at least 33
@@ -111,9 +112,10 @@ struct __align__(16) SmemCtl {
     int abort_flag;
     int merge_last;
 };
-constexpr int kSmemX = 0;                                      // two buffers of X1a X1b X2a X2b; the tile's results leave through its own
+constexpr int kSmemX = 0;                                      // two buffers of X1a X1b X2a X2b
 constexpr int kSmemRing = 2 * 4 * kTileBytes;
-constexpr int kSmemCtl = kSmemRing + kStages * 2 * kTileBytes;
+constexpr int kSmemOut = kSmemRing + kStages * 2 * kTileBytes;    // four tiles on their way out
+constexpr int kSmemCtl = kSmemOut + 4 * kTileBytes;
 constexpr int kSmemBytes = kSmemCtl + (int)sizeof(SmemCtl) + 1024;   // + slack for the 1024-byte alignment
 static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
 
@@ -480,8 +482,9 @@ __device__ __forceinline__ void accumulate_role(const KernelParams& p, SmemCtl* 
         have_p = mbar_test(&ctl->p_full[buf], par);
         info = ld_shared(&ctl->info[stg]);                      // (read again if the entry is not there yet)
         tc_commit(done);
-        if (now & kInfoLast) {                      // (the tile's scores and elementwise work are done as well)
+        if (now & kInfoLast) {                      // (the tile's scores and elementwise work are done as well: its rows may go)
             tc_commit(&ctl->acc_full);
+            tc_commit(&ctl->x_empty[(now & kInfoX) ? 1 : 0]);
             ++acc_n;
         }
     }
@@ -669,7 +672,8 @@ __device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ct
     const int quad = warp & 3, row = quad * 32 + lane, r64 = row & (kBlock - 1);
     const bool lower = row >= kBlock;
     const unsigned acc = tmem + ((unsigned)(quad * 32) << 16) + kColAcc;
-    const unsigned my_row = (lower ? kTileBytes : 0) + r64 * 128;     // of a 128 x 64 bf16 tile, swizzled
+    unsigned char* const stage = smem + kSmemOut;   // [accumulator][half of the tile]: 64 x 64 bf16, swizzled
+    const unsigned my_row = smem_u32(stage) + (lower ? kTileBytes : 0) + r64 * 128;
     unsigned slot_n = 0, acc_n = 0, sync_n = 0;
     bool have = false;                              // has the tile had any step
     int fail = 0;
@@ -688,28 +692,14 @@ __device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ct
             if (!BB_CHECK(slot->bh >= 0 && slot->bh < p.BH && slot->ra >= 0 && slot->ra < p.nb && slot->rb < p.nb &&
                           split < 2 * p.BH * p.global_tiles && slot->part >= 0 && slot->part < p.parts, 174)) break;
             const bool row_ok = ((lower ? slot->rbits_b : slot->rbits_a) >> r64) & 1ull;
-            if (!have && split < 0) {               // no steps, so no row buffer either: zeros, straight to the rows
-                const int blk = lower ? slot->rb : slot->ra;
-                if (blk >= 0)
-#pragma unroll 1
-                    for (int m = 0; m < (dkv ? 2 : 1); ++m) {
-                        uint4* dst = reinterpret_cast<uint4*>((dkv ? (m ? p.dv : p.dk) : p.dq) + (((size_t)slot->bh * p.nb + blk) * kBlock + r64) * kBlock);
-#pragma unroll 1
-                        for (int j = 0; j < 8; ++j) dst[j] = make_uint4(0u, 0u, 0u, 0u);
-                    }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&ctl->slot_empty[ss]);
-                ++slot_n;
-                continue;
-            }
-            const unsigned xs = acc_n & 1u;
-            unsigned char* const stage = smem + kSmemX + xs * 4 * kTileBytes;     // the tile's row buffer has been read: [accumulator][half of the tile]
+            // (a tile without a step is a part of a split one: one of its rows is a token, and a block is in its own list)
+            if (row == 0) bulk_wait_read();         // the previous tile has left the staging tiles
+            if (!epilogue_sync(ctl, sync_n)) { fail = 142; break; }
             if (have) {
                 if (!mbar_wait(&ctl->acc_full, acc_n & 1u, abort_flag)) { fail = 141; break; }
                 __syncwarp();
                 tc_fence_after();
                 ++acc_n;
-                if (split >= 0 && row == 0) mbar_arrive(&ctl->x_empty[xs]);
             }
             float* part = p.partials + ((size_t)max(split, 0) * p.parts + slot->part) * kPartialFloats + row * kBlock;
 #pragma unroll 1
@@ -732,7 +722,7 @@ __device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ct
                     // A padded row is zeroed by a select and not by a factor: a padded key takes part like any other up to here, and
                     // since its scores are not in lse, its sums may be infinite or NaN.
                     const float f = m ? 1.f : p.scale;
-                    const unsigned base = smem_u32(stage) + my_row + m * 2 * kTileBytes;
+                    const unsigned base = my_row + m * 2 * kTileBytes;
                     unsigned w[8];
 #pragma unroll
                     for (int j = 0; j < 8; ++j) w[j] = row_ok ? pack_bf16(o[2 * j] * f, o[2 * j + 1] * f) : 0u;
@@ -755,8 +745,6 @@ __device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ct
                         if (two) tma_store_tile(tm_dv, rb, stage + 3 * kTileBytes);
                     }
                     bulk_commit();
-                    bulk_wait_read();               // the row buffer may be filled again
-                    mbar_arrive(&ctl->x_empty[xs]);
                 }
             } else {
                 __threadfence();
