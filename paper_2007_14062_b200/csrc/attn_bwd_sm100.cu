@@ -13,10 +13,11 @@
 // two bf16 numbers (16 significant bits): the products keep the precision of the fp32 path to below the rounding of the
 // results, at twice the number of the accumulating MMAs.
 //
-// A block of the column side that only the upper rows of a tile attend shares a step with one that only the lower rows attend: each has
-// its products with all 128 rows, the second ones leaving the lanes of the upper half alone (the instruction's vector of disabled lanes).
-// The products are as many as if the two had a step of their own, but the way of a step through the hands of four warps is gone once and
-// not twice: 6312 steps instead of 8740 for the sparse tiles of the base layout, 12 heads, both kinds.
+// In the kernel's form for layouts with many of them (kShare), a block of the column side that only the upper rows of a tile attend shares
+// a step with one that only the lower rows attend: each has its products with all 128 rows, the second ones leaving the lanes of the upper
+// half alone (the instruction's vector of disabled lanes).  The products are as many as if the two had a step of their own, but the way of
+// a step through the hands of four warps is gone once and not twice: 6312 steps instead of 8740 for the sparse tiles of the base layout,
+// 12 heads, both kinds.
 //
 // Nothing carries over from step to step but the accumulators, so the steps of a tile are dealt in turn to three warpgroups
 // with a 128-column score buffer each.  One thread issues the scores of a step as soon as its buffer is free, another the
@@ -37,7 +38,7 @@
 // threads per row (24 warps) were no faster.
 //
 // With shared steps [8, 12, 4096] takes 419 us at full clocks (430 with a step for each block) and forward and gradients together 628
-// instead of 646 under the power cap.  A shared step takes two of the seven places in the ring of Y.  (Nine of them, for which a tile's
+// instead of 646 under the power cap; the launch says which layouts gain.  A shared step takes two of the seven places in the ring of Y.  (Nine of them, for which a tile's
 // results left through its own row buffer, were no faster there, and the tile after next waited for that buffer: [8, 12, 4224] ETC 359 us
 // against 345 under the power cap, [1, 2, 384] 13.5 against 13.35.)
 //
@@ -52,7 +53,8 @@ namespace {
 
 constexpr int kBufs = 3;                   // score buffers, each served by one warpgroup
 constexpr int kRing = 2 * kBufs;           // ring of steps
-constexpr int kStages = 7;                 // ring of Y1 | Y2 pairs: one for a step, two if the halves of the tile share it
+constexpr int kStages = 7;                 // ring of Y1 | Y2 pairs: one for a step, two if the halves of the tile share it (kShare; else step entry e has place e)
+static_assert(kRing <= kStages, "a place for each step");
 constexpr int kSlots = 3;                  // tiles (or segments of long ones) posted by the scheduler (two: [3, 16, 4096] ragged, forward and
                                            // gradients, 212.5 us against 209.2)
 constexpr int kSegSteps = 64;              // steps per posted segment, at least 33
@@ -72,7 +74,7 @@ constexpr int kStatFloats = 2 * kBlock;    // per block of query rows: 64 x (-ls
 constexpr int kPartialFloats = 2 * 128 * kBlock;   // one part of a split tile: acc0, acc1
 enum { kDkv = 0, kDq = 1 };
 enum { kSegFirst = 1, kSegLast = 2 };
-// A step: one block that both halves of the tile attend or only one of them, or (kSecond) one for the upper half and another for the
+// A step: one block that both halves of the tile attend or only one of them, or (kShare, kSecond) one for the upper half and another for the
 // lower, whose rows are computed with 128-row products that leave the lanes of the other half alone.
 enum { kAttends = 1, kPadded = 2, kSecond = 4 };        // of a half: it attends the step; some of its block's tokens are padding; its block is c1
 // what there is to know about a ring entry: the halves (kLower times the lower one's bits), kind, first and last step of its tile, the
@@ -81,10 +83,13 @@ enum { kLower = 8, kInfoShared = kSecond * kLower, kInfoDkv = 64, kInfoFirst = 1
 constexpr int kInfoStage = 12;
 static_assert(kStages <= 16, "bits of a place");
 
-struct __align__(16) StepEntry {
-    int c0, c1;                    // blocks of the column side; c1 < 0: none
-    int half[2];                   // kAttends, kPadded, kSecond of the upper and the lower half
-    unsigned long long kb[2];      // valid-token bits of c0 and c1 (never 0)
+struct __align__(16) StepPart {
+    int c;                         // block of the column side
+    int halves;                    // kAttends, kPadded, kSecond of the upper half, and kLower times those of the lower
+    unsigned long long kb;         // valid-token bits of the block (never 0)
+};
+struct StepEntry {
+    StepPart part[2];              // kShare: part[1].c < 0 if there is one block only; else part[0] alone is used
 };
 struct __align__(16) TileSlot {
     int w;                         // work index, -1 = no more work
@@ -152,6 +157,7 @@ __device__ __forceinline__ void clear_block(__nv_bfloat16* g, size_t block, int 
     for (int i = 0; i < 16; ++i) dst[32 * i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
+template <bool kShare>
 __device__ __forceinline__ void scheduler_role(const KernelParams& p, SmemCtl* ctl, int lane) {
     const unsigned lt_mask = (1u << lane) - 1u;
     unsigned slot_n = 0;
@@ -231,31 +237,27 @@ __device__ __forceinline__ void scheduler_role(const KernelParams& p, SmemCtl* c
                     ua = s.who != kLowerHalf && rbits_a != 0ull && kb != 0ull;
                     ub = s.who != kUpperHalf && rbits_b != 0ull && kb != 0ull;
                 }
-                // In turn a block of both halves and one of the upper half together with one of the lower (what is left of either
-                // by itself): steps of one and of two blocks alternate, so that the ring holds the same number of steps at any time.
-                const unsigned b_both = __ballot_sync(0xffffffffu, ua && ub), b_up = __ballot_sync(0xffffffffu, ua && !ub),
-                               b_lo = __ballot_sync(0xffffffffu, ub && !ua);
-                const int n_both = __popc(b_both), n_up = __popc(b_up), n_lo = __popc(b_lo), n_one = max(n_up, n_lo);
-                if (ua || ub) {
-                    const int rank = __popc((ua ? (ub ? b_both : b_up) : b_lo) & lt_mask);
-                    const int at = ua && ub ? (rank < n_one ? 2 * rank : n_one + rank) : (rank < n_both ? 2 * rank + 1 : n_both + rank);
-                    const bool second = !ua && rank < n_up;
-                    const int flags = kAttends | (kb != ~0ull ? kPadded : 0);
-                    StepEntry* e = &slot->steps[count + at];
-                    e->kb[second ? 1 : 0] = kb;
-                    if (second) {
-                        e->c1 = c;
-                        e->half[1] = flags | kSecond;
-                    } else {
-                        e->c0 = c;
-                        e->half[0] = ua ? flags : 0;
-                        if (ub || rank >= n_lo) {
-                            e->c1 = -1;
-                            e->half[1] = ub ? flags : 0;
-                        }
+                const int flags = kAttends | (kb != ~0ull ? kPadded : 0), halves = (ua ? flags : 0) | (ub ? flags * kLower : 0);
+                if constexpr (kShare) {
+                    // In turn a block of both halves and one of the upper half together with one of the lower (what is left of either
+                    // by itself): steps of one and of two blocks alternate, so that the ring holds the same number of steps at any time.
+                    const unsigned b_both = __ballot_sync(0xffffffffu, ua && ub), b_up = __ballot_sync(0xffffffffu, ua && !ub),
+                                   b_lo = __ballot_sync(0xffffffffu, ub && !ua);
+                    const int n_both = __popc(b_both), n_up = __popc(b_up), n_lo = __popc(b_lo), n_one = max(n_up, n_lo);
+                    if (ua || ub) {
+                        const int rank = __popc((ua ? (ub ? b_both : b_up) : b_lo) & lt_mask);
+                        const int at = rank + (ua && ub ? min(rank, n_one) : min(rank + 1, n_both));
+                        const bool second = !ua && rank < n_up, alone = !second && (ub || rank >= n_lo);
+                        StepPart* part = slot->steps[count + at].part;
+                        part[second ? 1 : 0] = StepPart{c, halves | (second ? kSecond * kLower : 0), kb};
+                        if (alone) part[1] = StepPart{-1, 0, 0ull};
                     }
+                    count += n_both + n_one;
+                } else {
+                    const unsigned bal = __ballot_sync(0xffffffffu, ua || ub);
+                    if (ua || ub) slot->steps[count + __popc(bal & lt_mask)].part[0] = StepPart{c, halves, kb};
+                    count += __popc(bal);
                 }
-                count += n_both + n_one;
                 i0 += 32;
             }
             __syncwarp();
@@ -285,6 +287,7 @@ __device__ __forceinline__ void scheduler_role(const KernelParams& p, SmemCtl* c
 }
 
 // ------------------------------------------------------------------------------------------------ TMA producer (one thread)
+template <bool kShare>
 __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ctl, unsigned char* smem, const CUtensorMap* tm_q,
                                               const CUtensorMap* tm_k, const CUtensorMap* tm_v, const CUtensorMap* tm_do) {
     int* abort_flag = &ctl->abort_flag;
@@ -294,6 +297,7 @@ __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ct
     int fail = 0;
     // room for a step of `blocks` blocks
     auto room = [&](unsigned blocks) -> bool {
+        if constexpr (!kShare) return mbar_wait(&ctl->empty[step_n % kRing], ((step_n / kRing) & 1u) ^ 1u, abort_flag);
         while (free_stages < blocks || step_n - done_n == (unsigned)kRing) {
             if (!mbar_wait(&ctl->empty[done_n % kRing], (done_n / kRing) & 1u, abort_flag)) return false;
             free_stages += 1u + ((shared_steps >> (done_n & 31u)) & 1u);
@@ -320,9 +324,11 @@ __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ct
         if (flags & kSegFirst) fresh = true;
         const CUtensorMap *tm1 = dkv ? tm_q : tm_k, *tm2 = dkv ? tm_do : tm_v;
         for (int i = 0; i < n; ++i) {
-            const StepEntry* e = &slot->steps[i];
-            const int c0 = e->c0, c1 = e->c1;
-            unsigned info = (unsigned)(e->half[0] | e->half[1] * kLower) | (dkv ? kInfoDkv : 0) | (i == n - 1 && (flags & kSegLast) ? kInfoLast : 0);
+            const StepPart e0 = slot->steps[i].part[0];
+            StepPart e1{-1, 0, 0ull};
+            if constexpr (kShare) e1 = slot->steps[i].part[1];
+            const int c0 = e0.c, c1 = e1.c;
+            unsigned info = (unsigned)(e0.halves | e1.halves) | (dkv ? kInfoDkv : 0) | (i == n - 1 && (flags & kSegLast) ? kInfoLast : 0);
             if (fresh) {
                 const int ra = slot->ra, rb = slot->rb;
                 const unsigned xs = tile_n & 1u;
@@ -347,13 +353,18 @@ __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ct
             if (!BB_CHECK(n <= kSegSteps && c0 >= 0 && c0 < p.nb && c1 < p.nb && (c1 >= 0) == ((info & kInfoShared) != 0), 173)) return;
             const unsigned blocks = c1 >= 0 ? 2u : 1u, g = step_n % kRing;
             if (!room(blocks)) { fail = 110; break; }
-            free_stages -= blocks;
-            const unsigned bit = 1u << (step_n & 31u);
-            shared_steps = c1 >= 0 ? shared_steps | bit : shared_steps & ~bit;
-            const unsigned next = stage + 1 == kStages ? 0u : stage + 1;
-            ctl->info[g] = info | (stage << kInfoStage) | (next << (kInfoStage + 4));
-            ctl->bits[g][0] = e->kb[0];
-            ctl->bits[g][1] = e->kb[1];
+            if constexpr (kShare) {
+                free_stages -= blocks;
+                const unsigned bit = 1u << (step_n & 31u);
+                shared_steps = c1 >= 0 ? shared_steps | bit : shared_steps & ~bit;
+                const unsigned next = stage + 1 == kStages ? 0u : stage + 1;
+                ctl->info[g] = info | (stage << kInfoStage) | (next << (kInfoStage + 4));
+                ctl->bits[g][1] = e1.kb;
+            } else {
+                ctl->info[g] = info;
+                stage = g;                          // a place for each entry
+            }
+            ctl->bits[g][0] = e0.kb;
             mbar_expect_tx(&ctl->full[g], blocks * (2 * kTileBytes + (dkv ? kStatFloats * 4 : 0)));
 #pragma unroll 1
             for (unsigned j = 0; j < blocks; ++j) {
@@ -362,7 +373,7 @@ __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ct
                 tma_load_tile(y, tm1, row * kBlock, &ctl->full[g]);
                 tma_load_tile(y + kTileBytes, tm2, row * kBlock, &ctl->full[g]);
                 if (dkv) bulk_load(ctl->y_stats[stage], p.stats + (size_t)row * kStatFloats, kStatFloats * 4, &ctl->full[g]);
-                if (++stage == kStages) stage = 0;
+                if (kShare && ++stage == kStages) stage = 0;
             }
             ++step_n;
         }
@@ -380,6 +391,7 @@ __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ct
 // that says what there is to know about the step.  full[] tells both of a loaded entry, empty[] (committed behind a step's
 // accumulation) frees the ring entry and its Y for the producer and, three steps on, the score buffer for the first thread.  The tests for
 // the next step come before a step's commit: behind it they cost four times as much.
+template <bool kShare>
 __device__ __forceinline__ void score_role(const KernelParams& p, SmemCtl* ctl, unsigned char* smem, unsigned tmem) {
     int* abort_flag = &ctl->abort_flag;
     constexpr unsigned kStageDesc = (2 * kTileBytes) >> 4, kTileDesc = kTileBytes >> 4;
@@ -406,12 +418,12 @@ __device__ __forceinline__ void score_role(const KernelParams& p, SmemCtl* ctl, 
             x1 = x0 + xs * 4 * kTileDesc;
         }
         tc_fence_after();
-        const unsigned y1 = ring0 + ((info >> kInfoStage) & 15u) * kStageDesc, d = tmem + buf * kBufCols;
+        const unsigned y1 = ring0 + (kShare ? (info >> kInfoStage) & 15u : stg) * kStageDesc, d = tmem + buf * kBufCols;
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) mma_ss_lo(d, x1 + kk * 2, y1 + kk * 2, kIdescQK64, kk > 0);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) mma_ss_lo(d + 64, x1 + 2 * kTileDesc + kk * 2, y1 + kTileDesc + kk * 2, kIdescQK64, kk > 0);
-        if (info & kInfoShared) {                   // over the lanes of the lower half: with its own block
+        if (kShare && (info & kInfoShared)) {       // over the lanes of the lower half: with its own block
             const unsigned z1 = ring0 + ((info >> (kInfoStage + 4)) & 15u) * kStageDesc;
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) mma_ss_half(d, x1 + kk * 2, z1 + kk * 2, kIdescQK64, kk > 0, ~0u, 0u);
@@ -429,6 +441,7 @@ __device__ __forceinline__ void score_role(const KernelParams& p, SmemCtl* ctl, 
     if (fail) give_up(abort_flag, p.status, fail);
 }
 
+template <bool kShare>
 __device__ __forceinline__ void accumulate_role(const KernelParams& p, SmemCtl* ctl, unsigned char* smem, unsigned tmem) {
     int* abort_flag = &ctl->abort_flag;
     constexpr unsigned kStageDesc = (2 * kTileBytes) >> 4, kTileDesc = kTileBytes >> 4;
@@ -449,29 +462,48 @@ __device__ __forceinline__ void accumulate_role(const KernelParams& p, SmemCtl* 
         if (!have_p && !mbar_wait(&ctl->p_full[buf], par, abort_flag)) { fail = 122; break; }
         tc_fence_after();
         const unsigned keep = (info & kInfoFirst) ? 0u : 1u;
-        unsigned y1 = ring0 + ((info >> kInfoStage) & 15u) * kStageDesc, skip_upper = 0u, skip_lower = (info & kInfoShared) ? ~0u : 0u;
+        // 16 tokens per MMA: 8 packed columns of A (the high halves, then the low halves), two 8-row groups of Y
+        if constexpr (kShare) {
+            unsigned y1 = ring0 + ((info >> kInfoStage) & 15u) * kStageDesc, skip_upper = 0u, skip_lower = (info & kInfoShared) ? ~0u : 0u;
 #pragma unroll 1
-        for (;;) {                                  // a shared step: the upper half's block, then the lower half's, each for its lanes
+            for (;;) {                                  // a shared step: the upper half's block, then the lower half's, each for its lanes
+                unsigned a = tmem + buf * kBufCols;
+                if (info & kInfoDkv) {
+                    const unsigned y2 = y1 + kTileDesc;
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk) {
+                        mma_ts_half(acc + 64, a + kk * 16, y2 + ((kk * 2048) >> 4), kIdescPV, kk > 0 ? 1u : keep, skip_upper, skip_lower);
+                        mma_ts_half(acc + 64, a + kk * 16 + 8, y2 + ((kk * 2048) >> 4), kIdescPV, 1u, skip_upper, skip_lower);
+                    }
+                    a += 64;
+                }
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                    mma_ts_half(acc, a + kk * 16, y1 + ((kk * 2048) >> 4), kIdescPV, kk > 0 ? 1u : keep, skip_upper, skip_lower);
+                    mma_ts_half(acc, a + kk * 16 + 8, y1 + ((kk * 2048) >> 4), kIdescPV, 1u, skip_upper, skip_lower);
+                }
+                if (!skip_lower) break;
+                y1 = ring0 + ((info >> (kInfoStage + 4)) & 15u) * kStageDesc;
+                skip_upper = ~0u;
+                skip_lower = 0u;
+            }
+        } else {
+            const unsigned y1 = ring0 + stg * kStageDesc;
             unsigned a = tmem + buf * kBufCols;
-            // 16 tokens per MMA: 8 packed columns of A (the high halves, then the low halves), two 8-row groups of Y
             if (info & kInfoDkv) {
                 const unsigned y2 = y1 + kTileDesc;
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {
-                    mma_ts_half(acc + 64, a + kk * 16, y2 + ((kk * 2048) >> 4), kIdescPV, kk > 0 ? 1u : keep, skip_upper, skip_lower);
-                    mma_ts_half(acc + 64, a + kk * 16 + 8, y2 + ((kk * 2048) >> 4), kIdescPV, 1u, skip_upper, skip_lower);
+                    mma_ts_lo(acc + 64, a + kk * 16, y2 + ((kk * 2048) >> 4), kIdescPV, kk > 0 ? 1u : keep);
+                    mma_ts_lo(acc + 64, a + kk * 16 + 8, y2 + ((kk * 2048) >> 4), kIdescPV, 1u);
                 }
                 a += 64;
             }
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
-                mma_ts_half(acc, a + kk * 16, y1 + ((kk * 2048) >> 4), kIdescPV, kk > 0 ? 1u : keep, skip_upper, skip_lower);
-                mma_ts_half(acc, a + kk * 16 + 8, y1 + ((kk * 2048) >> 4), kIdescPV, 1u, skip_upper, skip_lower);
+                mma_ts_lo(acc, a + kk * 16, y1 + ((kk * 2048) >> 4), kIdescPV, kk > 0 ? 1u : keep);
+                mma_ts_lo(acc, a + kk * 16 + 8, y1 + ((kk * 2048) >> 4), kIdescPV, 1u);
             }
-            if (!skip_lower) break;
-            y1 = ring0 + ((info >> (kInfoStage + 4)) & 15u) * kStageDesc;
-            skip_upper = ~0u;
-            skip_lower = 0u;
         }
         const unsigned now = info;
         unsigned long long* const done = &ctl->empty[stg];
@@ -570,6 +602,7 @@ __device__ __forceinline__ void dkv_columns(unsigned buf, float sl2, const float
 }
 
 // Like the issuing threads they walk the ring only: every third entry is theirs.
+template <bool kShare>
 __device__ __forceinline__ void elementwise_role(const KernelParams& p, SmemCtl* ctl, unsigned tmem, int warp, int lane) {
     int* abort_flag = &ctl->abort_flag;
     const unsigned g = (unsigned)warp >> 2;         // warpgroup = score buffer
@@ -586,7 +619,7 @@ __device__ __forceinline__ void elementwise_role(const KernelParams& p, SmemCtl*
         if (info & kInfoEnd) break;
         const bool dkv = info & kInfoDkv;
         const unsigned half = (info >> half_shift) & 7u;        // warp-uniform
-        const bool mine = half & kAttends, second = half & kSecond;
+        const bool mine = half & kAttends, second = kShare && (half & kSecond);
         float nl = 0.f, nd = 0.f;
         if (!dkv) {
             const unsigned xs = (info & kInfoX) ? 1u : 0u;
@@ -606,7 +639,7 @@ __device__ __forceinline__ void elementwise_role(const KernelParams& p, SmemCtl*
                 tmem_st32_zero(buf + 96);
             }
         } else if (dkv) {
-            const float2* st = reinterpret_cast<const float2*>(ctl->y_stats[(info >> (kInfoStage + (second ? 4 : 0))) & 15u]);
+            const float2* st = reinterpret_cast<const float2*>(ctl->y_stats[kShare ? (info >> (kInfoStage + (second ? 4 : 0))) & 15u : stage]);
             dkv_columns(buf, p.scale_log2, st, st + 32);
         } else {
             dq_columns(buf, p.scale_log2, nl, nd);
@@ -765,6 +798,7 @@ __device__ __forceinline__ void epilogue_role(const KernelParams& p, SmemCtl* ct
 }
 
 // ------------------------------------------------------------------------------------------------ the kernel
+template <bool kShare>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                       const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do,
@@ -800,16 +834,16 @@ attn_bwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
 
     if (warp < kWarpEpilogue) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsElem));
-        elementwise_role(p, ctl, tmem, warp, lane);
+        elementwise_role<kShare>(p, ctl, tmem, warp, lane);
     } else if (warp < kWarpScheduler) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsEpilogue));
         epilogue_role(p, ctl, smem, tmem, warp, lane, &tm_dq, &tm_dk, &tm_dv);
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLight));
-        if (warp == kWarpScheduler) scheduler_role(p, ctl, lane);
-        else if (warp == kWarpProducer) { if (elect_one()) producer_role(p, ctl, smem, &tm_q, &tm_k, &tm_v, &tm_do); }
-        else if (warp == kWarpScore) { if (elect_one()) score_role(p, ctl, smem, tmem); }
-        else if (elect_one()) accumulate_role(p, ctl, smem, tmem);
+        if (warp == kWarpScheduler) scheduler_role<kShare>(p, ctl, lane);
+        else if (warp == kWarpProducer) { if (elect_one()) producer_role<kShare>(p, ctl, smem, &tm_q, &tm_k, &tm_v, &tm_do); }
+        else if (warp == kWarpScore) { if (elect_one()) score_role<kShare>(p, ctl, smem, tmem); }
+        else if (elect_one()) accumulate_role<kShare>(p, ctl, smem, tmem);
     }
 
     // ------------------------------------------------------------------------------------------------ teardown
@@ -895,7 +929,8 @@ cudaError_t kernel_setup(int device, int* sm_count) {
     std::lock_guard<std::mutex> lock(g_bwd_mu);
     KernelDevice& d = g_bwd_dev[device];
     if (!d.ready) {
-        cudaError_t e = cudaFuncSetAttribute(attn_bwd_sm100_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+        cudaError_t e = cudaFuncSetAttribute(attn_bwd_sm100_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_bwd_sm100_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&d.sm_count, cudaDevAttrMultiProcessorCount, device);
         if (e != cudaSuccess) return e;
         d.ready = true;
@@ -984,7 +1019,12 @@ int launch_attn_bwd_sm100(const BwdArgs& a, const bigbird_layout& L, const Devic
                        (float*)ws, (unsigned long long*)(ws + off_bits), p.counter, (int)n_counters, (long long)rows, (int)a.N, a.H, row_ctas, (int)n_words);
     if (e == cudaSuccess) {
         ++*launches;
-        e = launch_chained(attn_bwd_sm100_kernel, (unsigned)std::min(sms, p.total_work), kThreads, kSmemBytes, a.stream, tm_q, tm_k, tm_v, tm_do, tm_dq, tm_dk, tm_dv, p);
+        // Shared steps where they make the sparse tiles' steps fewer by more than a fifth: what they cost every step (the places of Y are
+        // counted, three more ballots a list, more code) is more than they gain below.  Measured, a step for each block / shared, us:
+        // [8, 12, 4096] (28 % fewer) 483 / 474 under the power cap, [2, 12, 4096] 128.4 / 124.3, [4, 12, 4096] without random blocks, w = 1
+        // (25 %) 140 / 137, [3, 16, 1024] (21 %) 65.8 / 64.7; [8, 12, 4224] ETC (16 %) 334 / 346, [3, 16, 512] (none) 34.9 / 36.0.
+        const bool share = 5 * (L.tile_blocks - L.tile_steps_shared) > L.tile_blocks;
+        e = launch_chained(share ? attn_bwd_sm100_kernel<true> : attn_bwd_sm100_kernel<false>, (unsigned)std::min(sms, p.total_work), kThreads, kSmemBytes, a.stream, tm_q, tm_k, tm_v, tm_do, tm_dq, tm_dk, tm_dv, p);
         if (e == cudaSuccess) ++*launches;
     }
     const cudaError_t ef = cudaFreeAsync(ws, a.stream);

@@ -250,6 +250,15 @@ int build_layout_host(bigbird_layout* L) {
                 it.step_count = (int32_t)L->steps_t.size() - it.step_begin;
                 L->items_t.push_back(it);
             }
+        auto count = [&](const Item& it, const std::vector<Step>& steps) {
+            int64_t n[3] = {0, 0, 0};
+            for (int i = 0; i < it.step_count; ++i) ++n[steps[(size_t)it.step_begin + i].who];
+            L->tile_blocks += it.step_count;
+            L->tile_steps_shared += n[kBothHalves] + std::max(n[kUpperHalf], n[kLowerHalf]);
+        };
+        for (size_t i = 0; i < L->items_abs.size(); ++i)
+            if ((int)(i % L->items_per_head) >= n_gtiles) count(L->items_abs[i], L->steps);
+        for (const Item& it : L->items_t) count(it, L->steps_t);
     }
     return BIGBIRD_OK;
 }

@@ -74,6 +74,9 @@ struct bigbird_layout {
     std::vector<int32_t> block_order;
     std::vector<bigbird::Item> items_t;        // [H * sparse_tiles_per_head], step_begin absolute
     std::vector<bigbird::Step> steps_t;
+    // blocks in the lists of the sparse tiles of both kinds, and how many steps they are where a block of the upper half only and one of
+    // the lower half only share one (b == 64 only)
+    int64_t tile_blocks = 0, tile_steps_shared = 0;
     // device copies, made on first use
     mutable std::mutex mu;
     mutable bigbird::DeviceLayout dev;
