@@ -4,7 +4,7 @@
 // A CTA owns up to TM * TY rows of one block (TY = threads / 16 rows of threads, TM rows each) and walks the tokens of the
 // blocks in the rows' list, kc at a time, as one sequence: a chunk may begin in one block and end in the next, so block sizes
 // that are no multiple of the chunk waste nothing.  A thread's micro-tile is TM rows by kc / 16 tokens (scores) or by D / 16
-// columns (sums), which reads 12 to 14 shared-memory wavefronts per 64 to 96 FMAs of a warp.
+// columns (sums), which reads 12 to 15 shared-memory wavefronts per 64 to 112 FMAs of a warp.
 //
 // The tiles of global blocks have a list as long as the sequence.  The CTAs of a cluster share one such tile, each taking a
 // contiguous share of its chunks, and add up their results through distributed shared memory in the order of their ranks (no
@@ -88,7 +88,10 @@ __device__ __forceinline__ void mul2(f32x2& x, f32x2 a) { asm("mul.rn.f32x2 %0, 
 // acc[i][j] = sum_d a[i][d] b[16 j][d] over rows lda and ldb floats apart.  Even and odd d are summed apart and added at the end.
 // The loops of both products are bound by the latency of shared memory, so they are unrolled as far as it helps: [2, 12, 52 x 84, 64]
 // forward and gradients 2814 us with 4 rounds here and 2 in sum_tile, 2702 with 8 and 4, 2673 with 16 and 4, 2684 with 16 and 8;
-// [2, 8, 2560, 128] 308 with 4 and 2, 304.7 with 4 and 4, 301.5 with 8 and 8.
+// [2, 8, 2560, 128] 308 with 4 and 2, 304.7 with 4 and 4, 301.5 with 8 and 8.  That some instances spill a few registers outside of these
+// loops then (up to 200 bytes) costs less than it gains.  [2, 12, about 4096 tokens], 4 and 2 / as it is, forward and gradients: blocks
+// of 64 with D = 32 325 / 313 and 1040 / 1022, with D = 64 521 / 501 and 1713 / 1660, with D = 128 901 / 872 and 3465 / 3416; with D = 32
+// blocks of 16 111 / 107 and 353 / 342, of 96 428 / 420 and 1442 / 1420, of 169 787 / 772 and 2513 / 2468.
 template <int TM, int TN, int D>
 __device__ __forceinline__ void dot_tile(float (&acc)[TM][TN], const float* a, int lda, const float* b, int ldb) {
     f32x2 s[TM][TN];
@@ -231,28 +234,33 @@ struct Shape {
     int threads, grid;
 };
 // Two rows per thread where four would leave half of the GPU idle; else six where that covers a block with no more padding than four would
-// (the larger micro-tile reads less shared memory per FMA); seven where that pads no more than six: its CTAs have at most 192 threads,
-// so that a thread has 168 registers, and two CTAs of 192 fill the four sub-partitions evenly (84 rows: six warps instead of seven;
-// [2, 12, 52 x 84, 64] forward and gradients 2880 -> 2814 us).  Four for D = 128, whose sums take twice the registers.
+// (the larger micro-tile reads less shared memory per FMA).  Seven where that pads no more than six and gives a CTA all of its twelve
+// rows of threads: at most 192 threads have 168 registers each, and two CTAs of six warps fill the four sub-partitions evenly (84 rows:
+// six warps instead of seven).  With fewer warps it is the slower one: [2, 12, about 4096 tokens, 64], six / seven rows per thread,
+// forward and gradients in us: blocks of 84 688 / 679 and 2320 / 2297, of 160 1202 / 1180 and 3926 / 3850, of 70 (five warps) 595 / 674 and 2028 /
+// 2269, of 140 1080 / 1219 and 3593 / 3992, of 200 1505 / 1662 and 5095 / 5697, of 42 (three) 424 / 420 and 1395 / 1584.  Four for D = 128,
+// whose sums take twice the registers.
 constexpr int max_threads(int tm) { return tm == 7 ? 192 : 256; }
-inline int padded_rows(int tm, int b) {
-    const int cap = max_threads(tm) / 16 * tm, tiles = (b + cap - 1) / cap, rows = (b + tiles - 1) / tiles;
-    return tiles * std::max(2, ((rows + tm - 1) / tm + 1) / 2 * 2) * tm;
+inline int row_tiles(int tm, int b) { return (b + max_threads(tm) / 16 * tm - 1) / (max_threads(tm) / 16 * tm); }
+// Rows of threads of a CTA: an even number, so that a warp has two.
+inline int thread_rows(int tm, int b) {
+    const int tiles = row_tiles(tm, b), rows = (b + tiles - 1) / tiles;
+    return std::max(2, ((rows + tm - 1) / tm + 1) / 2 * 2);
 }
+inline int padded_rows(int tm, int b) { return row_tiles(tm, b) * thread_rows(tm, b) * tm; }
 inline int rows_per_thread(const bigbird_layout& L, int BH, int D, int slots) {
     if (2 * (int64_t)BH * L.nb * ((L.b + 63) / 64) <= slots) return 2;
     if (D > 64 || padded_rows(6, L.b) > padded_rows(4, L.b)) return 4;
-    return padded_rows(7, L.b) <= padded_rows(6, L.b) ? 7 : 6;
+    return padded_rows(7, L.b) <= padded_rows(6, L.b) && thread_rows(7, L.b) == max_threads(7) / 16 ? 7 : 6;
 }
 
 // tm: rows per thread; kc: tokens per chunk; slots: CTAs that fit the GPU at a time.
 inline Shape make_shape(int tm, const bigbird_layout& L, const DeviceLayout& dl, int BH, int slots, int kc) {
     Shape s{};
     const int b = L.b, nb = L.nb;
-    const int cap = max_threads(tm) / 16 * tm;
-    s.t.tiles = (b + cap - 1) / cap;
+    s.t.tiles = row_tiles(tm, b);
     s.t.rows = (b + s.t.tiles - 1) / s.t.tiles;
-    s.threads = 16 * std::max(2, ((s.t.rows + tm - 1) / tm + 1) / 2 * 2);
+    s.threads = 16 * thread_rows(tm, b);
     s.t.BH = BH;
     s.t.H = L.H;
     s.t.nb = nb;
