@@ -10,9 +10,9 @@ import paper_2007_14062_b200 as bb
 pytestmark = pytest.mark.gpu
 
 
-# 71, 83, 84: one tile of 12 rows of threads with seven rows each, full and with rows to spare; 85: just too many for it; 167, 168: two
-# such tiles; 96: six rows per thread; 64: four; 5: a tile of one warp
-@pytest.mark.parametrize("b", [5, 64, 71, 83, 84, 85, 96, 167, 168])
+# Rows per thread: four for 5 (a tile of one warp), 64 and 130; six for 42 (three warps), 65, 70, 71, 85, 96 and 140; seven for 83 and 84 (a tile
+# of twelve rows of threads, with a row to spare and full), 160, 167 and 168 (two such tiles).
+@pytest.mark.parametrize("b", [5, 42, 64, 65, 70, 71, 83, 84, 85, 96, 130, 140, 160, 167, 168])
 @pytest.mark.parametrize("D", [32, 64])
 def test_fp32_forward_and_gradients(b, D):
     B, H, nb = 2, 12, 24
