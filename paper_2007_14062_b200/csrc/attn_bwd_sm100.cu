@@ -297,13 +297,16 @@ __device__ __forceinline__ void producer_role(const KernelParams& p, SmemCtl* ct
     int fail = 0;
     // room for a step of `blocks` blocks
     auto room = [&](unsigned blocks) -> bool {
-        if constexpr (!kShare) return mbar_wait(&ctl->empty[step_n % kRing], ((step_n / kRing) & 1u) ^ 1u, abort_flag);
-        while (free_stages < blocks || step_n - done_n == (unsigned)kRing) {
-            if (!mbar_wait(&ctl->empty[done_n % kRing], (done_n / kRing) & 1u, abort_flag)) return false;
-            free_stages += 1u + ((shared_steps >> (done_n & 31u)) & 1u);
-            ++done_n;
+        if constexpr (kShare) {
+            while (free_stages < blocks || step_n - done_n == (unsigned)kRing) {
+                if (!mbar_wait(&ctl->empty[done_n % kRing], (done_n / kRing) & 1u, abort_flag)) return false;
+                free_stages += 1u + ((shared_steps >> (done_n & 31u)) & 1u);
+                ++done_n;
+            }
+            return true;
+        } else {
+            return mbar_wait(&ctl->empty[step_n % kRing], ((step_n / kRing) & 1u) ^ 1u, abort_flag);
         }
-        return true;
     };
     for (;;) {
         const unsigned ss = slot_n % kSlots;

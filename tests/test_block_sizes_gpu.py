@@ -10,8 +10,8 @@ import paper_2007_14062_b200 as bb
 pytestmark = pytest.mark.gpu
 
 
-# Rows per thread: four for 5 (a tile of one warp), 64 and 130; six for 42 (three warps), 65, 70, 71, 85, 96 and 140; seven for 83 and 84 (a tile
-# of twelve rows of threads, with a row to spare and full), 160, 167 and 168 (two such tiles).
+# Rows per thread: four for 5 (a tile of one warp) and 64; six for 42, 65, 70, 71, 85, 96, 130 and 140; seven for 83 and 84 (a tile of twelve
+# rows of threads, with a row to spare and full), 160, 167 and 168 (two such tiles).
 @pytest.mark.parametrize("b", [5, 42, 64, 65, 70, 71, 83, 84, 85, 96, 130, 140, 160, 167, 168])
 @pytest.mark.parametrize("D", [32, 64])
 def test_fp32_forward_and_gradients(b, D):
