@@ -36,8 +36,8 @@ NOMINAL_BF16_TFLOPS = 2250.0
 FALLBACK_PEAKS = {"bf16_tflops": 1590.0, "hbm_gbs": 6650.0}
 # dram__bytes_read.sum + dram__bytes_write.sum of one attn_fwd_sm100_kernel launch on this workload, from the
 # ncu capture summarised in profiles/ (None until a capture exists for the current kernel).
-NCU_DRAM_BYTES_PER_LAUNCH = {"c2_base_itc_bf16": 241.7e6}
-NCU_DRAM_BYTES_PER_BACKWARD_LAUNCH = {"c2_base_itc_bf16": 529.4e6}     # the same of attn_bwd_sm100_kernel
+NCU_DRAM_BYTES_PER_LAUNCH = {"c2_base_itc_bf16": 241.5e6}
+NCU_DRAM_BYTES_PER_BACKWARD_LAUNCH = {"c2_base_itc_bf16": 528.7e6}     # the same of attn_bwd_sm100_kernel
 
 
 def measured_peaks():

@@ -10,8 +10,8 @@
 // Both kinds of scores are register-tiled products over shared memory, and so are the sums, with P or dS passing through shared
 // memory between the 16 threads that share a row.  See simt.cuh for the tile shapes and for how clusters share the long tiles.
 // Padded query rows get dq = 0 and give nothing to dk, dv; padded keys get dk = dv = 0.
-// Bound by the FMA pipes (three products per pair of tokens by query, four by key).  Measured (four lanes per row with two
-// exchanges per score before): [2, 12, 52 x 84, 64] with three global blocks 12.16 -> 2.22 ms.
+// Bound by shared-memory latency and the FMA pipes (three products per pair of tokens by query, four by key).  Measured (four lanes per
+// row with two exchanges per score before): [2, 12, 52 x 84, 64] with three global blocks 12.16 -> 2.04 ms.
 #include "simt.cuh"
 
 namespace bigbird {

@@ -32,12 +32,12 @@
 // the same from one elected thread 557, columns 16 at a time with the next 16 on their way 527, two issuing threads 505, all
 // roles on the ring, tests ahead of the commits and rows written by TMA 497 us ([1, 12, 16384, 64] with 13000 valid tokens
 // 338 -> 193 us from the second of these to the last), and 189 with the parts of a cut tile fetched together ([2, 12, 1024]
-// 54 -> 39.5 us, there no longer cut); 430 us at full clocks.  A step took 1400 cycles then; its MMAs need 640 of the tensor pipe
-// (51% of the launch by its counter, 555 steps per SM), without any elementwise work it takes 1100, without any MMAs 1150: what is
+// 54 -> 39.5 us, there no longer cut, 40.1 now); 430 us at full clocks.  A step took 1400 cycles then; its MMAs need 640 of the tensor pipe
+// (51% of the launch by its counter then, 52% now; 555 steps per SM), without any elementwise work it takes 1100, without any MMAs 1150: what is
 // left is the way of a step through the hands of four warps with three steps in flight, which is all that tensor memory holds.  Two
 // threads per row (24 warps) were no faster.
 //
-// With shared steps [8, 12, 4096] takes 419 us at full clocks (430 with a step for each block) and forward and gradients together 628
+// With shared steps [8, 12, 4096] takes 417.5 us at full clocks (430 with a step for each block) and forward and gradients together 628
 // instead of 646 under the power cap; the launch says which layouts gain.  A shared step takes two of the seven places in the ring of Y.  (Nine of them, for which a tile's
 // results left through its own row buffer, were no faster there, and the tile after next waited for that buffer: [8, 12, 4224] ETC 359 us
 // against 345 under the power cap, [1, 2, 384] 13.5 against 13.35.)
@@ -976,10 +976,11 @@ int launch_attn_bwd_sm100(const BwdArgs& a, const bigbird_layout& L, const Devic
     // Tiles of global blocks have nb steps where the others have about ten: cut them into parts of about a third of what each
     // SM gets altogether, so that none of them is still running when the rest is done, but no more than one for every 16 steps
     // (rounded up: parts of 11 steps or more), and not at all up to 32 steps: adding the parts up takes about 5 us on the path of
-    // the last one (it was 24 when a thread fetched one value after the other), and at 32 steps that is more than a cut gains with
-    // few heads, less with many.  Measured, gradients of B, 12 heads, nb blocks in us: [2, nb 16] 39.5 uncut, 43.7 in two, 52 in four;
-    // [1, 32] 56.9 uncut, 54.6 in two; four heads [1, 32] 34.6, 38.2; [1, 64] 93.7 uncut, 79.7 in two, 74.6 in three, 75.2 in
-    // four, 78.5 in eight; [1, 256] 200 uncut, 190 in two, 191 in three; [3, 16 heads, 96] 212 uncut, 221 in two.
+    // the last one (it was 24 when a thread fetched one value after the other), and up to 32 steps that is more than a cut gains.
+    // Measured, gradients of B, 12 heads, nb blocks in us: [2, nb 16] 39.7 uncut, 48.2 in two, 52.5 in four; [1, 32] 41.5 uncut, 45.6 in
+    // two; four heads [1, 32] 33.6, 34.7; [1, 64] 68.0 uncut, 70.0 in two, 69.6 in three, 70.4 in four, 73.2 in eight; [1, 256] 255 uncut,
+    // 232 in two, 231 in three; [3, 16 heads, 96] 345 uncut, 356 in two (the last two under the power cap).  (With three tiles drawn ahead
+    // whatever the launch [1, 64] was 93.7 uncut and 74.6 in three, since a CTA with a whole global tile had two more tiles to do.)
     const int64_t steps = (int64_t)a.B * ((int64_t)L.steps.size() + (int64_t)L.steps_t.size() + (int64_t)a.H * L.global_tiles * a.nb);
     const int64_t want = std::max<int64_t>(16, steps / (3 * sms));
     const int want_parts = a.nb <= 32 ? 1 : (int)((a.nb + want - 1) / want);

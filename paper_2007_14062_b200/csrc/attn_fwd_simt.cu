@@ -6,7 +6,7 @@
 // The next chunk's K is on its way while the probabilities and sums are made; its V is requested when the sums are done, and both
 // are waited for at the top of the chunk.  See simt.cuh for the tile shapes and for how clusters share the long tiles.
 // Bound by shared-memory latency and the FMA pipes.  Measured (a warp per row before, no reuse of K and V in registers): [2, 12, 52 x 84,
-// 64] with three global blocks 3740 -> 655 us, [2, 8, 2560, 128] padded 1547 -> 302 us, [1, 2, 512, 64] 22.6 -> 13.8 us (18.5 with four rows per
+// 64] with three global blocks 3740 -> 640 us, [2, 8, 2560, 128] padded 1547 -> 300 us, [1, 2, 512, 64] 22.6 -> 13.8 us (18.5 with four rows per
 // thread and launches that wait for the kernel in front to drain).
 #include "simt.cuh"
 
